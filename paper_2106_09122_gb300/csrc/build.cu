@@ -588,8 +588,11 @@ cudaError_t psfsim_launch_build(psfsim_plan *h, cudaStream_t st) {
     // the whole quadrant, an upper bound, before the count was known).
     if (h->storage == PSFSIM_SPLIT_BF16_SYM) h->ld = psfsim_round_up(kv > 0 ? kv : 1, 64);
   }
-  if (h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16 || h->storage == PSFSIM_SPLIT_BF16_SYM)
-    return psfsim_launch_split_build(h, st);
+  psfsim_live_count(h);
+  if (h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16 || h->storage == PSFSIM_SPLIT_BF16_SYM) {
+    if ((e = psfsim_launch_split_build(h, st)) != cudaSuccess) return e;
+    return psfsim_launch_live_table(h, st);
+  }
   if (h->storage != PSFSIM_FP32 && h->storage != PSFSIM_FP32_SYM) return cudaErrorNotSupported;
   const bool compact = h->storage == PSFSIM_FP32_SYM;
 

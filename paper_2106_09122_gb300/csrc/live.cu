@@ -1,0 +1,140 @@
+// Tables of the live columns of a dense plan on a scene grid (live.cuh), in
+// the column-order part of the workspace, which nothing reads after the build:
+//   split storage   ktab[k_tiles]: first column (a multiple of 32) of every
+//                   64-column k-tile that holds a live column, then
+//                   dead[dead_groups]: the 32-column groups in no k-tile.
+// What that is worth depends on the grid: the wave of 50 scenes on ten split
+// plans (64..256 pixels a side, 12 lambda/D of PSFs in fields of 19 to 128)
+// streams 26 % of its k-tiles, 2680 -> 852 us; tiles start at multiples of 32
+// columns rather than 64 so that a narrow row needs one tile where it used to
+// touch two, and 32 columns are the 64 bytes that HBM moves at least.
+// The host counts the same tables by the same integer arithmetic, to size
+// launches without reading anything back.
+#include "live.cuh"
+#include "psfsim_internal.cuh"
+
+namespace {
+
+// Exclusive block scans over 1024 threads (max and sum), with the block total.
+__device__ __forceinline__ int scan_max(int v, int *sh, int &total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v = max(v, u);
+  }
+  if (lane == 31) sh[warp] = v;
+  __syncthreads();
+  int pre = -1;
+  total = -1;
+  for (int w = 0; w < 32; ++w) {
+    if (w < warp) pre = max(pre, sh[w]);
+    total = max(total, sh[w]);
+  }
+  __syncthreads();
+  return max(v, pre);  // inclusive
+}
+
+__device__ __forceinline__ int scan_sum(int v, int *sh, int &total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int x = v;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += u;
+  }
+  if (lane == 31) sh[warp] = x;
+  __syncthreads();
+  int pre = 0;
+  total = 0;
+  for (int w = 0; w < 32; ++w) {
+    if (w < warp) pre += sh[w];
+    total += sh[w];
+  }
+  __syncthreads();
+  return pre + x - v;  // exclusive
+}
+
+__device__ __forceinline__ bool group_live(int N, int64_t K, long long R2, int64_t g, int64_t groups) {
+  if (g < 0 || g >= groups) return false;
+  if (g == 0) {
+    if (R2 < (N & 1 ? 0 : 2)) return true;  // no live pixel at all: keep one tile
+  }
+  for (int64_t j = g * kLiveGroup; j < (g + 1) * kLiveGroup && j < K; ++j) {
+    const long long X = 2 * (j % N) - (N - 1), Y = 2 * (j / N) - (N - 1);
+    if (X * X + Y * Y <= R2) return true;
+  }
+  return false;
+}
+
+// One CTA walks the groups, 1024 at a time.  Within a run of live groups every
+// second one starts a k-tile; the group after a run of odd length falls inside
+// the run's last tile.
+__global__ void __launch_bounds__(1024) ktile_table_kernel(int N, int64_t K, long long R2, int *ktab, int k_tiles,
+                                                           int *dead, int64_t dead_groups) {
+  __shared__ int sh[32];
+  const int64_t groups = (K + kLiveGroup - 1) / kLiveGroup;
+  int run_carry = -1, tile_carry = 0, dead_carry = 0;
+  for (int64_t base = 0; base < groups; base += blockDim.x) {
+    const int64_t g = base + threadIdx.x;
+    const bool live = group_live(N, K, R2, g, groups), before = group_live(N, K, R2, g - 1, groups);
+    int total;
+    const int start = max(run_carry, scan_max(live && !before ? (int)g : -1, sh, total));  // of g's, or the last, run
+    run_carry = max(run_carry, total);
+    const bool tile = live && (((int)g - start) & 1) == 0;
+    const bool covered = live || (before && (((int)g - 1 - start) & 1) == 0);
+    const int t = tile_carry + scan_sum(tile ? 1 : 0, sh, total);
+    if (tile && t < k_tiles) ktab[t] = (int)(g * kLiveGroup);
+    tile_carry += total;
+    const int d = dead_carry + scan_sum(g < groups && !covered ? 1 : 0, sh, total);
+    if (g < groups && !covered && d < dead_groups) dead[d] = (int)g;
+    dead_carry += total;
+  }
+}
+
+}  // namespace
+
+void psfsim_live_count(psfsim_plan *h) {
+  const bool split = h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16;
+  h->live = false;
+  h->k_tiles = (int)(h->ld / 64);
+  h->dead_groups = 0;
+  if (h->N < 1 || h->quadrant || !split) return;
+  const long long R2 = live_r2(h->radii[h->n_r - 1], h->S);
+  const int64_t groups = (h->K + kLiveGroup - 1) / kLiveGroup;
+  int64_t tiles = 0, covered = 0, run0 = -1, run1 = -1;  // current run of live groups [run0, run1)
+  auto close = [&] {
+    if (run0 < 0) return;
+    const int64_t t = (run1 - run0 + 1) / 2, end = run0 + 2 * t;
+    tiles += t;
+    covered += (end < groups ? end : groups) - run0;
+  };
+  for (int iy = 0; iy < h->N; ++iy) {
+    int a, b;
+    live_row(h->N, R2, iy, a, b);
+    if (a == b) continue;
+    const int64_t g0 = ((int64_t)iy * h->N + a) / kLiveGroup, g1 = ((int64_t)iy * h->N + b - 1) / kLiveGroup + 1;
+    if (run0 >= 0 && g0 <= run1) {
+      run1 = g1;
+      continue;
+    }
+    close();
+    run0 = g0;
+    run1 = g1;
+  }
+  if (run0 < 0) {
+    run0 = 0;
+    run1 = 1;
+  }
+  close();
+  if (covered >= groups) return;  // nothing to skip
+  h->live = true;
+  h->k_tiles = (int)tiles;
+  h->dead_groups = groups - covered;
+}
+
+cudaError_t psfsim_launch_live_table(psfsim_plan *h, cudaStream_t st) {
+  if (!h->live) return cudaSuccess;
+  int *tab = reinterpret_cast<int *>(h->ws + h->order_off);
+  ktile_table_kernel<<<1, 1024, 0, st>>>(h->N, h->K, live_r2(h->radii[h->n_r - 1], h->S), tab, h->k_tiles,
+                                         tab + h->k_tiles, h->dead_groups);
+  return cudaGetLastError();
+}

@@ -41,6 +41,9 @@ struct psfsim_plan {
   int64_t a_off, lo_off, scale_off, geom_off, order_off, bstart_off, pts_off, status_off, libmax_off, plib_off,
       cols_off, mtorder_off;
   int device, num_sms;
+  bool live;            // products skip the zero columns listed in the workspace (live.cu)
+  int k_tiles;          // split storage: 64-column k-tiles the products read (ld / 64 when !live)
+  int64_t dead_groups;  // split storage: 32-column groups in none of them
   int fit_ks;           // column splits of the fit-gradient forward, fixed at first use (0: not yet)
   CUtensorMap lib_map;  // 3D tensor map over the library for TMA staging
 };
@@ -61,6 +64,11 @@ int64_t psfsim_fused_columns_bytes(int64_t K);
 // ... and its M-tile order (the image's 8 x 16 pixel tiles, nearest the centre first).
 int64_t psfsim_fused_mtile_order_bytes(int n);
 cudaError_t psfsim_launch_pair_library(psfsim_plan *h, cudaStream_t st);
+
+// Live (not identically zero) columns of a dense plan on a scene grid: counted
+// on the host, listed in the workspace by the build (live.cu).
+void psfsim_live_count(psfsim_plan *h);
+cudaError_t psfsim_launch_live_table(psfsim_plan *h, cudaStream_t st);
 
 // Kernel launchers (return cudaError_t of the launch).
 cudaError_t psfsim_launch_build(psfsim_plan *h, cudaStream_t st);

@@ -12,6 +12,10 @@
 // D[:, 0:2Bp] += hi * [x1 x2]^T, so the result carries the 2^-8 relative
 // storage error of hi and the dropped hi * x3 term (< 2^-16 relative).
 //
+// Dense plans on a scene grid are mostly zero columns (beyond the last library
+// radius): only the 64-column k-tiles that hold a live column are loaded
+// (live.cu; TMA starts them at multiples of 32 columns).
+//
 // Persistent warp-specialised kernel, one CTA per SM:
 //   warp 0  TMA producer (2D tiled loads, 128-byte swizzle) into a smem ring
 //   warp 1  MMA issuer (tcgen05.mma, accumulators in TMEM, double-buffered)
@@ -24,6 +28,7 @@
 
 #include <cstring>
 
+#include "live.cuh"
 #include "psfsim_internal.cuh"
 #include "ptx_util.cuh"
 
@@ -53,6 +58,7 @@ struct TcJob {
   int xparts;          // bf16 parts of x in the B operand: 3 (split-BF16) or 2 (BF16)
   int unit_begin;      // first work unit of this job
   int cap;             // scenes in the job's buffers (<= Bp)
+  const int *ktab;     // first column of every k-tile (NULL: k-tile t starts at column 64 t)
   const int *count;    // device int: scenes present (NULL: all cap)
   float *part;         // [KS][cap][rows]
 };
@@ -71,14 +77,27 @@ struct TcMulti {
   int64_t stall_it;  // test hook: the producer never issues this load (-1: none)
 };
 
+// xs[part][b][t]: the three bf16 parts of scene b at the t-th column that the
+// k-tiles cover, times the column's scale (width = 64 k-tiles columns).  The
+// columns in no k-tile are zero in A; a non-finite scene value there still
+// makes the whole image NaN (0 x inf), as it does when they are multiplied
+// out: position t adds 0 x for its share of them.
 __global__ void xsplit_kernel(const float *__restrict__ x, int B, const int *__restrict__ count, int Bp, int64_t K,
-                              int64_t ld, const float *__restrict__ scale, __nv_bfloat16 *__restrict__ xs) {
-  const int64_t total = (int64_t)Bp * ld;
+                              int64_t width, const int *__restrict__ ktab, int64_t dead_groups,
+                              const float *__restrict__ scale, __nv_bfloat16 *__restrict__ xs) {
+  const int64_t total = (int64_t)Bp * width;
   const int nb = count ? min(*count, B) : B;
+  const int *dead = ktab + width / BK;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(t / ld);
-    const int64_t j = t % ld;
-    const float v = (b < nb && j < K) ? x[(int64_t)b * K + j] * scale[j] : 0.f;
+    const int b = (int)(t / width);
+    const int64_t c = t % width;
+    const int64_t j = ktab ? ktab[c / BK] + c % BK : c;
+    float v = (b < nb && j < K) ? x[(int64_t)b * K + j] * scale[j] : 0.f;
+    if (b < nb)
+      for (int64_t e = c; e < dead_groups * kLiveGroup; e += width) {
+        const int64_t jd = (int64_t)dead[e / kLiveGroup] * kLiveGroup + e % kLiveGroup;
+        if (jd < K) v += 0.f * x[(int64_t)b * K + jd];
+      }
     const __nv_bfloat16 x1 = __float2bfloat16_rn(v);
     const float r1 = v - __bfloat162float(x1);
     const __nv_bfloat16 x2 = __float2bfloat16_rn(r1);
@@ -158,7 +177,11 @@ __global__ void __launch_bounds__(kThreads, 2) tc_gemm_kernel(const __grid_const
       const TcJob &J = P.job[jb];
       const int ks = lu / J.m_tiles, mt = lu % J.m_tiles;
       const uint32_t tx = (J.has_lo ? 2 : 1) * kTileBytes + (uint32_t)(J.xparts * J.Bp) * BK * 2;
-      for (int kt = k_begin(J, ks); kt < k_begin(J, ks + 1); ++kt, ++it) {
+      const int k0 = k_begin(J, ks), k1 = k_begin(J, ks + 1);
+      int next = J.ktab ? __ldg(J.ktab + k0) : 0;  // read one k-tile ahead of its use
+      for (int kt = k0; kt < k1; ++kt, ++it) {
+        const int col = J.ktab ? next : kt * BK;
+        if (J.ktab && kt + 1 < k1) next = __ldg(J.ktab + kt + 1);
         const int s = (int)(it % P.stages);
         if (!ptx::mbar_wait_bounded(&empty_bar[s], ((it / P.stages) & 1) ^ 1, lim)) {
           set_abort(&abort_flag, P.status);
@@ -168,8 +191,8 @@ __global__ void __launch_bounds__(kThreads, 2) tc_gemm_kernel(const __grid_const
         if ((int64_t)it == P.stall_it) continue;  // test hook: this stage is never filled
         uint8_t *st = smem + (size_t)s * P.stage_bytes;
         ptx::mbar_arrive_expect_tx(&full_bar[s], tx);
-        ptx::tma_load_2d(st, &P.map[jb][0], kt * BK, mt * BM, &full_bar[s]);
-        if (J.has_lo) ptx::tma_load_2d(st + kTileBytes, &P.map[jb][1], kt * BK, mt * BM, &full_bar[s]);
+        ptx::tma_load_2d(st, &P.map[jb][0], col, mt * BM, &full_bar[s]);
+        if (J.has_lo) ptx::tma_load_2d(st + kTileBytes, &P.map[jb][1], col, mt * BM, &full_bar[s]);
         ptx::tma_load_2d(st + P.x_off, &P.map[jb][2], kt * BK, 0, &full_bar[s]);
       }
     }
@@ -392,7 +415,7 @@ MultiPlan plan_multi(const JobSpec *jobs, int nj, const psfsim_tuning_t *tune) {
     p.Bp = (int)psfsim_round_up(jobs[j].cap, 16);
     p.rows = psfsim_round_up(h->M, BM);
     p.m_tiles = (int)(p.rows / BM);
-    p.k_tiles = (int)(h->ld / BK);
+    p.k_tiles = h->k_tiles;
     total += (int64_t)p.m_tiles * p.k_tiles;
   }
   const int64_t target_units = (int64_t)(ups ? ups : 4) * num_sms;
@@ -413,7 +436,7 @@ MultiPlan plan_multi(const JobSpec *jobs, int nj, const psfsim_tuning_t *tune) {
     Bp_max = p.Bp > Bp_max ? p.Bp : Bp_max;
     const psfsim_plan *h = jobs[j].h;
     p.xs_off = off;
-    off += (size_t)psfsim_round_up(3ll * p.Bp * h->ld * 2, 256);
+    off += (size_t)psfsim_round_up(3ll * p.Bp * p.k_tiles * BK * 2, 256);
     p.part_off = off;
     off += (size_t)psfsim_round_up((int64_t)p.KS * jobs[j].cap * p.rows * 4, 256);
   }
@@ -469,14 +492,14 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
     const JobPlan &p = mp.jp[j];
     __nv_bfloat16 *xs = reinterpret_cast<__nv_bfloat16 *>(base + p.xs_off);
     const float *scale = reinterpret_cast<const float *>(h->ws + h->scale_off);
-    xsplit_kernel<<<h->num_sms * 4, 256, 0, st>>>(jobs[j].x, jobs[j].cap, jobs[j].count, p.Bp, psfsim_cols(h), h->ld,
-                                                  scale,
-                                                  xs);
+    const int *ktab = h->live ? reinterpret_cast<const int *>(h->ws + h->order_off) : nullptr;
+    xsplit_kernel<<<h->num_sms * 4, 256, 0, st>>>(jobs[j].x, jobs[j].cap, jobs[j].count, p.Bp, psfsim_cols(h),
+                                                  (int64_t)p.k_tiles * BK, ktab, h->dead_groups, scale, xs);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const bool has_lo = h->lo_off >= 0;
     if (!encode_bf16_2d(&P.map[j][0], h->ws + h->a_off, (uint64_t)h->ld, (uint64_t)p.rows, BK, BM) ||
         (has_lo && !encode_bf16_2d(&P.map[j][1], h->ws + h->lo_off, (uint64_t)h->ld, (uint64_t)p.rows, BK, BM)) ||
-        !encode_bf16_2d(&P.map[j][2], xs, (uint64_t)h->ld, (uint64_t)(3 * p.Bp), BK,
+        !encode_bf16_2d(&P.map[j][2], xs, (uint64_t)p.k_tiles * BK, (uint64_t)(3 * p.Bp), BK,
                         (uint32_t)((has_lo ? 3 : 2) * p.Bp)))
       return cudaErrorInvalidValue;
     TcJob &J = P.job[j];
@@ -490,6 +513,7 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
     J.k_tiles = p.k_tiles;
     J.unit_begin = j == 0 ? 0 : P.job[j - 1].unit_begin + P.job[j - 1].m_tiles * P.job[j - 1].KS;
     J.cap = jobs[j].cap;
+    J.ktab = ktab;
     J.count = jobs[j].count;
     J.part = reinterpret_cast<float *>(base + p.part_off);
   }

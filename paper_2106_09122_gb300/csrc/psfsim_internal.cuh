@@ -90,6 +90,18 @@ cudaError_t psfsim_launch_split_build(psfsim_plan *h, cudaStream_t st);
 size_t psfsim_forward_tc_scratch(const psfsim_plan *h, int B);
 cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
                                      cudaStream_t st);
+cudaError_t psfsim_launch_forward_tc_sym(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
+                                         cudaStream_t st);
+// Images from the partial images of rotated scenes (sym.cu): rotated scene
+// q = 4 b + m is slot q % per of block q / per, whose partials are
+// part[KS][cap][rows]; y[b][i] = sum_m sum_ks part at P^-m(i).
+struct SymSum {
+  const float *part[16];
+  int cap[16], KS[16];
+  int per, n;
+  int64_t rows;
+};
+cudaError_t psfsim_launch_sym_sum(const SymSum &S, int B, float *y, cudaStream_t st);
 size_t psfsim_adjoint_split_scratch(const psfsim_plan *h, int B);
 // Test hook: the tensor-core forward of <= 80 scenes on one CTA with every
 // wait bounded by wait_ns and load number stall_it never issued.

@@ -66,6 +66,52 @@ __global__ void sym_permsum(const float *__restrict__ v, int B, int n, float *__
   }
 }
 
+// y[b][i] = sum_m sum_ks part_m[ks][P^-m(i)] (fixed order), one 32 x 32 pixel
+// block of an image per CTA: the quarter and three-quarter turns are read along
+// their own rows and transposed through shared memory, so every access is a run
+// of 32 pixels, and k-splits and rotations are added in one pass over the
+// partial images.  Bound by reading them; a thread has the 8 loads of its two
+// pixels in flight (one pixel of 1024 threads and two dependent rounds of
+// loads: 58 us for 256 rotated images of 256 x 256, 39 now; a copy per job
+// and a gather through the permutations took 154).
+constexpr int kSumThreads = 512;
+__global__ void __launch_bounds__(kSumThreads) sym_sum_kernel(const __grid_constant__ SymSum S, float *__restrict__ y) {
+  __shared__ float t1[32][33], t3[32][33];
+  constexpr int kRows = kSumThreads / 32, kPer = 32 / kRows;
+  const int n = S.n, b = blockIdx.z;
+  const int P0 = blockIdx.y * 32, Q0 = blockIdx.x * 32;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int blk = 4 * b / S.per, slot = 4 * b % S.per;  // a scene's four rotations share a block
+  const int64_t step = (int64_t)S.cap[blk] * S.rows;
+  const float *v = S.part[blk] + (int64_t)slot * S.rows;
+  float acc[kPer][4] = {};
+  for (int ks = 0; ks < S.KS[blk]; ++ks, v += step) {
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+      const int r = ty + e * kRows;
+      if (Q0 + r < n && P0 + tx < n) {  // P^-1(p, q) = (n-1-q, p), P^-3(p, q) = (q, n-1-p)
+        acc[e][1] += v[S.rows + (int64_t)(n - 1 - Q0 - r) * n + P0 + tx];
+        acc[e][3] += v[3 * S.rows + (int64_t)(Q0 + r) * n + n - 1 - P0 - tx];
+      }
+      if (P0 + r < n && Q0 + tx < n) {
+        acc[e][0] += v[(int64_t)(P0 + r) * n + Q0 + tx];
+        acc[e][2] += v[2 * S.rows + (int64_t)(n - 1 - P0 - r) * n + n - 1 - Q0 - tx];
+      }
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < kPer; ++e) {
+    t1[ty + e * kRows][tx] = acc[e][1];
+    t3[ty + e * kRows][tx] = acc[e][3];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < kPer; ++e) {
+    const int r = ty + e * kRows, p = P0 + r, q = Q0 + tx;
+    if (p < n && q < n) y[((int64_t)b * n + p) * n + q] = ((acc[e][0] + t1[tx][r]) + acc[e][2]) + t3[tx][r];
+  }
+}
+
 // gp[(b*4 + m) * M + i] = g[b][P^m(i)]
 __global__ void sym_gperm(const float *__restrict__ g, int B, int n, float *__restrict__ gp) {
   const int64_t M = (int64_t)n * n;
@@ -109,6 +155,12 @@ int sym_splits(const psfsim_plan *h) {
 }
 
 }  // namespace
+
+cudaError_t psfsim_launch_sym_sum(const SymSum &S, int B, float *y, cudaStream_t st) {
+  const unsigned t = (unsigned)((S.n + 31) / 32);
+  sym_sum_kernel<<<dim3(t, t, (unsigned)B), kSumThreads, 0, st>>>(S, y);
+  return cudaGetLastError();
+}
 
 size_t psfsim_forward_sym_scratch(const psfsim_plan *h, int B) {
   const size_t xc = (size_t)psfsim_round_up((int64_t)4 * B * h->K_valid * 4, 256);
@@ -156,31 +208,18 @@ cudaError_t psfsim_launch_adjoint_sym(const psfsim_plan *h, const float *g, int 
 }
 
 // ---- split-BF16 storage with the same compaction (PSFSIM_SPLIT_BF16_SYM) ----
-// Forward: the four rotated scenes of every scene are gathered as a batch of
-// 4B for the tcgen05 product over the compact columns, and the 4B partial
-// images are summed through the inverse quarter turns.  Adjoint: the residual
+// Forward: the four rotated scenes of every scene run as a batch of 4B through
+// the tcgen05 product over the compact columns (its scene split gathers them),
+// and the 4B partial images are summed through the inverse quarter turns.  Adjoint: the residual
 // turned four ways, the split adjoint over the compact columns, and a scatter
 // to the four rotated scene pixels.
 
-size_t psfsim_forward_split_sym_scratch(const psfsim_plan *h, int B) {
-  return (size_t)psfsim_round_up((int64_t)4 * B * h->ld * 4, 256) +
-         (size_t)psfsim_round_up((int64_t)4 * B * h->M * 4, 256) + psfsim_forward_tc_scratch(h, 4 * B);
-}
+size_t psfsim_forward_split_sym_scratch(const psfsim_plan *h, int B) { return psfsim_forward_tc_scratch(h, 4 * B); }
 
 cudaError_t psfsim_launch_forward_split_sym(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
                                             cudaStream_t st) {
-  const int *order = reinterpret_cast<const int *>(h->ws + h->order_off);
-  const int64_t Kv = h->K_valid;
-  float *xc = static_cast<float *>(scratch);
-  float *v = reinterpret_cast<float *>(static_cast<char *>(scratch) + psfsim_round_up((int64_t)4 * B * h->ld * 4, 256));
-  void *tc = reinterpret_cast<char *>(v) + psfsim_round_up((int64_t)4 * B * h->M * 4, 256);
-  if (Kv == 0) return cudaMemsetAsync(y, 0, (size_t)B * h->M * 4, st);
-  sym_gather<<<grid_for((int64_t)4 * B * Kv, h->num_sms), 256, 0, st>>>(x, B, h->N, Kv, order, xc);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if ((e = psfsim_launch_forward_tc(h, xc, 4 * B, v, tc, st)) != cudaSuccess) return e;
-  sym_permsum<<<grid_for((int64_t)B * h->M, h->num_sms), 256, 0, st>>>(v, B, h->n, y);
-  return cudaGetLastError();
+  if (h->K_valid == 0) return cudaMemsetAsync(y, 0, (size_t)B * h->M * 4, st);
+  return psfsim_launch_forward_tc_sym(h, x, B, y, scratch, st);
 }
 
 size_t psfsim_adjoint_split_sym_scratch(const psfsim_plan *h, int B) {

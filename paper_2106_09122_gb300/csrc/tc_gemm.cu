@@ -60,7 +60,8 @@ struct TcJob {
   int cap;             // scenes in the job's buffers (<= Bp)
   const int *ktab;     // first column of every k-tile (NULL: k-tile t starts at column 64 t)
   const int *count;    // device int: scenes present (NULL: all cap)
-  float *part;         // [KS][cap][rows]
+  float *out;          // partial images [KS][cap][out_ld]; with one split, the images themselves
+  int64_t out_ld, out_rows;  // out_ld = out_rows = rows, or M for the images themselves
 };
 
 // Kernel parameter block: tensor maps (hi, lo, x) and geometry of every job.
@@ -77,34 +78,117 @@ struct TcMulti {
   int64_t stall_it;  // test hook: the producer never issues this load (-1: none)
 };
 
-// xs[part][b][t]: the three bf16 parts of scene b at the t-th column that the
-// k-tiles cover, times the column's scale (width = 64 k-tiles columns).  The
-// columns in no k-tile are zero in A; a non-finite scene value there still
-// makes the whole image NaN (0 x inf), as it does when they are multiplied
-// out: position t adds 0 x for its share of them.
-__global__ void xsplit_kernel(const float *__restrict__ x, int B, const int *__restrict__ count, int Bp, int64_t K,
-                              int64_t width, const int *__restrict__ ktab, int64_t dead_groups,
-                              const float *__restrict__ scale, __nv_bfloat16 *__restrict__ xs) {
-  const int64_t total = (int64_t)Bp * width;
-  const int nb = count ? min(*count, B) : B;
-  const int *dead = ktab + width / BK;
+// One job's scene split (xsplit_kernel).
+struct XJob {
+  const float *x;
+  const int *count;    // scenes present (NULL: all B)
+  const int *ktab;     // k-tile table, dead groups after it (live.cu), or NULL
+  const int *order;    // compact storage: quadrant pixel of every column (else NULL)
+  const float *scale;
+  __nv_bfloat16 *xs;   // [3][Bp][width]
+  int64_t K, width, dead_groups;
+  int B, Bp, N, first; // compact storage: slot b is rotated scene first + b, i.e. scene / 4 turned % 4 times
+};
+struct XMulti {
+  XJob job[kMaxJobs];
+};
+
+// xs[part][b][t] of job blockIdx.y: the three bf16 parts of scene b at the t-th
+// column that the k-tiles cover, times the column's scale (width = 64 k-tiles
+// columns).  The columns in no k-tile are zero in A; a non-finite scene value
+// there still makes the whole image NaN (0 x inf), as it does when they are
+// multiplied out: position t adds 0 x for its share of them.  Compact storage
+// reads the four rotated pixels of a column straight from the scene.  One
+// launch serves every job (ten jobs: 12 us, against 33 us and the gaps of ten).
+__global__ void __launch_bounds__(256) xsplit_kernel(const __grid_constant__ XMulti P) {
+  const XJob &J = P.job[blockIdx.y];
+  const int64_t width = J.width, total = (int64_t)J.Bp * width;
+  const int nb = J.count ? min(*J.count, J.B) : J.B;
+  const int *dead = J.ktab + width / BK;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
     const int b = (int)(t / width);
     const int64_t c = t % width;
-    const int64_t j = ktab ? ktab[c / BK] + c % BK : c;
-    float v = (b < nb && j < K) ? x[(int64_t)b * K + j] * scale[j] : 0.f;
-    if (b < nb)
-      for (int64_t e = c; e < dead_groups * kLiveGroup; e += width) {
-        const int64_t jd = (int64_t)dead[e / kLiveGroup] * kLiveGroup + e % kLiveGroup;
-        if (jd < K) v += 0.f * x[(int64_t)b * K + jd];
+    float v = 0.f;
+    if (b < nb) {
+      if (J.order) {
+        if (c < J.K) {
+          const int H = J.N / 2, j0 = J.order[c], r = J.first + b;
+          int ix = H + j0 % H, iy = H + j0 / H;
+          for (int k = 0; k < (r & 3); ++k) {  // R(ix, iy) = (N-1-iy, ix)
+            const int nx = J.N - 1 - iy;
+            iy = ix;
+            ix = nx;
+          }
+          v = J.x[(int64_t)(r >> 2) * J.N * J.N + (int64_t)iy * J.N + ix] * J.scale[c];
+        }
+      } else {
+        const float *xb = J.x + (int64_t)b * J.K;
+        const int64_t j = J.ktab ? J.ktab[c / BK] + c % BK : c;
+        if (j < J.K) v = xb[j] * J.scale[j];
+#pragma unroll 4
+        for (int64_t e = c; e < J.dead_groups * kLiveGroup; e += width) {
+          const int64_t jd = (int64_t)dead[e / kLiveGroup] * kLiveGroup + e % kLiveGroup;
+          v += 0.f * xb[min(jd, J.K - 1)];
+        }
       }
+    }
     const __nv_bfloat16 x1 = __float2bfloat16_rn(v);
     const float r1 = v - __bfloat162float(x1);
     const __nv_bfloat16 x2 = __float2bfloat16_rn(r1);
     const float r2 = r1 - __bfloat162float(x2);
-    xs[t] = x1;
-    xs[total + t] = x2;
-    xs[2 * total + t] = __float2bfloat16_rn(r2);
+    J.xs[t] = x1;
+    J.xs[total + t] = x2;
+    J.xs[2 * total + t] = __float2bfloat16_rn(r2);
+  }
+}
+
+// One job's sum over its k-splits (tc_reduce_kernel).
+struct RJob {
+  const float *part;  // [KS][cap][rows]
+  float *y;           // [cap][M]
+  const int *count;
+  int64_t rows, M;
+  int KS, cap;
+};
+struct RMulti {
+  RJob job[kMaxJobs];
+};
+
+// y[b, i] = sum_ks part[ks, b, i] of job blockIdx.z in a fixed order, 128 rows
+// per CTA: its 8 warps take ks = warp, warp + 8, ... and combine through
+// shared memory.  One launch serves every job.
+constexpr int kRedRows = 128;
+__global__ void __launch_bounds__(256) tc_reduce_kernel(const __grid_constant__ RMulti P) {
+  __shared__ float4 red[8][32];
+  const RJob &J = P.job[blockIdx.z];
+  const int c4 = threadIdx.x & 31, grp = threadIdx.x >> 5;
+  const int64_t r = ((int64_t)blockIdx.x * 32 + c4) * 4;
+  const int b = blockIdx.y;
+  if (b >= J.cap || (int64_t)blockIdx.x * kRedRows >= J.M || (J.count && b >= *J.count)) return;
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (r < J.rows) {
+    const float *p = J.part + (int64_t)b * J.rows + r;
+    const int64_t step = (int64_t)J.cap * J.rows;
+#pragma unroll 4
+    for (int ks = grp; ks < J.KS; ks += 8) {
+      const float4 v = *reinterpret_cast<const float4 *>(p + ks * step);
+      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+  }
+  red[grp][c4] = s;
+  __syncthreads();
+  if (grp == 0 && r < J.M) {
+    float4 t = red[0][c4];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) {
+      const float4 v = red[k][c4];
+      t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
+    }
+    float *out = J.y + (int64_t)b * J.M + r;
+    out[0] = t.x;
+    if (r + 1 < J.M) out[1] = t.y;
+    if (r + 2 < J.M) out[2] = t.z;
+    if (r + 3 < J.M) out[3] = t.w;
   }
 }
 
@@ -315,10 +399,13 @@ __global__ void __launch_bounds__(kThreads, 2) tc_gemm_kernel(const __grid_const
       }
       if (!ok) break;
       const int nb = J.count ? min(*J.count, J.cap) : J.cap;
-      float *out = J.part + (int64_t)ks * J.cap * J.rows + (int64_t)mt * BM + row;
+      const int64_t i = (int64_t)mt * BM + row;
+      float *out = J.out + (int64_t)ks * J.cap * J.out_ld + i;
+      if (i < J.out_rows) {
 #pragma unroll
-      for (int t = 0; t < kMaxBp; ++t)
-        if (t < nb) out[(int64_t)t * J.rows] = sum[t];
+        for (int t = 0; t < kMaxBp; ++t)
+          if (t < nb) out[(int64_t)t * J.out_ld] = sum[t];
+      }
     }
   }
   __syncthreads();
@@ -380,6 +467,7 @@ struct JobSpec {
   float *y;
   int cap;
   const int *count;
+  int first;  // compact storage: x holds whole scenes, and slot b is rotated scene first + b (-1: plain)
 };
 
 struct JobPlan {
@@ -485,17 +573,35 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
                          const StallHook &hook = kNoStall) {
   char *base = static_cast<char *>(scratch);
   cudaError_t e;
-  TcMulti P;  // kernel parameter block, copied at launch
+  TcMulti P;  // kernel parameter blocks, copied at launch
+  XMulti XP;
+  RMulti RP;
   std::memset(&P, 0, sizeof(P));
+  std::memset(&XP, 0, sizeof(XP));
+  std::memset(&RP, 0, sizeof(RP));
+  int64_t x_blocks = 1, red_rows = 0;
+  int nred = 0, red_cap = 0;
   for (int j = 0; j < nj; ++j) {
     const psfsim_plan *h = jobs[j].h;
     const JobPlan &p = mp.jp[j];
     __nv_bfloat16 *xs = reinterpret_cast<__nv_bfloat16 *>(base + p.xs_off);
     const float *scale = reinterpret_cast<const float *>(h->ws + h->scale_off);
-    const int *ktab = h->live ? reinterpret_cast<const int *>(h->ws + h->order_off) : nullptr;
-    xsplit_kernel<<<h->num_sms * 4, 256, 0, st>>>(jobs[j].x, jobs[j].cap, jobs[j].count, p.Bp, psfsim_cols(h),
-                                                  (int64_t)p.k_tiles * BK, ktab, h->dead_groups, scale, xs);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    XJob &X = XP.job[j];
+    X.x = jobs[j].x;
+    X.count = jobs[j].count;
+    X.ktab = h->live ? reinterpret_cast<const int *>(h->ws + h->order_off) : nullptr;
+    X.order = jobs[j].first >= 0 ? reinterpret_cast<const int *>(h->ws + h->order_off) : nullptr;
+    X.scale = scale;
+    X.xs = xs;
+    X.K = psfsim_cols(h);
+    X.width = (int64_t)p.k_tiles * BK;
+    X.dead_groups = h->dead_groups;
+    X.B = jobs[j].cap;
+    X.Bp = p.Bp;
+    X.N = h->N;
+    X.first = jobs[j].first;
+    const int64_t blocks = ((int64_t)p.Bp * X.width + 255) / 256;
+    x_blocks = blocks > x_blocks ? blocks : x_blocks;
     const bool has_lo = h->lo_off >= 0;
     if (!encode_bf16_2d(&P.map[j][0], h->ws + h->a_off, (uint64_t)h->ld, (uint64_t)p.rows, BK, BM) ||
         (has_lo && !encode_bf16_2d(&P.map[j][1], h->ws + h->lo_off, (uint64_t)h->ld, (uint64_t)p.rows, BK, BM)) ||
@@ -513,10 +619,29 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
     J.k_tiles = p.k_tiles;
     J.unit_begin = j == 0 ? 0 : P.job[j - 1].unit_begin + P.job[j - 1].m_tiles * P.job[j - 1].KS;
     J.cap = jobs[j].cap;
-    J.ktab = ktab;
+    J.ktab = X.ktab;
     J.count = jobs[j].count;
-    J.part = reinterpret_cast<float *>(base + p.part_off);
+    // One split: the accumulated sums are the images (compact storage still
+    // has its four rotations to add).
+    const bool direct = p.KS == 1 && jobs[j].first < 0;
+    J.out = direct ? jobs[j].y : reinterpret_cast<float *>(base + p.part_off);
+    J.out_ld = J.out_rows = direct ? h->M : p.rows;
+    if (!direct) {
+      RJob &R = RP.job[nred++];
+      R.part = J.out;
+      R.y = jobs[j].y;
+      R.count = jobs[j].count;
+      R.rows = p.rows;
+      R.M = h->M;
+      R.KS = p.KS;
+      R.cap = jobs[j].cap;
+      red_rows = h->M > red_rows ? h->M : red_rows;
+      red_cap = R.cap > red_cap ? R.cap : red_cap;
+    }
   }
+  const int64_t x_cap = (int64_t)jobs[0].h->num_sms * 8;
+  xsplit_kernel<<<dim3((unsigned)(x_blocks < x_cap ? x_blocks : x_cap), (unsigned)nj), 256, 0, st>>>(XP);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   P.njobs = nj;
   P.units = mp.units;
   bool same = nj > 1;
@@ -540,13 +665,11 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
   const int slots = hook.one_cta ? 1 : num_sms * mp.ctas_per_sm;
   tc_gemm_kernel<<<mp.units < slots ? mp.units : slots, kThreads, mp.smem, st>>>(P);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  for (int j = 0; j < nj; ++j) {
-    const JobPlan &p = mp.jp[j];
-    if ((e = psfsim_launch_reduce_partials(reinterpret_cast<float *>(base + p.part_off), p.KS, jobs[j].cap, p.rows,
-                                           jobs[j].h->M, jobs[j].y, jobs[j].count, st)) != cudaSuccess)
-      return e;
-  }
-  return cudaSuccess;
+  if (jobs[0].first >= 0) return cudaSuccess;  // the caller adds the rotations (SymSum)
+  if (nred > 0)
+    tc_reduce_kernel<<<dim3((unsigned)((red_rows + kRedRows - 1) / kRedRows), (unsigned)red_cap, (unsigned)nred), 256, 0,
+                       st>>>(RP);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -560,7 +683,7 @@ int tc_jobs(const psfsim_plan *h, const float *x, int B, float *y, JobSpec *js) 
   int nj = 0;
   for (int b0 = 0; b0 < B && nj < kMaxJobs; b0 += kMaxBp, ++nj) {
     const int c = (B - b0) < kMaxBp ? (B - b0) : kMaxBp;
-    js[nj] = JobSpec{h, x ? x + (int64_t)b0 * cols : nullptr, y ? y + (int64_t)b0 * h->M : nullptr, c, nullptr};
+    js[nj] = JobSpec{h, x ? x + (int64_t)b0 * cols : nullptr, y ? y + (int64_t)b0 * h->M : nullptr, c, nullptr, -1};
   }
   return nj;
 }
@@ -588,6 +711,40 @@ cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B
   return cudaSuccess;
 }
 
+// Compact split storage: the four rotations of up to kMaxLaunchScenes / 4
+// scenes are the launch's jobs, gathered from the scenes by xsplit_kernel; the
+// partial images of all rotations are added through the inverse turns at the
+// end.
+cudaError_t psfsim_launch_forward_tc_sym(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
+                                         cudaStream_t st) {
+  constexpr int kScenes = kMaxLaunchScenes / 4;
+  static_assert(kMaxBp % 4 == 0, "a scene's rotations share a job");
+  for (int b0 = 0; b0 < B; b0 += kScenes) {
+    const int Bc = (B - b0) < kScenes ? (B - b0) : kScenes;
+    JobSpec js[kMaxJobs];
+    const int nj = tc_jobs(h, nullptr, 4 * Bc, nullptr, js);
+    for (int j = 0; j < nj; ++j) {
+      js[j].x = x + (int64_t)b0 * h->K;
+      js[j].first = j * kMaxBp;
+    }
+    const MultiPlan mp = plan_multi(js, nj, nullptr);
+    cudaError_t e = launch_multi(js, nj, mp, scratch, st);
+    if (e != cudaSuccess) return e;
+    SymSum S;
+    std::memset(&S, 0, sizeof(S));
+    S.per = kMaxBp;
+    S.rows = mp.jp[0].rows;
+    S.n = h->n;
+    for (int j = 0; j < nj; ++j) {
+      S.part[j] = reinterpret_cast<const float *>(static_cast<char *>(scratch) + mp.jp[j].part_off);
+      S.cap[j] = js[j].cap;
+      S.KS[j] = mp.jp[j].KS;
+    }
+    if ((e = psfsim_launch_sym_sum(S, Bc, y + (int64_t)b0 * h->M, st)) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 int psfsim_multi_validate(const psfsim_job_t *jobs, int njobs) {
   if (!jobs || njobs < 1 || njobs > kMaxJobs) return PSFSIM_ERR_ARG;
   for (int j = 0; j < njobs; ++j) {
@@ -602,14 +759,14 @@ int psfsim_multi_validate(const psfsim_job_t *jobs, int njobs) {
 
 size_t psfsim_forward_multi_scratch(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune) {
   JobSpec js[kMaxJobs];
-  for (int j = 0; j < njobs; ++j) js[j] = JobSpec{jobs[j].plan, jobs[j].d_x, jobs[j].d_y, jobs[j].capacity, jobs[j].d_count};
+  for (int j = 0; j < njobs; ++j) js[j] = JobSpec{jobs[j].plan, jobs[j].d_x, jobs[j].d_y, jobs[j].capacity, jobs[j].d_count, -1};
   return plan_multi(js, njobs, tune).scratch;
 }
 
 cudaError_t psfsim_launch_forward_multi(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune,
                                         void *scratch, cudaStream_t st) {
   JobSpec js[kMaxJobs];
-  for (int j = 0; j < njobs; ++j) js[j] = JobSpec{jobs[j].plan, jobs[j].d_x, jobs[j].d_y, jobs[j].capacity, jobs[j].d_count};
+  for (int j = 0; j < njobs; ++j) js[j] = JobSpec{jobs[j].plan, jobs[j].d_x, jobs[j].d_y, jobs[j].capacity, jobs[j].d_count, -1};
   return launch_multi(js, njobs, plan_multi(js, njobs, tune), scratch, st);
 }
 

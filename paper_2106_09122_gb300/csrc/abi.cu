@@ -73,6 +73,8 @@ int common_build(const float *d_lib, const double *h_radii, int n_r, int n, doub
   h->plib_off = L.plib_off;
   h->cols_off = L.cols_off;
   h->mtorder_off = L.mtorder_off;
+  // A workspace of the plain layout's size (or a field-point build) does without the pixel-wise build's tables.
+  h->pix_off = N > 0 && ws_bytes >= (size_t)L.total_pix ? L.pix_off : -1;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int rc = PSFSIM_OK;
   if (cudaGetDevice(&h->device) != cudaSuccess ||
@@ -114,7 +116,7 @@ int psfsim_workspace_bytes(int n, int n_r, int64_t K, int storage, size_t *bytes
   if (!bytes || n < 1 || n > 4096 || n_r < 2 || n_r > PSFSIM_MAX_RADII || K < 1 || K > (int64_t)1 << 30 ||
       !storage_ok(storage))
     return PSFSIM_ERR_ARG;
-  *bytes = (size_t)psfsim_layout(n, K, storage, n_r).total;
+  *bytes = (size_t)psfsim_layout(n, K, storage, n_r).total_pix;
   return PSFSIM_OK;
 }
 

@@ -504,8 +504,12 @@ WsLayout psfsim_layout(int n, int64_t K, int storage, int n_r) {
   // ... and the generators' column table.
   L.cols_off = storage == PSFSIM_FUSED ? take(psfsim_fused_columns_bytes(K)) : -1;
   L.mtorder_off = storage == PSFSIM_FUSED ? take(psfsim_fused_mtile_order_bytes(n)) : -1;
-  L.total = off;
-  (void)n_r;
+  L.total = L.total_pix = off;
+  L.pix_off = -1;
+  if (const int64_t extra = psfsim_pixel_build_bytes(n, K, storage, n_r)) {
+    L.pix_off = take(extra);
+    L.total_pix = off;
+  }
   return L;
 }
 
@@ -533,8 +537,8 @@ static bool encode_library_map(psfsim_plan *h, int Wp) {
 cudaError_t psfsim_launch_build(psfsim_plan *h, cudaStream_t st) {
   // Dense storage of an even grid is built from the x > 0, y > 0 quadrant's
   // columns, four quarter-turned copies each, so the geometry tables cover
-  // the quadrant only (entry (iy - N/2) (N/2) + ix - N/2).  The split builds
-  // take no column order.
+  // the quadrant only (entry (iy - N/2) (N/2) + ix - N/2).  The split
+  // builds without pair entries take no column order.
   const bool dense_split = h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16;
   const bool sym = !h->quadrant && h->N > 0 && h->N % 2 == 0 &&
                    (dense_split || (h->storage == PSFSIM_FP32 && h->n % kSymBlk == 0));
@@ -557,7 +561,7 @@ cudaError_t psfsim_launch_build(psfsim_plan *h, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   geom_kernel<<<(unsigned)((Kg + 255) / 256), 256, 0, st>>>(G, geom);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (!(sym && dense_split)) {
+  if (!(sym && dense_split && h->pix_off < 0)) {
     // chunks of at least 256 columns, and as many as fit in shared memory
     const int nb = psfsim_num_buckets(h->n_r);
     int W = (int)((Kg + 255) / 256);
@@ -570,6 +574,10 @@ cudaError_t psfsim_launch_build(psfsim_plan *h, cudaStream_t st) {
       return e;
     bracket_sort_kernel<<<1, 1024, smem, st>>>(geom, Kg, h->n_r, W, order, bstart);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (sym && dense_split) {
+      angle_sort_kernel<<<h->n_r - 1, 1024, 0, st>>>(geom, h->n_r, order, bstart);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
   }
   if (h->quadrant) {
     // The host needs the number of columns inside the last radius to size launches.

@@ -787,10 +787,14 @@ int64_t psfsim_fused_mtile_order_bytes(int n) {
   return (int64_t)((n + kTileW - 1) / kTileW) * ((n + kTileH - 1) / kTileH) * (int64_t)sizeof(int);
 }
 
+cudaError_t psfsim_launch_pair_entries(const float *lib, int n, int n_r, float *entries, int num_sms, cudaStream_t st) {
+  pair_library_kernel<<<num_sms * 4, 256, 0, st>>>(lib, n, n_r, entries);
+  return cudaGetLastError();
+}
+
 cudaError_t psfsim_launch_pair_library(psfsim_plan *h, cudaStream_t st) {
-  pair_library_kernel<<<h->num_sms * 4, 256, 0, st>>>(h->d_lib, h->n, h->n_r,
-                                                      reinterpret_cast<float *>(h->ws + h->plib_off));
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = psfsim_launch_pair_entries(h->d_lib, h->n, h->n_r, reinterpret_cast<float *>(h->ws + h->plib_off),
+                                             h->num_sms, st);
   if (e != cudaSuccess) return e;
   const int tiles_q = (h->n + kTileW - 1) / kTileW, m_tiles = tiles_q * ((h->n + kTileH - 1) / kTileH);
   mtile_order_kernel<<<(m_tiles + 255) / 256, 256, 0, st>>>(h->n, tiles_q, m_tiles,

@@ -54,13 +54,13 @@ __device__ __forceinline__ int scan_sum(int v, int *sh, int &total) {
 }
 
 __device__ __forceinline__ bool group_live(int N, int64_t K, long long R2, int64_t g, int64_t groups) {
-  if (g < 0 || g >= groups) return false;
-  if (g == 0) {
-    if (R2 < (N & 1 ? 0 : 2)) return true;  // no live pixel at all: keep one tile
-  }
-  for (int64_t j = g * kLiveGroup; j < (g + 1) * kLiveGroup && j < K; ++j) {
-    const long long X = 2 * (j % N) - (N - 1), Y = 2 * (j / N) - (N - 1);
-    if (X * X + Y * Y <= R2) return true;
+  if (g >= groups) return false;
+  if (g == 0 && R2 < (N & 1 ? 0 : 2)) return true;  // no live pixel at all: keep one tile
+  const int64_t j0 = g * kLiveGroup, j1 = min(j0 + kLiveGroup, K);
+  for (int iy = (int)(j0 / N); (int64_t)iy * N < j1; ++iy) {  // the one or two (narrow scenes: more) rows it spans
+    int a, b;
+    live_row(N, R2, iy, a, b);
+    if (a < b && (int64_t)iy * N + a < j1 && (int64_t)iy * N + b > j0) return true;
   }
   return false;
 }
@@ -71,11 +71,17 @@ __device__ __forceinline__ bool group_live(int N, int64_t K, long long R2, int64
 __global__ void __launch_bounds__(1024) ktile_table_kernel(int N, int64_t K, long long R2, int *ktab, int k_tiles,
                                                            int *dead, int64_t dead_groups) {
   __shared__ int sh[32];
+  __shared__ bool flag[1024];
+  bool carry = false;  // the last group of the block before is live
   const int64_t groups = (K + kLiveGroup - 1) / kLiveGroup;
   int run_carry = -1, tile_carry = 0, dead_carry = 0;
   for (int64_t base = 0; base < groups; base += blockDim.x) {
     const int64_t g = base + threadIdx.x;
-    const bool live = group_live(N, K, R2, g, groups), before = group_live(N, K, R2, g - 1, groups);
+    const bool live = group_live(N, K, R2, g, groups);
+    flag[threadIdx.x] = live;
+    __syncthreads();
+    const bool before = threadIdx.x ? flag[threadIdx.x - 1] : carry;
+    carry = flag[blockDim.x - 1];
     int total;
     const int start = max(run_carry, scan_max(live && !before ? (int)g : -1, sh, total));  // of g's, or the last, run
     run_carry = max(run_carry, total);

@@ -40,6 +40,7 @@ struct psfsim_plan {
   size_t ws_bytes;
   int64_t a_off, lo_off, scale_off, geom_off, order_off, bstart_off, pts_off, status_off, libmax_off, plib_off,
       cols_off, mtorder_off;
+  int64_t pix_off;  // split storage: pair entries and pixel order of the pixel-wise build (-1: another build)
   int device, num_sms;
   bool live;            // products skip the zero columns listed in the workspace (live.cu)
   int k_tiles;          // split storage: 64-column k-tiles the products read (ld / 64 when !live)
@@ -51,7 +52,8 @@ struct psfsim_plan {
 // Workspace layout for a given shape; returns total bytes.
 struct WsLayout {
   int64_t ld, a_off, lo_off, scale_off, geom_off, order_off, bstart_off, pts_off, status_off, libmax_off, plib_off,
-      cols_off, mtorder_off, total;
+      cols_off, mtorder_off, total;  // total: what a build needs
+  int64_t pix_off, total_pix;      // ... and with the pixel-wise split build's tables (total, -1 where it has none)
 };
 WsLayout psfsim_layout(int n, int64_t K, int storage, int n_r);
 // FUSED storage's copy of the library: one 32-byte pair entry per bracket
@@ -64,6 +66,9 @@ int64_t psfsim_fused_columns_bytes(int64_t K);
 // ... and its M-tile order (the image's 8 x 16 pixel tiles, nearest the centre first).
 int64_t psfsim_fused_mtile_order_bytes(int n);
 cudaError_t psfsim_launch_pair_library(psfsim_plan *h, cudaStream_t st);
+cudaError_t psfsim_launch_pair_entries(const float *lib, int n, int n_r, float *entries, int num_sms, cudaStream_t st);
+// Extra workspace of the pixel-wise dense split build of an even grid (0: it does not apply; split_build.cu).
+int64_t psfsim_pixel_build_bytes(int n, int64_t K, int storage, int n_r);
 
 // Live (not identically zero) columns of a dense plan on a scene grid: counted
 // on the host, listed in the workspace by the build (live.cu).

@@ -44,3 +44,48 @@ def test_non_finite_scene_value_at_a_skipped_column(storage, value):
         x[1, j] = value
         y = plan.forward(torch.from_numpy(x).to(DEV)).cpu().numpy()
         assert np.isfinite(y[0]).all() and np.isnan(y[1]).all()
+
+
+@pytest.mark.parametrize("storage", ["split_bf16", "bf16"])
+@pytest.mark.parametrize("n,N,interp", [(17, 48, "linear"), (96, 64, "linear"), (41, 50, "nearest"), (33, 66, "linear"),
+                                        (24, 320, "linear"), (20, 150, "linear")])
+def test_pixelwise_build_equals_direct_build_bit_for_bit(n, N, interp, storage):
+    """Dense split builds of an even grid (odd images, runs of 8 and ragged runs) against the
+    same grid given as field points, which takes the direct build; padding is zero."""
+    from paper_2106_09122_gb300 import Plan
+    rng = np.random.default_rng(n * N)
+    radii, S = np.linspace(0.0, 5.0, 4), 8.0 / N
+    lib = torch.from_numpy(rng.uniform(0.0, 1.0, (4, n, n)).astype(np.float32)).to(DEV)
+    c = (np.arange(N) - 0.5 * (N - 1)) * S
+    pts = np.stack([np.tile(c, N), np.repeat(c, N)], axis=1)
+    grid = Plan(lib, radii, 0.25, N=N, S=S, storage=storage, interp=interp)
+    direct = Plan(lib, radii, 0.25, points=pts, storage=storage, interp=interp)
+    for a, b in zip(grid.A_split(), direct.A_split()):
+        assert (a is None) == (b is None)
+        if a is not None:
+            assert torch.equal(a.view(torch.int16 if a.dtype == torch.bfloat16 else torch.int32),
+                               b.view(torch.int16 if b.dtype == torch.bfloat16 else torch.int32))
+
+
+def test_split_build_in_a_workspace_without_room_for_pair_entries():
+    """A workspace of the layout's size alone is enough: the block-wise build, the same bits."""
+    import ctypes
+    from paper_2106_09122_gb300 import Plan
+    from paper_2106_09122_gb300 import _binding as B
+    n, N, n_r = 33, 66, 4
+    rng = np.random.default_rng(3)
+    radii, S = np.linspace(0.0, 5.0, n_r), 8.0 / N
+    lib = torch.from_numpy(rng.uniform(0.0, 1.0, (n_r, n, n)).astype(np.float32)).to(DEV)
+    plan = Plan(lib, radii, 0.25, N=N, S=S, storage="split_bf16")
+    up = lambda v: (v + 255) // 256 * 256
+    extra = up(((n_r - 1) * (n + 1) ** 2 + 1) * 32) + up(n * n * 4)
+    ws = torch.zeros(plan.workspace.numel() - extra, dtype=torch.uint8, device=DEV)
+    h, L = ctypes.c_void_p(), B.load()
+    args = (ctypes.c_void_p(lib.data_ptr()), radii.ctypes.data_as(ctypes.c_void_p), n_r, n, 0.25, N, S,
+            B.SPLIT_BF16, B.LINEAR, ctypes.c_void_p(ws.data_ptr()))
+    assert L.psfsim_build(*args, ws.numel() - 256, None, ctypes.byref(h)) == B.ERR_WORKSPACE
+    B.check(L.psfsim_build(*args, ws.numel(), None, ctypes.byref(h)), "psfsim_build")
+    torch.cuda.synchronize()
+    end = plan.info.scale_offset + 4 * plan.info.ld
+    assert torch.equal(ws[:end], plan.workspace[:end])
+    L.psfsim_free(h)

@@ -217,7 +217,7 @@ int psfsim_forward(psfsim_t h, const float *d_x, int B, float *d_y, void *d_scra
   if (h->storage == PSFSIM_FP32) {
     const size_t need = psfsim_forward_fp32_scratch(h, B);
     if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
-    return psfsim_launch_forward_fp32(h, d_x, B, d_y, d_scratch, st) == cudaSuccess ? PSFSIM_OK
+    return psfsim_launch_forward_fp32(h, d_x, B, d_y, d_scratch, false, st) == cudaSuccess ? PSFSIM_OK
                                                                                     : PSFSIM_ERR_CUDA;
   }
   if (h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16) {
@@ -248,7 +248,7 @@ int psfsim_forward(psfsim_t h, const float *d_x, int B, float *d_y, void *d_scra
 int psfsim_forward_sparse_scratch_bytes(psfsim_t h, int B, size_t *bytes) {
   if (!h || !bytes || B < 1) return PSFSIM_ERR_ARG;
   if (h->storage != PSFSIM_FP32) return PSFSIM_ERR_UNSUPPORTED;
-  *bytes = psfsim_forward_sparse_scratch(h, B);
+  *bytes = psfsim_forward_fp32_scratch(h, B);
   return PSFSIM_OK;
 }
 
@@ -256,9 +256,9 @@ int psfsim_forward_sparse(psfsim_t h, const float *d_x, int B, float *d_y, void 
                           void *stream) {
   if (!h || !d_x || !d_y || B < 1) return PSFSIM_ERR_ARG;
   if (h->storage != PSFSIM_FP32) return PSFSIM_ERR_UNSUPPORTED;
-  const size_t need = psfsim_forward_sparse_scratch(h, B);
+  const size_t need = psfsim_forward_fp32_scratch(h, B);
   if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
-  return psfsim_launch_forward_sparse(h, d_x, B, d_y, d_scratch, static_cast<cudaStream_t>(stream)) == cudaSuccess
+  return psfsim_launch_forward_fp32(h, d_x, B, d_y, d_scratch, true, static_cast<cudaStream_t>(stream)) == cudaSuccess
              ? PSFSIM_OK
              : PSFSIM_ERR_CUDA;
 }

@@ -513,6 +513,8 @@ WsLayout psfsim_layout(int n, int64_t K, int storage, int n_r) {
   return L;
 }
 
+static cudaError_t launch_tables_and_build(psfsim_plan *h, cudaStream_t st);
+
 static bool encode_library_map(psfsim_plan *h, int Wp) {
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   if (!encode) {
@@ -535,6 +537,12 @@ static bool encode_library_map(psfsim_plan *h, int Wp) {
 }
 
 cudaError_t psfsim_launch_build(psfsim_plan *h, cudaStream_t st) {
+  const cudaError_t e = launch_tables_and_build(h, st);
+  if (e != cudaSuccess || h->storage == PSFSIM_FUSED) return e;
+  return psfsim_launch_live_table(h, st);  // the column order is free from here on
+}
+
+static cudaError_t launch_tables_and_build(psfsim_plan *h, cudaStream_t st) {
   // Dense storage of an even grid is built from the x > 0, y > 0 quadrant's
   // columns, four quarter-turned copies each, so the geometry tables cover
   // the quadrant only (entry (iy - N/2) (N/2) + ix - N/2).  The split
@@ -597,10 +605,8 @@ cudaError_t psfsim_launch_build(psfsim_plan *h, cudaStream_t st) {
     if (h->storage == PSFSIM_SPLIT_BF16_SYM) h->ld = psfsim_round_up(kv > 0 ? kv : 1, 64);
   }
   psfsim_live_count(h);
-  if (h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16 || h->storage == PSFSIM_SPLIT_BF16_SYM) {
-    if ((e = psfsim_launch_split_build(h, st)) != cudaSuccess) return e;
-    return psfsim_launch_live_table(h, st);
-  }
+  if (h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16 || h->storage == PSFSIM_SPLIT_BF16_SYM)
+    return psfsim_launch_split_build(h, st);
   if (h->storage != PSFSIM_FP32 && h->storage != PSFSIM_FP32_SYM) return cudaErrorNotSupported;
   const bool compact = h->storage == PSFSIM_FP32_SYM;
 

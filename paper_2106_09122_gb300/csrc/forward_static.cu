@@ -88,7 +88,7 @@ extern "C" int psfsim_forward_static(psfsim_t h, const float *d_x, int B, float 
   if (int rc = scratch_address(device, &scratch)) return rc;
   // Every launch overwrites all the partial sums it later reads, so the
   // previous call's contents never need clearing.
-  return psfsim_launch_forward_fp32(h, d_x, B, d_y, scratch, static_cast<cudaStream_t>(stream)) == cudaSuccess
+  return psfsim_launch_forward_fp32(h, d_x, B, d_y, scratch, false, static_cast<cudaStream_t>(stream)) == cudaSuccess
              ? PSFSIM_OK
              : PSFSIM_ERR_CUDA;
 }

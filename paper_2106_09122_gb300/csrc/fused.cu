@@ -861,7 +861,7 @@ static cudaError_t launch_fused(const psfsim_plan *h, const float *x, int B, flo
     const int units = f.m_tiles * f.KS;
     kernel<<<units < max_ctas ? units : max_ctas, kThreads, f.smem, st>>>(mx, P);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = psfsim_launch_reduce_partials(part, 4 * f.KS, Bc, f.rows, h->M, y + (int64_t)b0 * h->M, nullptr, st)) !=
+    if ((e = psfsim_launch_reduce_partials(part, 4 * f.KS, Bc, f.rows, h->M, y + (int64_t)b0 * h->M, st)) !=
         cudaSuccess)
       return e;
   }

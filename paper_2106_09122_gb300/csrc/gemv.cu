@@ -10,20 +10,147 @@ using namespace psfsim_gemv;
 
 namespace {
 
-// part[(ks*B + b)*ld + r] = sum over the ks-th column chunk of A[r, j] x[b, j].
-template <int BB>
-__global__ void __launch_bounds__(kFwdThreads) fwd_partial_kernel(const float *__restrict__ A, int64_t ld,
-                                                                  int64_t K, const float *__restrict__ x,
-                                                                  int B, int b0, float *__restrict__ part) {
+// Forward partials: CTA (tile, ks) adds the ks-th share of the columns for 1024
+// rows and BB scenes, part[(ks B + b0 + b) ld + r].  Bound by reading A once
+// (B <= 16 scenes a pass; the FMAs of 16 take as long):
+//   * only live columns are read (live.cu; 44 % of them at 12 of 16 lambda/D),
+//     and with kFilter only those that are non-zero in some scene of the pass;
+//   * a share is every KS-th group of four columns, so a filtered scene's flux
+//     spreads evenly without a list made beforehand;
+//   * the share's scene values go through shared memory, 256 columns at a
+//     time, as BB contiguous floats a column: one 16-byte broadcast load
+//     serves four scenes.  Read from global memory per thread, a group of 8
+//     scenes ran at half the rate of one.
+// 11 scenes of the 128^2 plan: 660 us in passes of 8, 2 and 1 over all columns,
+// 92 us in one pass over the live ones (HBM floor 70).
+constexpr int kChunkCols = kFwdThreads;
+constexpr int kShare = 4;
+
+__host__ __device__ constexpr int fwd_min_ctas(int BB) { return BB == 1 ? 6 : BB == 4 ? 4 : BB == 8 ? 3 : 2; }
+
+template <int BB, bool kFilter, bool kSym>
+__global__ void __launch_bounds__(kFwdThreads, fwd_min_ctas(BB)) fwd_cols_kernel(const FwdCols P, int b0, int nb) {
+  __shared__ __align__(16) float xs[kChunkCols * BB];
+  __shared__ int js[kChunkCols];
+  __shared__ int used[kFwdThreads / 32];
+  __shared__ unsigned bad;  // scenes with a non-finite value at a column that is not read
   const int64_t r = (int64_t)blockIdx.x * kRowsPerCta + 4 * threadIdx.x;
   const int KS = gridDim.y, ks = blockIdx.y;
-  if (r >= ld) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int U = BB <= 4 ? 4 : 8;  // columns in flight per thread
   float acc[BB][4];
-  fwd_accumulate<BB>(A, ld, K, x, b0, r, K * ks / KS, K * (ks + 1) / KS, acc);
 #pragma unroll
-  for (int b = 0; b < BB; ++b)
-    *reinterpret_cast<float4 *>(part + ((int64_t)ks * B + b0 + b) * ld + r) =
-        make_float4(acc[b][0], acc[b][1], acc[b][2], acc[b][3]);
+  for (int b = 0; b < BB; ++b) acc[b][0] = acc[b][1] = acc[b][2] = acc[b][3] = 0.f;
+  if (threadIdx.x == 0) bad = 0u;
+  if (!kSym && P.dead) {
+    __syncthreads();
+    for (int64_t e = ks + (int64_t)KS * threadIdx.x; e < P.D; e += (int64_t)KS * kFwdThreads) {
+      const float *xj = P.x + (int64_t)b0 * P.K + P.dead[e];
+      for (int b = 0; b < nb; ++b)
+        if (!isfinite(xj[(int64_t)b * P.K])) atomicOr(&bad, 1u << b);
+    }
+  }
+  const float *A = P.A + r;
+  auto add = [&](const float4 &v, const float *xc) {
+#pragma unroll
+    for (int b = 0; b < BB; ++b) {
+      acc[b][0] = fmaf(v.x, xc[b], acc[b][0]);
+      acc[b][1] = fmaf(v.y, xc[b], acc[b][1]);
+      acc[b][2] = fmaf(v.z, xc[b], acc[b][2]);
+      acc[b][3] = fmaf(v.w, xc[b], acc[b][3]);
+    }
+  };
+  auto values = [&](int c, float (&xc)[BB]) {
+    if (BB == 1) {
+      xc[0] = xs[c];
+    } else {
+#pragma unroll
+      for (int b = 0; b < BB; b += 4) {
+        const float4 q = *reinterpret_cast<const float4 *>(xs + c * BB + b);
+        xc[b] = q.x;
+        xc[b + 1 < BB ? b + 1 : 0] = q.y;
+        xc[b + 2 < BB ? b + 2 : 0] = q.z;
+        xc[b + 3 < BB ? b + 3 : 0] = q.w;
+      }
+    }
+  };
+  const int64_t groups = (P.L + kShare - 1) / kShare;
+  for (int64_t base = 0; ks + KS * (base / kShare) < groups; base += kChunkCols) {
+    const int64_t i = (ks + KS * ((base + threadIdx.x) / kShare)) * kShare + threadIdx.x % kShare;
+    float xv[BB];
+    int j = 0;
+    bool take = i < P.L;
+    if (take) {
+      j = !kSym && P.live ? P.live[i] : (int)i;
+      bool any = false;
+#pragma unroll
+      for (int b = 0; b < BB; ++b) {
+        xv[b] = 0.f;
+        if (b < nb) {
+          if (kSym) {
+            const int H = P.N / 2, j0 = P.order[i], q = b0 + b;
+            int ix = H + j0 % H, iy = H + j0 / H;
+            for (int k = 0; k < (q & 3); ++k) {  // R(ix, iy) = (N-1-iy, ix)
+              const int nx = P.N - 1 - iy;
+              iy = ix;
+              ix = nx;
+            }
+            xv[b] = P.x[(int64_t)(q >> 2) * P.N * P.N + (int64_t)iy * P.N + ix];
+          } else {
+            xv[b] = P.x[(int64_t)(b0 + b) * P.K + j];
+          }
+          any = any || xv[b] != 0.f;
+        }
+      }
+      if (kFilter) take = any;
+    }
+    // slots: the columns taken, in order (without the filter they fill the front anyway)
+    const unsigned votes = __ballot_sync(0xffffffffu, take);
+    __syncthreads();  // the chunk before is consumed
+    if (lane == 0) used[warp] = __popc(votes);
+    __syncthreads();
+    int slot = __popc(votes & ((1u << lane) - 1u)), count = 0;
+#pragma unroll
+    for (int w = 0; w < kFwdThreads / 32; ++w) {
+      if (w < warp) slot += used[w];
+      count += used[w];
+    }
+    if (take) {
+      js[slot] = j;
+#pragma unroll
+      for (int b = 0; b < BB; ++b) xs[slot * BB + b] = xv[b];
+    }
+    __syncthreads();
+    if (r < P.ld) {
+      int c = 0;
+      for (; c + U <= count; c += U) {
+        float4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = ld_stream4(A + (int64_t)js[c + u] * P.ld);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          float xc[BB];
+          values(c + u, xc);
+          add(v[u], xc);
+        }
+      }
+      for (; c < count; ++c) {
+        const float4 v = ld_stream4(A + (int64_t)js[c] * P.ld);
+        float xc[BB];
+        values(c, xc);
+        add(v, xc);
+      }
+    }
+  }
+  if (!kSym && P.dead) __syncthreads();
+  if (r >= P.ld) return;
+#pragma unroll
+  for (int b = 0; b < BB; ++b) {
+    if (b >= nb) break;
+    const float z = !kSym && P.dead && (bad >> b & 1u) ? __int_as_float(0x7fffffff) : 0.f;
+    *reinterpret_cast<float4 *>(P.part + ((int64_t)ks * P.B + b0 + b) * P.ld + r) =
+        make_float4(acc[b][0] + z, acc[b][1] + z, acc[b][2] + z, acc[b][3] + z);
+  }
 }
 
 // y[b, i] = sum_ks part[ks, b, i] in a fixed order.  A CTA covers 128 rows;
@@ -31,13 +158,11 @@ __global__ void __launch_bounds__(kFwdThreads) fwd_partial_kernel(const float *_
 // through shared memory, so every output needs only ~KS/8 loads per thread.
 constexpr int kRedRows = 128;
 __global__ void __launch_bounds__(256) fwd_reduce_kernel(const float *__restrict__ part, int KS, int B,
-                                                         int64_t ld, int64_t M, float *__restrict__ y,
-                                                         const int *__restrict__ count) {
+                                                         int64_t ld, int64_t M, float *__restrict__ y) {
   __shared__ float4 red[8][32];
   const int c4 = threadIdx.x & 31, grp = threadIdx.x >> 5;
   const int64_t r = ((int64_t)blockIdx.x * 32 + c4) * 4;
   const int b = blockIdx.y;
-  if (count && b >= *count) return;  // scene slot not present in this call
   float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
   if (r < ld) {
     const float *p = part + (int64_t)b * ld + r;
@@ -66,21 +191,6 @@ __global__ void __launch_bounds__(256) fwd_reduce_kernel(const float *__restrict
   }
 }
 
-// Resident fwd_partial_kernel CTAs per SM (registers decide it), queried once.
-int fwd_ctas_per_sm() {
-  static const int per_sm = [] {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fwd_partial_kernel<1>, kFwdThreads, 0) != cudaSuccess) {
-      (void)cudaGetLastError();
-      n = 0;
-    }
-    return n > 0 ? n : 1;
-  }();
-  return per_sm;
-}
-
-int forward_splits(const psfsim_plan *h) { return psfsim_gemv_splits(h->ld, h->K, h->num_sms); }
-
 // gx[b, j] = sum_i A[i, j] g[b, i]; CTA c owns the contiguous column range
 // [K c / G, K (c+1) / G).
 template <int BB, bool kVec>
@@ -90,13 +200,42 @@ __global__ void __launch_bounds__(kAdjThreads) adj_kernel(const float *__restric
   adj_columns<BB, kVec>(A, ld, M, K, g, b0, gx, K * blockIdx.x / gridDim.x, K * (blockIdx.x + 1) / gridDim.x);
 }
 
-template <int BB>
-cudaError_t fwd_group(const psfsim_plan *h, const float *x, int B, int b0, float *part, int KS,
-                      cudaStream_t st) {
-  const float *A = reinterpret_cast<const float *>(h->ws + h->a_off);
-  dim3 grid((unsigned)((h->ld + kRowsPerCta - 1) / kRowsPerCta), (unsigned)KS);
-  fwd_partial_kernel<BB><<<grid, kFwdThreads, 0, st>>>(A, h->ld, h->K, x, B, b0, part);
-  return cudaGetLastError();
+// One pass: nb scenes from b0 with KS splits.
+cudaError_t fwd_pass(const FwdCols &P, int BB, int b0, int nb, int KS, bool filter, cudaStream_t st) {
+  const dim3 grid((unsigned)((P.ld + kRowsPerCta - 1) / kRowsPerCta), (unsigned)KS);
+  auto go = [&](auto kern) {
+    kern<<<grid, kFwdThreads, 0, st>>>(P, b0, nb);
+    return cudaGetLastError();
+  };
+#define PSFSIM_FWD(n)                                                                                          \
+  (P.order ? go(fwd_cols_kernel<n, false, true>)                                                               \
+           : filter ? go(fwd_cols_kernel<n, true, false>) : go(fwd_cols_kernel<n, false, false>))
+  switch (BB) {
+    case 1: return filter ? go(fwd_cols_kernel<1, true, false>) : go(fwd_cols_kernel<1, false, false>);
+    case 4: return PSFSIM_FWD(4);
+    case 8: return PSFSIM_FWD(8);
+    case 12: return PSFSIM_FWD(12);
+    default: return PSFSIM_FWD(16);
+  }
+#undef PSFSIM_FWD
+}
+
+FwdCols fwd_cols(const psfsim_plan *h, const float *x, int B, float *part) {
+  const int *list = reinterpret_cast<const int *>(h->ws + h->order_off);
+  FwdCols P;
+  P.A = reinterpret_cast<const float *>(h->ws + h->a_off);
+  P.ld = h->ld;
+  P.x = x;
+  P.K = h->K;
+  P.live = h->live ? list : nullptr;
+  P.L = h->live_cols;
+  P.dead = h->live ? list + h->live_cols : nullptr;
+  P.D = h->K - h->live_cols;
+  P.order = nullptr;
+  P.N = h->N;
+  P.B = B;
+  P.part = part;
+  return P;
 }
 
 template <int BB>
@@ -114,30 +253,34 @@ cudaError_t adj_group(const psfsim_plan *h, const float *g, int b0, float *gx, b
 
 }  // namespace
 
-cudaError_t psfsim_launch_gemv_partials(const float *A, int64_t ld, int64_t K, const float *x, int B, float *part,
-                                        int KS, cudaStream_t st) {
-  dim3 grid((unsigned)((ld + kRowsPerCta - 1) / kRowsPerCta), (unsigned)KS);
-  int b0 = 0;
-  while (b0 < B) {
-    const int left = B - b0;
-    if (left >= 8) { fwd_partial_kernel<8><<<grid, kFwdThreads, 0, st>>>(A, ld, K, x, B, b0, part); b0 += 8; }
-    else if (left >= 4) { fwd_partial_kernel<4><<<grid, kFwdThreads, 0, st>>>(A, ld, K, x, B, b0, part); b0 += 4; }
-    else if (left >= 2) { fwd_partial_kernel<2><<<grid, kFwdThreads, 0, st>>>(A, ld, K, x, B, b0, part); b0 += 2; }
-    else { fwd_partial_kernel<1><<<grid, kFwdThreads, 0, st>>>(A, ld, K, x, B, b0, part); b0 += 1; }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
-// Column splits: one wave of resident CTAs over the row tiles (at least 8
-// columns per split).
-int psfsim_gemv_splits(int64_t ld, int64_t K, int num_sms) {
+// Column splits the scratch of a forward allows: eight CTAs an SM over the row
+// tiles, at least 8 columns each.
+int psfsim_gemv_max_splits(int64_t ld, int64_t K, int num_sms) {
   const int64_t row_blocks = (ld + kRowsPerCta - 1) / kRowsPerCta;
-  int64_t ks = (int64_t)num_sms * fwd_ctas_per_sm() / row_blocks;
+  int64_t ks = (int64_t)num_sms * 8 / row_blocks;
   ks = ks < 1 ? 1 : ks;
   const int64_t max_ks = K / 8 > 0 ? K / 8 : 1;
   return (int)(ks < max_ks ? ks : max_ks);
+}
+
+// Passes of at most 16 scenes, evenly filled, with one wave of resident CTAs.
+cudaError_t psfsim_launch_gemv_partials(const FwdCols &P, int max_splits, int num_sms, bool skip_zeros, int *KS_out,
+                                        cudaStream_t st) {
+  const int passes = (P.B + 15) / 16, per0 = (P.B + passes - 1) / passes;
+  const int per = P.order ? (per0 + 3) / 4 * 4 : per0;  // a scene's rotations stay together
+  const int BB = per == 1 ? 1 : (per + 3) / 4 * 4;
+  const int64_t row_blocks = (P.ld + kRowsPerCta - 1) / kRowsPerCta;
+  int64_t KS = (int64_t)num_sms * fwd_min_ctas(BB) / row_blocks;
+  const int64_t max_ks = P.L / 8 > 0 ? P.L / 8 : 1;
+  KS = KS < 1 ? 1 : KS;
+  KS = KS < max_ks ? KS : max_ks;
+  KS = KS < max_splits ? KS : max_splits;
+  *KS_out = (int)KS;
+  for (int b0 = 0; b0 < P.B; b0 += per) {
+    const cudaError_t e = fwd_pass(P, BB, b0, P.B - b0 < per ? P.B - b0 : per, (int)KS, skip_zeros, st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t psfsim_launch_adjoint_cols(const float *A, int64_t ld, int64_t M, int64_t K, const float *g, int B,
@@ -168,32 +311,27 @@ cudaError_t psfsim_launch_adjoint_cols(const float *A, int64_t ld, int64_t M, in
 }
 
 size_t psfsim_forward_fp32_scratch(const psfsim_plan *h, int B) {
-  return (size_t)forward_splits(h) * (size_t)B * (size_t)h->ld * 4;
+  return (size_t)psfsim_gemv_max_splits(h->ld, h->K, h->num_sms) * (size_t)B * (size_t)h->ld * 4;
 }
 
+// skip_zeros: only the columns of scene pixels that are non-zero in some scene
+// of a pass.  Without zeros the columns, their shares and so the bits are those
+// of the dense forward.
 cudaError_t psfsim_launch_forward_fp32(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
-                                       cudaStream_t st) {
-  const int KS = forward_splits(h);
+                                       bool skip_zeros, cudaStream_t st) {
   float *part = reinterpret_cast<float *>(scratch);
-  cudaError_t e = cudaSuccess;
-  int b0 = 0;
-  while (b0 < B && e == cudaSuccess) {
-    const int left = B - b0;
-    if (left >= 8) { e = fwd_group<8>(h, x, B, b0, part, KS, st); b0 += 8; }
-    else if (left >= 4) { e = fwd_group<4>(h, x, B, b0, part, KS, st); b0 += 4; }
-    else if (left >= 2) { e = fwd_group<2>(h, x, B, b0, part, KS, st); b0 += 2; }
-    else { e = fwd_group<1>(h, x, B, b0, part, KS, st); b0 += 1; }
-  }
+  int KS = 1;
+  const cudaError_t e = psfsim_launch_gemv_partials(fwd_cols(h, x, B, part),
+                                                    psfsim_gemv_max_splits(h->ld, h->K, h->num_sms), h->num_sms,
+                                                    skip_zeros, &KS, st);
   if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)((h->ld + kRedRows - 1) / kRedRows), (unsigned)B);
-  fwd_reduce_kernel<<<grid, 256, 0, st>>>(part, KS, B, h->ld, h->M, y, nullptr);
-  return cudaGetLastError();
+  return psfsim_launch_reduce_partials(part, KS, B, h->ld, h->M, y, st);
 }
 
 cudaError_t psfsim_launch_reduce_partials(const float *part, int KS, int B, int64_t ld, int64_t M, float *y,
-                                          const int *count, cudaStream_t st) {
+                                          cudaStream_t st) {
   dim3 grid((unsigned)((ld + kRedRows - 1) / kRedRows), (unsigned)B);
-  fwd_reduce_kernel<<<grid, 256, 0, st>>>(part, KS, B, ld, M, y, count);
+  fwd_reduce_kernel<<<grid, 256, 0, st>>>(part, KS, B, ld, M, y);
   return cudaGetLastError();
 }
 

@@ -8,6 +8,7 @@
 // streams 26 % of its k-tiles, 2680 -> 852 us; tiles start at multiples of 32
 // columns rather than 64 so that a narrow row needs one tile where it used to
 // touch two, and 32 columns are the 64 bytes that HBM moves at least.
+//   FP32 storage    the live columns, ascending, then the others, ascending.
 // The host counts the same tables by the same integer arithmetic, to size
 // launches without reading anything back.
 #include "live.cuh"
@@ -96,6 +97,37 @@ __global__ void __launch_bounds__(1024) ktile_table_kernel(int N, int64_t K, lon
   }
 }
 
+// FP32 storage: list[0 .. L) the live columns, list[L .. K) the others.  A CTA
+// takes kListRows scene rows; the rows before them are counted by all threads.
+constexpr int kListRows = 8;
+__global__ void __launch_bounds__(256) column_list_kernel(int N, long long R2, int64_t live_cols, int *list) {
+  __shared__ int before[8];
+  const int y0 = blockIdx.x * kListRows;
+  int a, b, n = 0;
+  for (int iy = threadIdx.x; iy < y0; iy += blockDim.x) {
+    live_row(N, R2, iy, a, b);
+    n += b - a;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+  if ((threadIdx.x & 31) == 0) before[threadIdx.x >> 5] = n;
+  __syncthreads();
+  int64_t at = 0;
+  for (int w = 0; w < 8; ++w) at += before[w];
+  for (int iy = y0; iy < y0 + kListRows && iy < N; ++iy) {
+    live_row(N, R2, iy, a, b);
+    const int64_t row = (int64_t)iy * N;
+    int *dead = list + live_cols + (row - at);  // the row's others follow the others of the rows before
+    for (int ix = threadIdx.x; ix < N; ix += blockDim.x) {
+      if (ix >= a && ix < b)
+        list[at + ix - a] = (int)(row + ix);
+      else
+        dead[ix < a ? ix : ix - (b - a)] = (int)(row + ix);
+    }
+    at += b - a;
+  }
+}
+
 }  // namespace
 
 void psfsim_live_count(psfsim_plan *h) {
@@ -103,8 +135,20 @@ void psfsim_live_count(psfsim_plan *h) {
   h->live = false;
   h->k_tiles = (int)(h->ld / 64);
   h->dead_groups = 0;
-  if (h->N < 1 || h->quadrant || !split) return;
+  h->live_cols = psfsim_cols(h);
+  if (h->N < 1 || h->quadrant) return;
   const long long R2 = live_r2(h->radii[h->n_r - 1], h->S);
+  if (!split) {
+    int64_t cols = 0;
+    for (int iy = 0; iy < h->N; ++iy) {
+      int a, b;
+      live_row(h->N, R2, iy, a, b);
+      cols += b - a;
+    }
+    h->live = cols < h->K;
+    h->live_cols = cols;
+    return;
+  }
   const int64_t groups = (h->K + kLiveGroup - 1) / kLiveGroup;
   int64_t tiles = 0, covered = 0, run0 = -1, run1 = -1;  // current run of live groups [run0, run1)
   auto close = [&] {
@@ -140,6 +184,11 @@ void psfsim_live_count(psfsim_plan *h) {
 cudaError_t psfsim_launch_live_table(psfsim_plan *h, cudaStream_t st) {
   if (!h->live) return cudaSuccess;
   int *tab = reinterpret_cast<int *>(h->ws + h->order_off);
+  if (h->storage == PSFSIM_FP32) {
+    column_list_kernel<<<(unsigned)((h->N + kListRows - 1) / kListRows), 256, 0, st>>>(
+        h->N, live_r2(h->radii[h->n_r - 1], h->S), h->live_cols, tab);
+    return cudaGetLastError();
+  }
   ktile_table_kernel<<<1, 1024, 0, st>>>(h->N, h->K, live_r2(h->radii[h->n_r - 1], h->S), tab, h->k_tiles,
                                          tab + h->k_tiles, h->dead_groups);
   return cudaGetLastError();

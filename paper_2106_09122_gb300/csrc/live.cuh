@@ -5,8 +5,7 @@
 // pixels X = 2 ix - (N - 1), Y = 2 iy - (N - 1), X^2 + Y^2 <= R2 with
 // R2 = floor((2 r_last / S)^2 (1 + 1e-9)): integers, so host and device agree
 // exactly, and a superset of the columns that the build fills (its FP64 test
-// r <= r_last errs by some 1e-15).  At least pixel 0 is live, so that no
-// product is empty.
+// r <= r_last errs by some 1e-15).
 #pragma once
 
 #include <math.h>

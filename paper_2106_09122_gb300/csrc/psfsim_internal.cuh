@@ -43,6 +43,7 @@ struct psfsim_plan {
   int64_t pix_off;  // split storage: pair entries and pixel order of the pixel-wise build (-1: another build)
   int device, num_sms;
   bool live;            // products skip the zero columns listed in the workspace (live.cu)
+  int64_t live_cols;    // FP32 storage: columns the products read (all of them when !live)
   int k_tiles;          // split storage: 64-column k-tiles the products read (ld / 64 when !live)
   int64_t dead_groups;  // split storage: 32-column groups in none of them
   int fit_ks;           // column splits of the fit-gradient forward, fixed at first use (0: not yet)
@@ -77,19 +78,14 @@ cudaError_t psfsim_launch_live_table(psfsim_plan *h, cudaStream_t st);
 
 // Kernel launchers (return cudaError_t of the launch).
 cudaError_t psfsim_launch_build(psfsim_plan *h, cudaStream_t st);
-cudaError_t psfsim_launch_forward_fp32(const psfsim_plan *h, const float *x, int B, float *y,
-                                       void *scratch, cudaStream_t st);
+cudaError_t psfsim_launch_forward_fp32(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
+                                       bool skip_zeros, cudaStream_t st);
 size_t psfsim_forward_fp32_scratch(const psfsim_plan *h, int B);
-// FP32 forward over the scene pixels that are non-zero in some scene of the batch.
-size_t psfsim_forward_sparse_scratch(const psfsim_plan *h, int B);
-cudaError_t psfsim_launch_forward_sparse(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
-                                         cudaStream_t st);
 cudaError_t psfsim_launch_adjoint_fp32(const psfsim_plan *h, const float *g, int B, float *gx,
                                        cudaStream_t st);
 // y[b, i] = sum_ks part[(ks * B + b) * ld + i], fixed order.
-// Slots b >= *count (when count is not NULL) are skipped.
 cudaError_t psfsim_launch_reduce_partials(const float *part, int KS, int B, int64_t ld, int64_t M, float *y,
-                                          const int *count, cudaStream_t st);
+                                          cudaStream_t st);
 // Split-BF16 storage: build, tensor-core forward, CUDA-core adjoint.
 cudaError_t psfsim_launch_split_build(psfsim_plan *h, cudaStream_t st);
 size_t psfsim_forward_tc_scratch(const psfsim_plan *h, int B);
@@ -117,10 +113,24 @@ int psfsim_multi_validate(const psfsim_job_t *jobs, int njobs);
 size_t psfsim_forward_multi_scratch(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune);
 cudaError_t psfsim_launch_forward_multi(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune,
                                         void *scratch, cudaStream_t st);
-// Generic FP32 GEMV pieces (column-major A) used by several storages.
-int psfsim_gemv_splits(int64_t ld, int64_t K, int num_sms);
-cudaError_t psfsim_launch_gemv_partials(const float *A, int64_t ld, int64_t K, const float *x, int B, float *part,
-                                        int KS, cudaStream_t st);
+// FP32 forward products (column-major A, gemv.cu): partial images part[KS][B][ld].
+struct FwdCols {
+  const float *A;
+  int64_t ld;
+  const float *x;     // [B][K] scenes (or whole scenes whose rotations are the batch, see order)
+  int64_t K;          // scene pixels
+  const int *live;    // columns read, ascending (NULL: all)
+  int64_t L;          // how many
+  const int *dead;    // the other columns: zero in A, but a non-finite scene value there makes the image NaN
+  int64_t D;
+  const int *order;   // compact storage: quadrant pixel of every column; scene b / 4 turned b % 4 times is slot b
+  int N;
+  int B;
+  float *part;
+};
+int psfsim_gemv_max_splits(int64_t ld, int64_t K, int num_sms);  // sizes the caller's scratch
+cudaError_t psfsim_launch_gemv_partials(const FwdCols &P, int max_splits, int num_sms, bool skip_zeros, int *KS,
+                                        cudaStream_t st);
 cudaError_t psfsim_launch_adjoint_cols(const float *A, int64_t ld, int64_t M, int64_t K, const float *g, int B,
                                        float *gx, int num_sms, cudaStream_t st);
 // FP32 storage compacted by the quarter-turn symmetry and zero columns.

@@ -8,8 +8,8 @@
 // Forward:  S = sum_{m=0..3} P^m (A_Q0 X^(m)),  X^(m)_t = x_{R^m(j_t)};
 // adjoint:  (A^T g)_{R^m(j_t)} = (A_Q0^T (g o P^m))_t.
 // Both reuse the FP32 GEMV kernels on the compact matrix (K_valid columns)
-// with the four rotations as a batch of four; gather / permutation kernels
-// around them carry the symmetry.  Results equal the dense FP32 path up to
+// with the four rotations as a batch of four; the forward gathers them itself,
+// and permutation kernels carry the symmetry on the image side.  Results equal the dense FP32 path up to
 // the order of the FP32 sums.
 #include "psfsim_internal.cuh"
 
@@ -34,38 +34,6 @@ __device__ __forceinline__ int64_t perm_pixel(int n, int m, int64_t i) {
   return (int64_t)p * n + q;
 }
 
-// xc[(b*4 + m) * Kv + t] = x[b][R^m(order[t])]
-__global__ void sym_gather(const float *__restrict__ x, int B, int N, int64_t Kv, const int *__restrict__ order,
-                           float *__restrict__ xc) {
-  const int H = N / 2;
-  const int64_t total = (int64_t)B * 4 * Kv;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int bm = (int)(idx / Kv);
-    const int64_t t = idx % Kv;
-    const int b = bm >> 2, m = bm & 3;
-    const int j0 = order[t];
-    int ix = H + j0 % H, iy = H + j0 / H;
-    rotate_pixel(N, m, ix, iy);
-    xc[idx] = x[(int64_t)b * N * N + (int64_t)iy * N + ix];
-  }
-}
-
-// y[b][i] = sum_m v[b*4+m][P^-m(i)]  (fixed order; v already reduced over k-splits).
-__global__ void sym_permsum(const float *__restrict__ v, int B, int n, float *__restrict__ y) {
-  const int64_t M = (int64_t)n * n;
-  const int64_t total = (int64_t)B * M;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(idx / M);
-    const int64_t i = idx % M;
-    float s = 0.f;
-#pragma unroll
-    for (int m = 0; m < 4; ++m) s += v[(int64_t)(b * 4 + m) * M + perm_pixel(n, (4 - m) & 3, i)];  // P^-m = P^(4-m)
-    y[idx] = s;
-  }
-}
-
 // y[b][i] = sum_m sum_ks part_m[ks][P^-m(i)] (fixed order), one 32 x 32 pixel
 // block of an image per CTA: the quarter and three-quarter turns are read along
 // their own rows and transposed through shared memory, so every access is a run
@@ -85,6 +53,7 @@ __global__ void __launch_bounds__(kSumThreads) sym_sum_kernel(const __grid_const
   const int64_t step = (int64_t)S.cap[blk] * S.rows;
   const float *v = S.part[blk] + (int64_t)slot * S.rows;
   float acc[kPer][4] = {};
+#pragma unroll 4
   for (int ks = 0; ks < S.KS[blk]; ++ks, v += step) {
 #pragma unroll
     for (int e = 0; e < kPer; ++e) {
@@ -146,10 +115,10 @@ unsigned grid_for(int64_t total, int num_sms) {
   return (unsigned)(g < 1 ? 1 : (g < cap ? g : cap));
 }
 
-// K-splits for the compact GEMV: enough CTAs to fill the GPU, but partial sums
-// kept well below the bytes of the compact A (at least 64 columns per split).
+// K-splits for the compact GEMV: partial sums kept well below the bytes of the
+// compact A (at least 64 columns per split).
 int sym_splits(const psfsim_plan *h) {
-  int ks = psfsim_gemv_splits(h->ld, h->K_valid, h->num_sms);
+  const int ks = psfsim_gemv_max_splits(h->ld, h->K_valid, h->num_sms);
   const int64_t cap = h->K_valid / 64 > 0 ? h->K_valid / 64 : 1;
   return ks < cap ? ks : (int)cap;
 }
@@ -163,28 +132,35 @@ cudaError_t psfsim_launch_sym_sum(const SymSum &S, int B, float *y, cudaStream_t
 }
 
 size_t psfsim_forward_sym_scratch(const psfsim_plan *h, int B) {
-  const size_t xc = (size_t)psfsim_round_up((int64_t)4 * B * h->K_valid * 4, 256);
-  const size_t v = (size_t)psfsim_round_up((int64_t)4 * B * h->M * 4, 256);
-  return xc + v + (size_t)sym_splits(h) * 4 * B * h->ld * 4;
+  return (size_t)sym_splits(h) * 4 * B * h->ld * 4;
 }
 
+// Two launches: the product over the four rotations of every scene, gathered
+// by the product itself, and the sum over splits and rotations.
 cudaError_t psfsim_launch_forward_sym(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
                                       cudaStream_t st) {
-  const int *order = reinterpret_cast<const int *>(h->ws + h->order_off);
-  const float *A = reinterpret_cast<const float *>(h->ws + h->a_off);
-  float *xc = static_cast<float *>(scratch);
-  float *v = reinterpret_cast<float *>(static_cast<char *>(scratch) +
-                                       psfsim_round_up((int64_t)4 * B * h->K_valid * 4, 256));
-  float *part = reinterpret_cast<float *>(reinterpret_cast<char *>(v) + psfsim_round_up((int64_t)4 * B * h->M * 4, 256));
-  const int KS = sym_splits(h);
   if (h->K_valid == 0) return cudaMemsetAsync(y, 0, (size_t)B * h->M * 4, st);
-  sym_gather<<<grid_for((int64_t)4 * B * h->K_valid, h->num_sms), 256, 0, st>>>(x, B, h->N, h->K_valid, order, xc);
-  cudaError_t e = cudaGetLastError();
+  FwdCols P = {};
+  P.A = reinterpret_cast<const float *>(h->ws + h->a_off);
+  P.ld = h->ld;
+  P.x = x;
+  P.K = h->K;
+  P.L = h->K_valid;
+  P.order = reinterpret_cast<const int *>(h->ws + h->order_off);
+  P.N = h->N;
+  P.B = 4 * B;
+  P.part = static_cast<float *>(scratch);
+  int KS = 1;
+  const cudaError_t e = psfsim_launch_gemv_partials(P, sym_splits(h), h->num_sms, false, &KS, st);
   if (e != cudaSuccess) return e;
-  if ((e = psfsim_launch_gemv_partials(A, h->ld, h->K_valid, xc, 4 * B, part, KS, st)) != cudaSuccess) return e;
-  if ((e = psfsim_launch_reduce_partials(part, KS, 4 * B, h->ld, h->M, v, nullptr, st)) != cudaSuccess) return e;
-  sym_permsum<<<grid_for((int64_t)B * h->M, h->num_sms), 256, 0, st>>>(v, B, h->n, y);
-  return cudaGetLastError();
+  SymSum S = {};
+  S.part[0] = P.part;
+  S.cap[0] = P.B;
+  S.KS[0] = KS;
+  S.per = P.B;
+  S.rows = h->ld;
+  S.n = h->n;
+  return psfsim_launch_sym_sum(S, B, y, st);
 }
 
 size_t psfsim_adjoint_sym_scratch(const psfsim_plan *h, int B) {

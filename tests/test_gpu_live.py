@@ -23,27 +23,45 @@ def _plan(N, S, r_last, storage, n=20, n_r=5, seed=5):
     return plan, O.build_A(lib.astype(np.float64), radii, N, S), rng
 
 
-@pytest.mark.parametrize("storage,tol", [("split_bf16", 1e-5), ("bf16", 2.0 ** -8 + 2.5e-5)])
-@pytest.mark.parametrize("N,S,r_last", GRIDS)
-def test_forward_skips_only_zero_columns(N, S, r_last, storage, tol):
-    plan, A, rng = _plan(N, S, r_last, storage)
-    x = rng.uniform(0.0, 1.0, (3, N * N)).astype(np.float32)
-    y = plan.forward(torch.from_numpy(x).to(DEV)).double().cpu().numpy()
+def _check_forward(plan, A, x, tol, **kw):
+    y = plan.forward(torch.from_numpy(x).to(DEV), **kw).double().cpu().numpy()
     x64 = x.astype(np.float64)
     err = O.bound_relative_error(y, x64 @ A.T, x64 @ np.abs(A).T, floor=O.FLT_MIN).max()
     assert err <= tol and plan.sync_status() == 0, err
 
 
-@pytest.mark.parametrize("storage", ["split_bf16", "bf16"])
+@pytest.mark.parametrize("storage,tol", [("split_bf16", 1e-5), ("bf16", 2.0 ** -8 + 2.5e-5), ("fp32", 1e-5)])
+@pytest.mark.parametrize("N,S,r_last", GRIDS)
+def test_forward_skips_only_zero_columns(N, S, r_last, storage, tol):
+    plan, A, rng = _plan(N, S, r_last, storage)
+    _check_forward(plan, A, rng.uniform(0.0, 1.0, (3, N * N)).astype(np.float32), tol)
+
+
+@pytest.mark.parametrize("B", [1, 2, 4, 5, 8, 9, 12, 13, 16, 17, 33])
+@pytest.mark.parametrize("storage", ["fp32", "fp32_sym"])
+def test_fp32_forward_batches(B, storage):
+    """Every group width of the batched product, its remainders, and the filter for zero pixels;
+    an odd image (row quads cut at the end), more than one 256-column chunk per share."""
+    plan, A, rng = _plan(64, 0.125, 4.0, storage, n=17)
+    x = rng.uniform(0.0, 1.0, (B, 64 * 64)).astype(np.float32)
+    x[:, rng.uniform(size=64 * 64) < 0.7] = 0.0
+    _check_forward(plan, A, x, 1e-5)
+    if storage == "fp32":
+        _check_forward(plan, A, x, 1e-5, skip_zeros=True)
+
+
+@pytest.mark.parametrize("storage,kw", [("split_bf16", {}), ("bf16", {}), ("fp32", {}), ("fp32", {"skip_zeros": True})])
 @pytest.mark.parametrize("value", [float("nan"), float("inf"), -float("inf")])
-def test_non_finite_scene_value_at_a_skipped_column(storage, value):
+def test_non_finite_scene_value_at_a_skipped_column(storage, kw, value):
     plan, A, rng = _plan(64, 0.5, 4.0, storage)
     dead = np.nonzero(~A.any(axis=0))[0]
     for j in (dead[0], dead[len(dead) // 2], dead[-1]):
         x = rng.uniform(0.0, 1.0, (2, 64 * 64)).astype(np.float32)
         x[1, j] = value
-        y = plan.forward(torch.from_numpy(x).to(DEV)).cpu().numpy()
+        y = plan.forward(torch.from_numpy(x).to(DEV), **kw).cpu().numpy()
         assert np.isfinite(y[0]).all() and np.isnan(y[1]).all()
+        y = plan.forward(torch.from_numpy(x[1]).to(DEV), **kw).cpu().numpy()
+        assert np.isnan(y).all()
 
 
 @pytest.mark.parametrize("storage", ["split_bf16", "bf16"])

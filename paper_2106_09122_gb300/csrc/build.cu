@@ -569,7 +569,7 @@ static cudaError_t launch_tables_and_build(psfsim_plan *h, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   geom_kernel<<<(unsigned)((Kg + 255) / 256), 256, 0, st>>>(G, geom);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (!(sym && dense_split && h->pix_off < 0)) {
+  if (!dense_split || (sym && h->pix_off >= 0)) {
     // chunks of at least 256 columns, and as many as fit in shared memory
     const int nb = psfsim_num_buckets(h->n_r);
     int W = (int)((Kg + 255) / 256);
@@ -582,7 +582,7 @@ static cudaError_t launch_tables_and_build(psfsim_plan *h, cudaStream_t st) {
       return e;
     bracket_sort_kernel<<<1, 1024, smem, st>>>(geom, Kg, h->n_r, W, order, bstart);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (sym && dense_split) {
+    if (dense_split) {
       angle_sort_kernel<<<h->n_r - 1, 1024, 0, st>>>(geom, h->n_r, order, bstart);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

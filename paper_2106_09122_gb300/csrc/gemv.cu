@@ -157,8 +157,9 @@ __global__ void __launch_bounds__(kFwdThreads, fwd_min_ctas(BB)) fwd_cols_kernel
 // its 8 warps split the KS partials (ks = warp, warp + 8, ...) and combine
 // through shared memory, so every output needs only ~KS/8 loads per thread.
 constexpr int kRedRows = 128;
-__global__ void __launch_bounds__(256) fwd_reduce_kernel(const float *__restrict__ part, int KS, int B,
-                                                         int64_t ld, int64_t M, float *__restrict__ y) {
+// y may be part itself with M = ld: a CTA reads its rows before it writes them.
+__global__ void __launch_bounds__(256) fwd_reduce_kernel(const float *part, int KS, int B, int64_t ld, int64_t M,
+                                                         float *y) {
   __shared__ float4 red[8][32];
   const int c4 = threadIdx.x & 31, grp = threadIdx.x >> 5;
   const int64_t r = ((int64_t)blockIdx.x * 32 + c4) * 4;
@@ -191,13 +192,205 @@ __global__ void __launch_bounds__(256) fwd_reduce_kernel(const float *__restrict
   }
 }
 
-// gx[b, j] = sum_i A[i, j] g[b, i]; CTA c owns the contiguous column range
-// [K c / G, K (c+1) / G).
-template <int BB, bool kVec>
-__global__ void __launch_bounds__(kAdjThreads) adj_kernel(const float *__restrict__ A, int64_t ld, int64_t M,
-                                                          int64_t K, const float *__restrict__ g, int b0,
-                                                          float *__restrict__ gx) {
-  adj_columns<BB, kVec>(A, ld, M, K, g, b0, gx, K * blockIdx.x / gridDim.x, K * (blockIdx.x + 1) / gridDim.x);
+// One residual: gx[j] = sum_i A[i, j] g[i] for the CTA's contiguous range of the
+// live columns; the CTA's 256 threads split the rows (float4 strided), reduce in
+// registers, then across warps through a double-buffered shared array.  Fixed
+// assignment and order: deterministic.  The columns that are not read get zero,
+// or NaN when some residual value is not finite (0 x inf), which the first
+// column's pass over g finds out.
+template <bool kVec>
+__global__ void __launch_bounds__(kAdjThreads) adj_kernel(const AdjCols P, int b0) {
+  __shared__ float red[2][kAdjThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t t0 = P.L * blockIdx.x / gridDim.x, t1 = P.L * (blockIdx.x + 1) / gridDim.x;
+  const float *g = P.g + (int64_t)b0 * P.M;
+  float *gx = P.gx + (int64_t)b0 * P.K;
+  int parity = 0;
+  float zero = 0.f;  // 0, or NaN from this thread's rows
+  for (int64_t t = t0; t < t1; ++t, parity ^= 1) {
+    const int64_t j = P.live ? P.live[t] : t;
+    const float *col = P.A + j * P.ld;
+    const bool probe = P.dead && t == t0;
+    float acc = 0.f;
+    auto add = [&](const float4 &v, const float4 &gv) {
+      acc = fmaf(v.x, gv.x, acc);
+      acc = fmaf(v.y, gv.y, acc);
+      acc = fmaf(v.z, gv.z, acc);
+      acc = fmaf(v.w, gv.w, acc);
+      if (probe) zero += 0.f * gv.x + 0.f * gv.y + 0.f * gv.z + 0.f * gv.w;
+    };
+    if (kVec) {
+      const int64_t M4 = P.M >> 2;
+      const float4 *g4 = reinterpret_cast<const float4 *>(g);
+      int64_t i4 = threadIdx.x;
+      constexpr int T = kAdjThreads;
+      for (; i4 + 3 * T < M4; i4 += 4 * T) {
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = ld_stream4(col + 4 * (i4 + T * u));
+#pragma unroll
+        for (int u = 0; u < 4; ++u) add(v[u], __ldg(g4 + i4 + T * u));
+      }
+      for (; i4 < M4; i4 += T) add(ld_stream4(col + 4 * i4), __ldg(g4 + i4));
+    } else {
+      for (int64_t i = threadIdx.x; i < P.M; i += kAdjThreads) {
+        const float gi = __ldg(g + i);
+        acc = fmaf(__ldg(col + i), gi, acc);
+        if (probe) zero += 0.f * gi;
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) red[parity][warp] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      float s = red[parity][0];
+#pragma unroll
+      for (int w = 1; w < kAdjThreads / 32; ++w) s += red[parity][w];
+      gx[j] = s;
+    }
+  }
+  if (!P.dead) return;
+  if (t0 == t1)  // no column of its own to look at g with
+    for (int64_t i = threadIdx.x; i < P.M; i += kAdjThreads) zero += 0.f * g[i];
+  const bool bad = __syncthreads_or(zero != 0.f);
+  const int64_t d0 = P.D * blockIdx.x / gridDim.x, d1 = P.D * (blockIdx.x + 1) / gridDim.x;
+  for (int64_t e = d0 + threadIdx.x; e < d1; e += kAdjThreads) gx[P.dead[e]] = bad ? __int_as_float(0x7fffffff) : 0.f;
+}
+
+// Several residuals: a CTA owns a contiguous range of the live columns (at most
+// kAdjCols at a time) and walks the rows in tiles of 2048, eight rows a thread,
+// with the tile's BB residuals in registers, two columns in hand at once.  Their
+// 2 BB sums are halved across the warp's lanes until each group of lanes holds
+// one, which it adds to its place in shared memory.  Bound by reading A once per
+// BB residuals, then by issue: the more rows a thread has, the less the exchange
+// of its sums weighs (with four rows a thread and 32 sums it took as long as the
+// FMAs, 122 us for 8 residuals of the 128^2 plan; 102 now).  Reading the residuals from
+// L2 per column instead moved eight times A's bytes: 320 us.
+constexpr int kAdjCols = 64;
+__host__ __device__ constexpr int adj_min_ctas(int BB) { return BB == 8 ? 2 : 3; }
+
+template <int BB>
+__global__ void __launch_bounds__(kAdjThreads, adj_min_ctas(BB)) adj_batch_kernel(const AdjCols P, int b0, int nb) {
+  constexpr int R = 2;                        // row quads a thread holds
+  constexpr int kTile = 4 * R * kAdjThreads;  // rows per tile
+  constexpr int S = 2 * BB, kLanes = 32 / S;  // sums in hand; lanes that end with the same one
+  __shared__ float red[kAdjThreads / 32][kAdjCols * BB];
+  __shared__ int js[kAdjCols];
+  __shared__ unsigned bad;  // residuals with a non-finite value
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t t0 = P.L * blockIdx.x / gridDim.x, t1 = P.L * (blockIdx.x + 1) / gridDim.x;
+  const bool vec = P.M % 4 == 0 && (reinterpret_cast<uintptr_t>(P.g) & 15) == 0;
+  if (threadIdx.x == 0) bad = 0u;
+  unsigned mine = 0u;
+  bool probe = P.dead != nullptr;
+  for (int64_t p0 = t0; p0 < t1 || probe; p0 += kAdjCols) {
+    const int cols = (int)(t1 - p0 < kAdjCols ? t1 - p0 : kAdjCols);
+    if ((int)threadIdx.x < cols) js[threadIdx.x] = P.live ? P.live[p0 + threadIdx.x] : (int)(p0 + threadIdx.x);
+    __syncthreads();
+    // The thread's row quad h of a tile is r0 + 1024 h + 4 threadIdx.x.  A's
+    // padding rows are zero and allocated up to ld, a multiple of 32.
+    auto load_a = [&](int64_t r0, int q, float4 (&v)[2][R]) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const bool take = q + c < cols;
+        const float *col = P.A + (int64_t)js[take ? q + c : 0] * P.ld + 4 * threadIdx.x;
+#pragma unroll
+        for (int h = 0; h < R; ++h) {
+          const int64_t r = r0 + h * 4 * kAdjThreads;
+          v[c][h] = ld_stream4_if(col + r, take && r + 4 * threadIdx.x < P.M);
+        }
+      }
+    };
+    float4 v[2][R], gv[BB][R];
+    if (cols > 0) load_a(0, 0, v);
+    for (int64_t r0 = 0; r0 < P.M; r0 += kTile) {
+#pragma unroll
+      for (int h = 0; h < R; ++h) {
+        const int64_t r = r0 + h * 4 * kAdjThreads + 4 * threadIdx.x;
+#pragma unroll
+        for (int b = 0; b < BB; ++b) {
+          gv[b][h] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (b < nb && r < P.M) {
+            const float *gb = P.g + (int64_t)(b0 + b) * P.M + r;
+            if (vec) {
+              gv[b][h] = __ldg(reinterpret_cast<const float4 *>(gb));
+            } else {
+              gv[b][h].x = gb[0];
+              if (r + 1 < P.M) gv[b][h].y = gb[1];
+              if (r + 2 < P.M) gv[b][h].z = gb[2];
+              if (r + 3 < P.M) gv[b][h].w = gb[3];
+            }
+          }
+        }
+      }
+      if (probe)
+#pragma unroll
+        for (int b = 0; b < BB; ++b)
+#pragma unroll
+          for (int h = 0; h < R; ++h)
+            if (!(isfinite(gv[b][h].x) && isfinite(gv[b][h].y) && isfinite(gv[b][h].z) && isfinite(gv[b][h].w)))
+              mine |= 1u << b;
+      for (int q = 0; q < cols; q += 2) {
+        float s[S];
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int b = 0; b < BB; ++b) {
+            float t = 0.f;
+#pragma unroll
+            for (int h = 0; h < R; ++h) {
+              t = fmaf(v[c][h].x, gv[b][h].x, t);
+              t = fmaf(v[c][h].y, gv[b][h].y, t);
+              t = fmaf(v[c][h].z, gv[b][h].z, t);
+              t = fmaf(v[c][h].w, gv[b][h].w, t);
+            }
+            s[c * BB + b] = t;
+          }
+        // The next columns load while these sums are exchanged.
+        if (q + 2 < cols)
+          load_a(r0, q + 2, v);
+        else if (r0 + kTile < P.M)
+          load_a(r0 + kTile, 0, v);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          const int o = 16 >> k, n = S >> (k + 1);
+          if (n > 0) {  // a lane keeps the half of its sums that its bit o names
+#pragma unroll
+            for (int i = 0; i < BB; ++i)
+              if (i < n) {
+                const bool up = lane & o;
+                const float keep = up ? s[i + n] : s[i], give = up ? s[i] : s[i + n];
+                s[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+              }
+          } else {
+            s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+          }
+        }
+        if (lane % kLanes == 0) {  // sum lane / kLanes: column q + sum / BB, residual sum % BB
+          float *slot = &red[warp][q * BB + lane / kLanes];
+          *slot = r0 == 0 ? s[0] : *slot + s[0];
+        }
+      }
+    }
+    __syncthreads();
+    for (int o = threadIdx.x; o < cols * BB; o += kAdjThreads) {
+      const int b = o % BB;
+      float s = red[0][o];
+#pragma unroll
+      for (int w = 1; w < kAdjThreads / 32; ++w) s += red[w][o];
+      if (b < nb) P.gx[(int64_t)(b0 + b) * P.K + js[o / BB]] = s;
+    }
+    probe = false;
+    __syncthreads();
+  }
+  if (!P.dead) return;
+  if (mine) atomicOr(&bad, mine);
+  __syncthreads();
+  const int64_t d0 = P.D * blockIdx.x / gridDim.x, d1 = P.D * (blockIdx.x + 1) / gridDim.x;
+  for (int64_t e = d0 + threadIdx.x; e < d1; e += kAdjThreads)
+    for (int b = 0; b < nb; ++b)
+      P.gx[(int64_t)(b0 + b) * P.K + P.dead[e]] = bad >> b & 1u ? __int_as_float(0x7fffffff) : 0.f;
 }
 
 // One pass: nb scenes from b0 with KS splits.
@@ -238,19 +431,6 @@ FwdCols fwd_cols(const psfsim_plan *h, const float *x, int B, float *part) {
   return P;
 }
 
-template <int BB>
-cudaError_t adj_group(const psfsim_plan *h, const float *g, int b0, float *gx, bool vec, cudaStream_t st) {
-  const float *A = reinterpret_cast<const float *>(h->ws + h->a_off);
-  auto kern = vec ? adj_kernel<BB, true> : adj_kernel<BB, false>;
-  int per_sm = 1;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kAdjThreads, 0);
-  if (e != cudaSuccess) return e;
-  int64_t grid = (int64_t)h->num_sms * (per_sm < 1 ? 1 : per_sm);
-  if (grid > h->K) grid = h->K;
-  kern<<<(unsigned)grid, kAdjThreads, 0, st>>>(A, h->ld, h->M, h->K, g, b0, gx);
-  return cudaGetLastError();
-}
-
 }  // namespace
 
 // Column splits the scratch of a forward allows: eight CTAs an SM over the row
@@ -283,29 +463,29 @@ cudaError_t psfsim_launch_gemv_partials(const FwdCols &P, int max_splits, int nu
   return cudaSuccess;
 }
 
-cudaError_t psfsim_launch_adjoint_cols(const float *A, int64_t ld, int64_t M, int64_t K, const float *g, int B,
-                                       float *gx, int num_sms, cudaStream_t st) {
-  const bool vec = (M % 4 == 0) && ((reinterpret_cast<uintptr_t>(g) & 15) == 0);
-  int b0 = 0;
-  while (b0 < B) {
-    const int left = B - b0;
-    const int bb = left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
-    auto launch = [&](auto kern) -> cudaError_t {
-      int per_sm = 1;
-      cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kAdjThreads, 0);
-      if (e != cudaSuccess) return e;
-      int64_t grid = (int64_t)num_sms * (per_sm < 1 ? 1 : per_sm);
-      if (grid > K) grid = K;
-      kern<<<(unsigned)grid, kAdjThreads, 0, st>>>(A, ld, M, K, g, b0, gx);
-      return cudaGetLastError();
-    };
-    cudaError_t e;
-    if (bb == 8) e = vec ? launch(adj_kernel<8, true>) : launch(adj_kernel<8, false>);
-    else if (bb == 4) e = vec ? launch(adj_kernel<4, true>) : launch(adj_kernel<4, false>);
-    else if (bb == 2) e = vec ? launch(adj_kernel<2, true>) : launch(adj_kernel<2, false>);
-    else e = vec ? launch(adj_kernel<1, true>) : launch(adj_kernel<1, false>);
+// One residual at a time, or passes of 2 to 8.
+cudaError_t psfsim_launch_adjoint_cols(const AdjCols &P, int num_sms, cudaStream_t st) {
+  if (P.B == 1) {
+    const bool vec = (P.M % 4 == 0) && ((reinterpret_cast<uintptr_t>(P.g) & 15) == 0);
+    auto kern = vec ? adj_kernel<true> : adj_kernel<false>;
+    int per_sm = 1;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kAdjThreads, 0);
     if (e != cudaSuccess) return e;
-    b0 += bb;
+    int64_t grid = (int64_t)num_sms * (per_sm < 1 ? 1 : per_sm);
+    grid = grid < P.L ? grid : P.L;
+    kern<<<(unsigned)(grid < 1 ? 1 : grid), kAdjThreads, 0, st>>>(P, 0);
+    return cudaGetLastError();
+  }
+  const int passes = (P.B + 7) / 8, per = (P.B + passes - 1) / passes;
+  for (int b0 = 0; b0 < P.B; b0 += per) {
+    const int nb = P.B - b0 < per ? P.B - b0 : per;
+    const int per_sm = adj_min_ctas(nb <= 4 ? 4 : 8);
+    auto kern = nb <= 4 ? adj_batch_kernel<4> : adj_batch_kernel<8>;
+    int64_t grid = (P.L + 1) / 2;
+    grid = grid < (int64_t)per_sm * num_sms ? grid : (int64_t)per_sm * num_sms;
+    kern<<<(unsigned)(grid < 1 ? 1 : grid), kAdjThreads, 0, st>>>(P, b0, nb);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
@@ -336,15 +516,18 @@ cudaError_t psfsim_launch_reduce_partials(const float *part, int KS, int B, int6
 }
 
 cudaError_t psfsim_launch_adjoint_fp32(const psfsim_plan *h, const float *g, int B, float *gx, cudaStream_t st) {
-  const bool vec = (h->M % 4 == 0) && ((reinterpret_cast<uintptr_t>(g) & 15) == 0);
-  cudaError_t e = cudaSuccess;
-  int b0 = 0;
-  while (b0 < B && e == cudaSuccess) {
-    const int left = B - b0;
-    if (left >= 8) { e = adj_group<8>(h, g, b0, gx, vec, st); b0 += 8; }
-    else if (left >= 4) { e = adj_group<4>(h, g, b0, gx, vec, st); b0 += 4; }
-    else if (left >= 2) { e = adj_group<2>(h, g, b0, gx, vec, st); b0 += 2; }
-    else { e = adj_group<1>(h, g, b0, gx, vec, st); b0 += 1; }
-  }
-  return e;
+  const int *list = reinterpret_cast<const int *>(h->ws + h->order_off);
+  AdjCols P;
+  P.A = reinterpret_cast<const float *>(h->ws + h->a_off);
+  P.ld = h->ld;
+  P.M = h->M;
+  P.g = g;
+  P.gx = gx;
+  P.K = h->K;
+  P.live = h->live ? list : nullptr;
+  P.L = h->live_cols;
+  P.dead = h->live ? list + h->live_cols : nullptr;
+  P.D = h->K - h->live_cols;
+  P.B = B;
+  return psfsim_launch_adjoint_cols(P, h->num_sms, st);
 }

@@ -97,12 +97,12 @@ cudaError_t psfsim_launch_forward_tc_sym(const psfsim_plan *h, const float *x, i
 // q = 4 b + m is slot q % per of block q / per, whose partials are
 // part[KS][cap][rows]; y[b][i] = sum_m sum_ks part at P^-m(i).
 struct SymSum {
-  const float *part[16];
+  const float *part[16];  // the caller's scratch: several splits are added in place
   int cap[16], KS[16];
   int per, n;
   int64_t rows;
 };
-cudaError_t psfsim_launch_sym_sum(const SymSum &S, int B, float *y, cudaStream_t st);
+cudaError_t psfsim_launch_sym_sum(SymSum S, int B, float *y, cudaStream_t st);
 size_t psfsim_adjoint_split_scratch(const psfsim_plan *h, int B);
 // Test hook: the tensor-core forward of <= 80 scenes on one CTA with every
 // wait bounded by wait_ns and load number stall_it never issued.
@@ -131,8 +131,20 @@ struct FwdCols {
 int psfsim_gemv_max_splits(int64_t ld, int64_t K, int num_sms);  // sizes the caller's scratch
 cudaError_t psfsim_launch_gemv_partials(const FwdCols &P, int max_splits, int num_sms, bool skip_zeros, int *KS,
                                         cudaStream_t st);
-cudaError_t psfsim_launch_adjoint_cols(const float *A, int64_t ld, int64_t M, int64_t K, const float *g, int B,
-                                       float *gx, int num_sms, cudaStream_t st);
+// FP32 adjoint products: gx[b][column] = sum_i A[i, column] g[b][i].
+struct AdjCols {
+  const float *A;
+  int64_t ld, M;
+  const float *g;     // [B][M]
+  float *gx;          // [B][K]
+  int64_t K;
+  const int *live;    // columns read, ascending (NULL: all)
+  int64_t L;
+  const int *dead;    // the other columns: zero, or NaN for a residual that is not finite everywhere
+  int64_t D;
+  int B;
+};
+cudaError_t psfsim_launch_adjoint_cols(const AdjCols &P, int num_sms, cudaStream_t st);
 // FP32 storage compacted by the quarter-turn symmetry and zero columns.
 size_t psfsim_forward_sym_scratch(const psfsim_plan *h, int B);
 cudaError_t psfsim_launch_forward_sym(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,

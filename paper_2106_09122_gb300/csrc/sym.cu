@@ -81,16 +81,19 @@ __global__ void __launch_bounds__(kSumThreads) sym_sum_kernel(const __grid_const
   }
 }
 
-// gp[(b*4 + m) * M + i] = g[b][P^m(i)]
-__global__ void sym_gperm(const float *__restrict__ g, int B, int n, float *__restrict__ gp) {
+// gp[(b*4 + m) * M + i] = g[b][P^m(i)]; and gx (nz values) = 0, for the scene
+// pixels without a column.
+__global__ void sym_gperm(const float *__restrict__ g, int B, int n, float *__restrict__ gp, float *__restrict__ gx,
+                          int64_t nz) {
   const int64_t M = (int64_t)n * n;
   const int64_t total = (int64_t)B * 4 * M;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t idx = first; idx < total; idx += stride) {
     const int bm = (int)(idx / M);
     const int64_t i = idx % M;
     gp[idx] = g[(int64_t)(bm >> 2) * M + perm_pixel(n, bm & 3, i)];
   }
+  for (int64_t j = first; j < nz; j += stride) gx[j] = 0.f;
 }
 
 // gx[b][R^m(order[t])] = gc[(b*4 + m) * Kv + t]; every other scene pixel is zero.
@@ -125,7 +128,17 @@ int sym_splits(const psfsim_plan *h) {
 
 }  // namespace
 
-cudaError_t psfsim_launch_sym_sum(const SymSum &S, int B, float *y, cudaStream_t st) {
+// Several k-splits are added first, in place, by the reduction that spreads them
+// over a CTA's warps: 28 splits of one image's four rotations (16 CTAs here) took
+// 60 us in this kernel's own loop, which keeps at most two.
+cudaError_t psfsim_launch_sym_sum(SymSum S, int B, float *y, cudaStream_t st) {
+  for (int blk = 0; blk * S.per < 4 * B; ++blk)
+    if (S.KS[blk] > 2) {
+      float *part = const_cast<float *>(S.part[blk]);
+      const cudaError_t e = psfsim_launch_reduce_partials(part, S.KS[blk], S.cap[blk], S.rows, S.rows, part, st);
+      if (e != cudaSuccess) return e;
+      S.KS[blk] = 1;
+    }
   const unsigned t = (unsigned)((S.n + 31) / 32);
   sym_sum_kernel<<<dim3(t, t, (unsigned)B), kSumThreads, 0, st>>>(S, y);
   return cudaGetLastError();
@@ -173,12 +186,19 @@ cudaError_t psfsim_launch_adjoint_sym(const psfsim_plan *h, const float *g, int 
   const float *A = reinterpret_cast<const float *>(h->ws + h->a_off);
   float *gp = static_cast<float *>(scratch);
   float *gc = reinterpret_cast<float *>(static_cast<char *>(scratch) + psfsim_round_up((int64_t)4 * B * h->M * 4, 256));
-  cudaError_t e = cudaMemsetAsync(gx, 0, (size_t)B * h->K * 4, st);
-  if (e != cudaSuccess || h->K_valid == 0) return e;
-  sym_gperm<<<grid_for((int64_t)4 * B * h->M, h->num_sms), 256, 0, st>>>(g, B, h->n, gp);
+  if (h->K_valid == 0) return cudaMemsetAsync(gx, 0, (size_t)B * h->K * 4, st);
+  cudaError_t e;
+  sym_gperm<<<grid_for((int64_t)4 * B * h->M, h->num_sms), 256, 0, st>>>(g, B, h->n, gp, gx, (int64_t)B * h->K);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = psfsim_launch_adjoint_cols(A, h->ld, h->M, h->K_valid, gp, 4 * B, gc, h->num_sms, st)) != cudaSuccess)
-    return e;
+  AdjCols P = {};
+  P.A = A;
+  P.ld = h->ld;
+  P.M = h->M;
+  P.g = gp;
+  P.gx = gc;
+  P.K = P.L = h->K_valid;
+  P.B = 4 * B;
+  if ((e = psfsim_launch_adjoint_cols(P, h->num_sms, st)) != cudaSuccess) return e;
   sym_scatter<<<grid_for((int64_t)4 * B * h->K_valid, h->num_sms), 256, 0, st>>>(gc, B, h->N, h->K_valid, order, gx);
   return cudaGetLastError();
 }
@@ -211,9 +231,9 @@ cudaError_t psfsim_launch_adjoint_split_sym(const psfsim_plan *h, const float *g
   float *gp = static_cast<float *>(scratch);
   float *gc = reinterpret_cast<float *>(static_cast<char *>(scratch) + psfsim_round_up((int64_t)4 * B * h->M * 4, 256));
   void *part = reinterpret_cast<char *>(gc) + psfsim_round_up((int64_t)4 * B * (Kv > 0 ? Kv : 1) * 4, 256);
-  cudaError_t e = cudaMemsetAsync(gx, 0, (size_t)B * h->K * 4, st);
-  if (e != cudaSuccess || Kv == 0) return e;
-  sym_gperm<<<grid_for((int64_t)4 * B * h->M, h->num_sms), 256, 0, st>>>(g, B, h->n, gp);
+  if (Kv == 0) return cudaMemsetAsync(gx, 0, (size_t)B * h->K * 4, st);
+  cudaError_t e;
+  sym_gperm<<<grid_for((int64_t)4 * B * h->M, h->num_sms), 256, 0, st>>>(g, B, h->n, gp, gx, (int64_t)B * h->K);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = psfsim_launch_adjoint_split(h, gp, 4 * B, gc, part, st)) != cudaSuccess) return e;
   sym_scatter<<<grid_for((int64_t)4 * B * Kv, h->num_sms), 256, 0, st>>>(gc, B, h->N, Kv, order, gx);

@@ -196,7 +196,7 @@ int psfsim_adjoint_scratch_bytes(psfsim_t h, int B, size_t *bytes) {
     return PSFSIM_OK;
   }
   if (h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16) {
-    *bytes = psfsim_adjoint_split_scratch(h, B);
+    *bytes = psfsim_adjoint_tc_scratch(h, B);
     return PSFSIM_OK;
   }
   if (h->storage == PSFSIM_FP32_SYM) {
@@ -204,7 +204,7 @@ int psfsim_adjoint_scratch_bytes(psfsim_t h, int B, size_t *bytes) {
     return PSFSIM_OK;
   }
   if (h->storage == PSFSIM_SPLIT_BF16_SYM) {
-    *bytes = psfsim_adjoint_split_sym_scratch(h, B);
+    *bytes = psfsim_adjoint_tc_scratch(h, 4 * B);
     return PSFSIM_OK;
   }
   return PSFSIM_ERR_UNSUPPORTED;
@@ -270,9 +270,9 @@ int psfsim_adjoint(psfsim_t h, const float *d_g, int B, float *d_gx, void *d_scr
   if (h->storage == PSFSIM_FP32)
     return psfsim_launch_adjoint_fp32(h, d_g, B, d_gx, st) == cudaSuccess ? PSFSIM_OK : PSFSIM_ERR_CUDA;
   if (h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16) {
-    const size_t need = psfsim_adjoint_split_scratch(h, B);
+    const size_t need = psfsim_adjoint_tc_scratch(h, B);
     if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
-    return psfsim_launch_adjoint_split(h, d_g, B, d_gx, d_scratch, st) == cudaSuccess ? PSFSIM_OK
+    return psfsim_launch_adjoint_tc(h, d_g, B, d_gx, d_scratch, st) == cudaSuccess ? PSFSIM_OK
                                                                                       : PSFSIM_ERR_CUDA;
   }
   if (h->storage == PSFSIM_FP32_SYM) {
@@ -281,9 +281,9 @@ int psfsim_adjoint(psfsim_t h, const float *d_g, int B, float *d_gx, void *d_scr
     return psfsim_launch_adjoint_sym(h, d_g, B, d_gx, d_scratch, st) == cudaSuccess ? PSFSIM_OK : PSFSIM_ERR_CUDA;
   }
   if (h->storage == PSFSIM_SPLIT_BF16_SYM) {
-    const size_t need = psfsim_adjoint_split_sym_scratch(h, B);
+    const size_t need = psfsim_adjoint_tc_scratch(h, 4 * B);
     if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
-    return psfsim_launch_adjoint_split_sym(h, d_g, B, d_gx, d_scratch, st) == cudaSuccess ? PSFSIM_OK
+    return psfsim_launch_adjoint_tc(h, d_g, B, d_gx, d_scratch, st) == cudaSuccess ? PSFSIM_OK
                                                                                           : PSFSIM_ERR_CUDA;
   }
   return PSFSIM_ERR_UNSUPPORTED;

@@ -361,17 +361,6 @@ __device__ __forceinline__ void axis_weights(uint32_t f, float &w_near, float &w
 // offset).  The descriptor's other fields are those of the K-major one.
 constexpr uint32_t kAtomMN = 1024, kGroupK = 2048;
 
-__device__ __forceinline__ uint64_t smem_desc_mn_sw128(const void *tile) {
-  const uint64_t addr = ptx::smem_u32(tile);
-  uint64_t d = 0;
-  d |= (addr & 0x3FFFFull) >> 4;
-  d |= (uint64_t)(kAtomMN >> 4) << 16;
-  d |= (uint64_t)(kGroupK >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-
 // Tile-row block of pixel column du: rows 16 sigma(du) .. +15 (sigma swaps
 // bits 0 and 1), so that the two pixels of each 8-lane group (du = 2i, 2i + 1)
 // have rows 32 apart modulo 64 and their 16-byte stores meet 8 different
@@ -401,8 +390,8 @@ __device__ __forceinline__ void issue_stage_mmas(const FusedParams &P, uint8_t *
   ptx::tc_fence_after();
   const uint32_t idesc = ptx::idesc_bf16_f32(BM, 4 * P.Bp) | (1u << 15);  // A is M-major
   const uint32_t x2_off = (uint32_t)(4 * P.Bp) * 128;  // x2 rows follow the 4Bp rows of x1
-  const uint64_t dh = smem_desc_mn_sw128(stage);
-  const uint64_t dl = smem_desc_mn_sw128(stage + kTileBytes);
+  const uint64_t dh = ptx::smem_desc_mn_sw128(stage, kAtomMN, kGroupK);
+  const uint64_t dl = ptx::smem_desc_mn_sw128(stage + kTileBytes, kAtomMN, kGroupK);
   const uint64_t dx1 = ptx::smem_desc_sw128(stage + 2 * kTileBytes);
   const uint64_t dx2 = ptx::smem_desc_sw128(stage + 2 * kTileBytes + x2_off);
   const uint32_t d_tmem = tbase + acc * kAccStride;

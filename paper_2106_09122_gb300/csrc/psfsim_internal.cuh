@@ -103,7 +103,10 @@ struct SymSum {
   int64_t rows;
 };
 cudaError_t psfsim_launch_sym_sum(SymSum S, int B, float *y, cudaStream_t st);
-size_t psfsim_adjoint_split_scratch(const psfsim_plan *h, int B);
+// Adjoint of split and BF16 storage, dense or compact, on the tensor cores.
+size_t psfsim_adjoint_tc_scratch(const psfsim_plan *h, int B);
+cudaError_t psfsim_launch_adjoint_tc(const psfsim_plan *h, const float *g, int B, float *gx, void *scratch,
+                                     cudaStream_t st);
 // Test hook: the tensor-core forward of <= 80 scenes on one CTA with every
 // wait bounded by wait_ns and load number stall_it never issued.
 cudaError_t psfsim_launch_forward_tc_stall(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
@@ -160,8 +163,6 @@ cudaError_t psfsim_launch_forward_fused(const psfsim_plan *h, const float *x, in
 // bounded by wait_ns and the x load of k-tile number stall_load never issued.
 cudaError_t psfsim_launch_forward_fused_stall(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
                                               uint64_t wait_ns, int64_t stall_load, cudaStream_t st);
-cudaError_t psfsim_launch_adjoint_split(const psfsim_plan *h, const float *g, int B, float *gx, void *scratch,
-                                        cudaStream_t st);
 
 static inline int64_t psfsim_round_up(int64_t v, int64_t m) { return (v + m - 1) / m * m; }
 
@@ -171,9 +172,6 @@ static inline int64_t psfsim_cols(const psfsim_plan *h) { return h->quadrant ? h
 // Split-BF16 storage compacted by the quarter-turn symmetry (sym.cu).
 size_t psfsim_forward_split_sym_scratch(const psfsim_plan *h, int B);
 cudaError_t psfsim_launch_forward_split_sym(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
-                                            cudaStream_t st);
-size_t psfsim_adjoint_split_sym_scratch(const psfsim_plan *h, int B);
-cudaError_t psfsim_launch_adjoint_split_sym(const psfsim_plan *h, const float *g, int B, float *gx, void *scratch,
                                             cudaStream_t st);
 
 // Launch configuration with programmatic stream serialization: the kernel may

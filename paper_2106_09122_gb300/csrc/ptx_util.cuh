@@ -167,6 +167,19 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(const void *tile) {
   return d;
 }
 
+// As smem_desc_sw128 for an M-major tile: swizzle atoms of 64 elements of M x 8
+// of K (1024 bytes), `atom_mn` bytes apart along M and `group_k` along K.
+__device__ __forceinline__ uint64_t smem_desc_mn_sw128(const void *tile, uint32_t atom_mn, uint32_t group_k) {
+  const uint64_t addr = smem_u32(tile);
+  uint64_t d = 0;
+  d |= (addr & 0x3FFFFull) >> 4;
+  d |= (uint64_t)(atom_mn >> 4) << 16;
+  d |= (uint64_t)(group_k >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+
 // Instruction descriptor, kind::f16: bf16 A and B (both K-major), f32 accumulate.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);

@@ -206,9 +206,8 @@ cudaError_t psfsim_launch_adjoint_sym(const psfsim_plan *h, const float *g, int 
 // ---- split-BF16 storage with the same compaction (PSFSIM_SPLIT_BF16_SYM) ----
 // Forward: the four rotated scenes of every scene run as a batch of 4B through
 // the tcgen05 product over the compact columns (its scene split gathers them),
-// and the 4B partial images are summed through the inverse quarter turns.  Adjoint: the residual
-// turned four ways, the split adjoint over the compact columns, and a scatter
-// to the four rotated scene pixels.
+// and the 4B partial images are summed through the inverse quarter turns.  The
+// adjoint is tc_gemm.cu's, over the four turns of every residual.
 
 size_t psfsim_forward_split_sym_scratch(const psfsim_plan *h, int B) { return psfsim_forward_tc_scratch(h, 4 * B); }
 
@@ -216,26 +215,4 @@ cudaError_t psfsim_launch_forward_split_sym(const psfsim_plan *h, const float *x
                                             cudaStream_t st) {
   if (h->K_valid == 0) return cudaMemsetAsync(y, 0, (size_t)B * h->M * 4, st);
   return psfsim_launch_forward_tc_sym(h, x, B, y, scratch, st);
-}
-
-size_t psfsim_adjoint_split_sym_scratch(const psfsim_plan *h, int B) {
-  return (size_t)psfsim_round_up((int64_t)4 * B * h->M * 4, 256) +
-         (size_t)psfsim_round_up((int64_t)4 * B * (h->K_valid > 0 ? h->K_valid : 1) * 4, 256) +
-         psfsim_adjoint_split_scratch(h, 4 * B);
-}
-
-cudaError_t psfsim_launch_adjoint_split_sym(const psfsim_plan *h, const float *g, int B, float *gx, void *scratch,
-                                            cudaStream_t st) {
-  const int *order = reinterpret_cast<const int *>(h->ws + h->order_off);
-  const int64_t Kv = h->K_valid;
-  float *gp = static_cast<float *>(scratch);
-  float *gc = reinterpret_cast<float *>(static_cast<char *>(scratch) + psfsim_round_up((int64_t)4 * B * h->M * 4, 256));
-  void *part = reinterpret_cast<char *>(gc) + psfsim_round_up((int64_t)4 * B * (Kv > 0 ? Kv : 1) * 4, 256);
-  if (Kv == 0) return cudaMemsetAsync(gx, 0, (size_t)B * h->K * 4, st);
-  cudaError_t e;
-  sym_gperm<<<grid_for((int64_t)4 * B * h->M, h->num_sms), 256, 0, st>>>(g, B, h->n, gp, gx, (int64_t)B * h->K);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = psfsim_launch_adjoint_split(h, gp, 4 * B, gc, part, st)) != cudaSuccess) return e;
-  sym_scatter<<<grid_for((int64_t)4 * B * Kv, h->num_sms), 256, 0, st>>>(gc, B, h->N, Kv, order, gx);
-  return cudaGetLastError();
 }

@@ -12,6 +12,13 @@
 // D[:, 0:2Bp] += hi * [x1 x2]^T, so the result carries the 2^-8 relative
 // storage error of hi and the dropped hi * x3 term (< 2^-16 relative).
 //
+// The adjoint A^T g of the same storages is the same kernel with A's tiles
+// transposed: an M-tile is 128 columns (two 64-column k-tiles of the forward,
+// live ones only), the contraction runs over the image rows 64 at a time, A's
+// tiles arrive as two M-major boxes of 64 columns x 64 rows, and the residuals
+// take x's place, always in three parts.  adj_finish_kernel adds the k-splits
+// and scales the columns.
+//
 // Dense plans on a scene grid are mostly zero columns (beyond the last library
 // radius): only the 64-column k-tiles that hold a live column are loaded
 // (live.cu; TMA starts them at multiples of 32 columns).
@@ -54,6 +61,7 @@ constexpr int kMaxMmas = 64;     // accumulating MMAs between drains (bounds the
 struct TcJob {
   int64_t rows, M;
   int Bp, KS, m_tiles, k_tiles;
+  int tiles, ld;       // adjoint: 64-column tiles of A (ktab's), and A's row pitch
   int has_lo;          // split-BF16 (hi + lo) or BF16 (hi alone)
   int xparts;          // bf16 parts of x in the B operand: 3 (split-BF16) or 2 (BF16)
   int unit_begin;      // first work unit of this job
@@ -71,6 +79,7 @@ struct TcMulti {
   int njobs, units, stages, chunk;
   uint32_t stage_bytes;
   uint32_t x_off;  // byte offset of the x tile in a stage: after hi and lo, or after hi alone
+  int adjoint;     // A transposed: M-tiles of columns, k-tiles of 64 image rows
   int interleave;  // jobs share one A and one unit count: unit u is job u % njobs, unit u / njobs
   uint32_t tmem_cols, acc_stride;
   int *status;
@@ -84,7 +93,8 @@ struct XJob {
   const int *count;    // scenes present (NULL: all B)
   const int *ktab;     // k-tile table, dead groups after it (live.cu), or NULL
   const int *order;    // compact storage: quadrant pixel of every column (else NULL)
-  const float *scale;
+  int turn;            // adjoint of compact storage: image side n, x holds whole images (else 0)
+  const float *scale;  // per column (adjoint: NULL)
   __nv_bfloat16 *xs;   // [3][Bp][width]
   int64_t K, width, dead_groups;
   int B, Bp, N, first; // compact storage: slot b is rotated scene first + b, i.e. scene / 4 turned % 4 times
@@ -110,7 +120,18 @@ __global__ void __launch_bounds__(256) xsplit_kernel(const __grid_constant__ XMu
     const int64_t c = t % width;
     float v = 0.f;
     if (b < nb) {
-      if (J.order) {
+      if (J.turn) {
+        if (c < J.K) {
+          int p = (int)(c / J.turn), q = (int)(c % J.turn);
+          const int r = J.first + b;
+          for (int k = 0; k < (r & 3); ++k) {  // P(p, q) = (q, n-1-p)
+            const int np = q;
+            q = J.turn - 1 - p;
+            p = np;
+          }
+          v = J.x[(int64_t)(r >> 2) * J.K + (int64_t)p * J.turn + q];
+        }
+      } else if (J.order) {
         if (c < J.K) {
           const int H = J.N / 2, j0 = J.order[c], r = J.first + b;
           int ix = H + j0 % H, iy = H + j0 / H;
@@ -124,7 +145,7 @@ __global__ void __launch_bounds__(256) xsplit_kernel(const __grid_constant__ XMu
       } else {
         const float *xb = J.x + (int64_t)b * J.K;
         const int64_t j = J.ktab ? J.ktab[c / BK] + c % BK : c;
-        if (j < J.K) v = xb[j] * J.scale[j];
+        if (j < J.K) v = J.scale ? xb[j] * J.scale[j] : xb[j];
 #pragma unroll 4
         for (int64_t e = c; e < J.dead_groups * kLiveGroup; e += width) {
           const int64_t jd = (int64_t)dead[e / kLiveGroup] * kLiveGroup + e % kLiveGroup;
@@ -189,6 +210,83 @@ __global__ void __launch_bounds__(256) tc_reduce_kernel(const __grid_constant__ 
     if (r + 1 < J.M) out[1] = t.y;
     if (r + 2 < J.M) out[2] = t.z;
     if (r + 3 < J.M) out[3] = t.w;
+  }
+}
+
+// The adjoint's result from its partial sums, part[KS][cap][rows] per block of
+// kMaxBp residuals: thread t of residual b adds the k-splits of compact column
+// t, scales it and stores it at its column (dense), or at the turned pixel of
+// scene b / 4 (compact storage).  Threads beyond the compact columns serve the
+// columns in no tile: zero.  A residual value that is not finite gives NaN in
+// its split parts; such a column is summed again from the stored elements, as
+// the plain product would, so that infinities come out as they always did.
+struct AdjFinish {
+  const float *part[kMaxJobs];
+  int cap[kMaxJobs];
+  int KS, n, N;
+  int64_t rows, width, dead_groups, K, Kv, M, ld;  // width: compact columns
+  const int *ktab, *order;
+  const float *scale;
+  const __nv_bfloat16 *hi, *lo;
+  const float *g;
+  float *gx;
+};
+
+__device__ __noinline__ float plain_adjoint(const AdjFinish &P, int b, int64_t j) {
+  const float *g = P.g + (int64_t)(P.order ? b >> 2 : b) * P.M;
+  float acc = 0.f;
+#pragma unroll 4
+  for (int64_t i = 0; i < P.M; ++i) {
+    int64_t k = i;
+    if (P.order) {
+      int p = (int)(i / P.n), q = (int)(i % P.n);
+      for (int m = 0; m < (b & 3); ++m) {
+        const int np = q;
+        q = P.n - 1 - p;
+        p = np;
+      }
+      k = (int64_t)p * P.n + q;
+    }
+    const float a = __bfloat162float(P.hi[i * P.ld + j]) + (P.lo ? __bfloat162float(P.lo[i * P.ld + j]) : 0.f);
+    acc = fmaf(a, g[k], acc);
+  }
+  return acc;
+}
+
+__global__ void __launch_bounds__(256) adj_finish_kernel(const __grid_constant__ AdjFinish P) {
+  const int b = blockIdx.y, blk = b / kMaxBp, slot = b % kMaxBp;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const float *part = P.part[blk] + (int64_t)slot * P.rows;
+  const int64_t step = (int64_t)P.cap[blk] * P.rows;
+  auto sum = [&](int64_t at) {
+    float s = 0.f;
+#pragma unroll 4
+    for (int ks = 0; ks < P.KS; ++ks) s += part[ks * step + at];
+    return s;
+  };
+  if (t < P.width) {
+    const int64_t j = P.ktab ? P.ktab[t / BK] + t % BK : t;
+    if (j >= P.Kv) return;
+    float s = sum(t);
+    if (s != s) s = plain_adjoint(P, b, j);
+    s *= P.scale[j];
+    if (P.order) {
+      const int H = P.N / 2, j0 = P.order[j];
+      int ix = H + j0 % H, iy = H + j0 / H;
+      for (int k = 0; k < (b & 3); ++k) {  // R(ix, iy) = (N-1-iy, ix)
+        const int nx = P.N - 1 - iy;
+        iy = ix;
+        ix = nx;
+      }
+      P.gx[(int64_t)(b >> 2) * P.K + (int64_t)iy * P.N + ix] = s;
+    } else {
+      P.gx[(int64_t)b * P.K + j] = s;
+    }
+  } else if (t - P.width < P.dead_groups * kLiveGroup) {
+    const int64_t e = t - P.width, j = (int64_t)P.ktab[P.width / BK + e / kLiveGroup] * kLiveGroup + e % kLiveGroup;
+    if (j >= P.Kv) return;
+    const float s = sum(0);
+    P.gx[(int64_t)b * P.K + j] = s != s ? plain_adjoint(P, b, j) * P.scale[j] : 0.f;
   }
 }
 
@@ -262,10 +360,15 @@ __global__ void __launch_bounds__(kThreads, 2) tc_gemm_kernel(const __grid_const
       const int ks = lu / J.m_tiles, mt = lu % J.m_tiles;
       const uint32_t tx = (J.has_lo ? 2 : 1) * kTileBytes + (uint32_t)(J.xparts * J.Bp) * BK * 2;
       const int k0 = k_begin(J, ks), k1 = k_begin(J, ks + 1);
-      int next = J.ktab ? __ldg(J.ktab + k0) : 0;  // read one k-tile ahead of its use
+      int next = J.ktab && !P.adjoint ? __ldg(J.ktab + k0) : 0;  // read one k-tile ahead of its use
+      int ca = 0, cb = 0;  // adjoint: the M-tile's two runs of 64 columns (the last may be absent: past A's edge)
+      if (P.adjoint) {
+        ca = J.ktab ? __ldg(J.ktab + 2 * mt) : 2 * mt * BK;
+        cb = 2 * mt + 1 >= J.tiles ? J.ld : J.ktab ? __ldg(J.ktab + 2 * mt + 1) : (2 * mt + 1) * BK;
+      }
       for (int kt = k0; kt < k1; ++kt, ++it) {
         const int col = J.ktab ? next : kt * BK;
-        if (J.ktab && kt + 1 < k1) next = __ldg(J.ktab + kt + 1);
+        if (J.ktab && !P.adjoint && kt + 1 < k1) next = __ldg(J.ktab + kt + 1);
         const int s = (int)(it % P.stages);
         if (!ptx::mbar_wait_bounded(&empty_bar[s], ((it / P.stages) & 1) ^ 1, lim)) {
           set_abort(&abort_flag, P.status);
@@ -275,8 +378,15 @@ __global__ void __launch_bounds__(kThreads, 2) tc_gemm_kernel(const __grid_const
         if ((int64_t)it == P.stall_it) continue;  // test hook: this stage is never filled
         uint8_t *st = smem + (size_t)s * P.stage_bytes;
         ptx::mbar_arrive_expect_tx(&full_bar[s], tx);
-        ptx::tma_load_2d(st, &P.map[jb][0], col, mt * BM, &full_bar[s]);
-        if (J.has_lo) ptx::tma_load_2d(st + kTileBytes, &P.map[jb][1], col, mt * BM, &full_bar[s]);
+        if (P.adjoint) {
+          for (int part = 0; part < (J.has_lo ? 2 : 1); ++part) {
+            ptx::tma_load_2d(st + part * kTileBytes, &P.map[jb][part], ca, kt * BK, &full_bar[s]);
+            ptx::tma_load_2d(st + part * kTileBytes + kTileBytes / 2, &P.map[jb][part], cb, kt * BK, &full_bar[s]);
+          }
+        } else {
+          ptx::tma_load_2d(st, &P.map[jb][0], col, mt * BM, &full_bar[s]);
+          if (J.has_lo) ptx::tma_load_2d(st + kTileBytes, &P.map[jb][1], col, mt * BM, &full_bar[s]);
+        }
         ptx::tma_load_2d(st + P.x_off, &P.map[jb][2], kt * BK, 0, &full_bar[s]);
       }
     }
@@ -297,8 +407,9 @@ __global__ void __launch_bounds__(kThreads, 2) tc_gemm_kernel(const __grid_const
       const TcJob &J = P.job[jb];
       const int ks = lu / J.m_tiles;
       const int k0 = k_begin(J, ks), k1 = k_begin(J, ks + 1);
-      const uint32_t idesc3 = ptx::idesc_bf16_f32(BM, J.xparts * J.Bp);
-      const uint32_t idesc2 = ptx::idesc_bf16_f32(BM, 2 * J.Bp);
+      const uint32_t major = P.adjoint ? 1u << 15 : 0u;  // A is M-major
+      const uint32_t idesc3 = ptx::idesc_bf16_f32(BM, J.xparts * J.Bp) | major;
+      const uint32_t idesc2 = ptx::idesc_bf16_f32(BM, 2 * J.Bp) | major;
       const bool has_lo = J.has_lo != 0;
       for (int kc = k0; kc < k1 && ok; kc += P.chunk, ++c) {
         const int kc1 = min(kc + P.chunk, k1);
@@ -319,14 +430,16 @@ __global__ void __launch_bounds__(kThreads, 2) tc_gemm_kernel(const __grid_const
           }
           ptx::tc_fence_after();
           const uint8_t *st = smem + (size_t)s * P.stage_bytes;
-          const uint64_t dh = ptx::smem_desc_sw128(st);
-          const uint64_t dl = ptx::smem_desc_sw128(st + kTileBytes);
+          const uint64_t dh = P.adjoint ? ptx::smem_desc_mn_sw128(st, kTileBytes / 2, 1024) : ptx::smem_desc_sw128(st);
+          const uint64_t dl = P.adjoint ? ptx::smem_desc_mn_sw128(st + kTileBytes, kTileBytes / 2, 1024)
+                                        : ptx::smem_desc_sw128(st + kTileBytes);
           const uint64_t dx = ptx::smem_desc_sw128(st + P.x_off);
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk) {
             const uint64_t adv = (uint64_t)(kk * 32) >> 4;  // 16 bf16 = 32 bytes along K
-            ptx::mma_bf16(d_tmem, dh + adv, dx + adv, idesc3, (kt > kc || kk > 0) ? 1u : 0u);
-            if (has_lo) ptx::mma_bf16(d_tmem, dl + adv, dx + adv, idesc2, 1u);
+            const uint64_t adva = P.adjoint ? (uint64_t)(kk * 2048) >> 4 : adv;  // M-major: two groups of 8 rows
+            ptx::mma_bf16(d_tmem, dh + adva, dx + adv, idesc3, (kt > kc || kk > 0) ? 1u : 0u);
+            if (has_lo) ptx::mma_bf16(d_tmem, dl + adva, dx + adv, idesc2, 1u);
           }
           ptx::mma_commit(&empty_bar[s]);
         }
@@ -490,7 +603,7 @@ struct MultiPlan {
 // that the whole launch has about units_per_sm work units per SM (or, for a
 // single job without tuning, the smallest split that fills the SMs evenly);
 // as many smem stages as fit.
-MultiPlan plan_multi(const JobSpec *jobs, int nj, const psfsim_tuning_t *tune) {
+MultiPlan plan_multi(const JobSpec *jobs, int nj, const psfsim_tuning_t *tune, bool adjoint = false) {
   MultiPlan mp;
   std::memset(&mp, 0, sizeof(mp));
   mp.njobs = nj;
@@ -501,9 +614,9 @@ MultiPlan plan_multi(const JobSpec *jobs, int nj, const psfsim_tuning_t *tune) {
     const psfsim_plan *h = jobs[j].h;
     JobPlan &p = mp.jp[j];
     p.Bp = (int)psfsim_round_up(jobs[j].cap, 16);
-    p.rows = psfsim_round_up(h->M, BM);
+    p.rows = adjoint ? psfsim_round_up(h->k_tiles, 2) * BK : psfsim_round_up(h->M, BM);
     p.m_tiles = (int)(p.rows / BM);
-    p.k_tiles = h->k_tiles;
+    p.k_tiles = adjoint ? (int)(psfsim_round_up(h->M, BM) / BK) : h->k_tiles;
     total += (int64_t)p.m_tiles * p.k_tiles;
   }
   const int64_t target_units = (int64_t)(ups ? ups : 4) * num_sms;
@@ -537,7 +650,7 @@ MultiPlan plan_multi(const JobSpec *jobs, int nj, const psfsim_tuning_t *tune) {
   for (int j = 0; j < nj; ++j) {
     const bool lo = jobs[j].h->lo_off >= 0;
     any_lo = any_lo || lo;
-    const int r = (lo ? 3 : 2) * mp.jp[j].Bp;
+    const int r = (lo || adjoint ? 3 : 2) * mp.jp[j].Bp;
     x_rows = r > x_rows ? r : x_rows;
   }
   mp.x_off = (any_lo ? 2 : 1) * kTileBytes;
@@ -555,7 +668,7 @@ MultiPlan plan_multi(const JobSpec *jobs, int nj, const psfsim_tuning_t *tune) {
   // accumulate between drains.
   const int max_chunk = kMaxMmas / ((any_lo ? 2 : 1) * (BK / 16));
   mp.chunk = tune && tune->chunk > 0 ? (tune->chunk > max_chunk ? max_chunk : tune->chunk)
-                                     : (any_lo ? kDefaultChunk : (nj > 1 ? kDefaultChunkHiMulti : max_chunk));
+                                     : (any_lo || adjoint ? kDefaultChunk : (nj > 1 ? kDefaultChunkHiMulti : max_chunk));
   mp.smem = (size_t)mp.stages * mp.stage_bytes + 1024;
   return mp;
 }
@@ -570,7 +683,7 @@ struct StallHook {
 constexpr StallHook kNoStall = {2000000000ull, -1, false};
 
 cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void *scratch, cudaStream_t st,
-                         const StallHook &hook = kNoStall) {
+                         const StallHook &hook = kNoStall, bool adjoint = false) {
   char *base = static_cast<char *>(scratch);
   cudaError_t e;
   TcMulti P;  // kernel parameter blocks, copied at launch
@@ -590,12 +703,13 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
     X.x = jobs[j].x;
     X.count = jobs[j].count;
     X.ktab = h->live ? reinterpret_cast<const int *>(h->ws + h->order_off) : nullptr;
-    X.order = jobs[j].first >= 0 ? reinterpret_cast<const int *>(h->ws + h->order_off) : nullptr;
-    X.scale = scale;
+    X.order = jobs[j].first >= 0 && !adjoint ? reinterpret_cast<const int *>(h->ws + h->order_off) : nullptr;
+    X.turn = jobs[j].first >= 0 && adjoint ? h->n : 0;
+    X.scale = adjoint ? nullptr : scale;
     X.xs = xs;
-    X.K = psfsim_cols(h);
+    X.K = adjoint ? h->M : psfsim_cols(h);
     X.width = (int64_t)p.k_tiles * BK;
-    X.dead_groups = h->dead_groups;
+    X.dead_groups = adjoint ? 0 : h->dead_groups;
     X.B = jobs[j].cap;
     X.Bp = p.Bp;
     X.N = h->N;
@@ -603,14 +717,19 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
     const int64_t blocks = ((int64_t)p.Bp * X.width + 255) / 256;
     x_blocks = blocks > x_blocks ? blocks : x_blocks;
     const bool has_lo = h->lo_off >= 0;
-    if (!encode_bf16_2d(&P.map[j][0], h->ws + h->a_off, (uint64_t)h->ld, (uint64_t)p.rows, BK, BM) ||
-        (has_lo && !encode_bf16_2d(&P.map[j][1], h->ws + h->lo_off, (uint64_t)h->ld, (uint64_t)p.rows, BK, BM)) ||
+    const uint64_t a_rows = (uint64_t)psfsim_round_up(h->M, BM);
+    const uint32_t box_rows = adjoint ? BK : BM;
+    const int xparts = has_lo || adjoint ? 3 : 2;
+    if (!encode_bf16_2d(&P.map[j][0], h->ws + h->a_off, (uint64_t)h->ld, a_rows, BK, box_rows) ||
+        (has_lo && !encode_bf16_2d(&P.map[j][1], h->ws + h->lo_off, (uint64_t)h->ld, a_rows, BK, box_rows)) ||
         !encode_bf16_2d(&P.map[j][2], xs, (uint64_t)p.k_tiles * BK, (uint64_t)(3 * p.Bp), BK,
-                        (uint32_t)((has_lo ? 3 : 2) * p.Bp)))
+                        (uint32_t)(xparts * p.Bp)))
       return cudaErrorInvalidValue;
     TcJob &J = P.job[j];
     J.has_lo = has_lo ? 1 : 0;
-    J.xparts = has_lo ? 3 : 2;
+    J.xparts = xparts;
+    J.tiles = h->k_tiles;
+    J.ld = (int)h->ld;
     J.rows = p.rows;
     J.M = h->M;
     J.Bp = p.Bp;
@@ -620,13 +739,14 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
     J.unit_begin = j == 0 ? 0 : P.job[j - 1].unit_begin + P.job[j - 1].m_tiles * P.job[j - 1].KS;
     J.cap = jobs[j].cap;
     J.ktab = X.ktab;
+    if (adjoint) X.ktab = nullptr;
     J.count = jobs[j].count;
     // One split: the accumulated sums are the images (compact storage still
     // has its four rotations to add).
-    const bool direct = p.KS == 1 && jobs[j].first < 0;
+    const bool direct = p.KS == 1 && jobs[j].first < 0 && !adjoint;
     J.out = direct ? jobs[j].y : reinterpret_cast<float *>(base + p.part_off);
     J.out_ld = J.out_rows = direct ? h->M : p.rows;
-    if (!direct) {
+    if (!direct && !adjoint) {
       RJob &R = RP.job[nred++];
       R.part = J.out;
       R.y = jobs[j].y;
@@ -649,6 +769,7 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
     same = same && jobs[j].h == jobs[0].h &&
            mp.jp[j].m_tiles * mp.jp[j].KS == mp.jp[0].m_tiles * mp.jp[0].KS;
   P.interleave = same ? 1 : 0;
+  P.adjoint = adjoint ? 1 : 0;
   P.tmem_cols = mp.tmem_cols;
   P.acc_stride = mp.acc_stride;
   P.stages = mp.stages;
@@ -665,7 +786,7 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
   const int slots = hook.one_cta ? 1 : num_sms * mp.ctas_per_sm;
   tc_gemm_kernel<<<mp.units < slots ? mp.units : slots, kThreads, mp.smem, st>>>(P);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (jobs[0].first >= 0) return cudaSuccess;  // the caller adds the rotations (SymSum)
+  if (jobs[0].first >= 0 || adjoint) return cudaSuccess;  // the caller adds the rotations (SymSum), or finishes
   if (nred > 0)
     tc_reduce_kernel<<<dim3((unsigned)((red_rows + kRedRows - 1) / kRedRows), (unsigned)red_cap, (unsigned)nred), 256, 0,
                        st>>>(RP);
@@ -741,6 +862,64 @@ cudaError_t psfsim_launch_forward_tc_sym(const psfsim_plan *h, const float *x, i
       S.KS[j] = mp.jp[j].KS;
     }
     if ((e = psfsim_launch_sym_sum(S, Bc, y + (int64_t)b0 * h->M, st)) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// Compact storage: the four turns of the residuals are the batch.
+size_t psfsim_adjoint_tc_scratch(const psfsim_plan *h, int B) {
+  JobSpec js[kMaxJobs];
+  const int nj = tc_jobs(h, nullptr, B < kMaxLaunchScenes ? B : kMaxLaunchScenes, nullptr, js);
+  return plan_multi(js, nj, nullptr, true).scratch;
+}
+
+cudaError_t psfsim_launch_adjoint_tc(const psfsim_plan *h, const float *g, int B, float *gx, void *scratch,
+                                     cudaStream_t st) {
+  const int turns = h->quadrant ? 4 : 1;
+  if (h->quadrant) {  // scene pixels without a column
+    const cudaError_t e = cudaMemsetAsync(gx, 0, (size_t)B * h->K * 4, st);
+    if (e != cudaSuccess || h->K_valid == 0) return e;
+  }
+  const int most = kMaxLaunchScenes / turns;
+  for (int b0 = 0; b0 < B; b0 += most) {
+    const int Bc = turns * ((B - b0) < most ? (B - b0) : most);
+    const float *gb = g + (int64_t)b0 * h->M;
+    JobSpec js[kMaxJobs];
+    const int nj = tc_jobs(h, nullptr, Bc, nullptr, js);
+    for (int j = 0; j < nj; ++j) {
+      js[j].x = h->quadrant ? gb : gb + (int64_t)j * kMaxBp * h->M;
+      js[j].first = h->quadrant ? j * kMaxBp : -1;
+    }
+    const MultiPlan mp = plan_multi(js, nj, nullptr, true);
+    cudaError_t e = launch_multi(js, nj, mp, scratch, st, kNoStall, true);
+    if (e != cudaSuccess) return e;
+    AdjFinish F;
+    std::memset(&F, 0, sizeof(F));
+    for (int j = 0; j < nj; ++j) {
+      F.part[j] = reinterpret_cast<const float *>(static_cast<char *>(scratch) + mp.jp[j].part_off);
+      F.cap[j] = js[j].cap;
+    }
+    const int *tab = reinterpret_cast<const int *>(h->ws + h->order_off);
+    F.KS = mp.jp[0].KS;
+    F.n = h->n;
+    F.N = h->N;
+    F.rows = mp.jp[0].rows;
+    F.width = (int64_t)h->k_tiles * BK;
+    F.dead_groups = h->dead_groups;
+    F.K = h->K;
+    F.Kv = psfsim_cols(h);
+    F.M = h->M;
+    F.ld = h->ld;
+    F.ktab = h->live ? tab : nullptr;
+    F.order = h->quadrant ? tab : nullptr;
+    F.scale = reinterpret_cast<const float *>(h->ws + h->scale_off);
+    F.hi = reinterpret_cast<const __nv_bfloat16 *>(h->ws + h->a_off);
+    F.lo = h->lo_off >= 0 ? reinterpret_cast<const __nv_bfloat16 *>(h->ws + h->lo_off) : nullptr;
+    F.g = gb;
+    F.gx = gx + (int64_t)b0 * h->K;
+    const int64_t threads = F.width + F.dead_groups * kLiveGroup;
+    adj_finish_kernel<<<dim3((unsigned)((threads + 255) / 256), (unsigned)Bc), 256, 0, st>>>(F);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }

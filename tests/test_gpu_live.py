@@ -109,29 +109,39 @@ def test_split_build_in_a_workspace_without_room_for_pair_entries():
     L.psfsim_free(h)
 
 
-@pytest.mark.parametrize("storage,B", [("fp32", b) for b in (1, 2, 4, 5, 8, 9, 16, 17)] + [("fp32_sym", 1), ("fp32_sym", 3)])
+ADJOINT_TOL = {"fp32": 1e-5, "fp32_sym": 1e-5, "split_bf16": 1e-5, "split_bf16_sym": 1e-5, "bf16": 2.0 ** -8 + 1e-5}
+
+
+@pytest.mark.parametrize("storage,B", [("fp32", b) for b in (1, 2, 4, 5, 8, 9, 16, 17)] + [("fp32_sym", 1), ("fp32_sym", 3)] +
+                         [(s, b) for s in ("split_bf16", "bf16") for b in (1, 16, 17, 33, 80, 81)] +
+                         [("split_bf16_sym", b) for b in (1, 5, 21)])
 @pytest.mark.parametrize("n,N,S,r_last", [(20, 31, 0.5, 3.0), (17, 64, 0.5, 4.0), (33, 40, 0.25, 6.0), (20, 12, 1.0, 0.2)])
 def test_adjoint_reads_only_live_columns(storage, B, n, N, S, r_last):
     """Odd images (row quads cut at the end), more than one 64-column range per CTA or fewer
     columns than CTAs, no live column at all; a column beyond the last radius is exactly zero."""
-    if storage == "fp32_sym" and N % 2:
+    if storage.endswith("_sym") and N % 2:
         pytest.skip("an even scene grid")
     plan, A, rng = _plan(N, S, r_last, storage, n=n)
     g = rng.standard_normal((B, n * n)).astype(np.float32)
     gx = plan.adjoint(torch.from_numpy(g).to(DEV)).double().cpu().numpy()
     g64 = g.astype(np.float64)
     err = O.bound_relative_error(gx, g64 @ A, np.abs(g64) @ np.abs(A), floor=O.FLT_MIN).max()
-    assert err <= 1e-5, err
+    assert err <= ADJOINT_TOL[storage] and plan.sync_status() == 0, err
     assert np.all(gx[:, ~A.any(axis=0)] == 0.0)
 
 
+@pytest.mark.parametrize("storage", ["fp32", "split_bf16", "bf16"])
 @pytest.mark.parametrize("B", [1, 3, 9])
-@pytest.mark.parametrize("value", [float("nan"), float("inf")])
-def test_non_finite_residual_reaches_the_columns_not_read(B, value):
-    plan, A, rng = _plan(64, 0.5, 4.0, "fp32")
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), -float("inf")])
+def test_non_finite_residual_comes_out_as_multiplied_out(storage, B, value):
+    """An infinite residual value gives an infinity where its element of A is not zero, and NaN
+    (0 x inf) where it is: also in the columns that are not read."""
+    plan, A, rng = _plan(64, 0.5, 4.0, storage)
     for i in (0, 211, 399):
         g = rng.standard_normal((B, 400)).astype(np.float32)
         g[B - 1, i] = value
         gx = plan.adjoint(torch.from_numpy(g).to(DEV)).cpu().numpy()
         assert np.isfinite(gx[:B - 1]).all()
-        assert np.isnan(gx[B - 1, ~A.any(axis=0)]).all()
+        with np.errstate(invalid="ignore"):
+            want = np.where(A[i] == 0.0, np.nan, value * np.sign(A[i]))
+        assert np.array_equal(gx[B - 1], want.astype(np.float32), equal_nan=True)

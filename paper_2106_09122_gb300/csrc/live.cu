@@ -150,11 +150,12 @@ void psfsim_live_count(psfsim_plan *h) {
     return;
   }
   const int64_t groups = (h->K + kLiveGroup - 1) / kLiveGroup;
-  int64_t tiles = 0, covered = 0, run0 = -1, run1 = -1;  // current run of live groups [run0, run1)
+  int64_t runs = 0, tiles = 0, covered = 0, run0 = -1, run1 = -1;  // current run of live groups [run0, run1)
   auto close = [&] {
     if (run0 < 0) return;
     const int64_t t = (run1 - run0 + 1) / 2, end = run0 + 2 * t;
     tiles += t;
+    ++runs;
     covered += (end < groups ? end : groups) - run0;
   };
   for (int iy = 0; iy < h->N; ++iy) {
@@ -178,6 +179,7 @@ void psfsim_live_count(psfsim_plan *h) {
   if (covered >= groups) return;  // nothing to skip
   h->live = true;
   h->k_tiles = (int)tiles;
+  h->short_runs = 2 * tiles <= 5 * runs;
   h->dead_groups = groups - covered;
 }
 

@@ -45,6 +45,7 @@ struct psfsim_plan {
   bool live;            // products skip the zero columns listed in the workspace (live.cu)
   int64_t live_cols;    // FP32 storage: columns the products read (all of them when !live)
   int k_tiles;          // split storage: 64-column k-tiles the products read (ld / 64 when !live)
+  bool short_runs;      // split storage: at most 2.5 k-tiles on average between skipped ones
   int64_t dead_groups;  // split storage: 32-column groups in none of them
   int fit_ks;           // column splits of the fit-gradient forward, fixed at first use (0: not yet)
   CUtensorMap lib_map;  // 3D tensor map over the library for TMA staging

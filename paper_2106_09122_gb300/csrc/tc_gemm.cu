@@ -543,7 +543,7 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encoder() {
 }
 
 bool encode_bf16_2d(CUtensorMap *map, const void *base, uint64_t inner, uint64_t outer, uint32_t box_inner,
-                    uint32_t box_outer) {
+                    uint32_t box_outer, CUtensorMapL2promotion promotion = CU_TENSOR_MAP_L2_PROMOTION_L2_256B) {
   auto encode = get_encoder();
   if (!encode) return false;
   cuuint64_t dims[2] = {inner, outer};
@@ -551,7 +551,7 @@ bool encode_bf16_2d(CUtensorMap *map, const void *base, uint64_t inner, uint64_t
   cuuint32_t box[2] = {box_inner, box_outer};
   cuuint32_t estr[2] = {1, 1};
   return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, promotion,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -720,8 +720,17 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
     const uint64_t a_rows = (uint64_t)psfsim_round_up(h->M, BM);
     const uint32_t box_rows = adjoint ? BK : BM;
     const int xparts = has_lo || adjoint ? 3 : 2;
-    if (!encode_bf16_2d(&P.map[j][0], h->ws + h->a_off, (uint64_t)h->ld, a_rows, BK, box_rows) ||
-        (has_lo && !encode_bf16_2d(&P.map[j][1], h->ws + h->lo_off, (uint64_t)h->ld, a_rows, BK, box_rows)) ||
+    // What an L2 miss on A fetches.  256 bytes suit rows read from end to end
+    // (all of a 128^2 plan's columns: 185 us, 210 at 64 bytes) and still runs of
+    // three tiles a scene row (256^2, 12 of 16 lambda/D: 1752 against 1837); where
+    // a row holds a tile or two, half of it is thrown away (50 scenes on ten
+    // plans: 765 us, 703 at 64 bytes).  The adjoint reads a run's tiles side by
+    // side, and takes 64 bytes wherever columns are skipped (256^2: 1869 / 1460).
+    const auto promotion = h->live && (adjoint || h->short_runs) ? CU_TENSOR_MAP_L2_PROMOTION_L2_64B
+                                                                 : CU_TENSOR_MAP_L2_PROMOTION_L2_256B;
+    if (!encode_bf16_2d(&P.map[j][0], h->ws + h->a_off, (uint64_t)h->ld, a_rows, BK, box_rows, promotion) ||
+        (has_lo &&
+         !encode_bf16_2d(&P.map[j][1], h->ws + h->lo_off, (uint64_t)h->ld, a_rows, BK, box_rows, promotion)) ||
         !encode_bf16_2d(&P.map[j][2], xs, (uint64_t)p.k_tiles * BK, (uint64_t)(3 * p.Bp), BK,
                         (uint32_t)(xparts * p.Bp)))
       return cudaErrorInvalidValue;

@@ -539,7 +539,11 @@ static bool encode_library_map(psfsim_plan *h, int Wp) {
 cudaError_t psfsim_launch_build(psfsim_plan *h, cudaStream_t st) {
   const cudaError_t e = launch_tables_and_build(h, st);
   if (e != cudaSuccess || h->storage == PSFSIM_FUSED) return e;
-  return psfsim_launch_live_table(h, st);  // the column order is free from here on
+  if (const cudaError_t e2 = psfsim_launch_live_table(h, st)) return e2;  // the column order is free from here on
+  // The retrieval's forward kernels read A and the column list before they wait
+  // for the kernel ahead of them (programmatic launch), so that kernel must not
+  // be one that writes them: end with an operation that waits for those.
+  return cudaMemsetAsync(h->ws + h->status_off + 8, 0, 8, st);
 }
 
 static cudaError_t launch_tables_and_build(psfsim_plan *h, cudaStream_t st) {

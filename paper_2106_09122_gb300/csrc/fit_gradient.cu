@@ -8,6 +8,8 @@
 //   adj_chain_kernel       A^T r, its dot with dZ/dtheta, and the final sums
 //                          {L, dL/dtheta}.
 //
+// Both stream the columns inside the last radius only (128^2 fit workload, 44 %
+// of the columns: 359 -> 205 us a loss_and_grad call, host and copy included).
 // Both kernels are launched with programmatic stream serialization: the
 // forward computes its scene values and streams A before it waits for the
 // kernel ahead of it (griddepcontrol.wait), so back-to-back gradients overlap
@@ -34,41 +36,64 @@ constexpr int kSliceVec = kFwdThreads / kFwdCluster;  // row quads per slice (64
 static_assert(kSliceVec % 32 == 0 && kSliceVec <= kFwdThreads, "slices are whole warps");
 constexpr int kXCols = 2048;                          // most scene columns one CTA holds
 
-// CTA (tile, ks): rows [1024 tile, 1024 tile + 1024), columns
-// [K ks / KS, K (ks + 1) / KS) (at most kXCols).  Cluster rank q reduces
+// CTA (tile, ks): rows [1024 tile, 1024 tile + 1024), entries
+// [L ks / KS, L (ks + 1) / KS) (at most kXCols) of the list of columns that can
+// be non-zero (live.cu; NULL: every column).  The ring is also evaluated at the
+// ks-th share of the other columns: a value there that is not finite makes the
+// partial sums NaN, as 0 x inf would (a ring that overflows).  Z and dZ/dtheta
+// are stored for all K pixels.  Cluster rank q reduces
 // slice q (256 rows) of the tile over the cluster's kFwdCluster partials in
 // rank order and writes the group partial part[grp][rows]; the last of the
 // G = KS / kFwdCluster groups to arrive for a slice adds the group partials
 // in group order and forms y, r and the slice's loss partial
 // sum ((y - d)/sigma)^2.
 __global__ void __cluster_dims__(1, kFwdCluster, 1) __launch_bounds__(kFwdThreads, 6)
-    fwd_ring_loss_kernel(const float *__restrict__ A, int64_t ld, int64_t M, int64_t K, const RingParams P,
+    fwd_ring_loss_kernel(const float *__restrict__ A, int64_t ld, int64_t M, int64_t K, const int *__restrict__ list,
+                         int64_t L, const RingParams P,
                          float *__restrict__ z, float *__restrict__ jac, float *__restrict__ part,
                          const float *__restrict__ d, double sigma, float inv_s2, float *__restrict__ y,
                          float *__restrict__ res, double *__restrict__ loss_part, unsigned *__restrict__ slice_count,
                          unsigned *__restrict__ adj_count, int n_adj_count) {
   __shared__ float xs[kXCols];
+  __shared__ int js[kXCols];
   __shared__ float4 cpart[kFwdThreads];
+  __shared__ int bad;
   const int KS = gridDim.y, ks = blockIdx.y, G = KS / kFwdCluster, grp = ks / kFwdCluster;
-  const int64_t j0 = K * ks / KS, j1 = K * (ks + 1) / KS;
   const int64_t tile0 = (int64_t)blockIdx.x * kRowsPerCta;
   ptx::griddep_launch_dependents();
   // Until griddep_wait below, this kernel neither writes global memory nor
   // reads anything an earlier kernel writes: it may overlap the tail of the
   // kernel before it in the stream.
-  for (int64_t j = j0 + threadIdx.x; j < j1; j += kFwdThreads) xs[j - j0] = ring_eval<false>(P, j, nullptr);
-  __syncthreads();
   {
+    const int64_t l0 = L * ks / KS, D = K - L;
+    const int n = (int)(L * (ks + 1) / KS - l0);
+    const int64_t d0 = L + D * ks / KS, d1 = L + D * (ks + 1) / KS;  // the list goes on with the other columns
+    if (threadIdx.x == 0) bad = 0;
+    __syncthreads();
+    for (int64_t t = threadIdx.x; t < n + (d1 - d0); t += kFwdThreads) {
+      const int64_t e = t < n ? l0 + t : d0 + (t - n);
+      const int j = list ? __ldg(list + e) : (int)e;
+      const float z0 = ring_eval<false>(P, j, nullptr);
+      if (t < n) {
+        js[t] = j;
+        xs[t] = z0;
+      } else if (!isfinite(z0)) {
+        bad = 1;
+      }
+    }
+    __syncthreads();
     const int64_t r = tile0 + 4 * threadIdx.x;
-    float acc[1][4] = {{0.f, 0.f, 0.f, 0.f}};
-    if (r < ld) fwd_accumulate<1, true>(A, ld, K, xs, 0, r, j0, j1, acc);
-    cpart[threadIdx.x] = make_float4(acc[0][0], acc[0][1], acc[0][2], acc[0][3]);
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    if (r < ld) fwd_accumulate_list(A, ld, js, xs, n, r, acc);
+    const float z0 = bad ? __int_as_float(0x7fffffff) : 0.f;
+    cpart[threadIdx.x] = make_float4(acc[0] + z0, acc[1] + z0, acc[2] + z0, acc[3] + z0);
   }
   ptx::griddep_wait();
   if (blockIdx.x == 0 && blockIdx.y == 0)  // the adjoint that follows starts from zeroed counters
     for (int i = threadIdx.x; i < n_adj_count; i += kFwdThreads) adj_count[i] = 0u;
   // Z and dZ/dtheta of column j are stored by the CTA of tile j mod tiles,
   // which spreads that work over the tiles.
+  const int64_t j0 = K * ks / KS, j1 = K * (ks + 1) / KS;
   for (int64_t j = j0 + threadIdx.x; j < j1; j += kFwdThreads) {
     if (j % gridDim.x == blockIdx.x) {
       float J[5];
@@ -138,49 +163,60 @@ __global__ void __cluster_dims__(1, kFwdCluster, 1) __launch_bounds__(kFwdThread
 constexpr int kChainGroup = 32;  // CTAs whose chain partials one group sum covers
 
 
-// gz[j] = sum_i A[i, j] g[i] for j0 <= j < j1, two columns per pass: one
-// block barrier per pair of columns (the barrier after every column left the
-// stream with nothing in flight once per column) and each residual load
-// serves both.  Per column each thread adds its rows in ascending order
-// (strides of the block), then a fixed butterfly and a fixed sum over the
-// warps; stash[j - j0] = gz[j] for the first kStashCols columns.
+// gz[j] = sum_i A[i, j] g[i] for the columns j of list entries t0 <= t < t1, two
+// columns per pass: one block barrier per pair of columns (the barrier after
+// every column left the stream with nothing in flight once per column) and each
+// residual load serves both.  Per column each thread adds its rows in ascending
+// order (strides of the block), then a fixed butterfly and a fixed sum over the
+// warps; stash[t - t0] = gz[j] for the first kStashCols columns.  Returns, with
+// `probe`, NaN where one of the thread's residual values is not finite, else 0
+// (found on the first pair's pass over g).
 template <bool kVec>
-__device__ __forceinline__ void adj_pairs(const float *__restrict__ A, int64_t ld, int64_t M, int64_t K,
-                                          const float *__restrict__ g, float *__restrict__ gx, int64_t j0,
-                                          int64_t j1, float *stash) {
+__device__ __forceinline__ float adj_pairs(const float *__restrict__ A, int64_t ld, int64_t M,
+                                           const int *__restrict__ list, const float *__restrict__ g,
+                                           float *__restrict__ gx, int64_t t0, int64_t t1, float *stash, bool probe) {
   __shared__ float red2[2][kAdjThreads / 32][2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int parity = 0;
-  for (int64_t j = j0; j < j1; j += 2, parity ^= 1) {
-    const bool two = j + 1 < j1;
-    const float *c0 = A + j * ld;
-    const float *c1 = two ? c0 + ld : c0;
+  float zero = 0.f;
+  int64_t ja = 0, jb = 0;  // this pair's columns; the next pair's are read while this one streams
+  if (t0 < t1) {
+    ja = list ? list[t0] : t0;
+    jb = t0 + 1 < t1 ? (list ? list[t0 + 1] : t0 + 1) : ja;
+  }
+  for (int64_t t = t0; t < t1; t += 2, parity ^= 1) {
+    const bool two = t + 1 < t1;
+    const float *c0 = A + ja * ld, *c1 = A + jb * ld;
+    const int64_t na = t + 2 < t1 ? (list ? list[t + 2] : t + 2) : 0, nb = t + 3 < t1 ? (list ? list[t + 3] : t + 3) : na;
+    const bool look = probe && t == t0;
     float a0 = 0.f, a1 = 0.f;
+    auto add = [&](const float4 &u, const float4 &w, const float4 &gv) {
+      a0 = fmaf(u.x, gv.x, a0); a0 = fmaf(u.y, gv.y, a0); a0 = fmaf(u.z, gv.z, a0); a0 = fmaf(u.w, gv.w, a0);
+      a1 = fmaf(w.x, gv.x, a1); a1 = fmaf(w.y, gv.y, a1); a1 = fmaf(w.z, gv.z, a1); a1 = fmaf(w.w, gv.w, a1);
+      if (look) zero += 0.f * gv.x + 0.f * gv.y + 0.f * gv.z + 0.f * gv.w;
+    };
     if (kVec) {
       const int64_t M4 = M >> 2;
       constexpr int T = kAdjThreads;
+      const float4 *g4 = reinterpret_cast<const float4 *>(g);
       int64_t i4 = threadIdx.x;
       for (; i4 + T < M4; i4 += 2 * T) {
         const float4 u0 = ld_stream4(c0 + 4 * i4), w0 = ld_stream4(c1 + 4 * i4);
         const float4 u1 = ld_stream4(c0 + 4 * (i4 + T)), w1 = ld_stream4(c1 + 4 * (i4 + T));
-        const float4 g0 = __ldg(reinterpret_cast<const float4 *>(g) + i4);
-        const float4 g1 = __ldg(reinterpret_cast<const float4 *>(g) + i4 + T);
-        a0 = fmaf(u0.x, g0.x, a0); a0 = fmaf(u0.y, g0.y, a0); a0 = fmaf(u0.z, g0.z, a0); a0 = fmaf(u0.w, g0.w, a0);
-        a1 = fmaf(w0.x, g0.x, a1); a1 = fmaf(w0.y, g0.y, a1); a1 = fmaf(w0.z, g0.z, a1); a1 = fmaf(w0.w, g0.w, a1);
-        a0 = fmaf(u1.x, g1.x, a0); a0 = fmaf(u1.y, g1.y, a0); a0 = fmaf(u1.z, g1.z, a0); a0 = fmaf(u1.w, g1.w, a0);
-        a1 = fmaf(w1.x, g1.x, a1); a1 = fmaf(w1.y, g1.y, a1); a1 = fmaf(w1.z, g1.z, a1); a1 = fmaf(w1.w, g1.w, a1);
+        const float4 g0 = __ldg(g4 + i4), g1 = __ldg(g4 + i4 + T);
+        add(u0, w0, g0);
+        add(u1, w1, g1);
       }
       for (; i4 < M4; i4 += T) {
         const float4 u0 = ld_stream4(c0 + 4 * i4), w0 = ld_stream4(c1 + 4 * i4);
-        const float4 g0 = __ldg(reinterpret_cast<const float4 *>(g) + i4);
-        a0 = fmaf(u0.x, g0.x, a0); a0 = fmaf(u0.y, g0.y, a0); a0 = fmaf(u0.z, g0.z, a0); a0 = fmaf(u0.w, g0.w, a0);
-        a1 = fmaf(w0.x, g0.x, a1); a1 = fmaf(w0.y, g0.y, a1); a1 = fmaf(w0.z, g0.z, a1); a1 = fmaf(w0.w, g0.w, a1);
+        add(u0, w0, __ldg(g4 + i4));
       }
     } else {
       for (int64_t i = threadIdx.x; i < M; i += kAdjThreads) {
         const float gi = __ldg(g + i);
         a0 = fmaf(__ldg(c0 + i), gi, a0);
         a1 = fmaf(__ldg(c1 + i), gi, a1);
+        if (look) zero += 0.f * gi;
       }
     }
 #pragma unroll
@@ -194,13 +230,16 @@ __device__ __forceinline__ void adj_pairs(const float *__restrict__ A, int64_t l
     }
     __syncthreads();
     if (threadIdx.x < (two ? 2 : 1)) {
-      float t = red2[parity][0][threadIdx.x];
+      float s = red2[parity][0][threadIdx.x];
 #pragma unroll
-      for (int w = 1; w < kAdjThreads / 32; ++w) t += red2[parity][w][threadIdx.x];
-      gx[j + threadIdx.x] = t;
-      if (j + threadIdx.x - j0 < kStashCols) stash[j + threadIdx.x - j0] = t;
+      for (int w = 1; w < kAdjThreads / 32; ++w) s += red2[parity][w][threadIdx.x];
+      gx[threadIdx.x ? jb : ja] = s;
+      if (t + threadIdx.x - t0 < kStashCols) stash[t + threadIdx.x - t0] = s;
     }
+    ja = na;
+    jb = nb;
   }
+  return zero;
 }
 
 struct ChainArgs {
@@ -213,33 +252,42 @@ struct ChainArgs {
   double *out;              // {L, dL/dtheta_0..4}
 };
 
-// gz = A^T g over the CTA's contiguous column range (adj_pairs: two columns
-// per pass, four CTAs of 64 registers per SM so that the stream loop does not
-// spill), then warp 0 dots the range's gz with dZ/dtheta (both in shared memory: gz
+// gz = A^T g over the CTA's contiguous range of the listed columns (adj_pairs:
+// two columns per pass, four CTAs of 64 registers per SM so that the stream loop
+// does not spill); the columns outside the list get zero, or NaN when a residual
+// value is not finite; then warp 0 dots the range's gz with dZ/dtheta (both in shared memory: gz
 // stashed as it is produced, the Jacobian copied by cp.async while A
 // streams).  Partials are added in two levels, each by the last warp to
 // arrive: the 32 CTAs of a group in CTA order, then the groups in group order
 // together with the loss partials; the butterfly shuffles are a fixed tree.
 template <bool kVec>
 __global__ void __launch_bounds__(kAdjThreads, 4)
-    adj_chain_kernel(const float *__restrict__ A, int64_t ld, int64_t M, int64_t K, const float *__restrict__ g,
-                     float *__restrict__ gz, const ChainArgs c) {
+    adj_chain_kernel(const float *__restrict__ A, int64_t ld, int64_t M, int64_t K, const int *__restrict__ list,
+                     int64_t L, const float *__restrict__ g, float *__restrict__ gz, const ChainArgs c) {
   __shared__ float gzs[kStashCols];
   __shared__ float jacs[5][kStashCols];
   ptx::griddep_launch_dependents();
   ptx::griddep_wait();  // r and dZ/dtheta come from the forward kernel
   {
-    const int64_t j0 = K * blockIdx.x / gridDim.x, j1 = K * (blockIdx.x + 1) / gridDim.x;
+    const int64_t t0 = L * blockIdx.x / gridDim.x, t1 = L * (blockIdx.x + 1) / gridDim.x;
     for (int t = threadIdx.x; t < 5 * kStashCols; t += kAdjThreads) {
       const int m = t / kStashCols, col = t % kStashCols;
-      if (j0 + col < j1)
+      if (t0 + col < t1)
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(ptx::smem_u32(&jacs[m][col])),
-                     "l"(c.jac + m * K + j0 + col)
+                     "l"(c.jac + m * K + (list ? list[t0 + col] : t0 + col))
                      : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  adj_pairs<kVec>(A, ld, M, K, g, gz, K * blockIdx.x / gridDim.x, K * (blockIdx.x + 1) / gridDim.x, gzs);
+  float zero = adj_pairs<kVec>(A, ld, M, list, g, gz, L * blockIdx.x / gridDim.x, L * (blockIdx.x + 1) / gridDim.x, gzs,
+                               L < K);
+  if (L < K) {
+    if (L * blockIdx.x / gridDim.x == L * (blockIdx.x + 1) / gridDim.x)  // no column of its own to look at g with
+      for (int64_t i = threadIdx.x; i < M; i += kAdjThreads) zero += 0.f * g[i];
+    zero = __syncthreads_or(zero != 0.f) ? __int_as_float(0x7fffffff) : 0.f;
+    const int64_t D = K - L, d0 = L + D * blockIdx.x / gridDim.x, d1 = L + D * (blockIdx.x + 1) / gridDim.x;
+    for (int64_t e = d0 + threadIdx.x; e < d1; e += kAdjThreads) gz[list[e]] = zero;
+  }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();  // gzs (thread 0) and every thread's Jacobian copies are complete
   if (threadIdx.x >= 32) return;
@@ -249,10 +297,11 @@ __global__ void __launch_bounds__(kAdjThreads, 4)
   unsigned cta, ncta;
   asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(cta));
   asm volatile("mov.u32 %0, %%nctaid.x;" : "=r"(ncta));
-  const int64_t j0 = K * cta / ncta, j1 = K * (cta + 1) / ncta;
-  double acc[5] = {0, 0, 0, 0, 0};
-  for (int64_t j = j0 + lane; j < j1; j += 32) {
-    const int col = (int)(j - j0);
+  const int64_t t0 = L * cta / ncta, t1 = L * (cta + 1) / ncta;
+  double acc[5] = {zero, zero, zero, zero, zero};
+  for (int64_t t = t0 + lane; t < t1; t += 32) {
+    const int col = (int)(t - t0);
+    const int64_t j = list ? list[t] : t;
     const double gj = col < kStashCols ? (double)gzs[col] : (double)gz[j];
 #pragma unroll
     for (int m = 0; m < 5; ++m)
@@ -328,9 +377,9 @@ int forward_splits(psfsim_plan *h) {
     clusters = 0;
   }
   int64_t groups = clusters / tiles;
-  const int64_t max_groups = h->K / (8 * kFwdCluster);
+  const int64_t max_groups = h->live_cols / (8 * kFwdCluster);
   if (groups > max_groups) groups = max_groups;
-  const int64_t min_ks = (h->K + kXCols - 1) / kXCols;  // ceil(K / KS) <= kXCols
+  const int64_t min_ks = (h->live_cols + kXCols - 1) / kXCols;  // ceil(L / KS) <= kXCols
   const int64_t min_groups = (min_ks + kFwdCluster - 1) / kFwdCluster;
   if (groups < min_groups) groups = min_groups;
   if (groups < 1) groups = 1;
@@ -355,6 +404,11 @@ int adjoint_blocks(const psfsim_plan *h, bool vec) {
 int adjoint_max_blocks(const psfsim_plan *h) {
   const int64_t g = (int64_t)h->num_sms * (2048 / kAdjThreads);
   return (int)(g < h->K ? g : h->K);
+}
+
+// The columns the gradient reads, and how many: the plan's live ones.
+const int *column_list(const psfsim_plan *h) {
+  return h->live ? reinterpret_cast<const int *>(h->ws + h->order_off) : nullptr;
 }
 
 struct GradScratch {
@@ -429,7 +483,7 @@ int psfsim_ring_forward_loss(psfsim_t h, double r_max, const double *h_theta, co
   const cudaLaunchConfig_t cfg = psfsim_pdl_config(dim3((unsigned)forward_tiles(h), (unsigned)forward_splits(h)),
                                             kFwdThreads, static_cast<cudaStream_t>(stream), attr);
   const cudaError_t e = cudaLaunchKernelEx(
-      &cfg, fwd_ring_loss_kernel, A, h->ld, h->M, h->K, P, d_z, reinterpret_cast<float *>(base + g.jac),
+      &cfg, fwd_ring_loss_kernel, A, h->ld, h->M, h->K, column_list(h), h->live_cols, P, d_z, reinterpret_cast<float *>(base + g.jac),
       reinterpret_cast<float *>(base + g.part), d_target, sigma, (float)(1.0 / (sigma * sigma)), d_y, d_r,
       reinterpret_cast<double *>(base + g.loss), count, count + g.n_slices, g.n_groups + 1);
   return e == cudaSuccess ? PSFSIM_OK : PSFSIM_ERR_CUDA;
@@ -461,8 +515,8 @@ int psfsim_ring_adjoint_chain(psfsim_t h, double r_max, const double *h_theta, c
   cudaLaunchAttribute attr[1];
   const cudaLaunchConfig_t cfg =
       psfsim_pdl_config(dim3((unsigned)adjoint_blocks(h, vec)), kAdjThreads, static_cast<cudaStream_t>(stream), attr);
-  const cudaError_t e = vec ? cudaLaunchKernelEx(&cfg, adj_chain_kernel<true>, A, h->ld, h->M, h->K, d_r, d_gz, c)
-                            : cudaLaunchKernelEx(&cfg, adj_chain_kernel<false>, A, h->ld, h->M, h->K, d_r, d_gz, c);
+  auto kern = vec ? adj_chain_kernel<true> : adj_chain_kernel<false>;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, A, h->ld, h->M, h->K, column_list(h), h->live_cols, d_r, d_gz, c);
   return e == cudaSuccess ? PSFSIM_OK : PSFSIM_ERR_CUDA;
 }
 

@@ -77,6 +77,29 @@ __device__ __forceinline__ void fwd_accumulate(const float *__restrict__ A, int6
   }
 }
 
+// acc[e] = sum_c A[r + e, js[c]] xs[c] for the thread's 4 rows over n listed
+// columns, columns and values in shared memory.
+__device__ __forceinline__ void fwd_accumulate_list(const float *__restrict__ A, int64_t ld, const int *js,
+                                                    const float *xs, int n, int64_t r, float (&acc)[4]) {
+  acc[0] = acc[1] = acc[2] = acc[3] = 0.f;
+  const float *a = A + r;
+  auto add = [&](const float4 &v, float x) {
+    acc[0] = fmaf(v.x, x, acc[0]);
+    acc[1] = fmaf(v.y, x, acc[1]);
+    acc[2] = fmaf(v.z, x, acc[2]);
+    acc[3] = fmaf(v.w, x, acc[3]);
+  };
+  int c = 0;
+  for (; c + 4 <= n; c += 4) {
+    float4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = ld_stream4(a + (int64_t)js[c + u] * ld);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) add(v[u], xs[c + u]);
+  }
+  for (; c < n; ++c) add(ld_stream4(a + (int64_t)js[c] * ld), xs[c]);
+}
+
 constexpr int kAdjThreads = 256;
 constexpr int kStashCols = 128;
 

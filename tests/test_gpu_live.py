@@ -145,3 +145,36 @@ def test_non_finite_residual_comes_out_as_multiplied_out(storage, B, value):
         with np.errstate(invalid="ignore"):
             want = np.where(A[i] == 0.0, np.nan, value * np.sign(A[i]))
         assert np.array_equal(gx[B - 1], want.astype(np.float32), equal_nan=True)
+
+
+@pytest.mark.parametrize("n,N,S,r_last", [(20, 31, 0.5, 3.0), (17, 64, 0.5, 4.0), (32, 96, 0.5, 2.0), (21, 12, 1.0, 0.2)])
+def test_ring_gradient_reads_only_live_columns(n, N, S, r_last):
+    """The fused gradient against the separate operators: rings that reach beyond the last
+    radius, few or no live columns, odd images; zero gradient at the columns not read."""
+    from paper_2106_09122_gb300.fit import RingProblem
+    plan, A, rng = _plan(N, S, r_last, "fp32", n=n)
+    target = torch.from_numpy((rng.uniform(0.5, 1.5, n * n) * 1e-9).astype(np.float32)).to(DEV)
+    P = RingProblem(plan, N, S, 1.5 * r_last, target, 1e-11)
+    assert P.fused
+    theta = np.array([1.1 * r_last, r_last / 2, np.deg2rad(40.0), 0.3, 1e-9])
+    loss, grad = P.loss_and_grad(theta)
+    y, gz, z = P.y.clone(), P.gz.clone(), P.z.clone()
+    loss2, grad2 = P.loss_and_grad(theta)
+    assert loss2 == loss and np.array_equal(grad2, grad)
+    assert torch.all(gz[torch.from_numpy(~A.any(axis=0)).to(DEV)] == 0)
+    P.fused = False
+    loss_s, grad_s = P.loss_and_grad(theta)
+    assert torch.equal(P.z, z)
+    assert torch.allclose(P.y, y, rtol=1e-6, atol=0) and torch.allclose(P.gz, gz, rtol=1e-5, atol=1e-5 * float(gz.abs().max()))
+    assert loss == pytest.approx(loss_s, rel=1e-6)
+    np.testing.assert_allclose(grad, grad_s, rtol=1e-5, atol=1e-6 * np.abs(grad_s).max())
+
+
+def test_ring_gradient_with_a_target_that_is_not_finite():
+    from paper_2106_09122_gb300.fit import RingProblem
+    plan, A, rng = _plan(64, 0.5, 4.0, "fp32")
+    target = torch.full((400,), 1e-9, device=DEV)
+    target[123] = float("nan")
+    P = RingProblem(plan, 64, 0.5, 4.0, target, 1e-11)
+    loss, grad = P.loss_and_grad(np.array([2.0, 1.0, 0.5, 0.3, 1e-9]))
+    assert np.isnan(loss) and np.isnan(grad).all() and torch.isnan(P.gz).all() and torch.isfinite(P.y).all()

@@ -529,6 +529,199 @@ __global__ void __launch_bounds__(kThreads, 2) tc_gemm_kernel(const __grid_const
   }
 }
 
+// ---- many scenes of one plan -------------------------------------------------
+//
+// With scenes along the MMA's N, a step reads A's 128-row tiles and every x part
+// from shared memory for each of its two MMAs: about 200 bytes a clock against
+// the 128 it delivers, which held 256 rotated scenes of 256^2 to half the tensor
+// rate (998 us).  From some 100 scenes on the roles are swapped: 128 scenes are
+// the MMA's M, 256 image pixels its N, and all five products
+//     x1 hi + x2 hi + x3 hi + x1 lo + x2 lo      (BF16: x1 hi + x2 hi)
+// accumulate into one accumulator of 256 columns, two of which alternate, so
+// each MMA is a full 128 x 256 x 16 (96 bytes of operands a clock).  Every
+// k-tile is drained into FP32 sums by itself (20 accumulating MMAs: less drift
+// than the narrow form's 32), by eight epilogue warps of 128 pixels each.
+// Two stages of x (three parts of 128 scenes, 48 KB) and A (hi and lo of 256
+// pixels, 64 KB).  Blocks of 128 scenes interleave, so A comes from L2.
+constexpr int kWideScenes = 128, kWidePix = 256;
+constexpr int kWideThreads = 320;
+constexpr uint32_t kWideX = kWideScenes * BK * 2, kWideA = kWidePix * BK * 2;
+constexpr int kWideStages = 2;
+
+struct TcWide {
+  CUtensorMap hi, lo, x;
+  int njobs, KS, n_tiles, k_tiles, units, has_lo, scenes;
+  int x_rows;  // rows of one x part (128 njobs)
+  const int *ktab;
+  float *out;  // [KS][scenes][out_ld]
+  int64_t out_ld, out_rows;
+  int *status;
+  uint64_t wait_ns;
+};
+
+__global__ void __launch_bounds__(kWideThreads, 1) tc_wide_kernel(const __grid_constant__ TcWide P) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ __align__(8) uint64_t full_bar[kWideStages], empty_bar[kWideStages], tfull_bar[2], tempty_bar[2];
+  __shared__ __align__(8) uint64_t drain_bar;
+  __shared__ uint32_t tmem_base_sh;
+  __shared__ volatile int abort_flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint64_t lim = P.wait_ns;
+  const int xparts = P.has_lo ? 3 : 2;
+  const uint32_t a_off = 3 * kWideX, stage_bytes = a_off + 2 * kWideA;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kWideStages; ++s) {
+      ptx::mbar_init(&full_bar[s], 1);
+      ptx::mbar_init(&empty_bar[s], 1);
+    }
+    ptx::mbar_init(&drain_bar, 1);
+    for (int a = 0; a < 2; ++a) {
+      ptx::mbar_init(&tfull_bar[a], 1);
+      ptx::mbar_init(&tempty_bar[a], 8);
+    }
+    abort_flag = 0;
+    ptx::fence_mbar_init();
+  }
+  if (warp == 0) {
+    ptx::tmem_alloc(&tmem_base_sh, 512);
+    ptx::tmem_relinquish();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tbase = tmem_base_sh;
+  auto k_at = [&](int ks) { return (int)((int64_t)P.k_tiles * ks / P.KS); };
+
+  if (warp == 0 && lane == 0) {
+    // ---------------- TMA producer ----------------
+    uint32_t it = 0;
+    bool ok = true;
+    const uint32_t tx = xparts * kWideX + (P.has_lo ? 2 : 1) * kWideA;
+    for (int u = blockIdx.x; u < P.units && ok && !abort_flag; u += gridDim.x) {
+      const int jb = u % P.njobs, nt = u / P.njobs % P.n_tiles, ks = u / P.njobs / P.n_tiles;
+      const int k0 = k_at(ks), k1 = k_at(ks + 1);
+      int next = P.ktab ? __ldg(P.ktab + k0) : 0;
+      for (int kt = k0; kt < k1; ++kt, ++it) {
+        const int col = P.ktab ? next : kt * BK;
+        if (P.ktab && kt + 1 < k1) next = __ldg(P.ktab + kt + 1);
+        const int s = (int)(it % kWideStages);
+        if (!ptx::mbar_wait_bounded(&empty_bar[s], ((it / kWideStages) & 1) ^ 1, lim)) {
+          set_abort(&abort_flag, P.status);
+          ok = false;
+          break;
+        }
+        uint8_t *st = smem + (size_t)s * stage_bytes;
+        ptx::mbar_arrive_expect_tx(&full_bar[s], tx);
+        ptx::tma_load_2d(st + a_off, &P.hi, col, nt * kWidePix, &full_bar[s]);
+        if (P.has_lo) ptx::tma_load_2d(st + a_off + kWideA, &P.lo, col, nt * kWidePix, &full_bar[s]);
+        for (int part = 0; part < xparts; ++part)
+          ptx::tma_load_2d(st + part * kWideX, &P.x, kt * BK, part * P.x_rows + jb * kWideScenes, &full_bar[s]);
+      }
+    }
+    // Drain: the last loads issued may not have been consumed (as in tc_gemm_kernel).
+    for (uint32_t i = it > (uint32_t)kWideStages ? it - (uint32_t)kWideStages : 0u; i < it; ++i)
+      if (!ptx::mbar_wait_bounded(&full_bar[i % kWideStages], (i / kWideStages) & 1, lim)) set_abort(&abort_flag, P.status);
+  } else if (warp == 1 && lane == 0) {
+    // ---------------- MMA issuer ----------------
+    uint32_t it = 0;
+    bool ok = true;
+    const uint32_t idesc = ptx::idesc_bf16_f32(kWideScenes, kWidePix);
+    for (int u = blockIdx.x; u < P.units && ok && !abort_flag; u += gridDim.x) {
+      const int ks = u / P.njobs / P.n_tiles;
+      for (int kt = k_at(ks); kt < k_at(ks + 1); ++kt, ++it) {
+        const uint32_t acc = it & 1;
+        const int s = (int)(it % kWideStages);
+        if (!ptx::mbar_wait_bounded(&tempty_bar[acc], ((it >> 1) & 1) ^ 1, lim) ||
+            !ptx::mbar_wait_bounded(&full_bar[s], (it / kWideStages) & 1, lim)) {
+          set_abort(&abort_flag, P.status);
+          ok = false;
+          break;
+        }
+        ptx::tc_fence_after();
+        const uint8_t *st = smem + (size_t)s * stage_bytes;
+        const uint64_t x1 = ptx::smem_desc_sw128(st), x2 = ptx::smem_desc_sw128(st + kWideX),
+                       x3 = ptx::smem_desc_sw128(st + 2 * kWideX);
+        const uint64_t dh = ptx::smem_desc_sw128(st + a_off), dl = ptx::smem_desc_sw128(st + a_off + kWideA);
+        const uint32_t d = tbase + acc * 256;
+#pragma unroll
+        for (int kk = 0; kk < BK / 16; ++kk) {
+          const uint64_t adv = (uint64_t)(kk * 32) >> 4;
+          ptx::mma_bf16(d, x1 + adv, dh + adv, idesc, kk > 0 ? 1u : 0u);
+          ptx::mma_bf16(d, x2 + adv, dh + adv, idesc, 1u);
+          if (P.has_lo) {
+            ptx::mma_bf16(d, x3 + adv, dh + adv, idesc, 1u);
+            ptx::mma_bf16(d, x1 + adv, dl + adv, idesc, 1u);
+            ptx::mma_bf16(d, x2 + adv, dl + adv, idesc, 1u);
+          }
+        }
+        ptx::mma_commit(&empty_bar[s]);
+        ptx::mma_commit(&tfull_bar[acc]);
+      }
+    }
+    ptx::mma_commit(&drain_bar);
+    if (!ptx::mbar_wait_bounded(&drain_bar, 0, lim)) set_abort(&abort_flag, P.status);
+  } else if (warp >= 2) {
+    // ---------------- epilogue: scene 32 (warp % 4) + lane, pixels 128 half .. +127 ----------------
+    const int quarter = warp & 3, half = (warp - 2) >> 2;
+    uint32_t it = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; u < P.units && ok; u += gridDim.x) {
+      const int jb = u % P.njobs, nt = u / P.njobs % P.n_tiles, ks = u / P.njobs / P.n_tiles;
+      float sum[128];
+#pragma unroll
+      for (int t = 0; t < 128; ++t) sum[t] = 0.f;
+      for (int kt = k_at(ks); kt < k_at(ks + 1); ++kt, ++it) {
+        const uint32_t acc = it & 1;
+        int good = 0;
+        if (lane == 0) {
+          good = !abort_flag && ptx::mbar_wait_bounded(&tfull_bar[acc], (it >> 1) & 1, lim);
+          if (!good) set_abort(&abort_flag, P.status);
+        }
+        good = __shfl_sync(0xffffffffu, good, 0);
+        if (!good) {
+          ok = false;
+          break;
+        }
+        // Already complete (lane 0 saw it): this gives every lane its acquire.
+        if (!ptx::mbar_wait_bounded(&tfull_bar[acc], (it >> 1) & 1, lim)) set_abort(&abort_flag, P.status);
+        ptx::tc_fence_after();
+        const uint32_t t0 = tbase + ((uint32_t)(quarter * 32) << 16) + acc * 256 + half * 128;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          float v[16];
+          ptx::tmem_ld16(t0 + q * 16, v);
+          ptx::tmem_ld_wait();
+#pragma unroll
+          for (int t = 0; t < 16; ++t) sum[q * 16 + t] += v[t];
+        }
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&tempty_bar[acc]);
+      }
+      if (!ok) break;
+      const int scene = jb * kWideScenes + quarter * 32 + lane;
+      const int64_t px = (int64_t)nt * kWidePix + half * 128;
+      if (scene < P.scenes && px < P.out_rows) {
+        float *out = P.out + ((int64_t)ks * P.scenes + scene) * P.out_ld + px;
+#pragma unroll
+        for (int t = 0; t < 128; t += 8)
+          if (px + t < P.out_rows)
+            asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(out + t), "f"(sum[t]),
+                         "f"(sum[t + 1]), "f"(sum[t + 2]), "f"(sum[t + 3]), "f"(sum[t + 4]), "f"(sum[t + 5]),
+                         "f"(sum[t + 6]), "f"(sum[t + 7])
+                         : "memory");
+      }
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    __syncwarp();
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tbase, 512);
+  }
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 get_encoder() {
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   if (!encode) {
@@ -820,22 +1013,133 @@ int tc_jobs(const psfsim_plan *h, const float *x, int B, float *y, JobSpec *js) 
 
 constexpr int kMaxLaunchScenes = kMaxJobs * kMaxBp;
 
+// Whether `scenes` scenes (or rotated scenes) of a plan take the wide form.  One
+// job of up to 80 never does: the narrow form reads A at HBM rate there.  Beyond,
+// compact and BF16 storage always (us a call, narrow / wide: compact 128^2, 132
+// rotated scenes 91 / 71, 256: 129 / 76; BF16 128^2, 130 scenes 290 / 187); dense
+// split storage, whose A weighs twice, where its shared-memory traffic per
+// 128-pixel tile and k-tile is less, 1375 clocks per 128 scenes against 512 a job
+// and 8 a scene (128^2, 90 scenes: 268 narrow, 178 wide; 160: 275 and 292).
+bool wide_form(const psfsim_plan *h, int scenes) {
+  if (scenes <= kMaxBp) return false;
+  if (h->quadrant || h->lo_off < 0) return true;
+  const int narrow = 512 * ((scenes + kMaxBp - 1) / kMaxBp) + 8 * scenes;
+  return 1375 * ((scenes + kWideScenes - 1) / kWideScenes) < narrow;
+}
+
+struct WidePlan {
+  int njobs, KS, n_tiles, k_tiles;
+  int64_t rows;
+  size_t part_off, scratch;
+};
+
+WidePlan plan_wide(const psfsim_plan *h, int scenes) {
+  WidePlan w;
+  w.njobs = (scenes + kWideScenes - 1) / kWideScenes;
+  w.rows = psfsim_round_up(h->M, BM);
+  w.n_tiles = (int)((w.rows + kWidePix - 1) / kWidePix);
+  w.k_tiles = h->k_tiles;
+  // Splits by their cost in clocks: the rounds of units, a unit's k-tiles at 2750
+  // and its partial image's 128 KB at 6000, and the partial images read again at
+  // HBM rate.  (Filling the last round alone cost a 256^2 image of a 64^2 scene
+  // more in partial images than in products: 148 us for 32 scenes, 83 now.)
+  w.KS = 1;
+  double best = 1e300;
+  for (int ks = 1; ks <= 16 && ks <= w.k_tiles; ++ks) {
+    const int64_t units = (int64_t)w.n_tiles * w.njobs * ks, rounds = (units + h->num_sms - 1) / h->num_sms;
+    const double cost = (double)rounds * (2750.0 * ((w.k_tiles + ks - 1) / ks) + 6000.0) +
+                        (double)ks * (double)scenes * (double)w.rows * 4.0 / 3400.0;
+    if (cost < best) {
+      best = cost;
+      w.KS = ks;
+    }
+  }
+  w.part_off = (size_t)psfsim_round_up(3ll * kWideScenes * w.njobs * w.k_tiles * BK * 2, 256);
+  w.scratch = w.part_off + (size_t)w.KS * scenes * w.rows * 4;
+  return w;
+}
+
+// Partial images part[KS][scenes][rows] in the scratch; compact storage: x holds
+// whole scenes and the batch is their rotations.
+cudaError_t launch_wide(const psfsim_plan *h, const float *x, int scenes, const WidePlan &w, void *scratch,
+                        cudaStream_t st) {
+  __nv_bfloat16 *xs = static_cast<__nv_bfloat16 *>(scratch);
+  const int *tab = reinterpret_cast<const int *>(h->ws + h->order_off);
+  XMulti XP;
+  TcWide P;
+  std::memset(&XP, 0, sizeof(XP));
+  std::memset(&P, 0, sizeof(P));
+  XJob &X = XP.job[0];
+  X.x = x;
+  X.ktab = h->live ? tab : nullptr;
+  X.order = h->quadrant ? tab : nullptr;
+  X.scale = reinterpret_cast<const float *>(h->ws + h->scale_off);
+  X.xs = xs;
+  X.K = psfsim_cols(h);
+  X.width = (int64_t)w.k_tiles * BK;
+  X.dead_groups = h->dead_groups;
+  X.B = scenes;
+  X.Bp = kWideScenes * w.njobs;
+  X.N = h->N;
+  const int64_t blocks = ((int64_t)X.Bp * X.width + 255) / 256, cap = (int64_t)h->num_sms * 16;
+  xsplit_kernel<<<(unsigned)(blocks < cap ? blocks : cap), 256, 0, st>>>(XP);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  P.has_lo = h->lo_off >= 0 ? 1 : 0;
+  if (!encode_bf16_2d(&P.hi, h->ws + h->a_off, (uint64_t)h->ld, (uint64_t)w.rows, BK, kWidePix) ||
+      (P.has_lo && !encode_bf16_2d(&P.lo, h->ws + h->lo_off, (uint64_t)h->ld, (uint64_t)w.rows, BK, kWidePix)) ||
+      !encode_bf16_2d(&P.x, xs, (uint64_t)X.width, (uint64_t)(3 * X.Bp), BK, kWideScenes))
+    return cudaErrorInvalidValue;
+  P.njobs = w.njobs;
+  P.KS = w.KS;
+  P.n_tiles = w.n_tiles;
+  P.k_tiles = w.k_tiles;
+  P.units = w.njobs * w.n_tiles * w.KS;
+  P.scenes = scenes;
+  P.x_rows = X.Bp;
+  P.ktab = X.ktab;
+  P.out = reinterpret_cast<float *>(static_cast<char *>(scratch) + w.part_off);
+  P.out_ld = P.out_rows = w.rows;
+  P.status = reinterpret_cast<int *>(h->ws + h->status_off);
+  P.wait_ns = kNoStall.wait_ns;
+  const size_t smem = kWideStages * (3 * kWideX + 2 * kWideA) + 1024;
+  if ((e = cudaFuncSetAttribute(tc_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    return e;
+  tc_wide_kernel<<<P.units < h->num_sms ? P.units : h->num_sms, kWideThreads, smem, st>>>(P);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
+// A batch beyond kMaxLaunchScenes runs as several launches, the last of which
+// may be smaller and of the other form.
 size_t psfsim_forward_tc_scratch(const psfsim_plan *h, int B) {
-  JobSpec js[kMaxJobs];
-  const int nj = tc_jobs(h, nullptr, B < kMaxLaunchScenes ? B : kMaxLaunchScenes, nullptr, js);
-  return plan_multi(js, nj, nullptr).scratch;
+  size_t most = 0;
+  for (int c : {B < kMaxLaunchScenes ? B : kMaxLaunchScenes, B > kMaxLaunchScenes ? B % kMaxLaunchScenes : 0}) {
+    if (c == 0) continue;
+    JobSpec js[kMaxJobs];
+    const size_t need =
+        wide_form(h, c) ? plan_wide(h, c).scratch : plan_multi(js, tc_jobs(h, nullptr, c, nullptr, js), nullptr).scratch;
+    most = need > most ? need : most;
+  }
+  return most;
 }
 
 cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
                                      cudaStream_t st) {
   for (int b0 = 0; b0 < B; b0 += kMaxLaunchScenes) {
     const int Bc = (B - b0) < kMaxLaunchScenes ? (B - b0) : kMaxLaunchScenes;
-    JobSpec js[kMaxJobs];
-    const int nj = tc_jobs(h, x + (int64_t)b0 * psfsim_cols(h), Bc, y + (int64_t)b0 * h->M, js);
-    const MultiPlan mp = plan_multi(js, nj, nullptr);
-    cudaError_t e = launch_multi(js, nj, mp, scratch, st);
+    cudaError_t e;
+    if (wide_form(h, Bc)) {
+      const WidePlan w = plan_wide(h, Bc);
+      if ((e = launch_wide(h, x + (int64_t)b0 * h->K, Bc, w, scratch, st)) != cudaSuccess) return e;
+      e = psfsim_launch_reduce_partials(reinterpret_cast<const float *>(static_cast<char *>(scratch) + w.part_off), w.KS,
+                                        Bc, w.rows, h->M, y + (int64_t)b0 * h->M, st);
+    } else {
+      JobSpec js[kMaxJobs];
+      const int nj = tc_jobs(h, x + (int64_t)b0 * psfsim_cols(h), Bc, y + (int64_t)b0 * h->M, js);
+      e = launch_multi(js, nj, plan_multi(js, nj, nullptr), scratch, st);
+    }
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -851,6 +1155,20 @@ cudaError_t psfsim_launch_forward_tc_sym(const psfsim_plan *h, const float *x, i
   static_assert(kMaxBp % 4 == 0, "a scene's rotations share a job");
   for (int b0 = 0; b0 < B; b0 += kScenes) {
     const int Bc = (B - b0) < kScenes ? (B - b0) : kScenes;
+    if (wide_form(h, 4 * Bc)) {
+      const WidePlan w = plan_wide(h, 4 * Bc);
+      cudaError_t e = launch_wide(h, x + (int64_t)b0 * h->K, 4 * Bc, w, scratch, st);
+      if (e != cudaSuccess) return e;
+      SymSum S;
+      std::memset(&S, 0, sizeof(S));
+      S.part[0] = reinterpret_cast<const float *>(static_cast<char *>(scratch) + w.part_off);
+      S.cap[0] = S.per = 4 * Bc;
+      S.KS[0] = w.KS;
+      S.rows = w.rows;
+      S.n = h->n;
+      if ((e = psfsim_launch_sym_sum(S, Bc, y + (int64_t)b0 * h->M, st)) != cudaSuccess) return e;
+      continue;
+    }
     JobSpec js[kMaxJobs];
     const int nj = tc_jobs(h, nullptr, 4 * Bc, nullptr, js);
     for (int j = 0; j < nj; ++j) {

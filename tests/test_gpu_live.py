@@ -178,3 +178,14 @@ def test_ring_gradient_with_a_target_that_is_not_finite():
     P = RingProblem(plan, 64, 0.5, 4.0, target, 1e-11)
     loss, grad = P.loss_and_grad(np.array([2.0, 1.0, 0.5, 0.3, 1e-9]))
     assert np.isnan(loss) and np.isnan(grad).all() and torch.isnan(P.gz).all() and torch.isfinite(P.y).all()
+
+
+@pytest.mark.parametrize("storage,tol,B", [(s, t, b) for s, t in (("split_bf16", 1e-5), ("bf16", 2.0 ** -8 + 2.5e-5))
+                                           for b in (81, 100, 128, 129, 200, 256)] +
+                         [("split_bf16_sym", 1e-5, b) for b in (20, 21, 32, 33, 50, 64)])
+@pytest.mark.parametrize("n", [17, 24])
+def test_forward_of_many_scenes(storage, tol, B, n):
+    """Around the batch where scenes become the product's rows: partial blocks of 128, images
+    that end inside a tile of 256 pixels, skipped k-tiles."""
+    plan, A, rng = _plan(64, 0.125, 3.0, storage, n=n)
+    _check_forward(plan, A, rng.uniform(0.0, 1.0, (B, 64 * 64)).astype(np.float32), tol)

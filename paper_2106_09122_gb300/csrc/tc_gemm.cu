@@ -55,6 +55,11 @@ constexpr int kMaxBp = 80;       // 3 * Bp <= 256 (MMA N and TMA box limits), Bp
 constexpr int kMaxJobs = 16;
 constexpr int kDefaultChunk = 4; // k-tiles (of 64) per TMEM accumulation, split-BF16 storage
 constexpr int kDefaultChunkHiMulti = 2;  // BF16 storage (hi alone), several jobs in one launch
+// Adjoint of split storage: residuals change sign, so its sums cancel and the
+// drift weighs more (error against 64 bits 2.493e-6 with plain FP32 sums, 2.553
+// at 4 k-tiles, 2.492 at one; 8 residuals of 128^2 take 127 and 129 us, 64 of
+// 256^2 1.45 and 1.64 ms).
+constexpr int kAdjointChunk = 1;
 constexpr int kMaxMmas = 64;     // accumulating MMAs between drains (bounds the FP32 drift)
 
 // One product S_j = A_j Z_j of a (possibly multi-job) launch.
@@ -861,7 +866,7 @@ MultiPlan plan_multi(const JobSpec *jobs, int nj, const psfsim_tuning_t *tune, b
   // accumulate between drains.
   const int max_chunk = kMaxMmas / ((any_lo ? 2 : 1) * (BK / 16));
   mp.chunk = tune && tune->chunk > 0 ? (tune->chunk > max_chunk ? max_chunk : tune->chunk)
-                                     : (any_lo || adjoint ? kDefaultChunk : (nj > 1 ? kDefaultChunkHiMulti : max_chunk));
+                                     : (adjoint && any_lo ? kAdjointChunk : any_lo || adjoint ? kDefaultChunk : (nj > 1 ? kDefaultChunkHiMulti : max_chunk));
   mp.smem = (size_t)mp.stages * mp.stage_bytes + 1024;
   return mp;
 }

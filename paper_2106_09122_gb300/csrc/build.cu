@@ -213,29 +213,45 @@ struct BuildParams {
   int *status;
 };
 
-// One rotated + lerped element (a3-a4).  a2/b2 hold 2a and 2b in fixed point
-// with PSFSIM_FRAC_BITS fraction bits; taps come from `tap(psf, row, col)`.
+// Radial lerp of one library pixel (a3).  A PSF of weight zero above takes no
+// part (it may hold anything).
+__device__ __forceinline__ float lerp_pixel(float w0, float w1, float l0, float l1) {
+  const float t = __fmul_rn(w0, l0);
+  return w1 != 0.f ? fmaf(w1, l1, t) : t;
+}
+
+// Bilinear sample (a4) of a lerped 2 x 2 footprint at the 32-bit fractions fa
+// and fb of its column and row.  Each weight is formed from its own exact
+// integer, so a tiny one is accurate relative to itself too (2^32 - f as
+// (2^32 - 1 - f) + 1: the sum is exact below 2^24 and under half an ulp above).
+// Lerping before sampling halves the taps.  Every FP32 build samples with these
+// operations, so all store the same bits.
+__device__ __forceinline__ float bilinear(float t00, float t01, float t10, float t11, unsigned fa, unsigned fb) {
+  constexpr float kInv32 = 2.3283064365386963e-10f;  // 2^-32
+  const float wa1 = __uint2float_rn(fa) * kInv32, wa0 = (__uint2float_rn(~fa) + 1.f) * kInv32;
+  const float wb1 = __uint2float_rn(fb) * kInv32, wb0 = (__uint2float_rn(~fb) + 1.f) * kInv32;
+  const float r0 = fmaf(wa0, t00, __fmul_rn(wa1, t01));
+  const float r1 = fmaf(wa0, t10, __fmul_rn(wa1, t11));
+  return fmaf(wb0, r0, __fmul_rn(wb1, r1));
+}
+
+// One element from the two library PSFs: a2/b2 hold 2a and 2b in fixed point
+// with PSFSIM_FRAC_BITS fraction bits; tap(row, col, l0, l1) fetches both PSFs'
+// pixel (zeros outside).  The taps are all requested before any is used.
 template <typename TapFn>
-__device__ __forceinline__ float rotated_value(long long a2, long long b2, int n, float w0, float w1,
-                                               TapFn tap) {
+__device__ __forceinline__ float rotated_value(long long a2, long long b2, int n, float w0, float w1, TapFn tap) {
   constexpr int kShift = PSFSIM_FRAC_BITS + 1;
   const int q0 = (int)(a2 >> kShift);
   const int p0 = (int)(b2 >> kShift);
   if (q0 < -1 || q0 > n - 1 || p0 < -1 || p0 > n - 1) return 0.f;
-  const unsigned fa = (unsigned)((unsigned long long)a2 >> (kShift - 32));
-  const unsigned fb = (unsigned)((unsigned long long)b2 >> (kShift - 32));
-  constexpr float kInv32 = 2.3283064365386963e-10f;  // 2^-32
-  const float wa1 = __uint2float_rn(fa) * kInv32;
-  const float wa0 = fa ? __uint2float_rn(0u - fa) * kInv32 : 1.f;
-  const float wb1 = __uint2float_rn(fb) * kInv32;
-  const float wb0 = fb ? __uint2float_rn(0u - fb) * kInv32 : 1.f;
-  float v0 = wb0 * (wa0 * tap(0, p0, q0) + wa1 * tap(0, p0, q0 + 1)) +
-             wb1 * (wa0 * tap(0, p0 + 1, q0) + wa1 * tap(0, p0 + 1, q0 + 1));
-  float v1 = 0.f;
-  if (w1 != 0.f)
-    v1 = wb0 * (wa0 * tap(1, p0, q0) + wa1 * tap(1, p0, q0 + 1)) +
-         wb1 * (wa0 * tap(1, p0 + 1, q0) + wa1 * tap(1, p0 + 1, q0 + 1));
-  return w0 * v0 + w1 * v1;
+  float l0[4], l1[4];
+  tap(p0, q0, l0[0], l1[0]);
+  tap(p0, q0 + 1, l0[1], l1[1]);
+  tap(p0 + 1, q0, l0[2], l1[2]);
+  tap(p0 + 1, q0 + 1, l0[3], l1[3]);
+  return bilinear(lerp_pixel(w0, w1, l0[0], l1[0]), lerp_pixel(w0, w1, l0[1], l1[1]), lerp_pixel(w0, w1, l0[2], l1[2]),
+                  lerp_pixel(w0, w1, l0[3], l1[3]), (unsigned)((unsigned long long)a2 >> (kShift - 32)),
+                  (unsigned)((unsigned long long)b2 >> (kShift - 32)));
 }
 
 // Writes column j of A (FP32, column-major) with one warp.
@@ -253,13 +269,17 @@ __device__ __forceinline__ void build_column(const BuildParams &P, int j, int64_
   const float *L0 = P.lib + (int64_t)g.k * M;
   const float *L1 = L0 + M;
   const int Wp = P.Wp;
-  auto tap = [&](int which, int r, int c) -> float {
+  auto tap = [&](int r, int c, float &l0, float &l1) {
     if (kSmem) {
-      const float *s = which ? s1 : s0;
-      return s[(r + 1) * Wp + (c + 4)];
+      const int i = (r + 1) * Wp + (c + 4);
+      l0 = s0[i];
+      l1 = s1[i];
     } else {
-      if (r < 0 || r >= n || c < 0 || c >= n) return 0.f;
-      return __ldg((which ? L1 : L0) + r * n + c);
+      l0 = l1 = 0.f;
+      if (r >= 0 && r < n && c >= 0 && c < n) {
+        l0 = __ldg(L0 + r * n + c);
+        l1 = __ldg(L1 + r * n + c);
+      }
     }
   };
   const long long h = n - 1;
@@ -373,96 +393,205 @@ __global__ void __launch_bounds__(512) build_fp32_kernel(const __grid_constant__
 // every copy is 32 rows of 32 contiguous floats.
 constexpr int kSymBlk = 32, kSymPitch = 33;  // block side; shared pitch (transposed reads without conflicts)
 
-template <bool kSmem>
-__device__ __forceinline__ void build_block_sym(const BuildParams &P, int jq, int p0, int q0, const float *s0,
-                                                const float *s1, float *blk, int lane) {
-  const int N = P.N, n = P.n, H = N / 2;
+// A column of the x > 0, y > 0 quadrant and its three turned copies.
+struct TurnedColumns {
+  float *at[4];
+};
+__device__ __forceinline__ TurnedColumns turned_columns(const BuildParams &P, int jq) {
+  const int N = P.N, H = N / 2;
   const int iy = H + jq / H, ix = H + jq % H;  // quadrant entry jq
-  const int64_t j = (int64_t)iy * N + ix;
-  float *Am[4] = {P.A + j * P.ld, P.A + ((int64_t)ix * N + (N - 1 - iy)) * P.ld,
-                  P.A + ((int64_t)(N - 1 - iy) * N + (N - 1 - ix)) * P.ld, P.A + ((int64_t)(N - 1 - ix) * N + iy) * P.ld};
-  const ColGeom g = P.geom[jq];
+  return TurnedColumns{{P.A + ((int64_t)iy * N + ix) * P.ld, P.A + ((int64_t)ix * N + (N - 1 - iy)) * P.ld,
+                        P.A + ((int64_t)(N - 1 - iy) * N + (N - 1 - ix)) * P.ld,
+                        P.A + ((int64_t)(N - 1 - ix) * N + iy) * P.ld}};
+}
+
+// One 32 x 32 pixel block at (p0, q0) of a quadrant column, to its four turned
+// places.  value(a2, b2) samples; lane: pixel column q0 + lane, down the rows in
+// exact steps.  Copies 0 and 2 leave as the rows are made, 32 contiguous floats
+// each (copy 2 backwards); the block goes through shared memory for copies 1 and
+// 3, whose rows are its columns.
+template <class ValueFn, class RowFn>
+__device__ __forceinline__ void build_block_sym(int n, const ColGeom &g, const TurnedColumns &A, int p0, int q0,
+                                                float *blk, int lane, ValueFn value, RowFn each_row) {
   __syncwarp();  // the previous block's copies have read the buffer
-  if (g.k < 0) {  // beyond the last radius: zeros
-    for (int a = 0; a < kSymBlk; ++a) blk[a * kSymPitch + lane] = 0.f;
-  } else {
-    const int64_t M = (int64_t)n * n;
-    const float *L0 = P.lib + (int64_t)g.k * M;
-    const float *L1 = L0 + M;
-    const int Wp = P.Wp;
-    auto tap = [&](int which, int r, int c) -> float {
-      if (kSmem) {
-        const float *s = which ? s1 : s0;
-        return s[(r + 1) * Wp + (c + 4)];
-      } else {
-        if (r < 0 || r >= n || c < 0 || c >= n) return 0.f;
-        return __ldg((which ? L1 : L0) + r * n + c);
-      }
-    };
-    const long long h = n - 1;
-    const long long base = h << PSFSIM_FRAC_BITS;
-    // lane: pixel column q0 + lane, down the block's 32 rows (exact steps)
-    const int q = q0 + lane;
-    long long a2 = base + g.C * (2 * q - h) + g.Sn * (2 * p0 - h);
-    long long b2 = base - g.Sn * (2 * q - h) + g.C * (2 * p0 - h);
-    for (int a = 0; a < kSymBlk; ++a) {
-      blk[a * kSymPitch + lane] = rotated_value(a2, b2, n, g.w0, g.w1, tap);
-      a2 += 2 * g.Sn;
-      b2 += 2 * g.C;
-    }
+  const long long h = n - 1;
+  const long long base = h << PSFSIM_FRAC_BITS;
+  const int q = q0 + lane;
+  long long a2 = base + g.C * (2 * q - h) + g.Sn * (2 * p0 - h);
+  long long b2 = base - g.Sn * (2 * q - h) + g.C * (2 * p0 - h);
+  float *r0 = A.at[0] + (int64_t)p0 * n + q, *r2 = A.at[2] + (int64_t)(n - 1 - p0) * n + (n - 1 - q);
+#pragma unroll 4
+  for (int a = 0; a < kSymBlk; ++a, r0 += n, r2 -= n) {
+    each_row(a);
+    const float v = value(a2, b2);
+    blk[a * kSymPitch + lane] = v;
+    __stcs(r0, v);
+    __stcs(r2, v);
+    a2 += 2 * g.Sn;
+    b2 += 2 * g.C;
   }
   __syncwarp();
-  // Row r of each turned block: m = 0 row p0 + r; m = 1 row q0 + r (source
-  // column r, rows reversed); m = 2 row n-1-p0-r (reversed); m = 3 row
-  // n-1-q0-r (source column r).  Lane l writes floats 4 (l % 8) .. +3 of row
-  // r0 + l / 8, so one 16-byte store instruction covers four rows (the rows
-  // are 128-byte aligned: n, p0 and q0 are multiples of 32).
-  const int rr = lane >> 3, f = (lane & 7) * 4;
-  for (int r0 = 0; r0 < kSymBlk; r0 += 4) {
-    const int r = r0 + rr;
-    float4 v0, v1, v2, v3;
-    float *a0 = &v0.x, *a1 = &v1.x, *a2 = &v2.x, *a3 = &v3.x;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      a0[i] = blk[r * kSymPitch + f + i];
-      a1[i] = blk[(kSymBlk - 1 - f - i) * kSymPitch + r];
-      a2[i] = blk[r * kSymPitch + (kSymBlk - 1 - f - i)];
-      a3[i] = blk[(f + i) * kSymPitch + r];
-    }
-    __stcs(reinterpret_cast<float4 *>(Am[0] + (int64_t)(p0 + r) * n + q0 + f), v0);
-    __stcs(reinterpret_cast<float4 *>(Am[1] + (int64_t)(q0 + r) * n + (n - kSymBlk - p0) + f), v1);
-    __stcs(reinterpret_cast<float4 *>(Am[2] + (int64_t)(n - 1 - p0 - r) * n + (n - kSymBlk - q0) + f), v2);
-    __stcs(reinterpret_cast<float4 *>(Am[3] + (int64_t)(n - 1 - q0 - r) * n + p0 + f), v3);
+  // Copy 1: row q0 + r, columns n-32-p0 .. (source column r, rows reversed);
+  // copy 3: row n-1-q0-r, columns p0 .. (source column r).
+  float *r1 = A.at[1] + (int64_t)q0 * n + (n - kSymBlk - p0) + lane, *r3 = A.at[3] + (int64_t)(n - 1 - q0) * n + p0 + lane;
+#pragma unroll 4
+  for (int r = 0; r < kSymBlk; ++r, r1 += n, r3 -= n) {
+    __stcs(r1, blk[(kSymBlk - 1 - lane) * kSymPitch + r]);
+    __stcs(r3, blk[lane * kSymPitch + r]);
   }
 }
 
-// As build_fp32_kernel, over the bracket-sorted list of the quadrant's
-// columns, in (column, 32 x 32 pixel block) tasks; each warp also owns a
-// 32 x 33 float block buffer after the staged pair.
-template <bool kSmem>
-__global__ void __launch_bounds__(512, 1) build_fp32_sym_kernel(const __grid_constant__ CUtensorMap map,
-                                                             const BuildParams P) {
+// Dense FP32 storage of an even grid, n % 32 == 0: the CTAs deal the sorted
+// quadrant columns round-robin (neighbours in the list, so the same PSFs, are in
+// work at once, and the columns beyond the last radius spread evenly); the warps
+// of a CTA take the 32 x 32 blocks of its column.
+// kLerped: the column's lerped PSF sits in shared memory, zero-bordered by one
+// pixel, and while a column is sampled its CTA lerps the next one into the other
+// of two buffers, loads eight rows ahead of their use.  Four taps an element
+// instead of eight, at a row pitch where a rotated line of 32 taps meets few bank
+// conflicts, and half the passes through shared memory for the copies: 1156 ->
+// 960 us for the paper's 16384 x 65536 A (4.5 TB/s written; no pipe is the bound
+// alone: issue 55 %, L1 data pipe 55 %, with 16 warps an SM in shared memory's
+// reach).  32 warps of 16-row blocks, whose turned rows are 64 bytes: 1040 us.
+template <bool kLerped>
+__global__ void __launch_bounds__(512, 1) build_fp32_sym_kernel(const BuildParams P) {
   extern __shared__ __align__(128) float smem[];
-  __shared__ __align__(8) uint64_t mbar;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  const int pair_floats = kSmem ? 2 * (P.n + 2) * P.Wp : 0;
-  float *s0 = smem;
-  float *s1 = smem + (P.n + 2) * P.Wp;
-  float *blk = smem + pair_floats + warp * (kSymBlk * kSymPitch);
-  if (kSmem && threadIdx.x == 0) {
-    ptx::mbar_init(&mbar, 1);
-    ptx::fence_mbar_init();
-  }
-  __syncthreads();
-  const int nbq = P.n / kSymBlk, nblocks = nbq * nbq;
-  for_each_bracket_group<kSmem>(&map, P, s0, &mbar, [&](int64_t pos, int64_t gend) {
-    // the group's tasks, dealt round-robin to the warps
-    for (int64_t t = warp; t < (gend - pos) * nblocks; t += nwarps) {
-      const int jq = P.order[pos + t / nblocks];
-      const int b = (int)(t % nblocks);
-      build_block_sym<kSmem>(P, jq, (b / nbq) * kSymBlk, (b % nbq) * kSymBlk, s0, s1, blk, lane);
+  const int n = P.n, Wp = P.Wp, plane = kLerped ? (n + 2) * Wp : 0;
+  const int64_t M = (int64_t)n * n;
+  float *blk = smem + 2 * plane + warp * (kSymBlk * kSymPitch);
+  const int nbq = n / kSymBlk, nblocks = nbq * nbq;
+  if (kLerped)
+    for (int i = threadIdx.x; i < 2 * plane; i += blockDim.x) smem[i] = 0.f;  // the borders stay zero
+  // The thread's share of a column, two quads of pixels at a time: quads
+  // threadIdx.x + blockDim.x i of the plane.
+  constexpr int kBatch = 2;
+  const int quads = (int)(M >> 2), rowq = n >> 2;
+  const int per = (quads + (int)blockDim.x * kBatch - 1) / ((int)blockDim.x * kBatch);  // batches a thread
+  float4 l0[kBatch], l1[kBatch];
+  auto fetch = [&](const ColGeom &g, int batch) {
+    const float4 *L0 = reinterpret_cast<const float4 *>(P.lib + (int64_t)g.k * M) + threadIdx.x;
+    const float4 *L1 = reinterpret_cast<const float4 *>(P.lib + (int64_t)(g.k + 1) * M) + threadIdx.x;
+#pragma unroll
+    for (int e = 0; e < kBatch; ++e) {
+      const int i = (batch * kBatch + e) * (int)blockDim.x;
+      if (i + (int)threadIdx.x < quads) {
+        l0[e] = __ldg(L0 + i);
+        l1[e] = __ldg(L1 + i);
+      }
     }
-  });
+  };
+  auto put = [&](const ColGeom &g, int batch, float *dst) {
+#pragma unroll
+    for (int e = 0; e < kBatch; ++e) {
+      const int i = (batch * kBatch + e) * (int)blockDim.x + (int)threadIdx.x;
+      if (i < quads) {
+        const int r = i / rowq;
+        *reinterpret_cast<float4 *>(dst + (r + 1) * Wp + 4 * (i - r * rowq) + 4) =
+            make_float4(lerp_pixel(g.w0, g.w1, l0[e].x, l1[e].x), lerp_pixel(g.w0, g.w1, l0[e].y, l1[e].y),
+                        lerp_pixel(g.w0, g.w1, l0[e].z, l1[e].z), lerp_pixel(g.w0, g.w1, l0[e].w, l1[e].w));
+      }
+    }
+  };
+  ColGeom g;
+  int jq = 0;
+  int64_t pos = blockIdx.x;
+  if (pos < P.K) {
+    jq = P.order[pos];
+    g = P.geom[jq];
+  }
+  if (kLerped) {
+    __syncthreads();
+    if (pos < P.K && g.k >= 0)
+      for (int b = 0; b < per; ++b) {
+        fetch(g, b);
+        put(g, b, smem);
+      }
+    __syncthreads();
+  }
+  for (int buf = 0; pos < P.K; pos += gridDim.x, buf ^= 1) {
+    const bool more = pos + gridDim.x < P.K;
+    int jn = 0;
+    ColGeom gn;
+    gn.k = -1;
+    if (more) {
+      jn = P.order[pos + gridDim.x];
+      gn = P.geom[jn];
+    }
+    const float *cur = smem + buf * plane;
+    float *dst = smem + (buf ^ 1) * plane;
+    const bool lerp = kLerped && gn.k >= 0;
+    int fetched = 0, done = 0;  // batches of the next column loaded, and lerped
+    const TurnedColumns A = turned_columns(P, jq);
+    for (int b = warp; b < nblocks; b += nwarps) {
+      const int p0 = (b / nbq) * kSymBlk, q0 = (b % nbq) * kSymBlk;
+      if (g.k < 0) {  // beyond the last radius: zeros
+        build_block_sym(n, g, A, p0, q0, blk, lane, [](long long, long long) { return 0.f; }, [](int) {});
+      } else if (kLerped) {
+        build_block_sym(
+            n, g, A, p0, q0, blk, lane,
+            [&](long long a2, long long b2) {
+              // Pixel (p, q) sits at (p + 1, q + 4); a footprint wholly outside reads
+              // the zeros right of the first row's border.
+              constexpr int kShift = PSFSIM_FRAC_BITS + 1;
+              const unsigned qa = (unsigned)((int)(a2 >> kShift) + 1), pb = (unsigned)((int)(b2 >> kShift) + 1);
+              const bool in = qa <= (unsigned)n && pb <= (unsigned)n;
+              const float *t = cur + (in ? pb * (unsigned)Wp + qa + 3u : (unsigned)n + 4u);
+              return bilinear(t[0], t[1], t[Wp], t[Wp + 1], (unsigned)((unsigned long long)a2 >> (kShift - 32)),
+                              (unsigned)((unsigned long long)b2 >> (kShift - 32)));
+            },
+            [&](int a) {
+              if (lerp && (a & 7) == 0) {
+                if (done < fetched) put(gn, done++, dst);
+                if (fetched < per) fetch(gn, fetched++);
+              }
+            });
+      } else {
+        const float *L0 = P.lib + (int64_t)g.k * M, *L1 = L0 + M;
+        build_block_sym(
+            n, g, A, p0, q0, blk, lane,
+            [&](long long a2, long long b2) {
+              return rotated_value(a2, b2, n, g.w0, g.w1, [&](int r, int c, float &l0, float &l1) {
+                l0 = l1 = 0.f;
+                if (r >= 0 && r < n && c >= 0 && c < n) {
+                  l0 = __ldg(L0 + r * n + c);
+                  l1 = __ldg(L1 + r * n + c);
+                }
+              });
+            },
+            [](int) {});
+      }
+    }
+    if (kLerped) {
+      if (lerp) {
+        if (done < fetched) put(gn, done++, dst);
+        for (; fetched < per; ++fetched) {
+          fetch(gn, fetched);
+          put(gn, done++, dst);
+        }
+      }
+      __syncthreads();
+    }
+    jq = jn;
+    g = gn;
+  }
+}
+
+// Row pitch of a lerped plane: a multiple of 4 (quads of pixels are stored at
+// once), at least n + 8 (the border, and zeros beyond it).  Of those up to 28
+// more, 20 and then 28 mod 32 meet a rotated line of 32 taps with the fewest bank
+// conflicts over the angles (2.3 ways; 0 mod 32: 8), where two planes and the
+// block buffers then fit.
+constexpr size_t kSymSmem = 226 * 1024;
+inline size_t sym_smem(int n, int pitch, int warps) {
+  return (2ull * (n + 2) * pitch + (size_t)warps * kSymBlk * kSymPitch) * 4;
+}
+inline int sym_pitch(int n, int warps) {
+  for (int residue : {20, 28}) {
+    const int p = (n + 8 - residue + 31) / 32 * 32 + residue;
+    if (sym_smem(n, p, warps) <= kSymSmem) return p;
+  }
+  return n + 8;
 }
 
 }  // namespace
@@ -640,15 +769,17 @@ static cudaError_t launch_tables_and_build(psfsim_plan *h, cudaStream_t st) {
     // Even grid: the quadrant's columns (the sorted list holds just those),
     // four turned copies each.
     P.K = Kg;
-    const size_t blk_bytes = 16ull * kSymBlk * kSymPitch * 4;  // 16 warps
-    const bool staged = use_smem && smem + blk_bytes <= 220 * 1024;
-    const size_t total = (staged ? smem : 0) + blk_bytes;
-    auto kern = staged ? build_fp32_sym_kernel<true> : build_fp32_sym_kernel<false>;
+    const int nblocks = (n / kSymBlk) * (n / kSymBlk), warps = nblocks < 16 ? nblocks : 16;
+    P.Wp = sym_pitch(n, warps);
+    const bool lerped = sym_smem(n, P.Wp, warps) <= kSymSmem;
+    const size_t total = lerped ? sym_smem(n, P.Wp, warps) : (size_t)warps * kSymBlk * kSymPitch * 4;
+    auto kern = lerped ? build_fp32_sym_kernel<true> : build_fp32_sym_kernel<false>;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)total)) != cudaSuccess)
       return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 512, total)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * warps, total)) != cudaSuccess) return e;
     per_sm = per_sm < 1 ? 1 : per_sm;
-    kern<<<h->num_sms * per_sm, 512, total, st>>>(staged ? h->lib_map : dummy, P);
+    const int64_t grid = (int64_t)h->num_sms * per_sm;
+    kern<<<(unsigned)(grid < Kg ? grid : Kg), 32 * warps, total, st>>>(P);
     return cudaGetLastError();
   }
   if (use_smem) {

@@ -17,8 +17,8 @@ from . import _binding as B
 from .plan import Plan, _stream_ptr
 
 
-def _vp(t: torch.Tensor) -> ctypes.c_void_p:
-    return ctypes.c_void_p(t.data_ptr())
+def _vp(t: torch.Tensor) -> int:
+    return t.data_ptr()
 
 
 class RingProblem:
@@ -54,19 +54,21 @@ class RingProblem:
         self.fused = self.lib.psfsim_ring_gradient_scratch_bytes(plan.handle, ctypes.byref(nb)) == B.OK
         self.gscr = torch.zeros(max(nb.value, 256), **u8) if self.fused else None
         self.launches = 0
+        # Where loss_and_grad's result lands: pinned, so that the copy neither stages nor allocates.
+        self._host6 = torch.empty(6, dtype=torch.float64).pin_memory()
 
     # -- operators ---------------------------------------------------------
     def scene(self, theta, out: torch.Tensor | None = None) -> torch.Tensor:
         z = self.z if out is None else out
         th = np.ascontiguousarray(theta, dtype=np.float64)
-        B.check(self.lib.psfsim_ring_scene(self.N, self.S, self.r_max, th.ctypes.data_as(ctypes.c_void_p), _vp(z),
+        B.check(self.lib.psfsim_ring_scene(self.N, self.S, self.r_max, th.ctypes.data, _vp(z),
                                            _stream_ptr(None)), "psfsim_ring_scene")
         self.launches += 1
         return z
 
     def chain(self, theta, gz: torch.Tensor) -> torch.Tensor:
         th = np.ascontiguousarray(theta, dtype=np.float64)
-        B.check(self.lib.psfsim_ring_chain(self.N, self.S, self.r_max, th.ctypes.data_as(ctypes.c_void_p), _vp(gz),
+        B.check(self.lib.psfsim_ring_chain(self.N, self.S, self.r_max, th.ctypes.data, _vp(gz),
                                            _vp(self.dtheta), _vp(self.cscr), self.cscr.numel(), _stream_ptr(None)),
                 "psfsim_ring_chain")
         self.launches += 2
@@ -89,7 +91,7 @@ class RingProblem:
     def enqueue_forward_loss(self, theta) -> None:
         """First half (one launch): ring scene and Jacobian, S = A Z with residual and loss partials."""
         th = np.ascontiguousarray(theta, dtype=np.float64)
-        B.check(self.lib.psfsim_ring_forward_loss(self.plan.handle, self.r_max, th.ctypes.data_as(ctypes.c_void_p),
+        B.check(self.lib.psfsim_ring_forward_loss(self.plan.handle, self.r_max, th.ctypes.data,
                                                   _vp(self.target), self.sigma, _vp(self.z), _vp(self.y), _vp(self.r),
                                                   _vp(self.gscr), self.gscr.numel(), _stream_ptr(None)),
                 "psfsim_ring_forward_loss")
@@ -98,7 +100,7 @@ class RingProblem:
     def enqueue_adjoint_chain(self, theta) -> None:
         """Second half (one launch): A^T r, its dot with the stored Jacobian, the final sums into out6."""
         th = np.ascontiguousarray(theta, dtype=np.float64)
-        B.check(self.lib.psfsim_ring_adjoint_chain(self.plan.handle, self.r_max, th.ctypes.data_as(ctypes.c_void_p),
+        B.check(self.lib.psfsim_ring_adjoint_chain(self.plan.handle, self.r_max, th.ctypes.data,
                                                    _vp(self.r), _vp(self.gz), _vp(self.out6), _vp(self.gscr),
                                                    self.gscr.numel(), _stream_ptr(None)),
                 "psfsim_ring_adjoint_chain")
@@ -109,7 +111,7 @@ class RingProblem:
         in out6 = (loss, dL/dtheta)."""
         if self.fused:  # one C-ABI call enqueues both halves
             th = np.ascontiguousarray(theta, dtype=np.float64)
-            B.check(self.lib.psfsim_ring_gradient(self.plan.handle, self.r_max, th.ctypes.data_as(ctypes.c_void_p),
+            B.check(self.lib.psfsim_ring_gradient(self.plan.handle, self.r_max, th.ctypes.data,
                                                   _vp(self.target), self.sigma, _vp(self.z), _vp(self.y),
                                                   _vp(self.r), _vp(self.gz), _vp(self.out6), _vp(self.gscr),
                                                   self.gscr.numel(), _stream_ptr(None)),
@@ -128,7 +130,11 @@ class RingProblem:
 
     def loss_and_grad(self, theta):
         self.enqueue_gradient(theta)
-        out = self.out6.cpu().numpy()
+        out = self.out6
+        if out.is_cuda:
+            out = self._host6.copy_(out, non_blocking=True)
+        torch.cuda.current_stream().synchronize()
+        out = out.numpy()
         return float(out[0]), out[1:].copy()
 
     def gauss_newton_diagonal(self, theta) -> np.ndarray:

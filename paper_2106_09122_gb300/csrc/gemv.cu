@@ -5,6 +5,7 @@
 //            across the CTA, fixed-order reduction.
 #include "gemv_device.cuh"
 #include "psfsim_internal.cuh"
+#include "reduce.cuh"
 
 using namespace psfsim_gemv;
 
@@ -153,43 +154,12 @@ __global__ void __launch_bounds__(kFwdThreads, fwd_min_ctas(BB)) fwd_cols_kernel
   }
 }
 
-// y[b, i] = sum_ks part[ks, b, i] in a fixed order.  A CTA covers 128 rows;
-// its 8 warps split the KS partials (ks = warp, warp + 8, ...) and combine
-// through shared memory, so every output needs only ~KS/8 loads per thread.
-constexpr int kRedRows = 128;
-// y may be part itself with M = ld: a CTA reads its rows before it writes them.
+// y[b, i] = sum_ks part[ks, b, i] (reduce.cuh).  y may be part itself with M = ld.
 __global__ void __launch_bounds__(256) fwd_reduce_kernel(const float *part, int KS, int B, int64_t ld, int64_t M,
                                                          float *y) {
   __shared__ float4 red[8][32];
-  const int c4 = threadIdx.x & 31, grp = threadIdx.x >> 5;
-  const int64_t r = ((int64_t)blockIdx.x * 32 + c4) * 4;
   const int b = blockIdx.y;
-  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (r < ld) {
-    const float *p = part + (int64_t)b * ld + r;
-    const int64_t step = (int64_t)B * ld;
-    int ks = grp;
-#pragma unroll 4
-    for (; ks < KS; ks += 8) {
-      const float4 v = *reinterpret_cast<const float4 *>(p + ks * step);
-      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-    }
-  }
-  red[grp][c4] = s;
-  __syncthreads();
-  if (grp == 0 && r < M) {
-    float4 t = red[0][c4];
-#pragma unroll
-    for (int k = 1; k < 8; ++k) {
-      const float4 v = red[k][c4];
-      t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
-    }
-    float *out = y + (int64_t)b * M + r;
-    out[0] = t.x;
-    if (r + 1 < M) out[1] = t.y;
-    if (r + 2 < M) out[2] = t.z;
-    if (r + 3 < M) out[3] = t.w;
-  }
+  reduce_partials(part + (int64_t)b * ld, (int64_t)B * ld, KS, ld, M, y + (int64_t)b * M, red);
 }
 
 // One residual: gx[j] = sum_i A[i, j] g[i] for the CTA's contiguous range of the
@@ -510,7 +480,7 @@ cudaError_t psfsim_launch_forward_fp32(const psfsim_plan *h, const float *x, int
 
 cudaError_t psfsim_launch_reduce_partials(const float *part, int KS, int B, int64_t ld, int64_t M, float *y,
                                           cudaStream_t st) {
-  dim3 grid((unsigned)((ld + kRedRows - 1) / kRedRows), (unsigned)B);
+  dim3 grid((unsigned)reduce_ctas(KS, M), (unsigned)B);
   fwd_reduce_kernel<<<grid, 256, 0, st>>>(part, KS, B, ld, M, y);
   return cudaGetLastError();
 }

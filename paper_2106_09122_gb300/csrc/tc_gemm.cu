@@ -38,6 +38,7 @@
 #include "live.cuh"
 #include "psfsim_internal.cuh"
 #include "ptx_util.cuh"
+#include "reduce.cuh"
 
 namespace {
 
@@ -54,12 +55,19 @@ constexpr uint32_t kTileBytes = BM * BK * 2;
 constexpr int kMaxBp = 80;       // 3 * Bp <= 256 (MMA N and TMA box limits), Bp % 16 == 0
 constexpr int kMaxJobs = 16;
 constexpr int kDefaultChunk = 4; // k-tiles (of 64) per TMEM accumulation, split-BF16 storage
+// One job of split storage: fewer splits sum longer runs (choose_ks), and draining
+// more often pays that back without costing time: 16 scenes of 128^2 take 141 us at
+// 4, 2 and 1 k-tiles, their error is 3.9e-7, 2.1e-7 and 1.5e-7.  Accumulators of
+// more than 128 columns are drained slower than they fill: 64 scenes take 149 us
+// at 4 and 3, 155 at 2, 173 at 1.
+constexpr int kSingleChunk = 1, kSingleChunkWide = 3;
 constexpr int kDefaultChunkHiMulti = 2;  // BF16 storage (hi alone), several jobs in one launch
 // Adjoint of split storage: residuals change sign, so its sums cancel and the
 // drift weighs more (error against 64 bits 2.493e-6 with plain FP32 sums, 2.553
 // at 4 k-tiles, 2.492 at one; 8 residuals of 128^2 take 127 and 129 us, 64 of
 // 256^2 1.45 and 1.64 ms).
 constexpr int kAdjointChunk = 1;
+constexpr int kAdjointRun = 160;  // and the most k-tiles a unit adds up
 constexpr int kMaxMmas = 64;     // accumulating MMAs between drains (bounds the FP32 drift)
 
 // One product S_j = A_j Z_j of a (possibly multi-job) launch.
@@ -180,42 +188,13 @@ struct RMulti {
   RJob job[kMaxJobs];
 };
 
-// y[b, i] = sum_ks part[ks, b, i] of job blockIdx.z in a fixed order, 128 rows
-// per CTA: its 8 warps take ks = warp, warp + 8, ... and combine through
-// shared memory.  One launch serves every job.
-constexpr int kRedRows = 128;
+// y[b, i] = sum_ks part[ks, b, i] of job blockIdx.z (reduce.cuh).  One launch serves every job.
 __global__ void __launch_bounds__(256) tc_reduce_kernel(const __grid_constant__ RMulti P) {
   __shared__ float4 red[8][32];
   const RJob &J = P.job[blockIdx.z];
-  const int c4 = threadIdx.x & 31, grp = threadIdx.x >> 5;
-  const int64_t r = ((int64_t)blockIdx.x * 32 + c4) * 4;
   const int b = blockIdx.y;
-  if (b >= J.cap || (int64_t)blockIdx.x * kRedRows >= J.M || (J.count && b >= *J.count)) return;
-  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (r < J.rows) {
-    const float *p = J.part + (int64_t)b * J.rows + r;
-    const int64_t step = (int64_t)J.cap * J.rows;
-#pragma unroll 4
-    for (int ks = grp; ks < J.KS; ks += 8) {
-      const float4 v = *reinterpret_cast<const float4 *>(p + ks * step);
-      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-    }
-  }
-  red[grp][c4] = s;
-  __syncthreads();
-  if (grp == 0 && r < J.M) {
-    float4 t = red[0][c4];
-#pragma unroll
-    for (int k = 1; k < 8; ++k) {
-      const float4 v = red[k][c4];
-      t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
-    }
-    float *out = J.y + (int64_t)b * J.M + r;
-    out[0] = t.x;
-    if (r + 1 < J.M) out[1] = t.y;
-    if (r + 2 < J.M) out[2] = t.z;
-    if (r + 3 < J.M) out[3] = t.w;
-  }
+  if (b >= J.cap || (J.count && b >= *J.count)) return;
+  reduce_partials(J.part + (int64_t)b * J.rows, (int64_t)J.cap * J.rows, J.KS, J.rows, J.M, J.y + (int64_t)b * J.M, red);
 }
 
 // The adjoint's result from its partial sums, part[KS][cap][rows] per block of
@@ -754,24 +733,6 @@ bool encode_bf16_2d(CUtensorMap *map, const void *base, uint64_t inner, uint64_t
 }
 
 
-// Split factor over k: smallest KS whose unit count fills the SMs evenly.
-int choose_ks(int m_tiles, int k_tiles, int num_sms) {
-  int best = 1;
-  double best_eff = 0.0;
-  for (int ks = 1; ks <= 64 && ks <= k_tiles; ++ks) {
-    const int64_t units = (int64_t)m_tiles * ks;
-    const int64_t waves = (units + num_sms - 1) / num_sms;
-    const double eff = (double)units / (double)(waves * num_sms);
-    const bool enough = units >= 2 * num_sms || ks == k_tiles;
-    if (eff > best_eff + 1e-9 && (enough || eff > best_eff + 0.05)) {
-      best = ks;
-      best_eff = eff;
-    }
-    if (enough && eff >= 0.97) return ks;
-  }
-  return best;
-}
-
 struct JobSpec {
   const psfsim_plan *h;
   const float *x;
@@ -787,6 +748,46 @@ struct JobPlan {
   size_t xs_off, part_off;
 };
 
+// Split over k of a single job: the cheapest by the launch's clocks.  CTAs walk the
+// units in rounds of `slots`; a k-tile of a round takes what its TMA pipeline needs
+// alone (1750 clocks, 1300 without lo), its share of memory at 4000 bytes a clock,
+// or its SM's shared memory under the MMAs, whichever is longest.  A unit's start
+// and store cost 1800; partial images 2700 for their launch and their bytes
+// written and read again.  The constants are a fit to 96 products (64^2..256^2
+// pixels and grids, 1..64 scenes, both directions, both storages) at 15 splits
+// each: 1.4 % above the best split on average, 12 % at worst.  The smallest split
+// that fills the SMs evenly was 9.3 % above on average: 23 scenes of a 100^2 BF16
+// plan on 85^2 pixels ran 1817 units in 43 us, 237 in 37; 64 of a 256^2 one on
+// 64^2 pixels took 121 us in three splits, 78 in one.  At most `most` k-tiles a
+// unit: the drained sums add up one after another in FP32, and the adjoint of
+// 256^2 split storage erred 2 % more with its 1024 in one chain than in runs of
+// 146 (kAdjointRun; 1.32 ms, 1.30 in one).
+int choose_ks(const JobPlan &p, int cap, int x_rows, bool lo, bool direct1, int most, int slots,
+              int num_sms) {
+  const double a_bytes = lo ? 2.0 * kTileBytes : kTileBytes, x_bytes = x_rows * BK * 2.0;
+  const double alone = lo ? 1750.0 : 1300.0, mma = (lo ? 2.0 : 1.0) * (kTileBytes + x_bytes) / 48.0;
+  auto tile = [&](int64_t active) {
+    const double mem = (double)active * (a_bytes + x_bytes) / 4000.0;
+    const double sm = (double)((active + num_sms - 1) / num_sms) * mma;
+    return fmax(alone, fmax(mem, sm));
+  };
+  const int fewest = (p.k_tiles + most - 1) / most < 64 ? (p.k_tiles + most - 1) / most : 64;
+  int best = fewest;
+  double least = 1e300;
+  for (int ks = fewest; ks <= 64 && ks <= p.k_tiles; ++ks) {
+    const int64_t units = (int64_t)p.m_tiles * ks, full = units / slots, rest = units % slots;
+    const double kt = (p.k_tiles + ks - 1) / ks;
+    double cost = (double)full * (kt * tile(slots) + 1800.0);
+    if (rest) cost += kt * tile(rest) + 1800.0;
+    if (ks > 1 || !direct1) cost += 2700.0 + (double)ks * cap * (double)p.rows * 4.0 / 3000.0;
+    if (cost < least * 0.9999) {
+      least = cost;
+      best = ks;
+    }
+  }
+  return best;
+}
+
 struct MultiPlan {
   JobPlan jp[kMaxJobs];
   int njobs, units, stages, chunk, ctas_per_sm;
@@ -799,14 +800,17 @@ struct MultiPlan {
 // that fit for one job and kDefaultChunkHiMulti for several (the fastest
 // measured on one 128^2 job and on eight 256^2 jobs); split factors chosen so
 // that the whole launch has about units_per_sm work units per SM (or, for a
-// single job without tuning, the smallest split that fills the SMs evenly);
-// as many smem stages as fit.
+// single job without tuning, by choose_ks); as many smem stages as fit.
 MultiPlan plan_multi(const JobSpec *jobs, int nj, const psfsim_tuning_t *tune, bool adjoint = false) {
   MultiPlan mp;
   std::memset(&mp, 0, sizeof(mp));
   mp.njobs = nj;
   const int num_sms = jobs[0].h->num_sms;
   const int ups = tune && tune->units_per_sm > 0 ? tune->units_per_sm : 0;
+  // A stage holds hi, lo (when any job has one) and the x tile; without lo
+  // the stage is smaller, so more stages (bytes in flight) fit.
+  bool any_lo = false;
+  int x_rows = 0;  // largest B operand: x parts x Bp
   int64_t total = 0;
   for (int j = 0; j < nj; ++j) {
     const psfsim_plan *h = jobs[j].h;
@@ -816,15 +820,24 @@ MultiPlan plan_multi(const JobSpec *jobs, int nj, const psfsim_tuning_t *tune, b
     p.m_tiles = (int)(p.rows / BM);
     p.k_tiles = adjoint ? (int)(psfsim_round_up(h->M, BM) / BK) : h->k_tiles;
     total += (int64_t)p.m_tiles * p.k_tiles;
+    const bool lo = h->lo_off >= 0;
+    any_lo = any_lo || lo;
+    const int r = (lo || adjoint ? 3 : 2) * p.Bp;
+    x_rows = r > x_rows ? r : x_rows;
   }
+  // Accumulators of at most 128 columns: two CTAs per SM, each with half the
+  // shared memory and half the tensor memory.
+  const bool narrow = x_rows <= (int)kAccStrideNarrow;
+  mp.ctas_per_sm = narrow ? 2 : 1;
   const int64_t target_units = (int64_t)(ups ? ups : 4) * num_sms;
   const int64_t per_unit = (total + target_units - 1) / target_units;
-  int Bp_max = 16, units = 0;
+  int units = 0;
   size_t off = 0;
   for (int j = 0; j < nj; ++j) {
     JobPlan &p = mp.jp[j];
     if (nj == 1 && !ups) {
-      p.KS = choose_ks(p.m_tiles, p.k_tiles, num_sms);
+      p.KS = choose_ks(p, jobs[j].cap, x_rows, any_lo, jobs[j].first < 0 && !adjoint,
+                       adjoint && any_lo ? kAdjointRun : p.k_tiles, num_sms * mp.ctas_per_sm, num_sms);
     } else {
       int ks = (int)((p.k_tiles + per_unit - 1) / (per_unit > 0 ? per_unit : 1));
       ks = ks < 1 ? 1 : ks;
@@ -832,7 +845,6 @@ MultiPlan plan_multi(const JobSpec *jobs, int nj, const psfsim_tuning_t *tune, b
       p.KS = ks > p.k_tiles ? p.k_tiles : ks;
     }
     units += p.m_tiles * p.KS;
-    Bp_max = p.Bp > Bp_max ? p.Bp : Bp_max;
     const psfsim_plan *h = jobs[j].h;
     p.xs_off = off;
     off += (size_t)psfsim_round_up(3ll * p.Bp * p.k_tiles * BK * 2, 256);
@@ -841,22 +853,8 @@ MultiPlan plan_multi(const JobSpec *jobs, int nj, const psfsim_tuning_t *tune, b
   }
   mp.units = units;
   mp.scratch = off;
-  // A stage holds hi, lo (when any job has one) and the x tile; without lo
-  // the stage is smaller, so more stages (bytes in flight) fit.
-  bool any_lo = false;
-  int x_rows = 0;  // largest B operand: x parts x Bp
-  for (int j = 0; j < nj; ++j) {
-    const bool lo = jobs[j].h->lo_off >= 0;
-    any_lo = any_lo || lo;
-    const int r = (lo || adjoint ? 3 : 2) * mp.jp[j].Bp;
-    x_rows = r > x_rows ? r : x_rows;
-  }
   mp.x_off = (any_lo ? 2 : 1) * kTileBytes;
   mp.stage_bytes = (uint32_t)psfsim_round_up(mp.x_off + (int64_t)x_rows * BK * 2, 1024);
-  // Accumulators of at most 128 columns: two CTAs per SM, each with half the
-  // shared memory and half the tensor memory.
-  const bool narrow = x_rows <= (int)kAccStrideNarrow;
-  mp.ctas_per_sm = narrow ? 2 : 1;
   mp.tmem_cols = narrow ? kTmemColsNarrow : kTmemColsWide;
   mp.acc_stride = narrow ? kAccStrideNarrow : kAccStrideWide;
   int fit = (int)(((narrow ? 108 : 220) * 1024) / mp.stage_bytes);
@@ -866,7 +864,10 @@ MultiPlan plan_multi(const JobSpec *jobs, int nj, const psfsim_tuning_t *tune, b
   // accumulate between drains.
   const int max_chunk = kMaxMmas / ((any_lo ? 2 : 1) * (BK / 16));
   mp.chunk = tune && tune->chunk > 0 ? (tune->chunk > max_chunk ? max_chunk : tune->chunk)
-                                     : (adjoint && any_lo ? kAdjointChunk : any_lo || adjoint ? kDefaultChunk : (nj > 1 ? kDefaultChunkHiMulti : max_chunk));
+                                     : (adjoint && any_lo ? kAdjointChunk
+                                        : any_lo && !adjoint && nj == 1 ? (narrow ? kSingleChunk : kSingleChunkWide)
+                                        : any_lo || adjoint ? kDefaultChunk
+                                        : (nj > 1 ? kDefaultChunkHiMulti : max_chunk));
   mp.smem = (size_t)mp.stages * mp.stage_bytes + 1024;
   return mp;
 }
@@ -890,7 +891,7 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
   std::memset(&P, 0, sizeof(P));
   std::memset(&XP, 0, sizeof(XP));
   std::memset(&RP, 0, sizeof(RP));
-  int64_t x_blocks = 1, red_rows = 0;
+  int64_t x_blocks = 1, red_ctas = 0;
   int nred = 0, red_cap = 0;
   for (int j = 0; j < nj; ++j) {
     const psfsim_plan *h = jobs[j].h;
@@ -962,7 +963,8 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
       R.M = h->M;
       R.KS = p.KS;
       R.cap = jobs[j].cap;
-      red_rows = h->M > red_rows ? h->M : red_rows;
+      const int64_t ctas = reduce_ctas(p.KS, h->M);
+      red_ctas = ctas > red_ctas ? ctas : red_ctas;
       red_cap = R.cap > red_cap ? R.cap : red_cap;
     }
   }
@@ -995,8 +997,7 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (jobs[0].first >= 0 || adjoint) return cudaSuccess;  // the caller adds the rotations (SymSum), or finishes
   if (nred > 0)
-    tc_reduce_kernel<<<dim3((unsigned)((red_rows + kRedRows - 1) / kRedRows), (unsigned)red_cap, (unsigned)nred), 256, 0,
-                       st>>>(RP);
+    tc_reduce_kernel<<<dim3((unsigned)red_ctas, (unsigned)red_cap, (unsigned)nred), 256, 0, st>>>(RP);
   return cudaGetLastError();
 }
 

@@ -189,3 +189,24 @@ def test_forward_of_many_scenes(storage, tol, B, n):
     that end inside a tile of 256 pixels, skipped k-tiles."""
     plan, A, rng = _plan(64, 0.125, 3.0, storage, n=n)
     _check_forward(plan, A, rng.uniform(0.0, 1.0, (B, 64 * 64)).astype(np.float32), tol)
+
+
+@pytest.mark.parametrize("storage,tol", [("split_bf16", 1e-5), ("bf16", 2.0 ** -8 + 2.5e-5)])
+@pytest.mark.parametrize("units", [0, 1, 2, 40])
+@pytest.mark.parametrize("n,shift", [(17, 0), (33, 0), (32, 0), (32, 1), (40, 2)])
+def test_sum_over_splits(storage, tol, units, n, shift):
+    """One job's k-splits from none to more than 8 (both forms of their sum), into images whose
+    rows start at any 4-byte address, ending inside a thread's 4 rows and inside a CTA's 1024."""
+    from paper_2106_09122_gb300.serve import MultiForward
+    plan, A, rng = _plan(64, 0.125, 3.0, storage, n=n)
+    x = rng.uniform(0.0, 1.0, (5, 64 * 64)).astype(np.float32)
+    big = torch.full((5 * plan.M + 8,), float("nan"), device=DEV)
+    y = big[shift:shift + 5 * plan.M].view(5, plan.M)
+    mf = MultiForward([plan], [5], tuning=(0, units, 0) if units else None, y=[y])
+    mf.x[0].copy_(torch.from_numpy(x))
+    mf.count.fill_(4)
+    mf.enqueue()
+    x64 = x[:4].astype(np.float64)
+    err = O.bound_relative_error(y[:4].double().cpu().numpy(), x64 @ A.T, x64 @ np.abs(A).T, floor=O.FLT_MIN).max()
+    assert err <= tol and plan.sync_status() == 0, err
+    assert torch.isnan(big[:shift]).all() and torch.isnan(big[shift + 4 * plan.M:]).all()

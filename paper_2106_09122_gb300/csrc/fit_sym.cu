@@ -83,7 +83,7 @@ __global__ void __cluster_dims__(1, kCluster, 1) __launch_bounds__(kFwdThreads, 
   {
     const int64_t r = tile0 + 4 * threadIdx.x;
     float acc[4][4] = {};
-    if (r < ld) fwd_accumulate<4, true, kXCols>(A, ld, Kv, xs, 0, r, t0, t1, acc);
+    if (r < ld) fwd_accumulate<4, kXCols>(A, ld, xs, r, t0, t1, acc);
 #pragma unroll
     for (int m = 0; m < 4; ++m) cpart[m][threadIdx.x] = make_float4(acc[m][0], acc[m][1], acc[m][2], acc[m][3]);
   }

@@ -182,3 +182,20 @@ def test_gradient_reads_target_and_writes_result_in_pinned_host_memory():
     Q.enqueue_gradient(theta)
     torch.cuda.synchronize()
     assert out[0].item() == l_dev and np.array_equal(out[1:].numpy(), g_dev)
+
+
+@pytest.mark.parametrize("N,S,w,inc", [(64, 0.25, 1.0, 60.0), (41, 0.3, 0.3, 62.0), (40, 0.3, 0.5, -35.0), (21, 0.7, 2.0, 180.0)])
+def test_ring_scene_rounds_like_its_last_operations(N, S, w, inc):
+    """The distance from the ring is formed without rounding shared by pixels: 1e-6 for the exponential
+    and the phase function, and 3e-7 of the exponent, where R in one float alone gave 4e-6 at w = 0.3."""
+    from paper_2106_09122_gb300 import Plan
+    from paper_2106_09122_gb300.fit import RingProblem
+    plan = Plan(torch.rand(4, 8, 8, device=DEV), np.linspace(0.0, 6.0, 4), 0.3, N=N, S=S)
+    P = RingProblem(plan, N, S, 5.9, torch.zeros(64, device=DEV), 1e-14)
+    theta = np.array([5.1, w, np.deg2rad(inc), 0.3, 1.1e-9])
+    z = P.scene(theta).double().cpu().numpy().ravel()
+    ref = RO.ring_scene(theta, N, S, 5.9).ravel()
+    c = (np.arange(N) - 0.5 * (N - 1)) * S
+    rd = np.hypot(np.tile(c, N), np.repeat(c, N) / np.cos(theta[2]))
+    arg = 4.0 * np.log(2.0) * ((rd - theta[0]) / w) ** 2
+    assert np.all(np.abs(z - ref) <= ref * (1e-6 + 3e-7 * arg) + 1e-37)

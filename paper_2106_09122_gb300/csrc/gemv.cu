@@ -155,11 +155,11 @@ __global__ void __launch_bounds__(kFwdThreads, fwd_min_ctas(BB)) fwd_cols_kernel
 }
 
 // y[b, i] = sum_ks part[ks, b, i] (reduce.cuh).  y may be part itself with M = ld.
+template <bool kSerial>
 __global__ void __launch_bounds__(256) fwd_reduce_kernel(const float *part, int KS, int B, int64_t ld, int64_t M,
                                                          float *y) {
-  __shared__ float4 red[8][32];
   const int b = blockIdx.y;
-  reduce_partials(part + (int64_t)b * ld, (int64_t)B * ld, KS, ld, M, y + (int64_t)b * M, red);
+  reduce_partials<kSerial>(part + (int64_t)b * ld, (int64_t)B * ld, KS, ld, M, y + (int64_t)b * M);
 }
 
 // One residual: gx[j] = sum_i A[i, j] g[i] for the CTA's contiguous range of the
@@ -480,8 +480,12 @@ cudaError_t psfsim_launch_forward_fp32(const psfsim_plan *h, const float *x, int
 
 cudaError_t psfsim_launch_reduce_partials(const float *part, int KS, int B, int64_t ld, int64_t M, float *y,
                                           cudaStream_t st) {
-  dim3 grid((unsigned)reduce_ctas(KS, M), (unsigned)B);
-  fwd_reduce_kernel<<<grid, 256, 0, st>>>(part, KS, B, ld, M, y);
+  const bool serial = reduce_serial(KS, (int64_t)B * M);
+  const dim3 grid((unsigned)reduce_ctas(serial, M), (unsigned)B);
+  if (serial)
+    fwd_reduce_kernel<true><<<grid, 256, 0, st>>>(part, KS, B, ld, M, y);
+  else
+    fwd_reduce_kernel<false><<<grid, 256, 0, st>>>(part, KS, B, ld, M, y);
   return cudaGetLastError();
 }
 

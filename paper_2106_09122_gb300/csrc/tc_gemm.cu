@@ -189,12 +189,13 @@ struct RMulti {
 };
 
 // y[b, i] = sum_ks part[ks, b, i] of job blockIdx.z (reduce.cuh).  One launch serves every job.
+template <bool kSerial>
 __global__ void __launch_bounds__(256) tc_reduce_kernel(const __grid_constant__ RMulti P) {
-  __shared__ float4 red[8][32];
   const RJob &J = P.job[blockIdx.z];
   const int b = blockIdx.y;
   if (b >= J.cap || (J.count && b >= *J.count)) return;
-  reduce_partials(J.part + (int64_t)b * J.rows, (int64_t)J.cap * J.rows, J.KS, J.rows, J.M, J.y + (int64_t)b * J.M, red);
+  reduce_partials<kSerial>(J.part + (int64_t)b * J.rows, (int64_t)J.cap * J.rows, J.KS, J.rows, J.M,
+                           J.y + (int64_t)b * J.M);
 }
 
 // The adjoint's result from its partial sums, part[KS][cap][rows] per block of
@@ -518,7 +519,7 @@ __global__ void __launch_bounds__(kThreads, 2) tc_gemm_kernel(const __grid_const
 // With scenes along the MMA's N, a step reads A's 128-row tiles and every x part
 // from shared memory for each of its two MMAs: about 200 bytes a clock against
 // the 128 it delivers, which held 256 rotated scenes of 256^2 to half the tensor
-// rate (998 us).  From some 100 scenes on the roles are swapped: 128 scenes are
+// rate (998 us).  Beyond 80 scenes (wide_form) the roles are swapped: 128 scenes are
 // the MMA's M, 256 image pixels its N, and all five products
 //     x1 hi + x2 hi + x3 hi + x1 lo + x2 lo      (BF16: x1 hi + x2 hi)
 // accumulate into one accumulator of 256 columns, two of which alternate, so
@@ -891,8 +892,8 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
   std::memset(&P, 0, sizeof(P));
   std::memset(&XP, 0, sizeof(XP));
   std::memset(&RP, 0, sizeof(RP));
-  int64_t x_blocks = 1, red_ctas = 0;
-  int nred = 0, red_cap = 0;
+  int64_t x_blocks = 1, red_M = 0, red_rows = 0;
+  int nred = 0, red_cap = 0, red_KS = 1;
   for (int j = 0; j < nj; ++j) {
     const psfsim_plan *h = jobs[j].h;
     const JobPlan &p = mp.jp[j];
@@ -963,8 +964,9 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
       R.M = h->M;
       R.KS = p.KS;
       R.cap = jobs[j].cap;
-      const int64_t ctas = reduce_ctas(p.KS, h->M);
-      red_ctas = ctas > red_ctas ? ctas : red_ctas;
+      red_M = h->M > red_M ? h->M : red_M;
+      red_KS = p.KS > red_KS ? p.KS : red_KS;
+      red_rows += (int64_t)R.cap * h->M;
       red_cap = R.cap > red_cap ? R.cap : red_cap;
     }
   }
@@ -996,8 +998,14 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
   tc_gemm_kernel<<<mp.units < slots ? mp.units : slots, kThreads, mp.smem, st>>>(P);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (jobs[0].first >= 0 || adjoint) return cudaSuccess;  // the caller adds the rotations (SymSum), or finishes
-  if (nred > 0)
-    tc_reduce_kernel<<<dim3((unsigned)red_ctas, (unsigned)red_cap, (unsigned)nred), 256, 0, st>>>(RP);
+  if (nred > 0) {
+    const bool serial = reduce_serial(red_KS, red_rows);
+    const dim3 grid((unsigned)reduce_ctas(serial, red_M), (unsigned)red_cap, (unsigned)nred);
+    if (serial)
+      tc_reduce_kernel<true><<<grid, 256, 0, st>>>(RP);
+    else
+      tc_reduce_kernel<false><<<grid, 256, 0, st>>>(RP);
+  }
   return cudaGetLastError();
 }
 
@@ -1048,7 +1056,7 @@ WidePlan plan_wide(const psfsim_plan *h, int scenes) {
   // Splits by their cost in clocks: the rounds of units, a unit's k-tiles at 2750
   // and its partial image's 128 KB at 6000, and the partial images read again at
   // HBM rate.  (Filling the last round alone cost a 256^2 image of a 64^2 scene
-  // more in partial images than in products: 148 us for 32 scenes, 83 now.)
+  // more in partial images than in products: 148 us for 32 scenes, 75 now.)
   w.KS = 1;
   double best = 1e300;
   for (int ks = 1; ks <= 16 && ks <= w.k_tiles; ++ks) {

@@ -210,3 +210,23 @@ def test_sum_over_splits(storage, tol, units, n, shift):
     err = O.bound_relative_error(y[:4].double().cpu().numpy(), x64 @ A.T, x64 @ np.abs(A).T, floor=O.FLT_MIN).max()
     assert err <= tol and plan.sync_status() == 0, err
     assert torch.isnan(big[:shift]).all() and torch.isnan(big[shift + 4 * plan.M:]).all()
+
+
+@pytest.mark.parametrize("n", [251, 252])
+def test_sum_over_splits_of_many_rows(n):
+    """More than four splits summed by one thread (many rows): against one and two splits, each
+    within 1e-5 of sums of products that are not negative."""
+    from paper_2106_09122_gb300 import Plan
+    from paper_2106_09122_gb300.serve import MultiForward
+    rng = np.random.default_rng(3)
+    plan = Plan(torch.rand(4, n, n, device=DEV), np.linspace(0.0, 3.0, 4), 0.25, N=64, S=0.125, storage="split_bf16")
+    x = torch.from_numpy(rng.uniform(0.0, 1.0, (5, 64 * 64)).astype(np.float32))
+    out = []
+    for units in (1, 40):
+        mf = MultiForward([plan], [5], tuning=(0, units, 0))
+        mf.x[0].copy_(x)
+        mf.count.fill_(5)
+        mf.enqueue()
+        out.append(mf.y[0].double().cpu())
+    assert plan.sync_status() == 0
+    assert torch.all((out[0] - out[1]).abs() <= 2e-5 * out[0])

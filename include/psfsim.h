@@ -56,8 +56,7 @@ enum psfsim_status {
  * bf16 hi + lo with a power-of-two float32 scale per column, for the
  * tensor-core path.  BF16: the hi part alone (row-major bf16 with the same
  * per-column scale): half the bytes, each element rounded to 8 significant
- * bits, so results carry up to 2^-8 of the error bound (tensor-core forward,
- * CUDA-core adjoint).  FP32_SYM: FP32 columns of the x > 0, y > 0 quadrant only,
+ * bits, so results carry up to 2^-8 of the error bound.  FP32_SYM: FP32 columns of the x > 0, y > 0 quadrant only,
  * inside the last radius: the other three quadrants' columns are exact
  * quarter turns of these and the rest are zero (even N, grid builds only;
  * same results as FP32 up to the order of the sums).  SPLIT_BF16_SYM: the
@@ -99,6 +98,9 @@ const char *psfsim_status_string(int status);
 
 /* Bytes of workspace psfsim_build needs for an n x n library of n_r PSFs
  * applied to K columns (K = N*N for a scene grid) with the given storage.
+ * SPLIT_BF16 and BF16 grids of even N that build faster from pair entries of
+ * the library (32 bytes per bracket and pixel) get room for them; a workspace
+ * without that room is accepted too, and its A is the same.
  * Sec. 3: A has n^2 rows and N^2 columns.  Returns PSFSIM_ERR_ARG for bad sizes. */
 int psfsim_workspace_bytes(int n, int n_r, int64_t K, int storage, size_t *bytes);
 
@@ -150,8 +152,8 @@ int psfsim_forward(psfsim_t h, const float *d_x, int B, float *d_y, void *d_scra
  * masked disks and everything beyond the outer working angle leave those
  * columns unread.  FP32 storage only (else PSFSIM_ERR_UNSUPPORTED).  Same
  * arguments and result as psfsim_forward, up to the order of the float32 sums;
- * deterministic.  The list of columns is built on the device, so the call
- * never synchronises. */
+ * deterministic.  The scene is looked at on the device, by the product itself,
+ * so the call never synchronises. */
 int psfsim_forward_sparse_scratch_bytes(psfsim_t h, int B, size_t *bytes);
 int psfsim_forward_sparse(psfsim_t h, const float *d_x, int B, float *d_y, void *d_scratch,
                           size_t scratch_bytes, void *stream);
@@ -183,7 +185,7 @@ typedef struct {
 /* Batched S_j = A_j Z_j (Eq. 6) for several SPLIT_BF16 plans at once — e.g.
  * scenes of different sizes and pixel scales, each with its own A — in one
  * persistent tensor-core launch whose work units interleave all jobs (plus one
- * split and one reduction launch per job).  1 <= njobs <= 16, all plans on
+ * split and one reduction launch for all of them).  1 <= njobs <= 16, all plans on
  * the current device.  `tuning` may be NULL.  Deterministic. */
 int psfsim_forward_multi_scratch_bytes(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tuning,
                                        size_t *bytes);

@@ -9,7 +9,8 @@
 //                          {L, dL/dtheta}.
 //
 // Both stream the columns inside the last radius only (128^2 fit workload, 44 %
-// of the columns: 359 -> 205 us a loss_and_grad call, host and copy included).
+// of the columns: 359 -> 205 us a loss_and_grad call, host and copy included; 190
+// since the calls cost less on the host).
 // Both kernels are launched with programmatic stream serialization: the
 // forward computes its scene values and streams A before it waits for the
 // kernel ahead of it (griddepcontrol.wait), so back-to-back gradients overlap

@@ -5,9 +5,10 @@
 //                   dead[dead_groups]: the 32-column groups in no k-tile.
 // What that is worth depends on the grid: the wave of 50 scenes on ten split
 // plans (64..256 pixels a side, 12 lambda/D of PSFs in fields of 19 to 128)
-// streams 26 % of its k-tiles, 2680 -> 852 us; tiles start at multiples of 32
-// columns rather than 64 so that a narrow row needs one tile where it used to
-// touch two, and 32 columns are the 64 bytes that HBM moves at least.
+// streams 26 % of its k-tiles, 2680 -> 852 us (651 with tc_gemm.cu's other steps);
+// tiles start at multiples of 32 columns rather than 64 so that a narrow row needs
+// one tile where it used to touch two, and 32 columns are the 64 bytes that HBM
+// moves at least.
 //   FP32 storage    the live columns, ascending, then the others, ascending.
 // The host counts the same tables by the same integer arithmetic, to size
 // launches without reading anything back.

@@ -42,7 +42,7 @@ __device__ __forceinline__ float pow2_at_least(float m) {
 }
 
 struct SplitParams {
-  int n, pad;
+  int n;
   int64_t K, ld, M, rows;
   const ColGeom *geom;
   const int *order;  // compacted storage: column j is geometry entry order[j] (else null: entry j)
@@ -675,7 +675,6 @@ cudaError_t psfsim_launch_split_build(psfsim_plan *h, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   SplitParams P;
   P.n = h->n;
-  P.pad = 0;
   P.K = psfsim_cols(h);
   P.order = h->quadrant ? reinterpret_cast<const int *>(h->ws + h->order_off) : nullptr;
   P.ld = h->ld;

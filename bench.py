@@ -41,18 +41,14 @@ CSRC = os.path.join(ROOT, "paper_2106_09122_gb300", "csrc")
 # (sha256 prefix of the .cu file): a changed kernel reports traffic null until
 # it is captured again.
 NCU_TRAFFIC = {
-    "fused_kernel": {"file": "fused.cu", "sha": "cce2519e41c5fb90", "bytes": 1.043801e9 + 0.244421e9},
-    "fwd_ring_loss_kernel": {"file": "fit_gradient.cu", "sha": "b12c1c3a52352d28", "bytes": 1.073864e9 + 0.003710e9},
-    "adj_chain_kernel": {"file": "fit_gradient.cu", "sha": "b12c1c3a52352d28", "bytes": 1.074243e9 + 0.003091e9},
-    "tc_gemm_kernel_per_A_byte": {"file": "tc_gemm.cu", "sha": "643a1c8518b1b882",
-                                  "bytes": (1086370560 + 28214528) / (4 * 16384 * 16384)},
+    "fused_kernel": {"file": "fused.cu", "sha": "3177a1a66eb342cd", "bytes": 1.001071e9 + 0.242350e9},
+    "fwd_ring_loss_kernel": {"file": "fit_gradient.cu", "sha": "dd7e9d436729d8ef", "bytes": 0.474149e9 + 0.003329e9},
+    "adj_chain_kernel": {"file": "fit_gradient.cu", "sha": "dd7e9d436729d8ef", "bytes": 0.474374e9 + 0.000058e9},
 }
 
 
 def _traffic(name: str):
     t = NCU_TRAFFIC[name]
-    if t["sha"] is None:
-        return None
     with open(os.path.join(CSRC, t["file"]), "rb") as f:
         return t["bytes"] if hashlib.sha256(f.read()).hexdigest()[:16] == t["sha"] else None
 
@@ -176,6 +172,13 @@ def _timed_build(make, stream):
     e1.record(stream)
     torch.cuda.synchronize()
     return plan, e0.elapsed_time(e1)
+
+
+def _live(N, S, radii):
+    """Scene pixels inside the last library radius: the columns of A that are not zero, which is
+    what a product with a stored grid plan reads."""
+    c = (np.arange(N) - 0.5 * (N - 1)) * S
+    return int(np.count_nonzero(np.hypot(c[:, None], c[None, :]) <= radii[-1] * (1.0 + 1e-9)))
 
 
 def _build_roofline(a_bytes, ms, hbm):
@@ -571,7 +574,7 @@ def _entry_fit128(dev, stream, with_oracle, steps=1000):
     A = plan.A_fp32()
     cmp_ms = _timed(lambda: (torch.mv(A, x), torch.mv(A.t(), g)), 200, stream)
     hbm = _peaks()["hbm"]
-    a_bytes = w.M * w.K * 4
+    a_bytes = w.M * _live(w.N, w.S, w.radii) * 4
     fwd_bytes = a_bytes + 3 * w.M * 4 + 6 * w.K * 4
     adj_bytes = a_bytes + w.M * 4 + 6 * w.K * 4
     f0 = time.perf_counter()
@@ -585,7 +588,8 @@ def _entry_fit128(dev, stream, with_oracle, steps=1000):
            "build_ms": build_ms, "build_roofline": _build_roofline(4 * w.M * w.K, build_ms, _peaks()["hbm"]),
            "roofline": {"bound": "hbm", "achieved": adj_bytes / (adj_ms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
                         "frac": adj_bytes / (adj_ms / 1e3) / 1e9 / hbm, "traffic": _traffic("adj_chain_kernel"),
-                        "kernel": "adj_chain_kernel (event pair around psfsim_ring_adjoint_chain, timed alone)"},
+                        "kernel": "adj_chain_kernel (event pair around psfsim_ring_adjoint_chain, timed alone)",
+                        "bytes_note": "the columns inside the last radius"},
            "roofline_frac": {"forward": fwd_bytes / (fwd_ms / 1e3) / 1e9 / hbm,
                              "adjoint": adj_bytes / (adj_ms / 1e3) / 1e9 / hbm},
            "e2e": {"images_per_s": 1e3 / e2e_ms, "h2d_bytes_per_step": w.M * 4, "d2h_bytes_per_step": 48,
@@ -638,8 +642,8 @@ def _path_batched(dev, stream, hbm, with_oracle):
         mf.x[l].copy_(torch.from_numpy(xs))
     mf.count.fill_(B)
     ms = _timed(mf.enqueue, 10, stream)
-    a_bytes = nl * (4 * w.M * w.K + B * w.K * 4 + B * w.M * 4)
-    tr = _traffic("tc_gemm_kernel_per_A_byte")
+    live = _live(w.N, w.S, w.radii)
+    a_bytes = nl * (4 * w.M * live + B * w.K * 4 + B * w.M * 4)
     out = {"workload": "batched_split_bf16_256: 8 wavelengths x 64 scenes, 60 PSFs 256^2 per wavelength, "
                        "8 x A 65536^2 split-BF16 (137 GB) in one launch",
            "images_per_s": nl * B / (ms / 1e3), "ms_per_batch": ms, "build_ms_per_wavelength": build_ms,
@@ -647,7 +651,8 @@ def _path_batched(dev, stream, hbm, with_oracle):
            "gmac_per_s": nl * B * w.M * w.K / (ms / 1e3) / 1e9,
            "roofline": {"bound": "hbm", "achieved": a_bytes / (ms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
                         "frac": a_bytes / (ms / 1e3) / 1e9 / hbm, "kernel": "tc_gemm_kernel, 8 jobs (+ split, reduce)",
-                        "traffic": None if tr is None else tr * nl * 4 * w.M * w.K},
+                        "traffic": None,
+                        "bytes_note": f"the {live} of {w.K} columns inside the last radius"},
            "status": plans[0].sync_status()}
     Y0 = mf.y[0][:4].clone()
     per = []
@@ -730,7 +735,7 @@ def _path_uneven(dev, stream, hbm, with_oracle):
     for imgs, _ in server.run_waves(wave_items):
         outs += imgs
     total = time.perf_counter() - t0
-    a_bytes = sum(p.M * p.info.ld * 4 for p in plans.values())
+    a_bytes = sum(p.M * _live(N, S, w.radii) * 4 for (N, S), p in plans.items())
     wave_s = total / len(waves)
     out = {"workload": "uneven_500: 500 scenes, N in {64,96,128,192,256} x S in {0.3,0.5} lambda/D, per-bucket "
                        "split-BF16 A (17.3 GB), seeded arrival order, waves of 50; the kernels read the scenes from "
@@ -748,7 +753,7 @@ def _path_uneven(dev, stream, hbm, with_oracle):
            "roofline": {"bound": "hbm", "achieved": a_bytes / wave_s / 1e9, "peak": hbm, "unit": "GB/s",
                         "frac": a_bytes / wave_s / 1e9 / hbm,
                         "kernel": "served waves: packing, copies and the multi-job launch, back to back; A bytes "
-                                  "of all buckets per wave over the wave time"}}
+                                  "(columns inside the last radius) of all buckets per wave over the wave time"}}
     fp = {k: Plan(lib, w.radii, w.s, N=k[0], S=k[1]) for k in buckets}
     xs_dev = [torch.from_numpy(sc).to(dev) for sc in scenes]
     torch.cuda.synchronize()
@@ -866,7 +871,8 @@ def _path_bf16(dev, stream, hbm, with_oracle):
         mf.x[l].copy_(torch.from_numpy(xs))
     mf.count.fill_(B)
     ms = _timed(mf.enqueue, 10, stream)
-    a_bytes = nl * (2 * w.M * w.K + B * w.K * 4 + B * w.M * 4)
+    live = _live(w.N, w.S, w.radii)
+    a_bytes = nl * (2 * w.M * live + B * w.K * 4 + B * w.M * 4)
     out = {"workload": "batched_bf16_256: the batched 256^2 workload (8 wavelengths x 64 scenes) with BF16 "
                        "storage, 8 x A 65536^2 (69 GB) in one launch",
            "images_per_s": nl * B / (ms / 1e3), "ms_per_batch": ms, "build_ms_per_wavelength": build_ms,
@@ -875,6 +881,7 @@ def _path_bf16(dev, stream, hbm, with_oracle):
            "roofline": {"bound": "hbm", "achieved": a_bytes / (ms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
                         "frac": a_bytes / (ms / 1e3) / 1e9 / hbm,
                         "kernel": "tc_gemm_kernel, 8 jobs, one MMA (N = 2 x 64) per k-step (+ split, reduce)",
+                        "bytes_note": f"the {live} of {w.K} columns inside the last radius",
                         "intensity_note": "2 x 128 flop per 2-byte element = 128 flop/byte < bf16 ridge ~278"},
            "tolerance": 2.0 ** -8 + 2.5e-5,
            "status": plans[0].sync_status()}
@@ -1055,7 +1062,7 @@ def _path_ipac(dev, stream, hbm, with_oracle):
         y = torch.empty(w.M, device=dev)
         scr = torch.empty(plan.forward_scratch_bytes(1), dtype=torch.uint8, device=dev)
         ms = _timed(lambda: plan.forward(x, out=y, scratch=scr), 50, stream)
-        a_bytes = 4 * w.M * w.K + 4 * w.K + 4 * w.M
+        a_bytes = 4 * w.M * _live(w.N, w.S, w.radii) + 4 * w.K + 4 * w.M
         out[interp] = {"build_ms": build_ms, "build_roofline": _build_roofline(4 * w.M * w.K, build_ms, hbm),
                        "simulate_ms": ms,
                        "speedup_vs_paper_simulate": 164.2 / ms,

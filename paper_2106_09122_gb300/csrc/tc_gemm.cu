@@ -64,9 +64,8 @@ constexpr int kSingleChunk = 1, kSingleChunkWide = 3;
 constexpr int kDefaultChunkHiMulti = 2;  // BF16 storage (hi alone), several jobs in one launch
 // Adjoint of split storage: residuals change sign, so its sums cancel and the
 // drift weighs more (error against 64 bits 2.493e-6 with plain FP32 sums, 2.553
-// at 4 k-tiles, 2.492 at one; 8 residuals of 128^2 took 127 and 129 us (119 since
-// choose_ks), 64 of
-// 256^2 1.45 and 1.64 ms).
+// at 4 k-tiles, 2.492 at one; 8 residuals of 128^2 took 127 and 129 us, 119 since
+// choose_ks; 64 of 256^2 1.45 and 1.64 ms).
 constexpr int kAdjointChunk = 1;
 constexpr int kAdjointRun = 160;  // and the most k-tiles a unit adds up
 constexpr int kMaxMmas = 64;     // accumulating MMAs between drains (bounds the FP32 drift)

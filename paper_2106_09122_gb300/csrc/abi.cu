@@ -26,25 +26,9 @@ bool storage_ok(int storage) {
          storage == PSFSIM_FP32_SYM || storage == PSFSIM_FUSED || storage == PSFSIM_SPLIT_BF16_SYM;
 }
 
-int common_build(const float *d_lib, const double *h_radii, int n_r, int n, double s, int N, double S,
-                 const double *h_xy, int64_t K, int storage, int interp, void *d_ws, size_t ws_bytes,
-                 void *stream, psfsim_t *out) {
-  if (!out) return PSFSIM_ERR_ARG;
-  *out = nullptr;
-  if (!d_lib || !d_ws || n < 1 || n > 4096 || K < 1 || K > (int64_t)1 << 30) return PSFSIM_ERR_ARG;
-  if (!(s > 0.0) || !std::isfinite(s)) return PSFSIM_ERR_ARG;
-  if (!storage_ok(storage) || (interp != PSFSIM_LINEAR && interp != PSFSIM_NEAREST)) return PSFSIM_ERR_ARG;
-  if (!aligned(d_lib, 16)) return PSFSIM_ERR_ARG;
-  if (int rc = check_radii(h_radii, n_r)) return rc;
-  // FUSED and FP32_SYM use the exact quarter-turn symmetry of an even N x N scene grid.
-  const bool quadrant =
-      storage == PSFSIM_FUSED || storage == PSFSIM_FP32_SYM || storage == PSFSIM_SPLIT_BF16_SYM;
-  if (quadrant && (h_xy || N < 2 || (N & 1))) return PSFSIM_ERR_UNSUPPORTED;
-  const WsLayout L = psfsim_layout(n, K, storage, n_r);
-  if (!aligned(d_ws, 256) || ws_bytes < (size_t)L.total) return PSFSIM_ERR_WORKSPACE;
-
-  psfsim_plan *h = new (std::nothrow) psfsim_plan;
-  if (!h) return PSFSIM_ERR_ARG;
+// The host side of a plan's fields, which every product's launch shapes follow from.
+void fill_shape(psfsim_plan *h, const WsLayout &L, const double *h_radii, int n_r, int n, int N, double S, int64_t K,
+                int storage, int interp) {
   std::memset(h, 0, sizeof(*h));
   h->storage = storage;
   h->interp = interp;
@@ -55,12 +39,10 @@ int common_build(const float *d_lib, const double *h_radii, int n_r, int n, doub
   h->ld = L.ld;
   h->N = N;
   h->S = S;
-  h->quadrant = quadrant;
+  // FUSED and the compact storages use the exact quarter-turn symmetry of an even N x N scene grid.
+  h->quadrant = storage == PSFSIM_FUSED || storage == PSFSIM_FP32_SYM || storage == PSFSIM_SPLIT_BF16_SYM;
   h->Kg = h->quadrant ? K / 4 : K;
-  h->d_lib = d_lib;
   for (int i = 0; i < n_r; ++i) h->radii[i] = h_radii[i];
-  h->ws = static_cast<char *>(d_ws);
-  h->ws_bytes = ws_bytes;
   h->a_off = L.a_off;
   h->lo_off = L.lo_off;
   h->scale_off = L.scale_off;
@@ -73,6 +55,29 @@ int common_build(const float *d_lib, const double *h_radii, int n_r, int n, doub
   h->plib_off = L.plib_off;
   h->cols_off = L.cols_off;
   h->mtorder_off = L.mtorder_off;
+}
+
+int common_build(const float *d_lib, const double *h_radii, int n_r, int n, double s, int N, double S,
+                 const double *h_xy, int64_t K, int storage, int interp, void *d_ws, size_t ws_bytes,
+                 void *stream, psfsim_t *out) {
+  if (!out) return PSFSIM_ERR_ARG;
+  *out = nullptr;
+  if (!d_lib || !d_ws || n < 1 || n > 4096 || K < 1 || K > (int64_t)1 << 30) return PSFSIM_ERR_ARG;
+  if (!(s > 0.0) || !std::isfinite(s)) return PSFSIM_ERR_ARG;
+  if (!storage_ok(storage) || (interp != PSFSIM_LINEAR && interp != PSFSIM_NEAREST)) return PSFSIM_ERR_ARG;
+  if (!aligned(d_lib, 16)) return PSFSIM_ERR_ARG;
+  if (int rc = check_radii(h_radii, n_r)) return rc;
+  const bool quadrant = storage == PSFSIM_FUSED || storage == PSFSIM_FP32_SYM || storage == PSFSIM_SPLIT_BF16_SYM;
+  if (quadrant && (h_xy || N < 2 || (N & 1))) return PSFSIM_ERR_UNSUPPORTED;
+  const WsLayout L = psfsim_layout(n, K, storage, n_r);
+  if (!aligned(d_ws, 256) || ws_bytes < (size_t)L.total) return PSFSIM_ERR_WORKSPACE;
+
+  psfsim_plan *h = new (std::nothrow) psfsim_plan;
+  if (!h) return PSFSIM_ERR_ARG;
+  fill_shape(h, L, h_radii, n_r, n, N, S, K, storage, interp);
+  h->d_lib = d_lib;
+  h->ws = static_cast<char *>(d_ws);
+  h->ws_bytes = ws_bytes;
   // A workspace of the plain layout's size (or a field-point build) does without the pixel-wise build's tables.
   h->pix_off = N > 0 && ws_bytes >= (size_t)L.total_pix ? L.pix_off : -1;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -223,7 +228,8 @@ int psfsim_forward(psfsim_t h, const float *d_x, int B, float *d_y, void *d_scra
   if (h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16) {
     const size_t need = psfsim_forward_tc_scratch(h, B);
     if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
-    return psfsim_launch_forward_tc(h, d_x, B, d_y, d_scratch, st) == cudaSuccess ? PSFSIM_OK : PSFSIM_ERR_CUDA;
+    return psfsim_launch_forward_tc(h, d_x, B, d_y, d_scratch, scratch_bytes, st) == cudaSuccess ? PSFSIM_OK
+                                                                                                 : PSFSIM_ERR_CUDA;
   }
   if (h->storage == PSFSIM_FP32_SYM) {
     const size_t need = psfsim_forward_sym_scratch(h, B);
@@ -233,8 +239,9 @@ int psfsim_forward(psfsim_t h, const float *d_x, int B, float *d_y, void *d_scra
   if (h->storage == PSFSIM_SPLIT_BF16_SYM) {
     const size_t need = psfsim_forward_split_sym_scratch(h, B);
     if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
-    return psfsim_launch_forward_split_sym(h, d_x, B, d_y, d_scratch, st) == cudaSuccess ? PSFSIM_OK
-                                                                                         : PSFSIM_ERR_CUDA;
+    return psfsim_launch_forward_split_sym(h, d_x, B, d_y, d_scratch, scratch_bytes, st) == cudaSuccess
+               ? PSFSIM_OK
+               : PSFSIM_ERR_CUDA;
   }
   if (h->storage == PSFSIM_FUSED) {
     const size_t need = psfsim_forward_fused_scratch(h, B);
@@ -343,6 +350,32 @@ int psfsim_debug_forward_stall(psfsim_t h, const float *d_x, int B, float *d_y, 
                                         static_cast<cudaStream_t>(stream)) == cudaSuccess
              ? PSFSIM_OK
              : PSFSIM_ERR_CUDA;
+}
+
+int psfsim_debug_scratch(const double *h_radii, int n_r, int n, int N, double S, int storage, int num_sms, int B,
+                         size_t *reported, size_t *taken) {
+  if (!reported || !taken || n < 1 || n > 4096 || N < 1 || N > 32768 || !(S > 0.0) || num_sms < 1 || B < 1)
+    return PSFSIM_ERR_ARG;
+  if (int rc = check_radii(h_radii, n_r)) return rc;
+  const int64_t K = (int64_t)N * N;
+  psfsim_plan p;
+  if (storage != PSFSIM_SPLIT_BF16 && storage != PSFSIM_BF16 && storage != PSFSIM_SPLIT_BF16_SYM)
+    return PSFSIM_ERR_UNSUPPORTED;
+  fill_shape(&p, psfsim_layout(n, K, storage, n_r), h_radii, n_r, n, N, S, K, storage, PSFSIM_LINEAR);
+  p.num_sms = num_sms;
+  if (p.quadrant) {
+    if (N & 1) return PSFSIM_ERR_UNSUPPORTED;
+    for (int iy = N / 2; iy < N; ++iy)
+      for (int ix = N / 2; ix < N; ++ix) {
+        const double x = (ix - 0.5 * (N - 1)) * S, y = (iy - 0.5 * (N - 1)) * S;
+        p.K_valid += std::sqrt(x * x + y * y) <= h_radii[n_r - 1];
+      }
+    p.ld = psfsim_round_up(p.K_valid > 0 ? p.K_valid : 1, 64);
+  }
+  psfsim_live_count(&p);
+  if (int rc = psfsim_forward_scratch_bytes(&p, B, reported)) return rc;
+  *taken = psfsim_forward_tc_taken(&p, p.quadrant ? 4 * B : B);
+  return PSFSIM_OK;
 }
 
 void psfsim_free(psfsim_t h) { delete h; }

@@ -89,11 +89,12 @@ cudaError_t psfsim_launch_reduce_partials(const float *part, int KS, int B, int6
                                           cudaStream_t st);
 // Split-BF16 storage: build, tensor-core forward, CUDA-core adjoint.
 cudaError_t psfsim_launch_split_build(psfsim_plan *h, cudaStream_t st);
-size_t psfsim_forward_tc_scratch(const psfsim_plan *h, int B);
+size_t psfsim_forward_tc_scratch(const psfsim_plan *h, int B);  // compact storage: of B rotated scenes
+size_t psfsim_forward_tc_taken(const psfsim_plan *h, int B);    // what the launches themselves take
 cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
-                                     cudaStream_t st);
+                                     size_t scratch_bytes, cudaStream_t st);
 cudaError_t psfsim_launch_forward_tc_sym(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
-                                         cudaStream_t st);
+                                         size_t scratch_bytes, cudaStream_t st);
 // Images from the partial images of rotated scenes (sym.cu): rotated scene
 // q = 4 b + m is slot q % per of block q / per, whose partials are
 // part[KS][cap][rows]; y[b][i] = sum_m sum_ks part at P^-m(i).
@@ -173,7 +174,7 @@ static inline int64_t psfsim_cols(const psfsim_plan *h) { return h->quadrant ? h
 // Split-BF16 storage compacted by the quarter-turn symmetry (sym.cu).
 size_t psfsim_forward_split_sym_scratch(const psfsim_plan *h, int B);
 cudaError_t psfsim_launch_forward_split_sym(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
-                                            cudaStream_t st);
+                                            size_t scratch_bytes, cudaStream_t st);
 
 // Launch configuration with programmatic stream serialization: the kernel may
 // be scheduled while the previous kernel in the stream finishes; it calls

@@ -1013,14 +1013,14 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
 
 namespace {
 
-// A batch of B scenes against one plan as jobs of at most kMaxBp scenes (at
-// most kMaxJobs of them), run by one interleaved persistent launch.
-int tc_jobs(const psfsim_plan *h, const float *x, int B, float *y, JobSpec *js) {
-  const int64_t cols = psfsim_cols(h);
+// A batch of B scenes (compact storage: rotated scenes) against one plan as jobs
+// of at most kMaxBp scenes (at most kMaxJobs of them), run by one interleaved
+// persistent launch.  The launch fills in x and y.
+int tc_jobs(const psfsim_plan *h, int B, JobSpec *js) {
   int nj = 0;
   for (int b0 = 0; b0 < B && nj < kMaxJobs; b0 += kMaxBp, ++nj) {
     const int c = (B - b0) < kMaxBp ? (B - b0) : kMaxBp;
-    js[nj] = JobSpec{h, x ? x + (int64_t)b0 * cols : nullptr, y ? y + (int64_t)b0 * h->M : nullptr, c, nullptr, -1};
+    js[nj] = JobSpec{h, nullptr, nullptr, c, nullptr, h->quadrant ? b0 : -1};
   }
   return nj;
 }
@@ -1125,34 +1125,77 @@ cudaError_t launch_wide(const psfsim_plan *h, const float *x, int scenes, const 
 
 }  // namespace
 
+namespace {
+
+// One launch of a product of `count` scenes (compact storage: rotated scenes).
+// What sizes the scratch and what runs are this same plan.
+struct Launch {
+  bool wide;
+  int nj;
+  JobSpec js[kMaxJobs];
+  MultiPlan multi;
+  WidePlan w;
+  size_t scratch;
+};
+
+Launch plan_launch(const psfsim_plan *h, int count) {
+  Launch L;
+  L.wide = wide_form(h, count);
+  L.nj = 0;
+  if (L.wide) {
+    L.w = plan_wide(h, count);
+    L.scratch = L.w.scratch;
+  } else {
+    L.nj = tc_jobs(h, count, L.js);
+    L.multi = plan_multi(L.js, L.nj, nullptr);
+    L.scratch = L.multi.scratch;
+  }
+  return L;
+}
+
 // A batch beyond kMaxLaunchScenes runs as several launches, the last of which
-// may be smaller and of the other form.
+// may be smaller and of the other form: the scenes of launch i.
+int launch_count(int B, int i) {
+  const int64_t left = B - (int64_t)i * kMaxLaunchScenes;
+  return left < 0 ? 0 : (int)(left < kMaxLaunchScenes ? left : kMaxLaunchScenes);
+}
+
+}  // namespace
+
 size_t psfsim_forward_tc_scratch(const psfsim_plan *h, int B) {
+  const size_t first = plan_launch(h, launch_count(B, 0)).scratch;
+  if (B <= kMaxLaunchScenes) return first;
+  const size_t last = plan_launch(h, launch_count(B, (B - 1) / kMaxLaunchScenes)).scratch;  // those between are as the first
+  return last > first ? last : first;
+}
+
+size_t psfsim_forward_tc_taken(const psfsim_plan *h, int B) {
   size_t most = 0;
-  for (int c : {B < kMaxLaunchScenes ? B : kMaxLaunchScenes, B > kMaxLaunchScenes ? B % kMaxLaunchScenes : 0}) {
-    if (c == 0) continue;
-    JobSpec js[kMaxJobs];
-    const size_t need =
-        wide_form(h, c) ? plan_wide(h, c).scratch : plan_multi(js, tc_jobs(h, nullptr, c, nullptr, js), nullptr).scratch;
+  for (int i = 0, c; (c = launch_count(B, i)) > 0; ++i) {
+    const size_t need = plan_launch(h, c).scratch;
     most = need > most ? need : most;
   }
   return most;
 }
 
 cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
-                                     cudaStream_t st) {
-  for (int b0 = 0; b0 < B; b0 += kMaxLaunchScenes) {
-    const int Bc = (B - b0) < kMaxLaunchScenes ? (B - b0) : kMaxLaunchScenes;
+                                     size_t scratch_bytes, cudaStream_t st) {
+  for (int i = 0, c; (c = launch_count(B, i)) > 0; ++i) {
+    Launch L = plan_launch(h, c);
+    if (L.scratch > scratch_bytes) return cudaErrorInvalidValue;
+    const float *xb = x + (int64_t)i * kMaxLaunchScenes * h->K;
+    float *yb = y + (int64_t)i * kMaxLaunchScenes * h->M;
     cudaError_t e;
-    if (wide_form(h, Bc)) {
-      const WidePlan w = plan_wide(h, Bc);
-      if ((e = launch_wide(h, x + (int64_t)b0 * h->K, Bc, w, scratch, st)) != cudaSuccess) return e;
-      e = psfsim_launch_reduce_partials(reinterpret_cast<const float *>(static_cast<char *>(scratch) + w.part_off), w.KS,
-                                        Bc, w.rows, h->M, y + (int64_t)b0 * h->M, st);
+    if (L.wide) {
+      if ((e = launch_wide(h, xb, c, L.w, scratch, st)) != cudaSuccess) return e;
+      e = psfsim_launch_reduce_partials(reinterpret_cast<const float *>(static_cast<char *>(scratch) + L.w.part_off),
+                                        L.w.KS, c, L.w.rows, h->M, yb, st);
     } else {
-      JobSpec js[kMaxJobs];
-      const int nj = tc_jobs(h, x + (int64_t)b0 * psfsim_cols(h), Bc, y + (int64_t)b0 * h->M, js);
-      e = launch_multi(js, nj, plan_multi(js, nj, nullptr), scratch, st);
+      for (int j = 0; j < L.nj; ++j) {
+        L.js[j].x = xb + (int64_t)j * kMaxBp * h->K;
+        L.js[j].y = yb + (int64_t)j * kMaxBp * h->M;
+      }
+      e = launch_multi(L.js, L.nj, L.multi, scratch, st);
     }
     if (e != cudaSuccess) return e;
   }
@@ -1164,45 +1207,36 @@ cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B
 // partial images of all rotations are added through the inverse turns at the
 // end.
 cudaError_t psfsim_launch_forward_tc_sym(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
-                                         cudaStream_t st) {
+                                         size_t scratch_bytes, cudaStream_t st) {
   constexpr int kScenes = kMaxLaunchScenes / 4;
   static_assert(kMaxBp % 4 == 0, "a scene's rotations share a job");
-  for (int b0 = 0; b0 < B; b0 += kScenes) {
-    const int Bc = (B - b0) < kScenes ? (B - b0) : kScenes;
-    if (wide_form(h, 4 * Bc)) {
-      const WidePlan w = plan_wide(h, 4 * Bc);
-      cudaError_t e = launch_wide(h, x + (int64_t)b0 * h->K, 4 * Bc, w, scratch, st);
-      if (e != cudaSuccess) return e;
-      SymSum S;
-      std::memset(&S, 0, sizeof(S));
-      S.part[0] = reinterpret_cast<const float *>(static_cast<char *>(scratch) + w.part_off);
-      S.cap[0] = S.per = 4 * Bc;
-      S.KS[0] = w.KS;
-      S.rows = w.rows;
-      S.n = h->n;
-      if ((e = psfsim_launch_sym_sum(S, Bc, y + (int64_t)b0 * h->M, st)) != cudaSuccess) return e;
-      continue;
-    }
-    JobSpec js[kMaxJobs];
-    const int nj = tc_jobs(h, nullptr, 4 * Bc, nullptr, js);
-    for (int j = 0; j < nj; ++j) {
-      js[j].x = x + (int64_t)b0 * h->K;
-      js[j].first = j * kMaxBp;
-    }
-    const MultiPlan mp = plan_multi(js, nj, nullptr);
-    cudaError_t e = launch_multi(js, nj, mp, scratch, st);
-    if (e != cudaSuccess) return e;
+  for (int i = 0, c; (c = launch_count(4 * B, i)) > 0; ++i) {
+    Launch L = plan_launch(h, c);
+    if (L.scratch > scratch_bytes) return cudaErrorInvalidValue;
+    const float *xb = x + (int64_t)i * kScenes * h->K;
     SymSum S;
     std::memset(&S, 0, sizeof(S));
-    S.per = kMaxBp;
-    S.rows = mp.jp[0].rows;
     S.n = h->n;
-    for (int j = 0; j < nj; ++j) {
-      S.part[j] = reinterpret_cast<const float *>(static_cast<char *>(scratch) + mp.jp[j].part_off);
-      S.cap[j] = js[j].cap;
-      S.KS[j] = mp.jp[j].KS;
+    cudaError_t e;
+    if (L.wide) {
+      e = launch_wide(h, xb, c, L.w, scratch, st);
+      S.part[0] = reinterpret_cast<const float *>(static_cast<char *>(scratch) + L.w.part_off);
+      S.cap[0] = S.per = c;
+      S.KS[0] = L.w.KS;
+      S.rows = L.w.rows;
+    } else {
+      for (int j = 0; j < L.nj; ++j) L.js[j].x = xb;
+      e = launch_multi(L.js, L.nj, L.multi, scratch, st);
+      S.per = kMaxBp;
+      S.rows = L.multi.jp[0].rows;
+      for (int j = 0; j < L.nj; ++j) {
+        S.part[j] = reinterpret_cast<const float *>(static_cast<char *>(scratch) + L.multi.jp[j].part_off);
+        S.cap[j] = L.js[j].cap;
+        S.KS[j] = L.multi.jp[j].KS;
+      }
     }
-    if ((e = psfsim_launch_sym_sum(S, Bc, y + (int64_t)b0 * h->M, st)) != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;
+    if ((e = psfsim_launch_sym_sum(S, c / 4, y + (int64_t)i * kScenes * h->M, st)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
@@ -1210,7 +1244,7 @@ cudaError_t psfsim_launch_forward_tc_sym(const psfsim_plan *h, const float *x, i
 // Compact storage: the four turns of the residuals are the batch.
 size_t psfsim_adjoint_tc_scratch(const psfsim_plan *h, int B) {
   JobSpec js[kMaxJobs];
-  const int nj = tc_jobs(h, nullptr, B < kMaxLaunchScenes ? B : kMaxLaunchScenes, nullptr, js);
+  const int nj = tc_jobs(h, B < kMaxLaunchScenes ? B : kMaxLaunchScenes, js);
   return plan_multi(js, nj, nullptr, true).scratch;
 }
 
@@ -1226,11 +1260,8 @@ cudaError_t psfsim_launch_adjoint_tc(const psfsim_plan *h, const float *g, int B
     const int Bc = turns * ((B - b0) < most ? (B - b0) : most);
     const float *gb = g + (int64_t)b0 * h->M;
     JobSpec js[kMaxJobs];
-    const int nj = tc_jobs(h, nullptr, Bc, nullptr, js);
-    for (int j = 0; j < nj; ++j) {
-      js[j].x = h->quadrant ? gb : gb + (int64_t)j * kMaxBp * h->M;
-      js[j].first = h->quadrant ? j * kMaxBp : -1;
-    }
+    const int nj = tc_jobs(h, Bc, js);
+    for (int j = 0; j < nj; ++j) js[j].x = h->quadrant ? gb : gb + (int64_t)j * kMaxBp * h->M;
     const MultiPlan mp = plan_multi(js, nj, nullptr, true);
     cudaError_t e = launch_multi(js, nj, mp, scratch, st, kNoStall, true);
     if (e != cudaSuccess) return e;
@@ -1293,8 +1324,10 @@ cudaError_t psfsim_launch_forward_multi(const psfsim_job_t *jobs, int njobs, con
 cudaError_t psfsim_launch_forward_tc_stall(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
                                            uint64_t wait_ns, int64_t stall_it, cudaStream_t st) {
   JobSpec js[kMaxJobs];
-  const int nj = tc_jobs(h, x, B, y, js);
+  const int nj = tc_jobs(h, B, js);
   if (nj != 1) return cudaErrorInvalidValue;
+  js[0].x = x;
+  js[0].y = y;
   const StallHook hook = {wait_ns, stall_it, true};
   return launch_multi(js, nj, plan_multi(js, nj, nullptr), scratch, st, hook);
 }

@@ -1,0 +1,56 @@
+"""Scratch sizes against what the launches of a call take, on the host: the size that a caller asks
+for is never below the partial images and split scenes that the product then writes."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_2106_09122_gb300 import _binding as B
+
+STORAGES = {"split_bf16": B.SPLIT_BF16, "bf16": B.BF16, "split_bf16_sym": B.SPLIT_BF16_SYM}
+
+
+def _scratch(n, N, storage, batch, r_last=12.0, field=32.0, num_sms=152):
+    radii = np.linspace(0.0, r_last, 5)
+    reported, taken = ctypes.c_size_t(), ctypes.c_size_t()
+    B.check(B.load().psfsim_debug_scratch(radii.ctypes.data, 5, n, N, field / N, STORAGES[storage], num_sms, batch,
+                                          ctypes.byref(reported), ctypes.byref(taken)), "psfsim_debug_scratch")
+    return reported.value, taken.value
+
+
+@pytest.mark.parametrize("storage", STORAGES)
+@pytest.mark.parametrize("n", [16, 24, 64, 128, 160, 256])
+def test_forward_scratch_holds_every_launch(storage, n):
+    for N in (32, 60, 64, 96, 128, 200, 256):
+        for num_sms in (148, 152):
+            for batch in (1, 2, 3, 5, 10, 16, 17, 20, 21, 33, 64, 80, 81, 130, 320, 321, 336, 1280, 1281, 1340, 2480):
+                reported, taken = _scratch(n, N, storage, batch, num_sms=num_sms)
+                assert reported >= taken, (N, num_sms, batch)
+
+
+def _guarded(plan, product, x, need):
+    """The product with a scratch of exactly `need` bytes, and whether the 64 KiB after it are as they were."""
+    import torch
+    guard = 1 << 16
+    buf = torch.full((need + guard,), 0x5A, dtype=torch.uint8, device=x.device)
+    out = product(x, scratch=buf[:need])
+    assert plan.sync_status() == 0
+    return out, bool(torch.all(buf[need:] == 0x5A))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,N,batch", [(64, 32, 1), (64, 32, 16), (128, 32, 5), (160, 64, 10), (24, 96, 17)])
+def test_compact_forward_stays_inside_its_scratch(n, N, batch):
+    """Few columns, so that several splits are worth their partial images, which compact storage
+    always has.  Sums of products that are not negative: both within 1e-5 of the true ones."""
+    import torch
+    from paper_2106_09122_gb300 import Plan
+    rng = np.random.default_rng(n + N)
+    lib = torch.from_numpy(rng.uniform(0.0, 1.0, (5, n, n)).astype(np.float32)).cuda()
+    radii, S = np.linspace(0.0, 12.0, 5), 32.0 / N
+    x = torch.from_numpy(rng.uniform(0.0, 1.0, (batch, N * N)).astype(np.float32)).cuda()
+    split = Plan(lib, radii, 0.25, N=N, S=S, storage="split_bf16_sym")
+    y, clean = _guarded(split, split.forward, x, split.forward_scratch_bytes(batch))
+    assert clean
+    ref = Plan(lib, radii, 0.25, N=N, S=S, storage="fp32_sym").forward(x)
+    assert torch.all((y.double() - ref.double()).abs() <= 2e-5 * ref.double())

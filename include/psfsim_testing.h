@@ -32,12 +32,12 @@ extern "C" {
 int psfsim_debug_forward_stall(psfsim_t h, const float *d_x, int B, float *d_y, void *d_scratch,
                                size_t scratch_bytes, uint64_t wait_ns, int64_t stall_load, void *stream);
 
-/* Scratch of psfsim_forward for B scenes of a plan of this shape (SPLIT_BF16,
- * BF16 or SPLIT_BF16_SYM on a scene grid) on a device of num_sms SMs: what
- * psfsim_forward_scratch_bytes reports, and the most that a launch of the call
- * takes.  Host arithmetic only: no device is needed. */
-int psfsim_debug_scratch(const double *h_radii, int n_r, int n, int N, double S, int storage, int num_sms, int B,
-                         size_t *reported, size_t *taken);
+/* Scratch of psfsim_forward (adjoint: psfsim_adjoint) for a batch of B and a plan
+ * of this shape (SPLIT_BF16, BF16 or SPLIT_BF16_SYM on a scene grid) on a device
+ * of num_sms SMs: what psfsim_forward_scratch_bytes (psfsim_adjoint_scratch_bytes)
+ * reports, and the most that a launch of the call takes.  Host arithmetic only: no device is needed. */
+int psfsim_debug_scratch(const double *h_radii, int n_r, int n, int N, double S, int storage, int num_sms,
+                         int adjoint, int B, size_t *reported, size_t *taken);
 
 #ifdef __cplusplus
 }

@@ -279,8 +279,8 @@ int psfsim_adjoint(psfsim_t h, const float *d_g, int B, float *d_gx, void *d_scr
   if (h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16) {
     const size_t need = psfsim_adjoint_tc_scratch(h, B);
     if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
-    return psfsim_launch_adjoint_tc(h, d_g, B, d_gx, d_scratch, st) == cudaSuccess ? PSFSIM_OK
-                                                                                      : PSFSIM_ERR_CUDA;
+    return psfsim_launch_adjoint_tc(h, d_g, B, d_gx, d_scratch, scratch_bytes, st) == cudaSuccess ? PSFSIM_OK
+                                                                                                  : PSFSIM_ERR_CUDA;
   }
   if (h->storage == PSFSIM_FP32_SYM) {
     const size_t need = psfsim_adjoint_sym_scratch(h, B);
@@ -290,8 +290,8 @@ int psfsim_adjoint(psfsim_t h, const float *d_g, int B, float *d_gx, void *d_scr
   if (h->storage == PSFSIM_SPLIT_BF16_SYM) {
     const size_t need = psfsim_adjoint_tc_scratch(h, 4 * B);
     if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
-    return psfsim_launch_adjoint_tc(h, d_g, B, d_gx, d_scratch, st) == cudaSuccess ? PSFSIM_OK
-                                                                                          : PSFSIM_ERR_CUDA;
+    return psfsim_launch_adjoint_tc(h, d_g, B, d_gx, d_scratch, scratch_bytes, st) == cudaSuccess ? PSFSIM_OK
+                                                                                                  : PSFSIM_ERR_CUDA;
   }
   return PSFSIM_ERR_UNSUPPORTED;
 }
@@ -352,8 +352,8 @@ int psfsim_debug_forward_stall(psfsim_t h, const float *d_x, int B, float *d_y, 
              : PSFSIM_ERR_CUDA;
 }
 
-int psfsim_debug_scratch(const double *h_radii, int n_r, int n, int N, double S, int storage, int num_sms, int B,
-                         size_t *reported, size_t *taken) {
+int psfsim_debug_scratch(const double *h_radii, int n_r, int n, int N, double S, int storage, int num_sms,
+                         int adjoint, int B, size_t *reported, size_t *taken) {
   if (!reported || !taken || n < 1 || n > 4096 || N < 1 || N > 32768 || !(S > 0.0) || num_sms < 1 || B < 1)
     return PSFSIM_ERR_ARG;
   if (int rc = check_radii(h_radii, n_r)) return rc;
@@ -373,8 +373,9 @@ int psfsim_debug_scratch(const double *h_radii, int n_r, int n, int N, double S,
     p.ld = psfsim_round_up(p.K_valid > 0 ? p.K_valid : 1, 64);
   }
   psfsim_live_count(&p);
-  if (int rc = psfsim_forward_scratch_bytes(&p, B, reported)) return rc;
-  *taken = psfsim_forward_tc_taken(&p, p.quadrant ? 4 * B : B);
+  if (int rc = adjoint ? psfsim_adjoint_scratch_bytes(&p, B, reported) : psfsim_forward_scratch_bytes(&p, B, reported))
+    return rc;
+  *taken = psfsim_tc_taken(&p, p.quadrant ? 4 * B : B, adjoint != 0);
   return PSFSIM_OK;
 }
 

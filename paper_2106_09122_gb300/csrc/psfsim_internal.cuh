@@ -90,7 +90,7 @@ cudaError_t psfsim_launch_reduce_partials(const float *part, int KS, int B, int6
 // Split-BF16 storage: build, tensor-core forward, CUDA-core adjoint.
 cudaError_t psfsim_launch_split_build(psfsim_plan *h, cudaStream_t st);
 size_t psfsim_forward_tc_scratch(const psfsim_plan *h, int B);  // compact storage: of B rotated scenes
-size_t psfsim_forward_tc_taken(const psfsim_plan *h, int B);    // what the launches themselves take
+size_t psfsim_tc_taken(const psfsim_plan *h, int B, bool adjoint);  // the most that one of the launches takes
 cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
                                      size_t scratch_bytes, cudaStream_t st);
 cudaError_t psfsim_launch_forward_tc_sym(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
@@ -106,9 +106,9 @@ struct SymSum {
 };
 cudaError_t psfsim_launch_sym_sum(SymSum S, int B, float *y, cudaStream_t st);
 // Adjoint of split and BF16 storage, dense or compact, on the tensor cores.
-size_t psfsim_adjoint_tc_scratch(const psfsim_plan *h, int B);
+size_t psfsim_adjoint_tc_scratch(const psfsim_plan *h, int B);  // compact storage: of B turned residuals
 cudaError_t psfsim_launch_adjoint_tc(const psfsim_plan *h, const float *g, int B, float *gx, void *scratch,
-                                     cudaStream_t st);
+                                     size_t scratch_bytes, cudaStream_t st);
 // Test hook: the tensor-core forward of <= 80 scenes on one CTA with every
 // wait bounded by wait_ns and load number stall_it never issued.
 cudaError_t psfsim_launch_forward_tc_stall(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,

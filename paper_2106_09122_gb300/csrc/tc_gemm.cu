@@ -1127,8 +1127,8 @@ cudaError_t launch_wide(const psfsim_plan *h, const float *x, int scenes, const 
 
 namespace {
 
-// One launch of a product of `count` scenes (compact storage: rotated scenes).
-// What sizes the scratch and what runs are this same plan.
+// One launch of a product of `count` scenes or, adjoint, residuals (compact storage:
+// turned ones).  What sizes the scratch and what runs are this same plan.
 struct Launch {
   bool wide;
   int nj;
@@ -1138,16 +1138,16 @@ struct Launch {
   size_t scratch;
 };
 
-Launch plan_launch(const psfsim_plan *h, int count) {
+Launch plan_launch(const psfsim_plan *h, int count, bool adjoint) {
   Launch L;
-  L.wide = wide_form(h, count);
+  L.wide = !adjoint && wide_form(h, count);
   L.nj = 0;
   if (L.wide) {
     L.w = plan_wide(h, count);
     L.scratch = L.w.scratch;
   } else {
     L.nj = tc_jobs(h, count, L.js);
-    L.multi = plan_multi(L.js, L.nj, nullptr);
+    L.multi = plan_multi(L.js, L.nj, nullptr, adjoint);
     L.scratch = L.multi.scratch;
   }
   return L;
@@ -1160,19 +1160,22 @@ int launch_count(int B, int i) {
   return left < 0 ? 0 : (int)(left < kMaxLaunchScenes ? left : kMaxLaunchScenes);
 }
 
-}  // namespace
-
-size_t psfsim_forward_tc_scratch(const psfsim_plan *h, int B) {
-  const size_t first = plan_launch(h, launch_count(B, 0)).scratch;
+size_t tc_scratch(const psfsim_plan *h, int B, bool adjoint) {
+  const size_t first = plan_launch(h, launch_count(B, 0), adjoint).scratch;
   if (B <= kMaxLaunchScenes) return first;
-  const size_t last = plan_launch(h, launch_count(B, (B - 1) / kMaxLaunchScenes)).scratch;  // those between are as the first
+  // A remainder of fewer jobs may split k further and take more; those between are as the first.
+  const size_t last = plan_launch(h, launch_count(B, (B - 1) / kMaxLaunchScenes), adjoint).scratch;
   return last > first ? last : first;
 }
 
-size_t psfsim_forward_tc_taken(const psfsim_plan *h, int B) {
+}  // namespace
+
+size_t psfsim_forward_tc_scratch(const psfsim_plan *h, int B) { return tc_scratch(h, B, false); }
+
+size_t psfsim_tc_taken(const psfsim_plan *h, int B, bool adjoint) {
   size_t most = 0;
   for (int i = 0, c; (c = launch_count(B, i)) > 0; ++i) {
-    const size_t need = plan_launch(h, c).scratch;
+    const size_t need = plan_launch(h, c, adjoint).scratch;
     most = need > most ? need : most;
   }
   return most;
@@ -1181,7 +1184,7 @@ size_t psfsim_forward_tc_taken(const psfsim_plan *h, int B) {
 cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
                                      size_t scratch_bytes, cudaStream_t st) {
   for (int i = 0, c; (c = launch_count(B, i)) > 0; ++i) {
-    Launch L = plan_launch(h, c);
+    Launch L = plan_launch(h, c, false);
     if (L.scratch > scratch_bytes) return cudaErrorInvalidValue;
     const float *xb = x + (int64_t)i * kMaxLaunchScenes * h->K;
     float *yb = y + (int64_t)i * kMaxLaunchScenes * h->M;
@@ -1211,7 +1214,7 @@ cudaError_t psfsim_launch_forward_tc_sym(const psfsim_plan *h, const float *x, i
   constexpr int kScenes = kMaxLaunchScenes / 4;
   static_assert(kMaxBp % 4 == 0, "a scene's rotations share a job");
   for (int i = 0, c; (c = launch_count(4 * B, i)) > 0; ++i) {
-    Launch L = plan_launch(h, c);
+    Launch L = plan_launch(h, c, false);
     if (L.scratch > scratch_bytes) return cudaErrorInvalidValue;
     const float *xb = x + (int64_t)i * kScenes * h->K;
     SymSum S;
@@ -1242,34 +1245,29 @@ cudaError_t psfsim_launch_forward_tc_sym(const psfsim_plan *h, const float *x, i
 }
 
 // Compact storage: the four turns of the residuals are the batch.
-size_t psfsim_adjoint_tc_scratch(const psfsim_plan *h, int B) {
-  JobSpec js[kMaxJobs];
-  const int nj = tc_jobs(h, B < kMaxLaunchScenes ? B : kMaxLaunchScenes, js);
-  return plan_multi(js, nj, nullptr, true).scratch;
-}
+size_t psfsim_adjoint_tc_scratch(const psfsim_plan *h, int B) { return tc_scratch(h, B, true); }
 
 cudaError_t psfsim_launch_adjoint_tc(const psfsim_plan *h, const float *g, int B, float *gx, void *scratch,
-                                     cudaStream_t st) {
+                                     size_t scratch_bytes, cudaStream_t st) {
   const int turns = h->quadrant ? 4 : 1;
   if (h->quadrant) {  // scene pixels without a column
     const cudaError_t e = cudaMemsetAsync(gx, 0, (size_t)B * h->K * 4, st);
     if (e != cudaSuccess || h->K_valid == 0) return e;
   }
-  const int most = kMaxLaunchScenes / turns;
-  for (int b0 = 0; b0 < B; b0 += most) {
-    const int Bc = turns * ((B - b0) < most ? (B - b0) : most);
-    const float *gb = g + (int64_t)b0 * h->M;
-    JobSpec js[kMaxJobs];
-    const int nj = tc_jobs(h, Bc, js);
-    for (int j = 0; j < nj; ++j) js[j].x = h->quadrant ? gb : gb + (int64_t)j * kMaxBp * h->M;
-    const MultiPlan mp = plan_multi(js, nj, nullptr, true);
-    cudaError_t e = launch_multi(js, nj, mp, scratch, st, kNoStall, true);
+  for (int i = 0, c; (c = launch_count(turns * B, i)) > 0; ++i) {
+    Launch L = plan_launch(h, c, true);
+    if (L.scratch > scratch_bytes) return cudaErrorInvalidValue;
+    const MultiPlan &mp = L.multi;
+    const int64_t b0 = (int64_t)i * (kMaxLaunchScenes / turns);
+    const float *gb = g + b0 * h->M;
+    for (int j = 0; j < L.nj; ++j) L.js[j].x = h->quadrant ? gb : gb + (int64_t)j * kMaxBp * h->M;
+    cudaError_t e = launch_multi(L.js, L.nj, mp, scratch, st, kNoStall, true);
     if (e != cudaSuccess) return e;
     AdjFinish F;
     std::memset(&F, 0, sizeof(F));
-    for (int j = 0; j < nj; ++j) {
+    for (int j = 0; j < L.nj; ++j) {
       F.part[j] = reinterpret_cast<const float *>(static_cast<char *>(scratch) + mp.jp[j].part_off);
-      F.cap[j] = js[j].cap;
+      F.cap[j] = L.js[j].cap;
     }
     const int *tab = reinterpret_cast<const int *>(h->ws + h->order_off);
     F.KS = mp.jp[0].KS;
@@ -1288,9 +1286,9 @@ cudaError_t psfsim_launch_adjoint_tc(const psfsim_plan *h, const float *g, int B
     F.hi = reinterpret_cast<const __nv_bfloat16 *>(h->ws + h->a_off);
     F.lo = h->lo_off >= 0 ? reinterpret_cast<const __nv_bfloat16 *>(h->ws + h->lo_off) : nullptr;
     F.g = gb;
-    F.gx = gx + (int64_t)b0 * h->K;
+    F.gx = gx + b0 * h->K;
     const int64_t threads = F.width + F.dead_groups * kLiveGroup;
-    adj_finish_kernel<<<dim3((unsigned)((threads + 255) / 256), (unsigned)Bc), 256, 0, st>>>(F);
+    adj_finish_kernel<<<dim3((unsigned)((threads + 255) / 256), (unsigned)c), 256, 0, st>>>(F);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;

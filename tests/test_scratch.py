@@ -10,11 +10,11 @@ from paper_2106_09122_gb300 import _binding as B
 STORAGES = {"split_bf16": B.SPLIT_BF16, "bf16": B.BF16, "split_bf16_sym": B.SPLIT_BF16_SYM}
 
 
-def _scratch(n, N, storage, batch, r_last=12.0, field=32.0, num_sms=152):
+def _scratch(n, N, storage, batch, r_last=12.0, field=32.0, num_sms=152, adjoint=0):
     radii = np.linspace(0.0, r_last, 5)
     reported, taken = ctypes.c_size_t(), ctypes.c_size_t()
-    B.check(B.load().psfsim_debug_scratch(radii.ctypes.data, 5, n, N, field / N, STORAGES[storage], num_sms, batch,
-                                          ctypes.byref(reported), ctypes.byref(taken)), "psfsim_debug_scratch")
+    B.check(B.load().psfsim_debug_scratch(radii.ctypes.data, 5, n, N, field / N, STORAGES[storage], num_sms, adjoint,
+                                          batch, ctypes.byref(reported), ctypes.byref(taken)), "psfsim_debug_scratch")
     return reported.value, taken.value
 
 
@@ -26,6 +26,18 @@ def test_forward_scratch_holds_every_launch(storage, n):
             for batch in (1, 2, 3, 5, 10, 16, 17, 20, 21, 33, 64, 80, 81, 130, 320, 321, 336, 1280, 1281, 1340, 2480):
                 reported, taken = _scratch(n, N, storage, batch, num_sms=num_sms)
                 assert reported >= taken, (N, num_sms, batch)
+
+
+@pytest.mark.parametrize("storage", STORAGES)
+@pytest.mark.parametrize("n", [16, 18, 22, 24, 64, 160])
+def test_adjoint_scratch_holds_every_launch(storage, n):
+    """More than 1280 residuals (320 on compact storage) take several launches, of which the last
+    may split k further than the first.  All columns live, or 44 % of them."""
+    for N in (20, 32, 60, 64, 66, 100, 160):
+        for field, num_sms in ((32.0, 152), (32.0, 148), (16.0, 152)):
+            for batch in (1, 5, 20, 21, 80, 81, 320, 321, 350, 560, 600, 640, 1280, 1281, 1300, 1400, 2240, 2480, 2560):
+                reported, taken = _scratch(n, N, storage, batch, field=field, num_sms=num_sms, adjoint=1)
+                assert reported >= taken, (N, field, num_sms, batch)
 
 
 def _guarded(plan, product, x, need):
@@ -54,3 +66,24 @@ def test_compact_forward_stays_inside_its_scratch(n, N, batch):
     assert clean
     ref = Plan(lib, radii, 0.25, N=N, S=S, storage="fp32_sym").forward(x)
     assert torch.all((y.double() - ref.double()).abs() <= 2e-5 * ref.double())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,N,storage,batch", [(16, 60, "split_bf16", 1281), (16, 60, "bf16", 2480),
+                                               (16, 60, "split_bf16", 2480), (16, 60, "split_bf16_sym", 321),
+                                               (24, 100, "split_bf16_sym", 600)])
+def test_adjoint_of_several_launches_stays_inside_its_scratch(n, N, storage, batch):
+    """Residuals that are not negative: sums without cancellation, within 1e-5 of the true ones
+    (BF16: and 2^-8 of them)."""
+    import torch
+    from paper_2106_09122_gb300 import Plan
+    rng = np.random.default_rng(n + N)
+    lib = torch.from_numpy(rng.uniform(0.0, 1.0, (5, n, n)).astype(np.float32)).cuda()
+    radii, S = np.linspace(0.0, 12.0, 5), 16.0 / N
+    g = torch.from_numpy(rng.uniform(0.0, 1.0, (batch, n * n)).astype(np.float32)).cuda()
+    split = Plan(lib, radii, 0.25, N=N, S=S, storage=storage)
+    gx, clean = _guarded(split, split.adjoint, g, split.adjoint_scratch_bytes(batch))
+    assert clean
+    ref = Plan(lib, radii, 0.25, N=N, S=S).adjoint(g).double()
+    tol = 2e-5 + (2.0 ** -8 if storage == "bf16" else 0.0)
+    assert torch.all((gx.double() - ref).abs() <= tol * ref)

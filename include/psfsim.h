@@ -136,7 +136,9 @@ int psfsim_build_points(const float *d_lib, const double *h_radii, int n_r, int 
 /* Fill *info with the plan's layout. */
 int psfsim_info(psfsim_t h, psfsim_info_t *info);
 
-/* Scratch bytes psfsim_forward / psfsim_adjoint need for a batch of B. */
+/* Scratch bytes psfsim_forward / psfsim_adjoint need for a batch of B, or of
+ * any smaller number: one buffer for a caller's largest batch serves them all.
+ * Asked for once, not per call (tens of microseconds for a large batch). */
 int psfsim_forward_scratch_bytes(psfsim_t h, int B, size_t *bytes);
 int psfsim_adjoint_scratch_bytes(psfsim_t h, int B, size_t *bytes);
 

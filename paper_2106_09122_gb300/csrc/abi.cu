@@ -226,7 +226,7 @@ int psfsim_forward(psfsim_t h, const float *d_x, int B, float *d_y, void *d_scra
                                                                                     : PSFSIM_ERR_CUDA;
   }
   if (h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16) {
-    const size_t need = psfsim_forward_tc_scratch(h, B);
+    const size_t need = psfsim_tc_taken(h, B, false);
     if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
     return psfsim_launch_forward_tc(h, d_x, B, d_y, d_scratch, scratch_bytes, st) == cudaSuccess ? PSFSIM_OK
                                                                                                  : PSFSIM_ERR_CUDA;
@@ -237,7 +237,7 @@ int psfsim_forward(psfsim_t h, const float *d_x, int B, float *d_y, void *d_scra
     return psfsim_launch_forward_sym(h, d_x, B, d_y, d_scratch, st) == cudaSuccess ? PSFSIM_OK : PSFSIM_ERR_CUDA;
   }
   if (h->storage == PSFSIM_SPLIT_BF16_SYM) {
-    const size_t need = psfsim_forward_split_sym_scratch(h, B);
+    const size_t need = psfsim_tc_taken(h, 4 * B, false);
     if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
     return psfsim_launch_forward_split_sym(h, d_x, B, d_y, d_scratch, scratch_bytes, st) == cudaSuccess
                ? PSFSIM_OK
@@ -277,7 +277,7 @@ int psfsim_adjoint(psfsim_t h, const float *d_g, int B, float *d_gx, void *d_scr
   if (h->storage == PSFSIM_FP32)
     return psfsim_launch_adjoint_fp32(h, d_g, B, d_gx, st) == cudaSuccess ? PSFSIM_OK : PSFSIM_ERR_CUDA;
   if (h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16) {
-    const size_t need = psfsim_adjoint_tc_scratch(h, B);
+    const size_t need = psfsim_tc_taken(h, B, true);
     if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
     return psfsim_launch_adjoint_tc(h, d_g, B, d_gx, d_scratch, scratch_bytes, st) == cudaSuccess ? PSFSIM_OK
                                                                                                   : PSFSIM_ERR_CUDA;
@@ -288,7 +288,7 @@ int psfsim_adjoint(psfsim_t h, const float *d_g, int B, float *d_gx, void *d_scr
     return psfsim_launch_adjoint_sym(h, d_g, B, d_gx, d_scratch, st) == cudaSuccess ? PSFSIM_OK : PSFSIM_ERR_CUDA;
   }
   if (h->storage == PSFSIM_SPLIT_BF16_SYM) {
-    const size_t need = psfsim_adjoint_tc_scratch(h, 4 * B);
+    const size_t need = psfsim_tc_taken(h, 4 * B, true);
     if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
     return psfsim_launch_adjoint_tc(h, d_g, B, d_gx, d_scratch, scratch_bytes, st) == cudaSuccess ? PSFSIM_OK
                                                                                                   : PSFSIM_ERR_CUDA;
@@ -307,7 +307,7 @@ int psfsim_forward_multi_scratch_bytes(const psfsim_job_t *jobs, int njobs, cons
 int psfsim_forward_multi(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tuning, void *d_scratch,
                          size_t scratch_bytes, void *stream) {
   if (int rc = psfsim_multi_validate(jobs, njobs)) return rc;
-  if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < psfsim_forward_multi_scratch(jobs, njobs, tuning))
+  if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < psfsim_forward_multi_taken(jobs, njobs, tuning))
     return PSFSIM_ERR_WORKSPACE;
   return psfsim_launch_forward_multi(jobs, njobs, tuning, d_scratch, static_cast<cudaStream_t>(stream)) == cudaSuccess
              ? PSFSIM_OK
@@ -344,7 +344,7 @@ int psfsim_debug_forward_stall(psfsim_t h, const float *d_x, int B, float *d_y, 
                : PSFSIM_ERR_CUDA;
   }
   if (h->storage != PSFSIM_SPLIT_BF16 && h->storage != PSFSIM_BF16) return PSFSIM_ERR_UNSUPPORTED;
-  const size_t need = psfsim_forward_tc_scratch(h, B);
+  const size_t need = psfsim_tc_taken(h, B, false);
   if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
   return psfsim_launch_forward_tc_stall(h, d_x, B, d_y, d_scratch, wait_ns, stall_load,
                                         static_cast<cudaStream_t>(stream)) == cudaSuccess

@@ -87,10 +87,11 @@ cudaError_t psfsim_launch_adjoint_fp32(const psfsim_plan *h, const float *g, int
 // y[b, i] = sum_ks part[(ks * B + b) * ld + i], fixed order.
 cudaError_t psfsim_launch_reduce_partials(const float *part, int KS, int B, int64_t ld, int64_t M, float *y,
                                           cudaStream_t st);
-// Split-BF16 storage: build, tensor-core forward, CUDA-core adjoint.
+// Split-BF16 and BF16 storage: build, tensor-core forward and adjoint.  A product's
+// scratch is reported monotone in the batch and checked against what it takes.
 cudaError_t psfsim_launch_split_build(psfsim_plan *h, cudaStream_t st);
 size_t psfsim_forward_tc_scratch(const psfsim_plan *h, int B);  // compact storage: of B rotated scenes
-size_t psfsim_tc_taken(const psfsim_plan *h, int B, bool adjoint);  // the most that one of the launches takes
+size_t psfsim_tc_taken(const psfsim_plan *h, int B, bool adjoint);  // the call's own launches
 cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
                                      size_t scratch_bytes, cudaStream_t st);
 cudaError_t psfsim_launch_forward_tc_sym(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
@@ -116,6 +117,7 @@ cudaError_t psfsim_launch_forward_tc_stall(const psfsim_plan *h, const float *x,
 // Multi-job persistent tensor-core forward (several split-BF16 plans, one launch).
 int psfsim_multi_validate(const psfsim_job_t *jobs, int njobs);
 size_t psfsim_forward_multi_scratch(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune);
+size_t psfsim_forward_multi_taken(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune);
 cudaError_t psfsim_launch_forward_multi(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune,
                                         void *scratch, cudaStream_t st);
 // FP32 forward products (column-major A, gemv.cu): partial images part[KS][B][ld].

@@ -1160,25 +1160,32 @@ int launch_count(int B, int i) {
   return left < 0 ? 0 : (int)(left < kMaxLaunchScenes ? left : kMaxLaunchScenes);
 }
 
+// What the caller is told: enough for every batch up to B, so that a buffer for a
+// large batch serves a smaller one, whose split of k may be finer and take more
+// (and the remainder launch of a batch beyond kMaxLaunchScenes).
 size_t tc_scratch(const psfsim_plan *h, int B, bool adjoint) {
-  const size_t first = plan_launch(h, launch_count(B, 0), adjoint).scratch;
-  if (B <= kMaxLaunchScenes) return first;
-  // A remainder of fewer jobs may split k further and take more; those between are as the first.
-  const size_t last = plan_launch(h, launch_count(B, (B - 1) / kMaxLaunchScenes), adjoint).scratch;
-  return last > first ? last : first;
+  const int step = h->quadrant ? 4 : 1, top = launch_count(B, 0);
+  size_t most = 0;
+  for (int c = step; c <= top; c += step) {
+    // Narrow launches of equally many jobs split alike: the last of them takes the most.
+    if (c > kMaxBp && c % kMaxBp && c < top && (adjoint || !(wide_form(h, c) || wide_form(h, c + step)))) continue;
+    const size_t need = plan_launch(h, c, adjoint).scratch;
+    most = need > most ? need : most;
+  }
+  return most;
 }
 
 }  // namespace
 
 size_t psfsim_forward_tc_scratch(const psfsim_plan *h, int B) { return tc_scratch(h, B, false); }
 
+// What a call of B itself takes: its first launch's, or its last's (those between
+// are as the first).
 size_t psfsim_tc_taken(const psfsim_plan *h, int B, bool adjoint) {
-  size_t most = 0;
-  for (int i = 0, c; (c = launch_count(B, i)) > 0; ++i) {
-    const size_t need = plan_launch(h, c, adjoint).scratch;
-    most = need > most ? need : most;
-  }
-  return most;
+  const size_t first = plan_launch(h, launch_count(B, 0), adjoint).scratch;
+  if (B <= kMaxLaunchScenes) return first;
+  const size_t last = plan_launch(h, launch_count(B, (B - 1) / kMaxLaunchScenes), adjoint).scratch;
+  return last > first ? last : first;
 }
 
 cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
@@ -1306,10 +1313,22 @@ int psfsim_multi_validate(const psfsim_job_t *jobs, int njobs) {
   return PSFSIM_OK;
 }
 
-size_t psfsim_forward_multi_scratch(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune) {
+size_t psfsim_forward_multi_taken(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune) {
   JobSpec js[kMaxJobs];
   for (int j = 0; j < njobs; ++j) js[j] = JobSpec{jobs[j].plan, jobs[j].d_x, jobs[j].d_y, jobs[j].capacity, jobs[j].d_count, -1};
   return plan_multi(js, njobs, tune).scratch;
+}
+
+// Enough for smaller capacities too: one job's split of k depends on its capacity.
+size_t psfsim_forward_multi_scratch(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune) {
+  if (njobs > 1) return psfsim_forward_multi_taken(jobs, njobs, tune);
+  psfsim_job_t one = jobs[0];
+  size_t most = 0;
+  for (one.capacity = 1; one.capacity <= jobs[0].capacity; ++one.capacity) {
+    const size_t need = psfsim_forward_multi_taken(&one, 1, tune);
+    most = need > most ? need : most;
+  }
+  return most;
 }
 
 cudaError_t psfsim_launch_forward_multi(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune,

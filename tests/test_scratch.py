@@ -40,6 +40,17 @@ def test_adjoint_scratch_holds_every_launch(storage, n):
                 assert reported >= taken, (N, field, num_sms, batch)
 
 
+@pytest.mark.parametrize("storage", STORAGES)
+@pytest.mark.parametrize("n,N", [(64, 64), (16, 60), (24, 100), (100, 86), (128, 32), (160, 64), (256, 128)])
+def test_scratch_for_a_batch_serves_every_smaller_one(storage, n, N):
+    for adjoint in (0, 1):
+        most = 0
+        for batch in [*range(1, 100), 128, 129, 160, 161, 200, 256, 257, 320, 321, 400, 1280, 1281, 2480]:
+            reported, taken = _scratch(n, N, storage, batch, adjoint=adjoint)
+            assert reported >= max(most, taken), (adjoint, batch)
+            most = reported
+
+
 def _guarded(plan, product, x, need):
     """The product with a scratch of exactly `need` bytes, and whether the 64 KiB after it are as they were."""
     import torch
@@ -87,3 +98,33 @@ def test_adjoint_of_several_launches_stays_inside_its_scratch(n, N, storage, bat
     ref = Plan(lib, radii, 0.25, N=N, S=S).adjoint(g).double()
     tol = 2e-5 + (2.0 ** -8 if storage == "bf16" else 0.0)
     assert torch.all((gx.double() - ref).abs() <= tol * ref)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("storage,n,N", [("split_bf16", 64, 64), ("bf16", 100, 86)])
+def test_multi_forward_scratch_of_one_job_serves_smaller_capacities(storage, n, N):
+    import torch
+    from paper_2106_09122_gb300 import Plan
+    rng = np.random.default_rng(n)
+    lib = torch.from_numpy(rng.uniform(0.0, 1.0, (5, n, n)).astype(np.float32)).cuda()
+    plan = Plan(lib, np.linspace(0.0, 12.0, 5), 0.25, N=N, S=32.0 / N, storage=storage)
+    x = torch.from_numpy(rng.uniform(0.0, 1.0, (80, N * N)).astype(np.float32)).cuda()
+    y = torch.empty((80, n * n), device="cuda")
+    L, nb = B.load(), ctypes.c_size_t()
+
+    def job(cap):
+        return (B.Job * 1)(B.Job(plan.handle, x.data_ptr(), y.data_ptr(), cap, None))
+
+    B.check(L.psfsim_forward_multi_scratch_bytes(job(80), 1, None, ctypes.byref(nb)), "scratch")
+    scr = torch.empty(nb.value, dtype=torch.uint8, device="cuda")
+    ref = plan.forward(x)
+    most = 0
+    for cap in range(1, 81):
+        B.check(L.psfsim_forward_multi_scratch_bytes(job(cap), 1, None, ctypes.byref(nb)), "scratch")
+        assert nb.value >= most
+        most = nb.value
+        B.check(L.psfsim_forward_multi(job(cap), 1, None, scr.data_ptr(), scr.numel(),
+                                       torch.cuda.current_stream().cuda_stream), "psfsim_forward_multi")
+        tol = 2e-5 * ref[:cap]  # both sums of products that are not negative, split differently
+        assert torch.all((y[:cap] - ref[:cap]).abs() <= tol)
+    assert plan.sync_status() == 0

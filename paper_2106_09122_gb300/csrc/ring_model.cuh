@@ -60,7 +60,8 @@ __device__ __forceinline__ float ring_eval(const RingParams &P, int64_t j, float
   const float big = fmaxf(xx, yy), small = fminf(xx, yy);
   const float left = fmaf(-rd, rd, r2d) + ((small - (r2d - big)) + fmaf(x, x, -xx) + fmaf(yd, yd, -yy)) +
                      2.f * (x * x_lo + yd * y_lo);
-  const float dr = ((rd - P.R) - P.R_lo) + (pos ? 0.5f * left / rd : 0.f);
+  // Beyond 1.8e19 the squares overflow, and with them the rest: the distance is infinite.
+  const float dr = ((rd - P.R) - P.R_lo) + (pos && rd <= 3.402823466e38f ? 0.5f * left / rd : 0.f);
   const float G = expf(P.k * (dr * dr));
   const float ratio = 1.f / (fmaf(-P.q, mu, 1.f) - P.q_lo * mu);
   const float H = ratio * sqrtf(ratio), GH = G * H;
@@ -103,6 +104,7 @@ inline bool ring_params(int N, double S, double r_max, const double *th, RingPar
   ring_two(th[4], &P->B, &P->B_lo);
   const double c = std::cos(th[2]), g2 = 1.0 + th[3] * th[3];
   ring_two(S / c, &P->V, &P->V_lo);
+  if (!std::isfinite(P->V)) P->V = std::copysign(3.402823466e38f, P->V);  // row 0 of an odd grid: 0 x V
   P->sini = (float)std::sin(th[2]);
   P->cosi = (float)c;
   P->tani = (float)(std::sin(th[2]) / c);

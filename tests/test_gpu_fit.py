@@ -199,3 +199,15 @@ def test_ring_scene_rounds_like_its_last_operations(N, S, w, inc):
     rd = np.hypot(np.tile(c, N), np.repeat(c, N) / np.cos(theta[2]))
     arg = 4.0 * np.log(2.0) * ((rd - theta[0]) / w) ** 2
     assert np.all(np.abs(z - ref) <= ref * (1e-6 + 3e-7 * arg) + 1e-37)
+
+
+@pytest.mark.parametrize("N,S,inc", [(8, 1e19, 0.5), (7, 1e19, 0.5), (8, 4e18, 0.5), (7, 1e33, 0.5), (8, 1e13, 1.5707943)])
+def test_ring_scene_where_squared_coordinates_overflow(N, S, inc):
+    """Pixels whose x^2 + (y / cos i)^2 is beyond float32 are infinitely far from the ring: zero flux, not NaN."""
+    from paper_2106_09122_gb300 import _binding as B
+    theta = np.array([1.0, 1.0, inc, 0.3, 1.0])
+    z = torch.full((N, N), float("nan"), device=DEV)
+    B.check(B.load().psfsim_ring_scene(N, S, 1e36, theta.ctypes.data, z.data_ptr(),
+                                       torch.cuda.current_stream().cuda_stream), "psfsim_ring_scene")
+    ref = RO.ring_scene(theta, N, S, 1e36).reshape(N, N)
+    np.testing.assert_allclose(z.cpu().numpy(), ref, rtol=1e-5, atol=0)

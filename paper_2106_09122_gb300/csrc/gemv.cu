@@ -23,7 +23,7 @@ namespace {
 //     serves four scenes.  Read from global memory per thread, a group of 8
 //     scenes ran at half the rate of one.
 // 11 scenes of the 128^2 plan: 660 us in passes of 8, 2 and 1 over all columns,
-// 92 us in one pass over the live ones (HBM floor 70).
+// 95 us in one pass over the live ones (HBM floor 70).
 constexpr int kChunkCols = kFwdThreads;
 constexpr int kShare = 4;
 
@@ -413,7 +413,7 @@ int psfsim_gemv_max_splits(int64_t ld, int64_t K, int num_sms) {
   return (int)(ks < max_ks ? ks : max_ks);
 }
 
-// Passes of at most 16 scenes, evenly filled, with one wave of resident CTAs.
+// Passes of at most 16 scenes, evenly filled, with whole waves of resident CTAs.
 cudaError_t psfsim_launch_gemv_partials(const FwdCols &P, int max_splits, int num_sms, bool skip_zeros, int *KS_out,
                                         cudaStream_t st) {
   const int passes = (P.B + 15) / 16, per0 = (P.B + passes - 1) / passes;
@@ -423,6 +423,16 @@ cudaError_t psfsim_launch_gemv_partials(const FwdCols &P, int max_splits, int nu
   int64_t KS = (int64_t)num_sms * fwd_min_ctas(BB) / row_blocks;
   const int64_t max_ks = P.L / 8 > 0 ? P.L / 8 : 1;
   KS = KS < 1 ? 1 : KS;
+  // A thread adds its share's columns one after another, and 12 or 16 scenes leave
+  // few CTAs: where that chain is long, whole waves of shorter shares.  Image of 16
+  // scenes against 64 bits, one wave / now: 256^2 of 128^2 4.5e-7 / 1.4e-7, 160^2
+  // 2.2e-7 / 1.3e-7, 128^2 1.21e-7 / 0.89e-7; time 452 / 466, 252 / 261 and 114 / 121
+  // us (11 scenes: 93 / 95).  Shorter chains gain nothing that the longer sum over
+  // splits does not lose.  Sub-sums of 8 columns or sums folded into shared memory
+  // every 64 cost 8 to 13 % at all sizes.
+  const int64_t chain = P.L / KS, waves = chain > 320 && chain <= 512 ? 2 : (chain + 511) / 512;
+  const int64_t most = max_splits / KS > 1 ? max_splits / KS : 1;
+  KS *= waves < 1 ? 1 : waves < most ? waves : most;
   KS = KS < max_ks ? KS : max_ks;
   KS = KS < max_splits ? KS : max_splits;
   *KS_out = (int)KS;

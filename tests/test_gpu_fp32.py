@@ -174,3 +174,21 @@ def test_adjoint_workload_sampled_rows():
     lhs, rhs = yfull @ g.astype(np.float64), x64 @ gx
     scale = np.abs(yfull) @ np.abs(g.astype(np.float64))
     assert abs(lhs - rhs) <= 1e-5 * scale
+
+
+def test_many_scenes_of_a_large_image_do_not_drift():
+    """16 scenes leave few CTAs for a 256 x 256 image.  Every element is 1 and every scene value
+    1 + 2^-15, whose last bit a float32 sum beyond 1024 drops each time: a chain of all of a CTA's
+    1800 columns would lose 1e-5 (2^-15 of each term from 1024 on).  Chains of at most 512 keep it: what is left is the
+    elements' rounding (2^-23) and the sum over at most 19 splits (1.1e-6)."""
+    from paper_2106_09122_gb300 import Plan
+    n, N, B = 256, 128, 16
+    plan = Plan(torch.ones(2, n, n, device=DEV), np.array([0.0, 12.0]), 0.125, N=N, S=0.25)
+    x = torch.full((B, N * N), 1.0 + 2.0 ** -15, device=DEV)
+    c = (torch.arange(N, dtype=torch.float64) - 0.5 * (N - 1)) * 0.25
+    live = int((torch.hypot(c.view(1, -1), c.view(-1, 1)) <= 12.0).sum())
+    y = plan.forward(x).view(B, n, n).double().cpu()
+    p = torch.arange(n) - 0.5 * (n - 1)
+    inside = torch.hypot(p.view(1, -1), p.view(-1, 1)) < 0.5 * n - 2.0  # footprints inside at every angle
+    want = live * (1.0 + 2.0 ** -15)
+    assert float((y[:, inside] / want - 1.0).abs().max()) <= 3e-6

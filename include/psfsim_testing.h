@@ -35,9 +35,10 @@ int psfsim_debug_forward_stall(psfsim_t h, const float *d_x, int B, float *d_y, 
 /* Scratch of psfsim_forward (adjoint: psfsim_adjoint) for a batch of B and a plan
  * of this shape (SPLIT_BF16, BF16 or SPLIT_BF16_SYM on a scene grid) on a device
  * of num_sms SMs: what psfsim_forward_scratch_bytes (psfsim_adjoint_scratch_bytes)
- * reports, and the most that a launch of the call takes.  Host arithmetic only: no device is needed. */
+ * reports, the most that a launch of the call takes, and the most k-tiles (64
+ * columns, or image rows) whose sums a work unit adds one after another.  Host arithmetic only: no device is needed. */
 int psfsim_debug_scratch(const double *h_radii, int n_r, int n, int N, double S, int storage, int num_sms,
-                         int adjoint, int B, size_t *reported, size_t *taken);
+                         int adjoint, int B, size_t *reported, size_t *taken, int *run);
 
 #ifdef __cplusplus
 }

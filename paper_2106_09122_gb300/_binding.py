@@ -57,7 +57,8 @@ SIGNATURES = {
     "psfsim_sync_status": (i32, [vp, vp]),
     "psfsim_reset_status": (i32, [vp, vp]),
     "psfsim_debug_forward_stall": (i32, [vp, vp, i32, vp, vp, ctypes.c_size_t, ctypes.c_uint64, i64, vp]),
-    "psfsim_debug_scratch": (i32, [vp, i32, i32, i32, f64, i32, i32, i32, i32, c_size_p, c_size_p]),
+    "psfsim_debug_scratch": (i32, [vp, i32, i32, i32, f64, i32, i32, i32, i32, c_size_p, c_size_p,
+                                   ctypes.POINTER(i32)]),
     "psfsim_ring_chain_scratch_bytes": (i32, [i32, c_size_p]),
     "psfsim_loss_scratch_bytes": (i32, [i64, c_size_p]),
     "psfsim_ring_scene": (i32, [i32, f64, f64, vp, vp, vp]),

@@ -353,8 +353,8 @@ int psfsim_debug_forward_stall(psfsim_t h, const float *d_x, int B, float *d_y, 
 }
 
 int psfsim_debug_scratch(const double *h_radii, int n_r, int n, int N, double S, int storage, int num_sms,
-                         int adjoint, int B, size_t *reported, size_t *taken) {
-  if (!reported || !taken || n < 1 || n > 4096 || N < 1 || N > 32768 || !(S > 0.0) || num_sms < 1 || B < 1)
+                         int adjoint, int B, size_t *reported, size_t *taken, int *run) {
+  if (!reported || !taken || !run || n < 1 || n > 4096 || N < 1 || N > 32768 || !(S > 0.0) || num_sms < 1 || B < 1)
     return PSFSIM_ERR_ARG;
   if (int rc = check_radii(h_radii, n_r)) return rc;
   const int64_t K = (int64_t)N * N;
@@ -376,6 +376,7 @@ int psfsim_debug_scratch(const double *h_radii, int n_r, int n, int N, double S,
   if (int rc = adjoint ? psfsim_adjoint_scratch_bytes(&p, B, reported) : psfsim_forward_scratch_bytes(&p, B, reported))
     return rc;
   *taken = psfsim_tc_taken(&p, p.quadrant ? 4 * B : B, adjoint != 0);
+  *run = psfsim_tc_run(&p, p.quadrant ? 4 * B : B, adjoint != 0);
   return PSFSIM_OK;
 }
 

@@ -92,6 +92,7 @@ cudaError_t psfsim_launch_reduce_partials(const float *part, int KS, int B, int6
 cudaError_t psfsim_launch_split_build(psfsim_plan *h, cudaStream_t st);
 size_t psfsim_forward_tc_scratch(const psfsim_plan *h, int B);  // compact storage: of B rotated scenes
 size_t psfsim_tc_taken(const psfsim_plan *h, int B, bool adjoint);  // the call's own launches
+int psfsim_tc_run(const psfsim_plan *h, int B, bool adjoint);       // most k-tiles that one unit adds up
 cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
                                      size_t scratch_bytes, cudaStream_t st);
 cudaError_t psfsim_launch_forward_tc_sym(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,

@@ -841,7 +841,8 @@ MultiPlan plan_multi(const JobSpec *jobs, int nj, const psfsim_tuning_t *tune, b
                        adjoint && any_lo ? kAdjointRun : p.k_tiles, num_sms * mp.ctas_per_sm, num_sms);
     } else {
       int ks = (int)((p.k_tiles + per_unit - 1) / (per_unit > 0 ? per_unit : 1));
-      ks = ks < 1 ? 1 : ks;
+      const int fewest = adjoint && any_lo ? (p.k_tiles + kAdjointRun - 1) / kAdjointRun : 1;
+      ks = ks < fewest ? fewest : ks;
       ks = ks > 64 ? 64 : ks;
       p.KS = ks > p.k_tiles ? p.k_tiles : ks;
     }
@@ -1186,6 +1187,17 @@ size_t psfsim_tc_taken(const psfsim_plan *h, int B, bool adjoint) {
   if (B <= kMaxLaunchScenes) return first;
   const size_t last = plan_launch(h, launch_count(B, (B - 1) / kMaxLaunchScenes), adjoint).scratch;
   return last > first ? last : first;
+}
+
+int psfsim_tc_run(const psfsim_plan *h, int B, bool adjoint) {
+  int most = 0;
+  for (int i = 0, c; (c = launch_count(B, i)) > 0; ++i) {
+    const Launch L = plan_launch(h, c, adjoint);
+    const int k = L.wide ? L.w.k_tiles : L.multi.jp[0].k_tiles, ks = L.wide ? L.w.KS : L.multi.jp[0].KS;
+    const int run = (k + ks - 1) / ks;
+    most = run > most ? run : most;
+  }
+  return most;
 }
 
 cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,

@@ -12,10 +12,11 @@ STORAGES = {"split_bf16": B.SPLIT_BF16, "bf16": B.BF16, "split_bf16_sym": B.SPLI
 
 def _scratch(n, N, storage, batch, r_last=12.0, field=32.0, num_sms=152, adjoint=0):
     radii = np.linspace(0.0, r_last, 5)
-    reported, taken = ctypes.c_size_t(), ctypes.c_size_t()
+    reported, taken, run = ctypes.c_size_t(), ctypes.c_size_t(), ctypes.c_int()
     B.check(B.load().psfsim_debug_scratch(radii.ctypes.data, 5, n, N, field / N, STORAGES[storage], num_sms, adjoint,
-                                          batch, ctypes.byref(reported), ctypes.byref(taken)), "psfsim_debug_scratch")
-    return reported.value, taken.value
+                                          batch, ctypes.byref(reported), ctypes.byref(taken), ctypes.byref(run)),
+            "psfsim_debug_scratch")
+    return reported.value, taken.value, run.value
 
 
 @pytest.mark.parametrize("storage", STORAGES)
@@ -24,7 +25,7 @@ def test_forward_scratch_holds_every_launch(storage, n):
     for N in (32, 60, 64, 96, 128, 200, 256):
         for num_sms in (148, 152):
             for batch in (1, 2, 3, 5, 10, 16, 17, 20, 21, 33, 64, 80, 81, 130, 320, 321, 336, 1280, 1281, 1340, 2480):
-                reported, taken = _scratch(n, N, storage, batch, num_sms=num_sms)
+                reported, taken, _ = _scratch(n, N, storage, batch, num_sms=num_sms)
                 assert reported >= taken, (N, num_sms, batch)
 
 
@@ -36,7 +37,7 @@ def test_adjoint_scratch_holds_every_launch(storage, n):
     for N in (20, 32, 60, 64, 66, 100, 160):
         for field, num_sms in ((32.0, 152), (32.0, 148), (16.0, 152)):
             for batch in (1, 5, 20, 21, 80, 81, 320, 321, 350, 560, 600, 640, 1280, 1281, 1300, 1400, 2240, 2480, 2560):
-                reported, taken = _scratch(n, N, storage, batch, field=field, num_sms=num_sms, adjoint=1)
+                reported, taken, _ = _scratch(n, N, storage, batch, field=field, num_sms=num_sms, adjoint=1)
                 assert reported >= taken, (N, field, num_sms, batch)
 
 
@@ -46,9 +47,17 @@ def test_scratch_for_a_batch_serves_every_smaller_one(storage, n, N):
     for adjoint in (0, 1):
         most = 0
         for batch in [*range(1, 100), 128, 129, 160, 161, 200, 256, 257, 320, 321, 400, 1280, 1281, 2480]:
-            reported, taken = _scratch(n, N, storage, batch, adjoint=adjoint)
+            reported, taken, _ = _scratch(n, N, storage, batch, adjoint=adjoint)
             assert reported >= max(most, taken), (adjoint, batch)
             most = reported
+
+
+@pytest.mark.parametrize("storage", ["split_bf16", "split_bf16_sym"])
+@pytest.mark.parametrize("n,N", [(64, 64), (128, 128), (256, 128), (256, 256), (400, 64)])
+def test_adjoint_of_split_storage_adds_short_runs_whatever_the_batch(storage, n, N):
+    """At most 160 k-tiles of 64 image rows in one FP32 chain, with one job or several."""
+    for batch in (1, 8, 16, 20, 21, 64, 80, 81, 100, 160, 161, 320, 321, 1280, 1281):
+        assert _scratch(n, N, storage, batch, adjoint=1)[2] <= 160, batch
 
 
 def _guarded(plan, product, x, need):

@@ -132,3 +132,27 @@ def test_batched_256_workload_sampled_rows():
     Yr = Y[:, torch.from_numpy(rows).to(DEV)].double().cpu().numpy()
     rel = O.bound_relative_error(Yr, X64 @ A_r.T, np.abs(X64) @ np.abs(A_r).T, floor=O.FLT_MIN)
     assert rel.max() <= 1e-5, rel.max()
+
+
+def test_small_parts_are_not_cut_at_the_last_bit_of_large_sums():
+    """lo's products next to hi's 512 times larger ones, in one accumulation of 484 columns without
+    a split: elements of 1 - 2^-16 (hi = 1, lo = -2^-16) and scene values of 8 bits (x2 = x3 = 0), so that hi x1
+    adds up exactly and one rounding of the sum of both blocks is left, 2^-24; the stored elements
+    are read back.  Cut at the sum's last bit, 32 additions of lo lose 1e-6."""
+    from paper_2106_09122_gb300 import Plan
+    from paper_2106_09122_gb300.serve import MultiForward
+    n, N, B = 256, 22, 4
+    lib = torch.full((2, n, n), 1.0 - 2.0 ** -16, device=DEV)
+    plan = Plan(lib, np.array([0.0, 12.0]), 0.125, N=N, S=0.25, storage="split_bf16")
+    x = 1.0 + torch.from_numpy(np.random.default_rng(8).integers(0, 128, (B, N * N)).astype(np.float32)) / 128.0
+    mf = MultiForward([plan], [B], tuning=(8, 1, 0))
+    mf.x[0].copy_(x)
+    mf.count.fill_(B)
+    mf.enqueue()
+    hi, lo, scale = plan.A_split()
+    A = (hi[:plan.M, :plan.K].double() + lo[:plan.M, :plan.K].double()) * scale[:plan.K].double()
+    want = (x.to(DEV).double() @ A.t()).view(B, n, n).cpu()
+    p = torch.arange(n) - 0.5 * (n - 1)
+    inside = torch.hypot(p.view(1, -1), p.view(-1, 1)) < 0.5 * n - 2.0  # footprints inside at every angle
+    err = (mf.y[0].view(B, n, n).double().cpu() / want - 1.0)[:, inside].abs().max()
+    assert plan.sync_status() == 0 and float(err) <= 2.0 ** -23

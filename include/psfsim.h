@@ -100,9 +100,11 @@ const char *psfsim_status_string(int status);
  * applied to K columns (K = N*N for a scene grid) with the given storage.
  * SPLIT_BF16 and BF16 grids of even N that build faster from pair entries of
  * the library (32 bytes per bracket and pixel) get room for them; a workspace
- * without that room is accepted too, and its A is the same.
+ * of psfsim_workspace_min_bytes, without that room, is accepted too, and its A
+ * is the same.
  * Sec. 3: A has n^2 rows and N^2 columns.  Returns PSFSIM_ERR_ARG for bad sizes. */
 int psfsim_workspace_bytes(int n, int n_r, int64_t K, int storage, size_t *bytes);
+int psfsim_workspace_min_bytes(int n, int n_r, int64_t K, int storage, size_t *bytes);
 
 /* Build the interpolated PSF library A for a scene grid (Sec. 2, the loop over
  * all N^2 scene pixels; Eq. 4-5).
@@ -124,6 +126,16 @@ int psfsim_workspace_bytes(int n, int n_r, int64_t K, int storage, size_t *bytes
 int psfsim_build(const float *d_lib, const double *h_radii, int n_r, int n, double s,
                  int N, double S, int storage, int interp, void *d_workspace,
                  size_t workspace_bytes, void *stream, psfsim_t *out);
+
+/* psfsim_build with the pair entries (see psfsim_workspace_bytes) in a buffer of
+ * their own, for plans that should not hold them: d_tables, 256-byte aligned, of
+ * psfsim_workspace_bytes - psfsim_workspace_min_bytes bytes, is the caller's
+ * again once the stream has passed the build.  With NULL or fewer bytes the
+ * workspace serves if it has the room, else the build does without. */
+int psfsim_build_with_tables(const float *d_lib, const double *h_radii, int n_r, int n, double s,
+                             int N, double S, int storage, int interp, void *d_workspace,
+                             size_t workspace_bytes, void *d_tables, size_t tables_bytes, void *stream,
+                             psfsim_t *out);
 
 /* Same as psfsim_build for K arbitrary field points h_xy (host double [K][2],
  * (x, y) in lambda/D) instead of a scene grid; column j is the interpolated,

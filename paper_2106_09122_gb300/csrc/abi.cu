@@ -59,7 +59,7 @@ void fill_shape(psfsim_plan *h, const WsLayout &L, const double *h_radii, int n_
 
 int common_build(const float *d_lib, const double *h_radii, int n_r, int n, double s, int N, double S,
                  const double *h_xy, int64_t K, int storage, int interp, void *d_ws, size_t ws_bytes,
-                 void *stream, psfsim_t *out) {
+                 void *d_tables, size_t tables_bytes, void *stream, psfsim_t *out) {
   if (!out) return PSFSIM_ERR_ARG;
   *out = nullptr;
   if (!d_lib || !d_ws || n < 1 || n > 4096 || K < 1 || K > (int64_t)1 << 30) return PSFSIM_ERR_ARG;
@@ -70,7 +70,7 @@ int common_build(const float *d_lib, const double *h_radii, int n_r, int n, doub
   const bool quadrant = storage == PSFSIM_FUSED || storage == PSFSIM_FP32_SYM || storage == PSFSIM_SPLIT_BF16_SYM;
   if (quadrant && (h_xy || N < 2 || (N & 1))) return PSFSIM_ERR_UNSUPPORTED;
   const WsLayout L = psfsim_layout(n, K, storage, n_r);
-  if (!aligned(d_ws, 256) || ws_bytes < (size_t)L.total) return PSFSIM_ERR_WORKSPACE;
+  if (!aligned(d_ws, 256) || ws_bytes < (size_t)L.total || !aligned(d_tables, 256)) return PSFSIM_ERR_WORKSPACE;
 
   psfsim_plan *h = new (std::nothrow) psfsim_plan;
   if (!h) return PSFSIM_ERR_ARG;
@@ -78,8 +78,12 @@ int common_build(const float *d_lib, const double *h_radii, int n_r, int n, doub
   h->d_lib = d_lib;
   h->ws = static_cast<char *>(d_ws);
   h->ws_bytes = ws_bytes;
-  // A workspace of the plain layout's size (or a field-point build) does without the pixel-wise build's tables.
-  h->pix_off = N > 0 && ws_bytes >= (size_t)L.total_pix ? L.pix_off : -1;
+  // Without room for the pixel-wise build's tables (or for field points) another build runs.
+  const size_t extra = (size_t)(L.total_pix - L.total);
+  if (N > 0 && L.pix_off >= 0)
+    h->pix = d_tables && tables_bytes >= extra            ? static_cast<char *>(d_tables)
+             : ws_bytes >= (size_t)L.total_pix ? h->ws + L.pix_off
+                                               : nullptr;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int rc = PSFSIM_OK;
   if (cudaGetDevice(&h->device) != cudaSuccess ||
@@ -96,6 +100,7 @@ int common_build(const float *d_lib, const double *h_radii, int n_r, int n, doub
     delete h;
     return rc;
   }
+  h->pix = nullptr;  // the caller's again once the build has run
   *out = h;
   return PSFSIM_OK;
 }
@@ -125,15 +130,28 @@ int psfsim_workspace_bytes(int n, int n_r, int64_t K, int storage, size_t *bytes
   return PSFSIM_OK;
 }
 
+int psfsim_workspace_min_bytes(int n, int n_r, int64_t K, int storage, size_t *bytes) {
+  if (int rc = psfsim_workspace_bytes(n, n_r, K, storage, bytes)) return rc;
+  *bytes = (size_t)psfsim_layout(n, K, storage, n_r).total;
+  return PSFSIM_OK;
+}
+
 int psfsim_build(const float *d_lib, const double *h_radii, int n_r, int n, double s, int N, double S,
                  int storage, int interp, void *d_workspace, size_t workspace_bytes, void *stream,
                  psfsim_t *out) {
+  return psfsim_build_with_tables(d_lib, h_radii, n_r, n, s, N, S, storage, interp, d_workspace, workspace_bytes, nullptr,
+                                  0, stream, out);
+}
+
+int psfsim_build_with_tables(const float *d_lib, const double *h_radii, int n_r, int n, double s, int N, double S,
+                             int storage, int interp, void *d_workspace, size_t workspace_bytes, void *d_tables,
+                             size_t tables_bytes, void *stream, psfsim_t *out) {
   if (N < 1 || N > 32768 || !(S > 0.0) || !std::isfinite(S)) {
     if (out) *out = nullptr;
     return PSFSIM_ERR_ARG;
   }
   return common_build(d_lib, h_radii, n_r, n, s, N, S, nullptr, (int64_t)N * N, storage, interp, d_workspace,
-                      workspace_bytes, stream, out);
+                      workspace_bytes, d_tables, tables_bytes, stream, out);
 }
 
 int psfsim_build_points(const float *d_lib, const double *h_radii, int n_r, int n, double s, const double *h_xy,
@@ -149,7 +167,7 @@ int psfsim_build_points(const float *d_lib, const double *h_radii, int n_r, int 
       return PSFSIM_ERR_ARG;
     }
   return common_build(d_lib, h_radii, n_r, n, s, 0, 0.0, h_xy, K, storage, interp, d_workspace, workspace_bytes,
-                      stream, out);
+                      nullptr, 0, stream, out);
 }
 
 int psfsim_info(psfsim_t h, psfsim_info_t *info) {

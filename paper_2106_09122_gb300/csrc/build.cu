@@ -702,7 +702,7 @@ static cudaError_t launch_tables_and_build(psfsim_plan *h, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   geom_kernel<<<(unsigned)((Kg + 255) / 256), 256, 0, st>>>(G, geom);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (!dense_split || (sym && h->pix_off >= 0)) {
+  if (!dense_split || (sym && h->pix)) {
     // chunks of at least 256 columns, and as many as fit in shared memory
     const int nb = psfsim_num_buckets(h->n_r);
     int W = (int)((Kg + 255) / 256);

@@ -40,7 +40,7 @@ struct psfsim_plan {
   size_t ws_bytes;
   int64_t a_off, lo_off, scale_off, geom_off, order_off, bstart_off, pts_off, status_off, libmax_off, plib_off,
       cols_off, mtorder_off;
-  int64_t pix_off;  // split storage: pair entries and pixel order of the pixel-wise build (-1: another build)
+  char *pix;  // split storage, during the build: pair entries and pixel order of the pixel-wise build (NULL: another build)
   int device, num_sms;
   bool live;            // products skip the zero columns listed in the workspace (live.cu)
   int64_t live_cols;    // FP32 storage: columns the products read (all of them when !live)

@@ -697,8 +697,8 @@ cudaError_t psfsim_launch_split_build(psfsim_plan *h, cudaStream_t st) {
           (e = cudaMemset2DAsync(a + P.K, row_bytes, 0, (size_t)(P.ld - P.K) * 2, (size_t)P.M, st)) != cudaSuccess)
         return e;
     }
-    if (h->pix_off >= 0) {
-      char *pix = h->ws + h->pix_off;
+    if (h->pix) {
+      char *pix = h->pix;
       float *entries = reinterpret_cast<float *>(pix);
       int *pair_order = reinterpret_cast<int *>(pix + psfsim_round_up(psfsim_pair_library_bytes(h->n, h->n_r), 256));
       // the quadrant's geometry leaves three quarters of its table free

@@ -60,8 +60,29 @@ class Plan:
         else:
             K = int(N) * int(N)
         self.K, self.M = K, self.n * self.n
-        ws = workspace_bytes(self.n, self.n_r, K, storage)
-        self.workspace = torch.empty(ws, dtype=torch.uint8, device=lib.device)
+        least = ctypes.c_size_t()
+        B.check(self._lib.psfsim_workspace_min_bytes(self.n, self.n_r, K, _STORAGE[storage], ctypes.byref(least)),
+                "workspace_min_bytes")
+        ws, tables = least.value, None
+        extra = workspace_bytes(self.n, self.n_r, K, storage) - ws if points is None else 0
+        # What only the build reads stays in the workspace where it is small, else in a buffer that
+        # goes back to the allocator; without memory for it A is built without (the same A).
+        if extra and 16 * extra <= ws:
+            ws += extra
+        elif extra:
+            try:
+                tables = torch.empty(extra, dtype=torch.uint8, device=lib.device)
+                if stream is not None:
+                    tables.record_stream(stream)
+            except torch.cuda.OutOfMemoryError:
+                pass
+        try:
+            self.workspace = torch.empty(ws, dtype=torch.uint8, device=lib.device)
+        except torch.cuda.OutOfMemoryError:
+            if ws == least.value and tables is None:
+                raise
+            ws, tables = least.value, None
+            self.workspace = torch.empty(ws, dtype=torch.uint8, device=lib.device)
         h = ctypes.c_void_p()
         rp = self.radii.ctypes.data_as(ctypes.c_void_p)
         if points is not None:
@@ -70,9 +91,10 @@ class Plan:
                 pts.ctypes.data_as(ctypes.c_void_p), K, _STORAGE[storage], _INTERP[interp],
                 ctypes.c_void_p(self.workspace.data_ptr()), ws, _stream_ptr(stream), ctypes.byref(h))
         else:
-            rc = self._lib.psfsim_build(
+            rc = self._lib.psfsim_build_with_tables(
                 ctypes.c_void_p(lib.data_ptr()), rp, self.n_r, self.n, float(s), int(N), float(S),
                 _STORAGE[storage], _INTERP[interp], ctypes.c_void_p(self.workspace.data_ptr()), ws,
+                None if tables is None else tables.data_ptr(), 0 if tables is None else extra,
                 _stream_ptr(stream), ctypes.byref(h))
         B.check(rc, "psfsim_build")
         self.handle = h

@@ -103,3 +103,18 @@ def test_status_and_testing_hooks_reject_null_handles(lib):
     assert lib.psfsim_reset_status(None, None) == B.ERR_ARG
     assert lib.psfsim_sync_status(None, None) == B.ERR_ARG
     assert lib.psfsim_debug_forward_stall(None, None, 1, None, None, 0, 1_000_000, 0, None) == B.ERR_ARG
+
+
+def test_smallest_workspace_is_the_layout_without_the_builds_tables(lib):
+    least, full = ctypes.c_size_t(), ctypes.c_size_t()
+    for storage in (B.FP32, B.SPLIT_BF16, B.BF16, B.FUSED, B.FP32_SYM, B.SPLIT_BF16_SYM):
+        for n, N, n_r in ((128, 64, 60), (33, 66, 4), (64, 63, 20), (100, 20, 5)):
+            assert lib.psfsim_workspace_min_bytes(n, n_r, N * N, storage, ctypes.byref(least)) == B.OK
+            assert lib.psfsim_workspace_bytes(n, n_r, N * N, storage, ctypes.byref(full)) == B.OK
+            tables = storage in (B.SPLIT_BF16, B.BF16) and N in (64, 66)
+            assert (least.value < full.value) if tables else (least.value == full.value)
+    assert lib.psfsim_workspace_min_bytes(0, 4, 10, B.FP32, ctypes.byref(least)) == B.ERR_ARG
+    r = np.array([0.0, 1.0, 2.0])
+    h = ctypes.c_void_p()
+    assert lib.psfsim_build_with_tables(0x1000, r.ctypes.data, 3, 16, 0.5, 8, 0.5, B.SPLIT_BF16, B.LINEAR, 0x100000, 1 << 40,
+                                        0x100010, 1 << 20, None, ctypes.byref(h)) == B.ERR_WORKSPACE  # tables misaligned

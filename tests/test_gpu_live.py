@@ -230,3 +230,42 @@ def test_sum_over_splits_of_many_rows(n):
         out.append(mf.y[0].double().cpu())
     assert plan.sync_status() == 0
     assert torch.all((out[0] - out[1]).abs() <= 2e-5 * out[0])
+
+
+@pytest.mark.parametrize("n,N,n_r,held", [(128, 64, 60, False), (33, 66, 4, True)])
+@pytest.mark.parametrize("storage", ["split_bf16", "bf16"])
+def test_plan_holds_no_large_tables_and_builds_without_memory_for_them(n, N, n_r, held, storage, monkeypatch):
+    """What only the build reads is held where it is small beside A, else given back; when there is
+    no memory for it the same A comes out."""
+    import ctypes
+    from paper_2106_09122_gb300 import Plan, workspace_bytes
+    from paper_2106_09122_gb300 import _binding as B
+    radii, S = np.linspace(0.0, 5.0, n_r), 8.0 / N
+    lib = torch.from_numpy(np.random.default_rng(3).uniform(0.0, 1.0, (n_r, n, n)).astype(np.float32)).to(DEV)
+    code = B.SPLIT_BF16 if storage == "split_bf16" else B.BF16
+    least, L = ctypes.c_size_t(), B.load()
+    B.check(L.psfsim_workspace_min_bytes(n, n_r, N * N, code, ctypes.byref(least)), "workspace_min_bytes")
+    full = workspace_bytes(n, n_r, N * N, storage)
+    assert full > least.value
+    plan = Plan(lib, radii, 0.25, N=N, S=S, storage=storage)
+    assert plan.workspace.numel() == (full if held else least.value)
+    end = plan.info.scale_offset + 4 * plan.info.ld
+    ws, h = torch.zeros(full, dtype=torch.uint8, device=DEV), ctypes.c_void_p()
+    B.check(L.psfsim_build(lib.data_ptr(), radii.ctypes.data, n_r, n, 0.25, N, S, code, B.LINEAR, ws.data_ptr(), full, None,
+                           ctypes.byref(h)), "psfsim_build")
+    torch.cuda.synchronize()
+    assert torch.equal(ws[:end], plan.workspace[:end])
+    L.psfsim_free(h)
+    real, refused = torch.empty, []
+
+    def empty(size, *args, **kw):
+        if size == (full if held else full - least.value):
+            refused.append(size)
+            raise torch.cuda.OutOfMemoryError("no memory")
+        return real(size, *args, **kw)
+
+    monkeypatch.setattr(torch, "empty", empty)
+    small = Plan(lib, radii, 0.25, N=N, S=S, storage=storage)
+    monkeypatch.undo()
+    assert refused and small.workspace.numel() == least.value
+    assert torch.equal(small.workspace[:end], plan.workspace[:end]) and small.sync_status() == 0

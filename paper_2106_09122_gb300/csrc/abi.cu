@@ -350,7 +350,7 @@ int psfsim_reset_status(psfsim_t h, void *stream) {
 
 int psfsim_debug_forward_stall(psfsim_t h, const float *d_x, int B, float *d_y, void *d_scratch,
                                size_t scratch_bytes, uint64_t wait_ns, int64_t stall_load, void *stream) {
-  if (!h || !d_x || !d_y || B < 1 || B > 80) return PSFSIM_ERR_ARG;
+  if (!h || !d_x || !d_y || B < 1) return PSFSIM_ERR_ARG;
   if (wait_ns < 1000 || wait_ns > 2000000000ull || stall_load < -1) return PSFSIM_ERR_ARG;
   if (h->storage == PSFSIM_FUSED) {
     if (B > 64) return PSFSIM_ERR_ARG;
@@ -362,9 +362,10 @@ int psfsim_debug_forward_stall(psfsim_t h, const float *d_x, int B, float *d_y, 
                : PSFSIM_ERR_CUDA;
   }
   if (h->storage != PSFSIM_SPLIT_BF16 && h->storage != PSFSIM_BF16) return PSFSIM_ERR_UNSUPPORTED;
+  if (!psfsim_forward_tc_one_launch(h, B)) return PSFSIM_ERR_ARG;
   const size_t need = psfsim_tc_taken(h, B, false);
   if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
-  return psfsim_launch_forward_tc_stall(h, d_x, B, d_y, d_scratch, wait_ns, stall_load,
+  return psfsim_launch_forward_tc_stall(h, d_x, B, d_y, d_scratch, scratch_bytes, wait_ns, stall_load,
                                         static_cast<cudaStream_t>(stream)) == cudaSuccess
              ? PSFSIM_OK
              : PSFSIM_ERR_CUDA;

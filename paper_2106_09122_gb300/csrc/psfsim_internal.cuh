@@ -111,10 +111,11 @@ cudaError_t psfsim_launch_sym_sum(SymSum S, int B, float *y, cudaStream_t st);
 size_t psfsim_adjoint_tc_scratch(const psfsim_plan *h, int B);  // compact storage: of B turned residuals
 cudaError_t psfsim_launch_adjoint_tc(const psfsim_plan *h, const float *g, int B, float *gx, void *scratch,
                                      size_t scratch_bytes, cudaStream_t st);
-// Test hook: the tensor-core forward of <= 80 scenes on one CTA with every
-// wait bounded by wait_ns and load number stall_it never issued.
+// Test hook: a tensor-core forward of one job, or of the wide form, on one CTA with
+// every wait bounded by wait_ns and load number stall_it never issued.
+bool psfsim_forward_tc_one_launch(const psfsim_plan *h, int B);
 cudaError_t psfsim_launch_forward_tc_stall(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
-                                           uint64_t wait_ns, int64_t stall_it, cudaStream_t st);
+                                           size_t scratch_bytes, uint64_t wait_ns, int64_t stall_it, cudaStream_t st);
 // Multi-job persistent tensor-core forward (several split-BF16 plans, one launch).
 int psfsim_multi_validate(const psfsim_job_t *jobs, int njobs);
 size_t psfsim_forward_multi_scratch(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune);

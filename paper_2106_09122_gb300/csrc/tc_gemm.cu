@@ -548,6 +548,7 @@ struct TcWide {
   int64_t out_ld, out_rows;
   int *status;
   uint64_t wait_ns;
+  int64_t stall_it;  // test hook: the producer never issues this load (-1: none)
 };
 
 __global__ void __launch_bounds__(kWideThreads, 1) tc_wide_kernel(const __grid_constant__ TcWide P) {
@@ -602,6 +603,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) tc_wide_kernel(const __grid_c
           ok = false;
           break;
         }
+        if ((int64_t)it == P.stall_it) continue;  // test hook: this stage is never filled
         uint8_t *st = smem + (size_t)s * stage_bytes;
         ptx::mbar_arrive_expect_tx(&full_bar[s], tx);
         ptx::tma_load_2d(st + a_off, &P.hi, col, nt * kWidePix, &full_bar[s]);
@@ -612,7 +614,8 @@ __global__ void __launch_bounds__(kWideThreads, 1) tc_wide_kernel(const __grid_c
     }
     // Drain: the last loads issued may not have been consumed (as in tc_gemm_kernel).
     for (uint32_t i = it > (uint32_t)kWideStages ? it - (uint32_t)kWideStages : 0u; i < it; ++i)
-      if (!ptx::mbar_wait_bounded(&full_bar[i % kWideStages], (i / kWideStages) & 1, lim)) set_abort(&abort_flag, P.status);
+      if ((int64_t)i != P.stall_it && !ptx::mbar_wait_bounded(&full_bar[i % kWideStages], (i / kWideStages) & 1, lim))
+        set_abort(&abort_flag, P.status);
   } else if (warp == 1 && lane == 0) {
     // ---------------- MMA issuer ----------------
     uint32_t it = 0;
@@ -1083,7 +1086,7 @@ WidePlan plan_wide(const psfsim_plan *h, int scenes) {
 // Partial images part[KS][scenes][rows] in the scratch; compact storage: x holds
 // whole scenes and the batch is their rotations.
 cudaError_t launch_wide(const psfsim_plan *h, const float *x, int scenes, const WidePlan &w, void *scratch,
-                        cudaStream_t st) {
+                        cudaStream_t st, const StallHook &hook = kNoStall) {
   __nv_bfloat16 *xs = static_cast<__nv_bfloat16 *>(scratch);
   const int *tab = reinterpret_cast<const int *>(h->ws + h->order_off);
   XMulti XP;
@@ -1122,11 +1125,13 @@ cudaError_t launch_wide(const psfsim_plan *h, const float *x, int scenes, const 
   P.out = reinterpret_cast<float *>(static_cast<char *>(scratch) + w.part_off);
   P.out_ld = P.out_rows = w.rows;
   P.status = reinterpret_cast<int *>(h->ws + h->status_off);
-  P.wait_ns = kNoStall.wait_ns;
+  P.wait_ns = hook.wait_ns;
+  P.stall_it = hook.stall_it;
   const size_t smem = kWideStages * (3 * kWideX + 2 * kWideA) + 1024;
   if ((e = cudaFuncSetAttribute(tc_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
     return e;
-  tc_wide_kernel<<<P.units < h->num_sms ? P.units : h->num_sms, kWideThreads, smem, st>>>(P);
+  const int slots = hook.one_cta ? 1 : h->num_sms;
+  tc_wide_kernel<<<P.units < slots ? P.units : slots, kWideThreads, smem, st>>>(P);
   return cudaGetLastError();
 }
 
@@ -1206,8 +1211,8 @@ int psfsim_tc_run(const psfsim_plan *h, int B, bool adjoint) {
   return most;
 }
 
-cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
-                                     size_t scratch_bytes, cudaStream_t st) {
+static cudaError_t launch_forward(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
+                                  size_t scratch_bytes, cudaStream_t st, const StallHook &hook) {
   for (int i = 0, c; (c = launch_count(B, i)) > 0; ++i) {
     Launch L = plan_launch(h, c, false);
     if (L.scratch > scratch_bytes) return cudaErrorInvalidValue;
@@ -1215,7 +1220,7 @@ cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B
     float *yb = y + (int64_t)i * kMaxLaunchScenes * h->M;
     cudaError_t e;
     if (L.wide) {
-      if ((e = launch_wide(h, xb, c, L.w, scratch, st)) != cudaSuccess) return e;
+      if ((e = launch_wide(h, xb, c, L.w, scratch, st, hook)) != cudaSuccess) return e;
       e = psfsim_launch_reduce_partials(reinterpret_cast<const float *>(static_cast<char *>(scratch) + L.w.part_off),
                                         L.w.KS, c, L.w.rows, h->M, yb, st);
     } else {
@@ -1223,11 +1228,16 @@ cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B
         L.js[j].x = xb + (int64_t)j * kMaxBp * h->K;
         L.js[j].y = yb + (int64_t)j * kMaxBp * h->M;
       }
-      e = launch_multi(L.js, L.nj, L.multi, scratch, st);
+      e = launch_multi(L.js, L.nj, L.multi, scratch, st, hook);
     }
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+
+cudaError_t psfsim_launch_forward_tc(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
+                                     size_t scratch_bytes, cudaStream_t st) {
+  return launch_forward(h, x, B, y, scratch, scratch_bytes, st, kNoStall);
 }
 
 // Compact split storage: the four rotations of up to kMaxLaunchScenes / 4
@@ -1356,13 +1366,12 @@ cudaError_t psfsim_launch_forward_multi(const psfsim_job_t *jobs, int njobs, con
   return launch_multi(js, njobs, plan_multi(js, njobs, tune), scratch, st);
 }
 
+bool psfsim_forward_tc_one_launch(const psfsim_plan *h, int B) {
+  return B <= kMaxBp || (B <= kMaxLaunchScenes && wide_form(h, B));
+}
+
 cudaError_t psfsim_launch_forward_tc_stall(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
-                                           uint64_t wait_ns, int64_t stall_it, cudaStream_t st) {
-  JobSpec js[kMaxJobs];
-  const int nj = tc_jobs(h, B, js);
-  if (nj != 1) return cudaErrorInvalidValue;
-  js[0].x = x;
-  js[0].y = y;
+                                           size_t scratch_bytes, uint64_t wait_ns, int64_t stall_it, cudaStream_t st) {
   const StallHook hook = {wait_ns, stall_it, true};
-  return launch_multi(js, nj, plan_multi(js, nj, nullptr), scratch, st, hook);
+  return launch_forward(h, x, B, y, scratch, scratch_bytes, st, hook);
 }

@@ -158,3 +158,66 @@ def test_fused_stall_hook_rejects_batches_beyond_one_launch():
     scr = torch.empty(plan.forward_scratch_bytes(65), dtype=torch.uint8, device=DEV)
     assert _stall(plan, x, y, scr, 1_000_000, 0) == B.ERR_ARG
     plan.free()
+
+
+def _wide_plan(storage, scenes):
+    """More than 80 scenes, in the form with scenes as the product's rows."""
+    from paper_2106_09122_gb300 import Plan
+    rng = np.random.default_rng(505)
+    n, N, S = 40, 32, 0.3
+    radii = np.linspace(0.0, 4.5, 12)
+    lib32 = rng.uniform(0.0, 1.0, (12, n, n)).astype(np.float32)
+    plan = Plan(torch.from_numpy(lib32).to(DEV), radii, 0.5, N=N, S=S, storage=storage)
+    A = O.build_A(lib32.astype(np.float64), radii, N, S)
+    return plan, A, rng.uniform(0.0, 1.0, (scenes, N * N)).astype(np.float32)
+
+
+def _check_wide(y, A, x, storage):
+    x64 = x.astype(np.float64)
+    rel = O.bound_relative_error(y.astype(np.float64), x64 @ A.T, np.abs(x64) @ np.abs(A).T, floor=O.FLT_MIN)
+    assert rel.max() <= (1e-5 if storage == "split_bf16" else 2.0 ** -8 + 2.5e-5), rel.max()
+
+
+@pytest.mark.parametrize("storage,scenes", [("split_bf16", 90), ("bf16", 130)])
+@pytest.mark.parametrize("stall_load", [0, 1, 5])
+def test_wide_wait_that_runs_out_reports_timeout_and_leaves_the_plan_usable(storage, scenes, stall_load):
+    from paper_2106_09122_gb300 import _binding as B
+    plan, A, x_np = _wide_plan(storage, scenes)
+    x = torch.from_numpy(x_np).to(DEV)
+    y = torch.zeros((scenes, plan.M), device=DEV)
+    scr = torch.empty(plan.forward_scratch_bytes(scenes), dtype=torch.uint8, device=DEV)
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    assert _stall(plan, x, y, scr, 1_000_000, stall_load) == B.OK
+    assert plan.sync_status() == B.ERR_TIMEOUT
+    assert time.perf_counter() - t0 < 1.5
+    assert plan._lib.psfsim_reset_status(plan.handle, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)) == B.OK
+    assert plan.sync_status() == B.OK
+    y2 = plan.forward(x)
+    assert plan.sync_status() == B.OK
+    _check_wide(y2.cpu().numpy(), A, x_np, storage)
+    plan.free()
+
+
+@pytest.mark.parametrize("storage,scenes", [("split_bf16", 90), ("bf16", 130)])
+def test_wide_stall_hook_without_a_stall_is_a_correct_one_cta_forward(storage, scenes):
+    from paper_2106_09122_gb300 import _binding as B
+    plan, A, x_np = _wide_plan(storage, scenes)
+    x = torch.from_numpy(x_np).to(DEV)
+    y = torch.full((scenes, plan.M), float("nan"), device=DEV)
+    scr = torch.empty(plan.forward_scratch_bytes(scenes), dtype=torch.uint8, device=DEV)
+    assert _stall(plan, x, y, scr, 1_000_000_000, -1) == B.OK
+    assert plan.sync_status() == B.OK
+    _check_wide(y.cpu().numpy(), A, x_np, storage)
+    plan.free()
+
+
+def test_stall_hook_rejects_batches_of_several_launches():
+    from paper_2106_09122_gb300 import _binding as B
+    plan, _, _ = _wide_plan("split_bf16", 1)
+    for scenes in (160, 1281):  # two interleaved jobs; two launches
+        x = torch.zeros((scenes, plan.K), device=DEV)
+        y = torch.zeros((scenes, plan.M), device=DEV)
+        scr = torch.empty(plan.forward_scratch_bytes(scenes), dtype=torch.uint8, device=DEV)
+        assert _stall(plan, x, y, scr, 1_000_000, 0) == B.ERR_ARG
+    plan.free()

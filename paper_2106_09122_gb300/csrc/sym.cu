@@ -128,9 +128,9 @@ int sym_splits(const psfsim_plan *h) {
 
 }  // namespace
 
-// Several k-splits are added first, in place, by the reduction that spreads them
-// over a CTA's warps: 28 splits of one image's four rotations (16 CTAs here) took
-// 60 us in this kernel's own loop, which keeps at most two.
+// Several k-splits are added first, in place, by the reduction (reduce.cuh): 28
+// splits of one image's four rotations (16 CTAs here) took 60 us in this kernel's
+// own loop, which keeps at most two.
 cudaError_t psfsim_launch_sym_sum(SymSum S, int B, float *y, cudaStream_t st) {
   for (int blk = 0; blk * S.per < 4 * B; ++blk)
     if (S.KS[blk] > 2) {

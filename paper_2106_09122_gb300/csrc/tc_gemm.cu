@@ -61,23 +61,22 @@ constexpr int kMaxBp = 80;       // 3 * Bp <= 256 (MMA N and TMA box limits), Bp
 constexpr int kMaxJobs = 16;
 constexpr int kDefaultChunk = 4; // k-tiles (of 64) per TMEM accumulation, split-BF16 storage
 // One job of split storage: fewer splits sum longer runs (choose_ks), and draining
-// more often pays that back without costing time: 16 scenes of 128^2 take 141 us at
-// 4, 2 and 1 k-tiles, their error is 3.9e-7, 2.1e-7 and 1.5e-7.  Accumulators of
-// more than 128 columns are drained slower than they fill: 64 scenes take 149 us
-// at 4 and 3, 155 at 2, 173 at 1.
+// more often pays that back without costing time: 16 scenes of 128^2 take 142 us at
+// 4, 2 and 1 k-tiles, and their product errs 4.2e-7, 2.5e-7 and 1.7e-7 (against the
+// stored A in 64 bits).  Accumulators of more than 128 columns are drained slower
+// than they fill: 64 scenes take 156 us at 4 and 3, 159 at 2, 176 at 1.
 constexpr int kSingleChunk = 1, kSingleChunkWide = 3;
 constexpr int kDefaultChunkHiMulti = 2;  // BF16 storage (hi alone), several jobs in one launch
 // Adjoint of split storage: residuals change sign, so its sums cancel and the
-// drift weighs more (error against 64 bits 2.493e-6 with plain FP32 sums, 2.553
-// at 4 k-tiles, 2.492 at one; 8 residuals of 128^2 took 127 and 129 us, 119 since
-// choose_ks; 64 of 256^2 1.45 and 1.64 ms).
+// drift weighs more: 8 residuals of 128^2 err 2.537e-6 against 64 bits with plain
+// FP32 sums, 2.552 at 4 k-tiles, 2.537 at one; 124 us a call either way (8 of 256^2
+// 1.50 and 1.51 ms).
 constexpr int kAdjointChunk = 1;
-constexpr int kAdjointRun = 160;  // and the most k-tiles a unit adds up
+constexpr int kAdjointRun = 160;  // and the most k-tiles a unit adds up, with one job or several
 constexpr int kMaxMmas = 64;     // accumulating MMAs between drains (bounds the FP32 drift)
 
 // One product S_j = A_j Z_j of a (possibly multi-job) launch.
 struct TcJob {
-  int64_t rows, M;
   int Bp, KS, m_tiles, k_tiles;
   int tiles, ld;       // adjoint: 64-column tiles of A (ktab's), and A's row pitch
   int has_lo;          // split-BF16 (hi + lo) or BF16 (hi alone)
@@ -770,8 +769,8 @@ struct JobPlan {
 // plan on 85^2 pixels ran 1817 units in 43 us, 237 in 37; 64 of a 256^2 one on
 // 64^2 pixels took 121 us in three splits, 78 in one.  At most `most` k-tiles a
 // unit: the drained sums add up one after another in FP32, and the adjoint of
-// 256^2 split storage erred 2 % more with its 1024 in one chain than in runs of
-// 146 (kAdjointRun; 1.32 ms, 1.30 in one).
+// 256^2 split storage errs 2 % more with its 1024 in one chain than in runs of
+// 146 (kAdjointRun; 8 residuals 1.51 ms, 1.45 in one).
 int choose_ks(const JobPlan &p, int cap, int x_rows, bool lo, bool direct1, int most, int slots,
               int num_sms) {
   const double a_bytes = lo ? 2.0 * kTileBytes : kTileBytes, x_bytes = x_rows * BK * 2.0;
@@ -949,8 +948,6 @@ cudaError_t launch_multi(const JobSpec *jobs, int nj, const MultiPlan &mp, void 
     J.xparts = xparts;
     J.tiles = h->k_tiles;
     J.ld = (int)h->ld;
-    J.rows = p.rows;
-    J.M = h->M;
     J.Bp = p.Bp;
     J.KS = p.KS;
     J.m_tiles = p.m_tiles;

@@ -583,7 +583,7 @@ def _entry_fit128(dev, stream, with_oracle, steps=1000):
     out = {"workload": "adjoint_fit_128: 40 PSFs 128^2 at 0.25 lambda/D, A 16384^2 FP32 (1.07 GB); step = one fit "
                        "gradient in two launches",
            "images_per_s": 1e3 / step_ms, "ms_per_step": step_ms,
-           "gmac_per_s": 2 * w.M * w.K / (step_ms / 1e3) / 1e9,
+           "gmac_per_s": 2 * w.M * _live(w.N, w.S, w.radii) / (step_ms / 1e3) / 1e9,
            "kernels_ms": {"forward_loss": fwd_ms, "adjoint_chain": adj_ms},
            "build_ms": build_ms, "build_roofline": _build_roofline(4 * w.M * w.K, build_ms, _peaks()["hbm"]),
            "roofline": {"bound": "hbm", "achieved": adj_bytes / (adj_ms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
@@ -648,7 +648,7 @@ def _path_batched(dev, stream, hbm, with_oracle):
                        "8 x A 65536^2 split-BF16 (137 GB) in one launch",
            "images_per_s": nl * B / (ms / 1e3), "ms_per_batch": ms, "build_ms_per_wavelength": build_ms,
            "build_roofline": _build_roofline(4 * w.M * w.K, build_ms, hbm),
-           "gmac_per_s": nl * B * w.M * w.K / (ms / 1e3) / 1e9,
+           "gmac_per_s": nl * B * w.M * live / (ms / 1e3) / 1e9,
            "roofline": {"bound": "hbm", "achieved": a_bytes / (ms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
                         "frac": a_bytes / (ms / 1e3) / 1e9 / hbm, "kernel": "tc_gemm_kernel, 8 jobs (+ split, reduce)",
                         "traffic": None,
@@ -806,11 +806,9 @@ def _path_split_sym(dev, stream, hbm, with_oracle):
     kst = plans[0].info.K_stored
     ld = plans[0].info.ld
     rows = (w.M + 127) // 128 * 128
-    # the 4B = 256 rotated scenes run as interleaved jobs of at most 80 (padded to 16) against
-    # one A: per job, MMAs of N = 3 Bp (hi) and 2 Bp (lo) over every (row, column) of A
-    jobs = [min(80, 4 * B - b0) for b0 in range(0, 4 * B, 80)]
-    bps = [-(-c // 16) * 16 for c in jobs]
-    tc_flops = nl * 2.0 * rows * ld * sum(5 * bp for bp in bps)
+    # the 4B = 256 rotated scenes are the rows of two 128-row blocks against 256 image pixels at a
+    # time: five products (hi with three parts of x, lo with two) over every (pixel, column) of A
+    tc_flops = nl * 2.0 * (-(-rows // 256) * 256) * ld * 5 * (-(-4 * B // 128) * 128)
     # the method's own work on this storage: every stored column against the 4B rotated scenes
     method_flops = nl * 2.0 * w.M * kst * 4 * B
     bf16_peak = _peaks()["bf16"]
@@ -821,16 +819,16 @@ def _path_split_sym(dev, stream, hbm, with_oracle):
            "method_gmac_per_s": method_flops / 2 / (ms / 1e3) / 1e9,
            "roofline": {"bound": "tensor", "achieved": method_flops / (ms / 1e3) / 1e12, "peak": bf16_peak,
                         "unit": "TFLOP/s", "frac": method_flops / (ms / 1e3) / 1e12 / bf16_peak,
-                        "kernel": "gather + tc_gemm_kernel (the 256 rotated scenes as 4 interleaved jobs against "
+                        "kernel": "gather + tc_wide_kernel (the 256 rotated scenes as two blocks of 128 rows against "
                                   "the compact A) + turned sum",
                         "numerator": "the method's MACs x 2: rows x stored columns x 4 rotations x scenes",
                         "issued_tflops": tc_flops / (ms / 1e3) / 1e12,
                         "issued_frac": tc_flops / (ms / 1e3) / 1e12 / bf16_peak,
                         "issued_note": "the tensor pipe issues 5 bf16 products per MAC for the 2^-17 split "
-                                       "precision (hi x 3 parts of x, lo x 2) on scene counts padded to 16, so "
+                                       "precision (hi x 3 parts of x, lo x 2) on scene counts padded to 128, so "
                                        "it is busy at issued_frac while the method's own work is frac; A "
                                        f"({4 * rows * ld / 1e9:.2f} GB per wavelength) is read from HBM once per "
-                                       "wavelength and served from L2 to the other jobs"},
+                                       "wavelength and served from L2 to the other block"},
            "status": plans[0].sync_status()}
     if with_oracle:
         per = []
@@ -877,7 +875,7 @@ def _path_bf16(dev, stream, hbm, with_oracle):
                        "storage, 8 x A 65536^2 (69 GB) in one launch",
            "images_per_s": nl * B / (ms / 1e3), "ms_per_batch": ms, "build_ms_per_wavelength": build_ms,
            "build_roofline": _build_roofline(2 * w.M * w.K, build_ms, hbm),
-           "gmac_per_s": nl * B * w.M * w.K / (ms / 1e3) / 1e9,
+           "gmac_per_s": nl * B * w.M * live / (ms / 1e3) / 1e9,
            "roofline": {"bound": "hbm", "achieved": a_bytes / (ms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
                         "frac": a_bytes / (ms / 1e3) / 1e9 / hbm,
                         "kernel": "tc_gemm_kernel, 8 jobs, one MMA (N = 2 x 64) per k-step (+ split, reduce)",
@@ -1142,6 +1140,14 @@ def _profile_case(name: str) -> None:
         for _ in range(3):
             plan.forward(x)
             plan.adjoint(g)
+    elif name == "fp32_batch128":
+        w = workloads.adjoint_128()
+        plan = Plan(torch.from_numpy(w.library().astype(np.float32)).to(dev), w.radii, w.s, N=w.N, S=w.S)
+        X = torch.rand(11, w.K, device=dev)
+        g = torch.rand(8, w.M, device=dev)
+        for _ in range(3):
+            plan.forward(X)
+            plan.adjoint(g)
     elif name == "sparse128":
         from synth import scenes
         w = workloads.adjoint_128()
@@ -1198,7 +1204,7 @@ def main():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--main-only", action="store_true", help="skip the other workloads' measurements")
     ap.add_argument("--case", default=None,
-                    help="run one small profiling case (fp32_128, fit128, sym128, sparse128, splitsym128, tc128, "
+                    help="run one small profiling case (fp32_128, fp32_batch128, fit128, sym128, sparse128, splitsym128, tc128, "
                          "bf16_128, fused512, builds)")
     args = ap.parse_args()
     if args.case:

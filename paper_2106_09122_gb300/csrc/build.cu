@@ -451,7 +451,7 @@ __device__ __forceinline__ void build_block_sym(int n, const ColGeom &g, const T
 // instead of eight, at a row pitch where a rotated line of 32 taps meets few bank
 // conflicts, and half the passes through shared memory for the copies: 1156 ->
 // 960 us for the paper's 16384 x 65536 A (4.5 TB/s written; no pipe is the bound
-// alone: issue 55 %, L1 data pipe 55 %, with 16 warps an SM in shared memory's
+// alone: issue 55 %, L1 data pipe 58 %, with 16 warps an SM in shared memory's
 // reach).  32 warps of 16-row blocks, whose turned rows are 64 bytes: 1040 us.
 template <bool kLerped>
 __global__ void __launch_bounds__(512, 1) build_fp32_sym_kernel(const BuildParams P) {

@@ -530,7 +530,8 @@ __device__ __forceinline__ void store_one(const PixParams &P, uint32_t w, int64_
 // thread interleaves the two halves of the work: while the footprints of the
 // next pixels' columns are on their way it stores runs of the current pixels.
 // 3.36 ms for one 256^2 wavelength (17.2 GB, 5.1 TB/s; block-wise 11.6 ms); what
-// is left above the stores is the L1 data pipe (70 %) and issue (59 %).
+// is left above the stores is L1 (71 % busy, its data pipe 67 %) and issue (58 %;
+// counters of 128^2 images on 256^2 pixels).
 // Apart, the halves take 1.5 ms (generation) and 2.6 ms (stores, the HBM floor)
 // at 256^2, and alternating them, by phases of one CTA or by two CTAs an SM,
 // takes their sum: a burst of stores fills the SM's request queue and the other

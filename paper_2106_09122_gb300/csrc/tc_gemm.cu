@@ -208,11 +208,15 @@ __global__ void __launch_bounds__(256) tc_reduce_kernel(const __grid_constant__ 
 // scene b / 4 (compact storage).  Threads beyond the compact columns serve the
 // columns in no tile: zero.  A residual value that is not finite gives NaN in
 // its split parts; such a column is summed again from the stored elements, as
-// the plain product would, so that infinities come out as they always did.
+// the plain product would, so that infinities come out as they always did.  So is
+// a sum below M 2^-108, which a column has where it meets only values below 2^-108
+// (M rows of elements up to 1): the lesser bf16 parts of still smaller ones are
+// subnormal and have lost bits (residuals of 2^-112 err 1.7e-6, of 2^-120 2.5e-5).
 struct AdjFinish {
   const float *part[kMaxJobs];
   int cap[kMaxJobs];
   int KS, n, N;
+  long long R2;        // dense grid: live pixels are within it (live.cuh); else -1
   int64_t rows, width, dead_groups, K, Kv, M, ld;  // width: compact columns
   const int *ktab, *order;
   const float *scale;
@@ -253,11 +257,34 @@ __global__ void __launch_bounds__(256) adj_finish_kernel(const __grid_constant__
     for (int ks = 0; ks < P.KS; ++ks) s += part[ks * step + at];
     return s;
   };
-  if (t < P.width) {
-    const int64_t j = P.ktab ? P.ktab[t / BK] + t % BK : t;
-    if (j >= P.Kv) return;
-    float s = sum(t);
-    if (s != s) s = plain_adjoint(P, b, j);
+  const int64_t j = t >= P.width ? P.Kv : P.ktab ? P.ktab[t / BK] + t % BK : t;
+  const bool column = j < P.Kv;
+  float s = column ? sum(t) : 0.f;
+  // A sum of zero that is not a dead column's (the k-tiles hold some): zero it is
+  // where the residual has a larger value, which the CTA looks for.
+  bool again = s != s || (column && s != 0.f && fabsf(s) < (float)P.M * 0x1p-108f);
+  bool zero = column && s == 0.f;
+  if (zero && P.R2 >= 0) {
+    const long long X = 2 * (j % P.N) - (P.N - 1), Y = 2 * (j / P.N) - (P.N - 1);
+    zero = X * X + Y * Y <= P.R2;
+  }
+  if (__syncthreads_or(zero)) {
+    const float *g = P.g + (int64_t)(P.order ? b >> 2 : b) * P.M;
+    bool some = false, large = false;
+    for (int64_t i0 = 0; !large && i0 < P.M; i0 += 4 * 256) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int64_t i = i0 + 256 * u + threadIdx.x;
+        const float v = i < P.M ? fabsf(g[i]) : 0.f;
+        some = some || v != 0.f;
+        large = large || v >= 0x1p-108f;
+      }
+      large = __syncthreads_or(large);
+    }
+    if (!large && __syncthreads_or(some)) again = again || zero;
+  }
+  if (column) {
+    if (again) s = plain_adjoint(P, b, j);
     s *= P.scale[j];
     if (P.order) {
       const int H = P.N / 2, j0 = P.order[j];
@@ -271,11 +298,11 @@ __global__ void __launch_bounds__(256) adj_finish_kernel(const __grid_constant__
     } else {
       P.gx[(int64_t)b * P.K + j] = s;
     }
-  } else if (t - P.width < P.dead_groups * kLiveGroup) {
-    const int64_t e = t - P.width, j = (int64_t)P.ktab[P.width / BK + e / kLiveGroup] * kLiveGroup + e % kLiveGroup;
-    if (j >= P.Kv) return;
-    const float s = sum(0);
-    P.gx[(int64_t)b * P.K + j] = s != s ? plain_adjoint(P, b, j) * P.scale[j] : 0.f;
+  } else if (t >= P.width && t - P.width < P.dead_groups * kLiveGroup) {
+    const int64_t e = t - P.width, jd = (int64_t)P.ktab[P.width / BK + e / kLiveGroup] * kLiveGroup + e % kLiveGroup;
+    if (jd >= P.Kv) return;
+    const float s0 = sum(0);
+    P.gx[(int64_t)b * P.K + jd] = s0 != s0 ? plain_adjoint(P, b, jd) * P.scale[jd] : 0.f;
   }
 }
 
@@ -1305,6 +1332,7 @@ cudaError_t psfsim_launch_adjoint_tc(const psfsim_plan *h, const float *g, int B
     F.KS = mp.jp[0].KS;
     F.n = h->n;
     F.N = h->N;
+    F.R2 = h->N > 0 && !h->quadrant ? live_r2(h->radii[h->n_r - 1], h->S) : -1;
     F.rows = mp.jp[0].rows;
     F.width = (int64_t)h->k_tiles * BK;
     F.dead_groups = h->dead_groups;

@@ -269,3 +269,23 @@ def test_plan_holds_no_large_tables_and_builds_without_memory_for_them(n, N, n_r
     monkeypatch.undo()
     assert refused and small.workspace.numel() == least.value
     assert torch.equal(small.workspace[:end], plan.workspace[:end]) and small.sync_status() == 0
+
+
+@pytest.mark.parametrize("storage,B", [("split_bf16", 1), ("split_bf16", 9), ("bf16", 3), ("split_bf16_sym", 2)])
+@pytest.mark.parametrize("power", [-99, -101, -112, -120, -124])
+def test_adjoint_of_very_small_residuals(storage, B, power):
+    """Residuals near the bottom of float32's normal range, whose lesser bf16 parts are subnormal: each
+    result as exact as for ordinary ones; one residual of ordinary size, one with a few ordinary values
+    far from its start, and one of zeros beside them."""
+    plan, A, rng = _plan(64, 0.25, 4.0, storage, n=33)
+    g = rng.standard_normal((B, 33 * 33)).astype(np.float32)
+    g *= np.float32(2.0) ** np.float32(power)
+    if B >= 9:
+        g[3] = rng.standard_normal(33 * 33)
+        g[5, -7:] = 1.0
+        g[7] = 0.0
+    gx = plan.adjoint(torch.from_numpy(g).to(DEV)).double().cpu().numpy()
+    g64 = g.astype(np.float64)
+    err = O.bound_relative_error(gx, g64 @ A, np.abs(g64) @ np.abs(A), floor=O.FLT_MIN).max()
+    assert err <= ADJOINT_TOL[storage] and plan.sync_status() == 0, err
+    assert np.all(gx[:, ~A.any(axis=0)] == 0.0)

@@ -228,6 +228,77 @@ __global__ void __launch_bounds__(kAdjThreads) adj_kernel(const AdjCols P, int b
   for (int64_t e = d0 + threadIdx.x; e < d1; e += kAdjThreads) gx[P.dead[e]] = bad ? __int_as_float(0x7fffffff) : 0.f;
 }
 
+// 2, 4 or 8 residuals and few columns: a CTA per column, the threads splitting the
+// rows, every residual read from L2 once per column.  Where the batched kernel below
+// has a CTA for two columns, its tiles of rows come one after another and that is what
+// it takes.  8 residuals, this form / batched: 128^2 on 452 columns 14 / 21 us, on 608
+// 15 / 21, 640 26 / 28, 1000 29 / 29; 160^2 on 452 21 / 32; a call of 64 on 64^2, 452
+// columns 50 / 66.  A thread adds 16 products by themselves before its sum (the same
+// time; 64 registers, four CTAs an SM).
+template <int BB, bool kVec>
+__global__ void __launch_bounds__(kAdjThreads) adj_few_kernel(const AdjCols P, int b0) {
+  __shared__ float red[2][kAdjThreads / 32][BB];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t t0 = P.L * blockIdx.x / gridDim.x, t1 = P.L * (blockIdx.x + 1) / gridDim.x;
+  const float *g = P.g + (int64_t)b0 * P.M;
+  int parity = 0;
+  for (int64_t t = t0; t < t1; ++t, parity ^= 1) {
+    const int64_t j = P.live ? P.live[t] : t;
+    const float *col = P.A + j * P.ld;
+    float acc[BB];
+#pragma unroll
+    for (int b = 0; b < BB; ++b) acc[b] = 0.f;
+    if (kVec) {
+      const int64_t M4 = P.M >> 2;
+      int64_t i4 = threadIdx.x;
+      constexpr int T = kAdjThreads;
+      auto add = [&](const float4 &v, int64_t at, float (&s)[BB]) {
+#pragma unroll
+        for (int b = 0; b < BB; ++b) {
+          const float4 gv = __ldg(reinterpret_cast<const float4 *>(g + (int64_t)b * P.M) + at);
+          s[b] = fmaf(v.x, gv.x, s[b]);
+          s[b] = fmaf(v.y, gv.y, s[b]);
+          s[b] = fmaf(v.z, gv.z, s[b]);
+          s[b] = fmaf(v.w, gv.w, s[b]);
+        }
+      };
+      for (; i4 + 3 * T < M4; i4 += 4 * T) {
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = ld_stream4(col + 4 * (i4 + T * u));
+        float s[BB];
+#pragma unroll
+        for (int b = 0; b < BB; ++b) s[b] = 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) add(v[u], i4 + T * u, s);
+#pragma unroll
+        for (int b = 0; b < BB; ++b) acc[b] += s[b];
+      }
+      for (; i4 < M4; i4 += T) add(ld_stream4(col + 4 * i4), i4, acc);
+    } else {
+      for (int64_t i = threadIdx.x; i < P.M; i += kAdjThreads) {
+        const float v = __ldg(col + i);
+#pragma unroll
+        for (int b = 0; b < BB; ++b) acc[b] = fmaf(v, __ldg(g + (int64_t)b * P.M + i), acc[b]);
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < BB; ++b) {
+      float s = acc[b];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) red[parity][warp][b] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x < BB) {
+      float s = red[parity][0][threadIdx.x];
+#pragma unroll
+      for (int w = 1; w < kAdjThreads / 32; ++w) s += red[parity][w][threadIdx.x];
+      P.gx[(int64_t)(b0 + threadIdx.x) * P.K + j] = s;
+    }
+  }
+}
+
 // Several residuals: a CTA owns a contiguous range of the live columns (at most
 // kAdjCols at a time) and walks the rows in tiles of 2048, eight rows a thread,
 // with the tile's BB residuals in registers, two columns in hand at once.  Their
@@ -443,27 +514,41 @@ cudaError_t psfsim_launch_gemv_partials(const FwdCols &P, int max_splits, int nu
   return cudaSuccess;
 }
 
-// One residual at a time, or passes of 2 to 8.
+// One residual at a time, or passes of 2 to 8.  The form for few columns takes those of
+// a compact plan or of field points (dense grids also have their dead columns to fill,
+// for which every CTA would look through the residuals) where each has a CTA resident
+// at once, four an SM.  Passes of 2 and 4 also between 6 and 8 columns an SM, two rounds
+// of it where the batched form's CTAs, three an SM, have more than a pair each: 4
+// residuals of 128^2 on 1000 columns 20 / 25 us, 160^2 on 1200 30 / 38; between 4 and 6
+// both take the same.  Passes of 3, 5, 6 or 7 never do: that form would make two of them.
 cudaError_t psfsim_launch_adjoint_cols(const AdjCols &P, int num_sms, cudaStream_t st) {
-  if (P.B == 1) {
-    const bool vec = (P.M % 4 == 0) && ((reinterpret_cast<uintptr_t>(P.g) & 15) == 0);
-    auto kern = vec ? adj_kernel<true> : adj_kernel<false>;
-    int per_sm = 1;
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kAdjThreads, 0);
-    if (e != cudaSuccess) return e;
-    int64_t grid = (int64_t)num_sms * (per_sm < 1 ? 1 : per_sm);
-    grid = grid < P.L ? grid : P.L;
-    kern<<<(unsigned)(grid < 1 ? 1 : grid), kAdjThreads, 0, st>>>(P, 0);
-    return cudaGetLastError();
-  }
-  const int passes = (P.B + 7) / 8, per = (P.B + passes - 1) / passes;
-  for (int b0 = 0; b0 < P.B; b0 += per) {
-    const int nb = P.B - b0 < per ? P.B - b0 : per;
-    const int per_sm = adj_min_ctas(nb <= 4 ? 4 : 8);
-    auto kern = nb <= 4 ? adj_batch_kernel<4> : adj_batch_kernel<8>;
-    int64_t grid = (P.L + 1) / 2;
-    grid = grid < (int64_t)per_sm * num_sms ? grid : (int64_t)per_sm * num_sms;
-    kern<<<(unsigned)(grid < 1 ? 1 : grid), kAdjThreads, 0, st>>>(P, b0, nb);
+  const bool vec = (P.M % 4 == 0) && ((reinterpret_cast<uintptr_t>(P.g) & 15) == 0);
+  auto grid_of = [](int64_t n) { return (unsigned)(n < 1 ? 1 : n); };
+  for (int b0 = 0, nb; b0 < P.B; b0 += nb) {
+    const int left = P.B - b0;
+    if (left == 1) {
+      nb = 1;
+      auto kern = vec ? adj_kernel<true> : adj_kernel<false>;
+      int per_sm = 1;
+      const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kAdjThreads, 0);
+      if (e != cudaSuccess) return e;
+      const int64_t grid = (int64_t)num_sms * (per_sm < 1 ? 1 : per_sm);
+      kern<<<grid_of(grid < P.L ? grid : P.L), kAdjThreads, 0, st>>>(P, b0);
+    } else if (!P.dead && (left >= 8 || left == 4 || left == 2) &&
+               (P.L <= 4ll * num_sms || (left < 8 && P.L > 6ll * num_sms && P.L <= 8ll * num_sms))) {
+      nb = left >= 8 ? 8 : left;
+      auto kern = nb == 8   ? (vec ? adj_few_kernel<8, true> : adj_few_kernel<8, false>)
+                  : nb == 4 ? (vec ? adj_few_kernel<4, true> : adj_few_kernel<4, false>)
+                            : (vec ? adj_few_kernel<2, true> : adj_few_kernel<2, false>);
+      kern<<<grid_of(P.L), kAdjThreads, 0, st>>>(P, b0);
+    } else {
+      const int passes = (left + 7) / 8;
+      nb = (left + passes - 1) / passes;
+      const int per_sm = adj_min_ctas(nb <= 4 ? 4 : 8);
+      auto kern = nb <= 4 ? adj_batch_kernel<4> : adj_batch_kernel<8>;
+      const int64_t grid = (P.L + 1) / 2, most = (int64_t)per_sm * num_sms;
+      kern<<<grid_of(grid < most ? grid : most), kAdjThreads, 0, st>>>(P, b0, nb);
+    }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

@@ -289,3 +289,27 @@ def test_adjoint_of_very_small_residuals(storage, B, power):
     err = O.bound_relative_error(gx, g64 @ A, np.abs(g64) @ np.abs(A), floor=O.FLT_MIN).max()
     assert err <= ADJOINT_TOL[storage] and plan.sync_status() == 0, err
     assert np.all(gx[:, ~A.any(axis=0)] == 0.0)
+
+
+@pytest.mark.parametrize("storage,n,N,r_last", [("fp32", 17, 20, 4.0), ("fp32", 40, 24, 30.0), ("fp32", 33, 30, 30.0),
+                                                ("fp32", 64, 36, 30.0), ("fp32_sym", 41, 24, 4.0), ("fp32_sym", 32, 48, 30.0),
+                                                ("fp32_sym", 24, 52, 30.0), ("fp32_sym", 20, 66, 30.0), ("fp32_sym", 21, 72, 30.0)])
+def test_adjoint_of_few_columns(storage, n, N, r_last):
+    """Passes of 8, 4 and 2 residuals on few columns (up to 608 and 1216 of them on 152 SMs, between and
+    above), the remainders that take the batched form, odd images, residuals at any 4-byte address; a
+    dense grid with and without dead columns, and infinities."""
+    plan, A, rng = _plan(N, 8.0 / N, r_last, storage, n=n)
+    for B in (1, 2, 3, 4, 7, 8, 9, 10, 12, 15, 16, 18):
+        big = torch.from_numpy(rng.standard_normal(B * n * n + 1).astype(np.float32)).to(DEV)
+        for shift in (0, 1):
+            g = big[shift:shift + B * n * n].view(B, n * n)
+            gx = plan.adjoint(g).double().cpu().numpy()
+            g64 = g.double().cpu().numpy()
+            err = O.bound_relative_error(gx, g64 @ A, np.abs(g64) @ np.abs(A), floor=O.FLT_MIN).max()
+            assert err <= 1e-5 and plan.sync_status() == 0, (B, shift, err)
+            assert np.all(gx[:, ~A.any(axis=0)] == 0.0)
+    if storage == "fp32":
+        g = big[:8 * n * n].view(8, n * n).clone()
+        g[5, 3] = float("inf")
+        gx = plan.adjoint(g).cpu().numpy()
+        assert np.isfinite(gx[[0, 1, 2, 3, 4, 6, 7]]).all() and not np.isfinite(gx[5][A[3] == 0.0]).any()

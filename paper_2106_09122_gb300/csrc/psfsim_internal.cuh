@@ -111,6 +111,10 @@ cudaError_t psfsim_launch_sym_sum(SymSum S, int B, float *y, cudaStream_t st);
 size_t psfsim_adjoint_tc_scratch(const psfsim_plan *h, int B);  // compact storage: of B turned residuals
 cudaError_t psfsim_launch_adjoint_tc(const psfsim_plan *h, const float *g, int B, float *gx, void *scratch,
                                      size_t scratch_bytes, cudaStream_t st);
+// ... of one residual where (nearly) every column is read, on CUDA cores (split_adjoint.cu).
+bool psfsim_adjoint_one_better(const psfsim_plan *h);
+size_t psfsim_adjoint_one_scratch(const psfsim_plan *h);
+cudaError_t psfsim_launch_adjoint_one(const psfsim_plan *h, const float *g, float *gx, void *scratch, cudaStream_t st);
 // Test hook: a tensor-core forward of one job, or of the wide form, on one CTA with
 // every wait bounded by wait_ns and load number stall_it never issued.
 bool psfsim_forward_tc_one_launch(const psfsim_plan *h, int B);

@@ -17,7 +17,8 @@
 // D[:, 0:2Bp] += hi * [x1 x2]^T, so the result carries the 2^-8 relative
 // storage error of hi and the dropped hi * x3 term (< 2^-16 relative).
 //
-// The adjoint A^T g of the same storages is the same kernel with A's tiles
+// The adjoint A^T g of the same storages (but of one residual where nearly all columns
+// are read: split_adjoint.cu) is the same kernel with A's tiles
 // transposed: an M-tile is 128 columns (two 64-column k-tiles of the forward,
 // live ones only), the contraction runs over the image rows 64 at a time, A's
 // tiles arrive as two M-major boxes of 64 columns x 64 rows, and the residuals
@@ -1166,7 +1167,8 @@ namespace {
 // One launch of a product of `count` scenes or, adjoint, residuals (compact storage:
 // turned ones).  What sizes the scratch and what runs are this same plan.
 struct Launch {
-  bool wide;
+  bool wide;  // forward: scenes as the product's rows
+  bool one;   // adjoint: one residual on CUDA cores
   int nj;
   JobSpec js[kMaxJobs];
   MultiPlan multi;
@@ -1177,8 +1179,11 @@ struct Launch {
 Launch plan_launch(const psfsim_plan *h, int count, bool adjoint) {
   Launch L;
   L.wide = !adjoint && wide_form(h, count);
+  L.one = adjoint && count == 1 && psfsim_adjoint_one_better(h);
   L.nj = 0;
-  if (L.wide) {
+  if (L.one) {
+    L.scratch = psfsim_adjoint_one_scratch(h);
+  } else if (L.wide) {
     L.w = plan_wide(h, count);
     L.scratch = L.w.scratch;
   } else {
@@ -1228,6 +1233,7 @@ int psfsim_tc_run(const psfsim_plan *h, int B, bool adjoint) {
   int most = 0;
   for (int i = 0, c; (c = launch_count(B, i)) > 0; ++i) {
     const Launch L = plan_launch(h, c, adjoint);
+    if (L.one) continue;
     const int k = L.wide ? L.w.k_tiles : L.multi.jp[0].k_tiles, ks = L.wide ? L.w.KS : L.multi.jp[0].KS;
     const int run = (k + ks - 1) / ks;
     most = run > most ? run : most;
@@ -1319,6 +1325,11 @@ cudaError_t psfsim_launch_adjoint_tc(const psfsim_plan *h, const float *g, int B
     const MultiPlan &mp = L.multi;
     const int64_t b0 = (int64_t)i * (kMaxLaunchScenes / turns);
     const float *gb = g + b0 * h->M;
+    if (L.one) {
+      const cudaError_t e = psfsim_launch_adjoint_one(h, gb, gx + b0 * h->K, scratch, st);
+      if (e != cudaSuccess) return e;
+      continue;
+    }
     for (int j = 0; j < L.nj; ++j) L.js[j].x = h->quadrant ? gb : gb + (int64_t)j * kMaxBp * h->M;
     cudaError_t e = launch_multi(L.js, L.nj, mp, scratch, st, kNoStall, true);
     if (e != cudaSuccess) return e;

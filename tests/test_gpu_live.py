@@ -313,3 +313,25 @@ def test_adjoint_of_few_columns(storage, n, N, r_last):
         g[5, 3] = float("inf")
         gx = plan.adjoint(g).cpu().numpy()
         assert np.isfinite(gx[[0, 1, 2, 3, 4, 6, 7]]).all() and not np.isfinite(gx[5][A[3] == 0.0]).any()
+
+
+@pytest.mark.parametrize("storage", ["split_bf16", "bf16"])
+@pytest.mark.parametrize("n,N,r_last", [(17, 91, 30.0), (16, 128, 12.0), (33, 96, 30.0), (24, 90, 30.0)])
+def test_adjoint_of_one_residual_where_nearly_all_columns_are_read(storage, n, N, r_last):
+    """One residual on CUDA cores (from 8192 columns on) and, below, on the tensor cores: odd images and
+    grids, column counts off the 8 of a thread; the same residual in a batch; infinities; small values."""
+    plan, A, rng = _plan(N, 8.0 / N, r_last, storage, n=n)
+    g = rng.standard_normal((2, n * n)).astype(np.float32)
+    for x in (g, np.float32(2.0 ** -120) * g):
+        x64 = x.astype(np.float64)
+        one = plan.adjoint(torch.from_numpy(x[0]).to(DEV)).double().cpu().numpy()
+        two = plan.adjoint(torch.from_numpy(x).to(DEV)).double().cpu().numpy()
+        for y, r in ((one[None], x64[:1]), (two, x64)):
+            err = O.bound_relative_error(y, r @ A, np.abs(r) @ np.abs(A), floor=O.FLT_MIN).max()
+            assert err <= ADJOINT_TOL[storage] and plan.sync_status() == 0, err
+        assert np.all(one[~A.any(axis=0)] == 0.0)
+    g[0, 5] = -np.inf
+    y = plan.adjoint(torch.from_numpy(g[0]).to(DEV)).cpu().numpy()
+    with np.errstate(invalid="ignore"):
+        want = np.where(A[5] == 0.0, np.nan, -np.inf)
+    assert np.array_equal(y, want.astype(np.float32), equal_nan=True)

@@ -21,6 +21,10 @@ int check_radii(const double *r, int n_r) {
   return PSFSIM_OK;
 }
 
+int product_status(cudaError_t e) {
+  return e == cudaSuccess ? PSFSIM_OK : e == kScratchTooSmall ? PSFSIM_ERR_WORKSPACE : PSFSIM_ERR_CUDA;
+}
+
 bool storage_ok(int storage) {
   return storage == PSFSIM_FP32 || storage == PSFSIM_SPLIT_BF16 || storage == PSFSIM_BF16 ||
          storage == PSFSIM_FP32_SYM || storage == PSFSIM_FUSED || storage == PSFSIM_SPLIT_BF16_SYM;
@@ -244,10 +248,8 @@ int psfsim_forward(psfsim_t h, const float *d_x, int B, float *d_y, void *d_scra
                                                                                     : PSFSIM_ERR_CUDA;
   }
   if (h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16) {
-    const size_t need = psfsim_tc_taken(h, B, false);
-    if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
-    return psfsim_launch_forward_tc(h, d_x, B, d_y, d_scratch, scratch_bytes, st) == cudaSuccess ? PSFSIM_OK
-                                                                                                 : PSFSIM_ERR_CUDA;
+    if (!d_scratch || !aligned(d_scratch, 256)) return PSFSIM_ERR_WORKSPACE;
+    return product_status(psfsim_launch_forward_tc(h, d_x, B, d_y, d_scratch, scratch_bytes, st));
   }
   if (h->storage == PSFSIM_FP32_SYM) {
     const size_t need = psfsim_forward_sym_scratch(h, B);
@@ -255,11 +257,8 @@ int psfsim_forward(psfsim_t h, const float *d_x, int B, float *d_y, void *d_scra
     return psfsim_launch_forward_sym(h, d_x, B, d_y, d_scratch, st) == cudaSuccess ? PSFSIM_OK : PSFSIM_ERR_CUDA;
   }
   if (h->storage == PSFSIM_SPLIT_BF16_SYM) {
-    const size_t need = psfsim_tc_taken(h, 4 * B, false);
-    if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
-    return psfsim_launch_forward_split_sym(h, d_x, B, d_y, d_scratch, scratch_bytes, st) == cudaSuccess
-               ? PSFSIM_OK
-               : PSFSIM_ERR_CUDA;
+    if (!d_scratch || !aligned(d_scratch, 256)) return PSFSIM_ERR_WORKSPACE;
+    return product_status(psfsim_launch_forward_split_sym(h, d_x, B, d_y, d_scratch, scratch_bytes, st));
   }
   if (h->storage == PSFSIM_FUSED) {
     const size_t need = psfsim_forward_fused_scratch(h, B);
@@ -295,10 +294,8 @@ int psfsim_adjoint(psfsim_t h, const float *d_g, int B, float *d_gx, void *d_scr
   if (h->storage == PSFSIM_FP32)
     return psfsim_launch_adjoint_fp32(h, d_g, B, d_gx, st) == cudaSuccess ? PSFSIM_OK : PSFSIM_ERR_CUDA;
   if (h->storage == PSFSIM_SPLIT_BF16 || h->storage == PSFSIM_BF16) {
-    const size_t need = psfsim_tc_taken(h, B, true);
-    if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
-    return psfsim_launch_adjoint_tc(h, d_g, B, d_gx, d_scratch, scratch_bytes, st) == cudaSuccess ? PSFSIM_OK
-                                                                                                  : PSFSIM_ERR_CUDA;
+    if (!d_scratch || !aligned(d_scratch, 256)) return PSFSIM_ERR_WORKSPACE;
+    return product_status(psfsim_launch_adjoint_tc(h, d_g, B, d_gx, d_scratch, scratch_bytes, st));
   }
   if (h->storage == PSFSIM_FP32_SYM) {
     const size_t need = psfsim_adjoint_sym_scratch(h, B);
@@ -306,10 +303,8 @@ int psfsim_adjoint(psfsim_t h, const float *d_g, int B, float *d_gx, void *d_scr
     return psfsim_launch_adjoint_sym(h, d_g, B, d_gx, d_scratch, st) == cudaSuccess ? PSFSIM_OK : PSFSIM_ERR_CUDA;
   }
   if (h->storage == PSFSIM_SPLIT_BF16_SYM) {
-    const size_t need = psfsim_tc_taken(h, 4 * B, true);
-    if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
-    return psfsim_launch_adjoint_tc(h, d_g, B, d_gx, d_scratch, scratch_bytes, st) == cudaSuccess ? PSFSIM_OK
-                                                                                                  : PSFSIM_ERR_CUDA;
+    if (!d_scratch || !aligned(d_scratch, 256)) return PSFSIM_ERR_WORKSPACE;
+    return product_status(psfsim_launch_adjoint_tc(h, d_g, B, d_gx, d_scratch, scratch_bytes, st));
   }
   return PSFSIM_ERR_UNSUPPORTED;
 }
@@ -325,11 +320,9 @@ int psfsim_forward_multi_scratch_bytes(const psfsim_job_t *jobs, int njobs, cons
 int psfsim_forward_multi(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tuning, void *d_scratch,
                          size_t scratch_bytes, void *stream) {
   if (int rc = psfsim_multi_validate(jobs, njobs)) return rc;
-  if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < psfsim_forward_multi_taken(jobs, njobs, tuning))
-    return PSFSIM_ERR_WORKSPACE;
-  return psfsim_launch_forward_multi(jobs, njobs, tuning, d_scratch, static_cast<cudaStream_t>(stream)) == cudaSuccess
-             ? PSFSIM_OK
-             : PSFSIM_ERR_CUDA;
+  if (!d_scratch || !aligned(d_scratch, 256)) return PSFSIM_ERR_WORKSPACE;
+  return product_status(psfsim_launch_forward_multi(jobs, njobs, tuning, d_scratch, scratch_bytes,
+                                                    static_cast<cudaStream_t>(stream)));
 }
 
 int psfsim_sync_status(psfsim_t h, void *stream) {
@@ -363,12 +356,9 @@ int psfsim_debug_forward_stall(psfsim_t h, const float *d_x, int B, float *d_y, 
   }
   if (h->storage != PSFSIM_SPLIT_BF16 && h->storage != PSFSIM_BF16) return PSFSIM_ERR_UNSUPPORTED;
   if (!psfsim_forward_tc_one_launch(h, B)) return PSFSIM_ERR_ARG;
-  const size_t need = psfsim_tc_taken(h, B, false);
-  if (!d_scratch || !aligned(d_scratch, 256) || scratch_bytes < need) return PSFSIM_ERR_WORKSPACE;
-  return psfsim_launch_forward_tc_stall(h, d_x, B, d_y, d_scratch, scratch_bytes, wait_ns, stall_load,
-                                        static_cast<cudaStream_t>(stream)) == cudaSuccess
-             ? PSFSIM_OK
-             : PSFSIM_ERR_CUDA;
+  if (!d_scratch || !aligned(d_scratch, 256)) return PSFSIM_ERR_WORKSPACE;
+  return product_status(psfsim_launch_forward_tc_stall(h, d_x, B, d_y, d_scratch, scratch_bytes, wait_ns, stall_load,
+                                                       static_cast<cudaStream_t>(stream)));
 }
 
 int psfsim_debug_scratch(const double *h_radii, int n_r, int n, int N, double S, int storage, int num_sms,

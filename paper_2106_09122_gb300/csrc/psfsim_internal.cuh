@@ -88,7 +88,10 @@ cudaError_t psfsim_launch_adjoint_fp32(const psfsim_plan *h, const float *g, int
 cudaError_t psfsim_launch_reduce_partials(const float *part, int KS, int B, int64_t ld, int64_t M, float *y,
                                           cudaStream_t st);
 // Split-BF16 and BF16 storage: build, tensor-core forward and adjoint.  A product's
-// scratch is reported monotone in the batch and checked against what it takes.
+// scratch is reported monotone in the batch; the launchers check it against what
+// the call takes, before they enqueue anything (kScratchTooSmall), so that a call is
+// planned once.
+constexpr cudaError_t kScratchTooSmall = cudaErrorMemoryValueTooLarge;
 cudaError_t psfsim_launch_split_build(psfsim_plan *h, cudaStream_t st);
 size_t psfsim_forward_tc_scratch(const psfsim_plan *h, int B);  // compact storage: of B rotated scenes
 size_t psfsim_tc_taken(const psfsim_plan *h, int B, bool adjoint);  // the call's own launches
@@ -123,9 +126,8 @@ cudaError_t psfsim_launch_forward_tc_stall(const psfsim_plan *h, const float *x,
 // Multi-job persistent tensor-core forward (several split-BF16 plans, one launch).
 int psfsim_multi_validate(const psfsim_job_t *jobs, int njobs);
 size_t psfsim_forward_multi_scratch(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune);
-size_t psfsim_forward_multi_taken(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune);
 cudaError_t psfsim_launch_forward_multi(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune,
-                                        void *scratch, cudaStream_t st);
+                                        void *scratch, size_t scratch_bytes, cudaStream_t st);
 // FP32 forward products (column-major A, gemv.cu): partial images part[KS][B][ld].
 struct FwdCols {
   const float *A;

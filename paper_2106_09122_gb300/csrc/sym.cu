@@ -213,6 +213,5 @@ size_t psfsim_forward_split_sym_scratch(const psfsim_plan *h, int B) { return ps
 
 cudaError_t psfsim_launch_forward_split_sym(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
                                             size_t scratch_bytes, cudaStream_t st) {
-  if (h->K_valid == 0) return cudaMemsetAsync(y, 0, (size_t)B * h->M * 4, st);
   return psfsim_launch_forward_tc_sym(h, x, B, y, scratch, scratch_bytes, st);
 }

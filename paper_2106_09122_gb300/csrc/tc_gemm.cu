@@ -1241,11 +1241,17 @@ int psfsim_tc_run(const psfsim_plan *h, int B, bool adjoint) {
   return most;
 }
 
+// A call of several launches is refused whole: the first launch refuses by itself.
+static bool fits(const psfsim_plan *h, int total, bool adjoint, size_t scratch_bytes) {
+  return total <= kMaxLaunchScenes || psfsim_tc_taken(h, total, adjoint) <= scratch_bytes;
+}
+
 static cudaError_t launch_forward(const psfsim_plan *h, const float *x, int B, float *y, void *scratch,
                                   size_t scratch_bytes, cudaStream_t st, const StallHook &hook) {
+  if (!fits(h, B, false, scratch_bytes)) return kScratchTooSmall;
   for (int i = 0, c; (c = launch_count(B, i)) > 0; ++i) {
     Launch L = plan_launch(h, c, false);
-    if (L.scratch > scratch_bytes) return cudaErrorInvalidValue;
+    if (L.scratch > scratch_bytes) return kScratchTooSmall;
     const float *xb = x + (int64_t)i * kMaxLaunchScenes * h->K;
     float *yb = y + (int64_t)i * kMaxLaunchScenes * h->M;
     cudaError_t e;
@@ -1278,9 +1284,11 @@ cudaError_t psfsim_launch_forward_tc_sym(const psfsim_plan *h, const float *x, i
                                          size_t scratch_bytes, cudaStream_t st) {
   constexpr int kScenes = kMaxLaunchScenes / 4;
   static_assert(kMaxBp % 4 == 0, "a scene's rotations share a job");
+  if (!fits(h, 4 * B, false, scratch_bytes)) return kScratchTooSmall;
   for (int i = 0, c; (c = launch_count(4 * B, i)) > 0; ++i) {
     Launch L = plan_launch(h, c, false);
-    if (L.scratch > scratch_bytes) return cudaErrorInvalidValue;
+    if (L.scratch > scratch_bytes) return kScratchTooSmall;
+    if (h->K_valid == 0) return cudaMemsetAsync(y, 0, (size_t)B * h->M * 4, st);
     const float *xb = x + (int64_t)i * kScenes * h->K;
     SymSum S;
     std::memset(&S, 0, sizeof(S));
@@ -1315,13 +1323,14 @@ size_t psfsim_adjoint_tc_scratch(const psfsim_plan *h, int B) { return tc_scratc
 cudaError_t psfsim_launch_adjoint_tc(const psfsim_plan *h, const float *g, int B, float *gx, void *scratch,
                                      size_t scratch_bytes, cudaStream_t st) {
   const int turns = h->quadrant ? 4 : 1;
-  if (h->quadrant) {  // scene pixels without a column
-    const cudaError_t e = cudaMemsetAsync(gx, 0, (size_t)B * h->K * 4, st);
-    if (e != cudaSuccess || h->K_valid == 0) return e;
-  }
+  if (!fits(h, turns * B, true, scratch_bytes)) return kScratchTooSmall;
   for (int i = 0, c; (c = launch_count(turns * B, i)) > 0; ++i) {
     Launch L = plan_launch(h, c, true);
-    if (L.scratch > scratch_bytes) return cudaErrorInvalidValue;
+    if (L.scratch > scratch_bytes) return kScratchTooSmall;
+    if (h->quadrant && i == 0) {  // scene pixels without a column
+      const cudaError_t e = cudaMemsetAsync(gx, 0, (size_t)B * h->K * 4, st);
+      if (e != cudaSuccess || h->K_valid == 0) return e;
+    }
     const MultiPlan &mp = L.multi;
     const int64_t b0 = (int64_t)i * (kMaxLaunchScenes / turns);
     const float *gb = g + b0 * h->M;
@@ -1377,29 +1386,30 @@ int psfsim_multi_validate(const psfsim_job_t *jobs, int njobs) {
   return PSFSIM_OK;
 }
 
-size_t psfsim_forward_multi_taken(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune) {
-  JobSpec js[kMaxJobs];
+static MultiPlan plan_jobs(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune, JobSpec *js) {
   for (int j = 0; j < njobs; ++j) js[j] = JobSpec{jobs[j].plan, jobs[j].d_x, jobs[j].d_y, jobs[j].capacity, jobs[j].d_count, -1};
-  return plan_multi(js, njobs, tune).scratch;
+  return plan_multi(js, njobs, tune);
 }
 
 // Enough for smaller capacities too: one job's split of k depends on its capacity.
 size_t psfsim_forward_multi_scratch(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune) {
-  if (njobs > 1) return psfsim_forward_multi_taken(jobs, njobs, tune);
+  JobSpec js[kMaxJobs];
+  if (njobs > 1) return plan_jobs(jobs, njobs, tune, js).scratch;
   psfsim_job_t one = jobs[0];
   size_t most = 0;
   for (one.capacity = 1; one.capacity <= jobs[0].capacity; ++one.capacity) {
-    const size_t need = psfsim_forward_multi_taken(&one, 1, tune);
+    const size_t need = plan_jobs(&one, 1, tune, js).scratch;
     most = need > most ? need : most;
   }
   return most;
 }
 
 cudaError_t psfsim_launch_forward_multi(const psfsim_job_t *jobs, int njobs, const psfsim_tuning_t *tune,
-                                        void *scratch, cudaStream_t st) {
+                                        void *scratch, size_t scratch_bytes, cudaStream_t st) {
   JobSpec js[kMaxJobs];
-  for (int j = 0; j < njobs; ++j) js[j] = JobSpec{jobs[j].plan, jobs[j].d_x, jobs[j].d_y, jobs[j].capacity, jobs[j].d_count, -1};
-  return launch_multi(js, njobs, plan_multi(js, njobs, tune), scratch, st);
+  const MultiPlan mp = plan_jobs(jobs, njobs, tune, js);
+  if (mp.scratch > scratch_bytes) return kScratchTooSmall;
+  return launch_multi(js, njobs, mp, scratch, st);
 }
 
 bool psfsim_forward_tc_one_launch(const psfsim_plan *h, int B) {

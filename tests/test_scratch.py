@@ -137,3 +137,38 @@ def test_multi_forward_scratch_of_one_job_serves_smaller_capacities(storage, n, 
         tol = 2e-5 * ref[:cap]  # both sums of products that are not negative, split differently
         assert torch.all((y[:cap] - ref[:cap]).abs() <= tol)
     assert plan.sync_status() == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("storage", STORAGES)
+@pytest.mark.parametrize("batch", [1, 17, 90, 350, 1300])
+def test_scratch_below_what_a_call_takes_is_refused_before_anything_runs(storage, batch):
+    import torch
+    from paper_2106_09122_gb300 import Plan
+    n, N = 16, 24
+    rng = np.random.default_rng(5)
+    lib = torch.from_numpy(rng.uniform(0.0, 1.0, (5, n, n)).astype(np.float32)).cuda()
+    L, st = B.load(), torch.cuda.current_stream().cuda_stream
+    for radii in (np.linspace(0.0, 12.0, 5), np.linspace(0.0, 0.1, 5)):  # the second: no column at all
+        plan = Plan(lib, radii, 0.25, N=N, S=1.0, storage=storage)
+        x, g = torch.ones(batch, N * N, device="cuda"), torch.ones(batch, n * n, device="cuda")
+        for call, a, out, nbytes in ((L.psfsim_forward, x, torch.full_like(g, 7.0), plan.forward_scratch_bytes(batch)),
+                                     (L.psfsim_adjoint, g, torch.full_like(x, 7.0), plan.adjoint_scratch_bytes(batch))):
+            scr = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+
+            def run(size, ptr=scr.data_ptr()):
+                return call(plan.handle, a.data_ptr(), batch, out.data_ptr(), ptr, size, st)
+
+            assert run(0) == B.ERR_WORKSPACE and run(255) == B.ERR_WORKSPACE and run(nbytes, None) == B.ERR_WORKSPACE
+            assert run(nbytes, scr.data_ptr() + 16) == B.ERR_WORKSPACE
+            low, high = 255, nbytes  # the least that is accepted; everything below is refused and leaves the output alone
+            while high - low > 1:
+                mid = (low + high) // 2
+                torch.cuda.synchronize()
+                before = out.clone()
+                rc = run(mid)
+                assert rc in (B.OK, B.ERR_WORKSPACE)
+                torch.cuda.synchronize()
+                assert rc == B.OK or torch.equal(out, before)
+                low, high = (low, mid) if rc == B.OK else (mid, high)
+            assert run(high) == B.OK and plan.sync_status() == 0

@@ -671,7 +671,9 @@ cudaError_t psfsim_launch_build(psfsim_plan *h, cudaStream_t st) {
   if (const cudaError_t e2 = psfsim_launch_live_table(h, st)) return e2;  // the column order is free from here on
   // The retrieval's forward kernels read A and the column list before they wait
   // for the kernel ahead of them (programmatic launch), so that kernel must not
-  // be one that writes them: end with an operation that waits for those.
+  // be one that writes them: end with an operation that waits for those (split
+  // storages have no such reader).
+  if (h->storage != PSFSIM_FP32 && h->storage != PSFSIM_FP32_SYM) return cudaSuccess;
   return cudaMemsetAsync(h->ws + h->status_off + 8, 0, 8, st);
 }
 
